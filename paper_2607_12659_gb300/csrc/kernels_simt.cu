@@ -216,73 +216,121 @@ __global__ void __launch_bounds__(256) k_mod_gemv(const TW* __restrict__ Wm, con
 // ---------------------------------------------------------------------------------------------
 // Token embedding: row 0 of each request is the state token, rows 1..nctx-1 the correction
 // items (context tokens, taken as given), then the C action tokens.
-// Block = 128 features of one token. For the tensor-core path it also writes the operand of
-// the first layer's norm-fed projection (xs = bf16((1 + sigma) * h) at row xs_row(m), and beta in
-// the last row of tile m while m < xs_tiles) and that slice's sum of squares (ss[slice][m]).
-__global__ void __launch_bounds__(128) k_embed(
-    float* __restrict__ hres, __nv_bfloat16* __restrict__ xs, const float* __restrict__ sigma,
-    const float* __restrict__ beta, float* __restrict__ ss, int ss_ld,
-    const float* __restrict__ state,
-    const float* __restrict__ x, const float* __restrict__ Ws, const float* __restrict__ bs,
-    const float* __restrict__ Wa, const float* __restrict__ ba, const float* __restrict__ corr, int nctx,
-    int S, int C, int W, int Sd, int A) {
-    __shared__ float scratch[32];
-    const int m = blockIdx.y;
-    const int b = m / S, i = m % S;
-    const float* in = nullptr;
-    const float* Wm = nullptr;
-    const float* bias = nullptr;
-    int K = 0;
-    if (i == 0) {
-        in = state + (size_t)b * Sd; Wm = Ws; bias = bs; K = Sd;
-    } else if (i >= nctx) {
-        in = x + ((size_t)b * C + (i - nctx)) * A; Wm = Wa; bias = ba; K = A;
-    }
-    const int n = blockIdx.x * 128 + threadIdx.x;
-    // Everything but x (the previous step's actions) is ready before the dependency wait: the
-    // first EMB_K weights of this feature's row, its bias and the norm's scale and shift.
-    constexpr int EMB_K = 32;
+// Block = 128 features of up to TPB tokens that share one input matrix: blockIdx.y counts groups of
+// action tokens first, then groups of state and context tokens. A thread keeps its feature's weight
+// row in registers for all of them (its 128 bytes are a line of their own, so with one token per
+// block every token fetched 16 KB of weights per 128 features again: 382 us at 3264 tokens x 1024
+// features, bound by those reads; the outputs alone are 20 MB, 3 us) and reads the tokens' inputs
+// from shared memory as broadcasts. The sums keep the order of one token at a time.
+// For the tensor-core path it also writes the operand of the first layer's norm-fed projection
+// (xs = bf16((1 + sigma) * h) at row xs_row(m), and beta in the last row of every 64-row tile) and
+// each token's sum of squares over the 128 features (ss[slice][m]).
+struct EmbedArgs {
+    float* hres;
+    __nv_bfloat16* xs;   // null without the tensor-core path (as is ss)
+    const float *sigma, *beta;
+    float* ss;
+    int ss_ld;
+    const float *state, *x, *Ws, *bs, *Wa, *ba, *corr;
+    int nctx, B, S, C, W, Sd, A;
+    int tpb, action_groups;   // tokens per block; groups of action tokens
+};
+constexpr int EMB_MAX_TPB = 16;
+constexpr int EMB_K = 32;     // inputs per token kept in registers / shared memory
+
+__global__ void __launch_bounds__(128) k_embed(const EmbedArgs a) {
+    __shared__ __align__(16) float in_s[EMB_MAX_TPB][EMB_K];
+    __shared__ float part[EMB_MAX_TPB][4];
+    const int tid = threadIdx.x;
+    const bool act = (int)blockIdx.y < a.action_groups;
+    // Tokens [j0, j0 + nt) of this block's kind: action token j = (request j / C, action j mod C),
+    // else context token j = (request j / nctx, row j mod nctx).
+    const int per = act ? a.C : a.nctx;
+    const int j0 = (act ? blockIdx.y : blockIdx.y - a.action_groups) * a.tpb;
+    const int nt = min(a.tpb, a.B * per - j0);
+    const int K = act ? a.A : a.Sd;
+    const int Kr = min(K, EMB_K);
+    const float* Wm = act ? a.Wa : a.Ws;
+    const int n = blockIdx.x * 128 + tid;
+    const bool live = n < a.W;
+    // Everything but x (the previous step's actions) is ready before the dependency wait.
     float wv[EMB_K];
     float bv = 0.f, sg = 0.f, bt = 0.f;
-    const bool lin = n < W && !(i > 0 && i < nctx);
-    if (lin) {
+    if (live) {
+        const float* wr = Wm + (size_t)n * K;
+        if (K % 4 == 0) {
 #pragma unroll
-        for (int k = 0; k < EMB_K; ++k) wv[k] = k < K ? Wm[(size_t)n * K + k] : 0.f;
-        bv = bias[n];
-    }
-    if (n < W && xs) {
-        sg = sigma[n];
-        bt = beta[n];
+            for (int k = 0; k < EMB_K; k += 4) {
+                const float4 w4 = k < K ? __ldg(reinterpret_cast<const float4*>(wr + k)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                wv[k] = w4.x;
+                wv[k + 1] = w4.y;
+                wv[k + 2] = w4.z;
+                wv[k + 3] = w4.w;
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < EMB_K; ++k) wv[k] = k < K ? wr[k] : 0.f;
+        }
+        bv = (act ? a.ba : a.bs)[n];
+        if (a.xs) {
+            sg = a.sigma[n];
+            bt = a.beta[n];
+        }
     }
     // Launched with programmatic dependent launch: x comes from the previous step's final kernel;
     // the next kernel may start its weight prefetch at once.
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-    float v = 0.f;
-    if (n < W) {
-        if (!lin) {
-            v = corr[((size_t)b * (nctx - 1) + (i - 1)) * W + n];
-        } else {
-            // The inputs of this row loaded together, then summed in k order.
-            float acc = 0.f;
-            float iv[EMB_K];
+    // Inputs of token j: its action row, or its request's state (context rows past 0 have none).
+    auto input = [&](int j) { return act ? a.x + (size_t)j * a.A : a.state + (size_t)(j / a.nctx) * a.Sd; };
+    for (int i = tid; i < nt * EMB_K; i += 128) {
+        const int tt = i / EMB_K, k = i % EMB_K;
+        in_s[tt][k] = k < Kr ? input(j0 + tt)[k] : 0.f;
+    }
+    __syncthreads();
+    for (int tt = 0; tt < nt; ++tt) {
+        const int j = j0 + tt;
+        const int b = j / per, i = (act ? a.nctx : 0) + j - b * per;   // request, row in its suffix
+        const int m = b * a.S + i;
+        float v = 0.f;
+        if (live) {
+            if (!act && i > 0) {
+                v = a.corr[((size_t)b * (a.nctx - 1) + (i - 1)) * a.W + n];
+            } else {
+                float acc = 0.f;
+                const float4* iv = reinterpret_cast<const float4*>(in_s[tt]);
 #pragma unroll
-            for (int k = 0; k < EMB_K; ++k) iv[k] = k < K ? in[k] : 0.f;
-#pragma unroll
-            for (int k = 0; k < EMB_K; ++k)
-                if (k < K) acc = fmaf(wv[k], iv[k], acc);
-            for (int k = EMB_K; k < K; ++k) acc = fmaf(Wm[(size_t)n * K + k], in[k], acc);
-            v = acc + bv;
+                for (int k = 0; k < EMB_K; k += 4) {
+                    const float4 x4 = iv[k / 4];
+                    if (k < K) acc = fmaf(wv[k], x4.x, acc);
+                    if (k + 1 < K) acc = fmaf(wv[k + 1], x4.y, acc);
+                    if (k + 2 < K) acc = fmaf(wv[k + 2], x4.z, acc);
+                    if (k + 3 < K) acc = fmaf(wv[k + 3], x4.w, acc);
+                }
+                const float* in = input(j);
+                for (int k = EMB_K; k < K; ++k) acc = fmaf(Wm[(size_t)n * K + k], in[k], acc);
+                v = acc + bv;
+            }
+            a.hres[(size_t)m * a.W + n] = v;
+            if (a.xs) a.xs[(size_t)xs_row(m) * a.W + n] = __float2bfloat16_rn((1.f + sg) * v);
         }
-        hres[(size_t)m * W + n] = v;
-        if (xs) {
-            xs[(size_t)xs_row(m) * W + n] = __float2bfloat16_rn((1.f + sg) * v);
-            if (m < xs_tiles(gridDim.y)) xs[((size_t)m * 64 + 63) * W + n] = __float2bfloat16_rn(bt);
+        if (a.ss) {
+            const float t = warp_sum(v * v);
+            if ((tid & 31) == 0) part[tt][tid >> 5] = t;
         }
     }
-    if (ss) {
-        const float t = block_sum(v * v, scratch);
-        if (threadIdx.x == 0) ss[(size_t)blockIdx.x * ss_ld + m] = t;
+    if (a.xs && live) {
+        // Tile z's beta row: block y takes tiles y tpb .. (the blocks' token slots cover the tiles).
+        const int z0 = blockIdx.y * a.tpb, z1 = min(z0 + a.tpb, xs_tiles(a.B * a.S));
+        for (int z = z0; z < z1; ++z) a.xs[((size_t)z * 64 + 63) * a.W + n] = __float2bfloat16_rn(bt);
+    }
+    if (a.ss) {
+        __syncthreads();
+        if (tid < nt) {
+            const int j = j0 + tid, b = j / per, i = (act ? a.nctx : 0) + j - b * per;
+            a.ss[(size_t)blockIdx.x * a.ss_ld + b * a.S + i] =
+                (part[tid][0] + part[tid][2]) + (part[tid][1] + part[tid][3]);
+        }
     }
 }
 
@@ -776,14 +824,38 @@ jpi_status launch_time_conditioning_into(jpi_handle* h, double t, float* temb, f
 }
 
 jpi_status launch_embed(jpi_handle* h, int step, int B, int C, const float* x, cudaStream_t st) {
-    const int S = C + h->n_ctx();
+    const int slices = (h->W + 127) / 128, nctx = h->n_ctx();
     // Scale and shift of layer 0's attention norm at this step.
     const float* ms = h->mods + (size_t)step * mod_rows(h->L) * h->W;
-    launch_pdl(h, dim3((h->W + 127) / 128, B * S), dim3(128), 0, st, k_embed,
-               h->h, h->tc ? (__nv_bfloat16*)h->hx : nullptr, ms, ms + h->W, h->tc ? h->ss : nullptr, h->maxMt,
-               (const float*)h->state, x, (const float*)h->state_in_w, (const float*)h->state_in_b,
-               (const float*)h->action_in_w, (const float*)h->action_in_b, (const float*)h->corr, h->n_ctx(), S, C,
-               h->W, h->Sd, h->A);
+    EmbedArgs a;
+    a.hres = h->h;
+    a.xs = h->tc ? (__nv_bfloat16*)h->hx : nullptr;
+    a.sigma = ms;
+    a.beta = ms + h->W;
+    a.ss = h->tc ? h->ss : nullptr;
+    a.ss_ld = h->maxMt;
+    a.state = h->state;
+    a.x = x;
+    a.Ws = h->state_in_w;
+    a.bs = h->state_in_b;
+    a.Wa = h->action_in_w;
+    a.ba = h->action_in_b;
+    a.corr = h->corr;
+    a.nctx = nctx;
+    a.B = B;
+    a.S = C + nctx;
+    a.C = C;
+    a.W = h->W;
+    a.Sd = h->Sd;
+    a.A = h->A;
+    // About eight blocks per SM (a small batch keeps one token per block, the shortest chain), at
+    // most EMB_MAX_TPB tokens each.
+    const long long want = 8ll * h->num_sms;
+    const long long tpb = ((long long)B * a.S * slices + want - 1) / want;
+    a.tpb = (int)(tpb < 1 ? 1 : tpb > EMB_MAX_TPB ? EMB_MAX_TPB : tpb);
+    a.action_groups = (B * C + a.tpb - 1) / a.tpb;
+    const int groups = a.action_groups + (B * nctx + a.tpb - 1) / a.tpb;
+    launch_pdl(h, dim3(slices, groups), dim3(128), 0, st, k_embed, a);
     return check_launch("embed");
 }
 
