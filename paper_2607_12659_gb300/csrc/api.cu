@@ -408,13 +408,7 @@ JPI_API jpi_status jpi_set_prefix_kv(jpi_handle* h, const void* const* k_layers,
     for (int l = 0; l < h->L; ++l)
         if (!k_layers[l] || !v_layers[l]) return fail(JPI_ERR_INVALID_ARG, "layer %d K or V is NULL", l);
     cudaStream_t st = (cudaStream_t)stream;
-    const size_t layer_elems = (size_t)h->maxB * h->kv_rows * h->D;
-    for (int l = 0; l < h->L; ++l) {
-        JPI_TRY(launch_convert_kv(h, k_layers[l], kv_is_fp32, tw_offset(h, h->kv_k, l * layer_elems),
-                                  batch, prefix_len, st));
-        JPI_TRY(launch_convert_kv(h, v_layers[l], kv_is_fp32, tw_offset(h, h->kv_v, l * layer_elems),
-                                  batch, prefix_len, st));
-    }
+    JPI_TRY(launch_load_prefix(h, k_layers, v_layers, kv_is_fp32, batch, prefix_len, st));
     h->cur_batch = batch;
     h->cur_prefix = prefix_len;
     h->prefix_ready = true;

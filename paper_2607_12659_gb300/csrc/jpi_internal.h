@@ -208,8 +208,8 @@ jpi_status launch_op_simt(jpi_handle* h, int op, int layer, int step, int batch,
                           cudaStream_t st);
 jpi_status launch_final(jpi_handle* h, int step, int batch, int chunk, float delta,
                         float* x_inout, float* v_out, float* out_copy, cudaStream_t st);
-jpi_status launch_convert_kv(jpi_handle* h, const void* src, int src_fp32, void* dst,
-                             int batch, int prefix_len, cudaStream_t st);
+jpi_status launch_load_prefix(jpi_handle* h, const void* const* k_layers, const void* const* v_layers, int src_fp32,
+                              int B, int P, cudaStream_t st);
 
 // Entry-point helpers (api.cu). check_call: host-side checks of a denoise or forward call of
 // `B` requests, `C` actions and `N` steps against the handle's maxima, its prefix and its

@@ -600,15 +600,100 @@ __global__ void __launch_bounds__(FIN_THREADS) k_final(const float* __restrict__
 }
 
 // ---------------------------------------------------------------------------------------------
-// Prefix KV into the store: src [batch][P][D] (fp32 or bf16) -> dst [batch][kv_rows][D].
-template <typename TS, typename TD>
-__global__ void k_convert_kv(const TS* __restrict__ src, TD* __restrict__ dst, int P, int D,
-                             int kv_rows, long long total) {
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const long long d = idx % D, p = (idx / D) % P, b = idx / ((long long)D * P);
-        dst[((size_t)b * kv_rows + p) * D + d] = cvt<TD>(ldf(src + idx));
+// Prefix KV into the store, every layer's K and V in one launch: tensor y (K then V of layer y / 2)
+// src [batch][P][D] (fp32 or bf16) -> dst [batch][kv_rows][D]. A request's P D elements are
+// contiguous on both sides; a thread moves KV_CH chunks of 8 elements (16 bytes of bf16), all loads
+// before the stores. Bound by launches before (one kernel of 2-byte accesses per tensor: 36 launches
+// of 4.4 us each for 15 MB at 18 layers x 816 tokens); the copy alone is 30 MB of traffic, 4.4 us at
+// the copy peak. VEC: the sources are 16-byte aligned.
+constexpr int KV_CH = 4;
+constexpr int KV_MAX_TENSORS = 128;
+struct KvLoadArgs {
+    const void* src[KV_MAX_TENSORS];
+    void* dst[KV_MAX_TENSORS];
+    int B;
+    long long per;          // elements per request: P D (a multiple of 32)
+    long long dst_stride;   // elements between requests of the store
+};
+
+template <typename T> struct Chunk8;   // 8 consecutive elements
+template <> struct Chunk8<__nv_bfloat16> {
+    uint4 v;
+    __device__ __forceinline__ void load(const __nv_bfloat16* p) { v = *reinterpret_cast<const uint4*>(p); }
+    __device__ __forceinline__ void load1(const __nv_bfloat16* p) {
+        const unsigned short* u = reinterpret_cast<const unsigned short*>(p);
+        v = make_uint4(u[0] | (uint32_t)u[1] << 16, u[2] | (uint32_t)u[3] << 16, u[4] | (uint32_t)u[5] << 16,
+                       u[6] | (uint32_t)u[7] << 16);
     }
+    __device__ __forceinline__ void store(__nv_bfloat16* p) const { *reinterpret_cast<uint4*>(p) = v; }
+    __device__ __forceinline__ void store(float* p) const {
+        const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+        float f[8];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            f[2 * i] = __uint_as_float(u[i] << 16);
+            f[2 * i + 1] = __uint_as_float(u[i] & 0xFFFF0000u);
+        }
+        reinterpret_cast<float4*>(p)[0] = make_float4(f[0], f[1], f[2], f[3]);
+        reinterpret_cast<float4*>(p)[1] = make_float4(f[4], f[5], f[6], f[7]);
+    }
+};
+template <> struct Chunk8<float> {
+    float4 a, b;
+    __device__ __forceinline__ void load(const float* p) {
+        a = reinterpret_cast<const float4*>(p)[0];
+        b = reinterpret_cast<const float4*>(p)[1];
+    }
+    __device__ __forceinline__ void load1(const float* p) {
+        a = make_float4(p[0], p[1], p[2], p[3]);
+        b = make_float4(p[4], p[5], p[6], p[7]);
+    }
+    __device__ __forceinline__ static uint32_t pack(float lo, float hi) {
+        const __nv_bfloat162 t = __floats2bfloat162_rn(lo, hi);
+        return *reinterpret_cast<const uint32_t*>(&t);
+    }
+    __device__ __forceinline__ void store(__nv_bfloat16* p) const {
+        *reinterpret_cast<uint4*>(p) = make_uint4(pack(a.x, a.y), pack(a.z, a.w), pack(b.x, b.y), pack(b.z, b.w));
+    }
+    __device__ __forceinline__ void store(float* p) const {
+        reinterpret_cast<float4*>(p)[0] = a;
+        reinterpret_cast<float4*>(p)[1] = b;
+    }
+};
+
+template <typename TS, typename TD, bool VEC>
+__global__ void __launch_bounds__(256) k_load_prefix(const __grid_constant__ KvLoadArgs a) {
+    const TS* src0 = static_cast<const TS*>(a.src[blockIdx.y]);
+    TD* dst0 = static_cast<TD*>(a.dst[blockIdx.y]);
+    const long long nch = a.per / 8, step = (long long)gridDim.x * 256 * KV_CH;
+    for (int b = blockIdx.z; b < a.B; b += gridDim.z) {
+        const TS* src = src0 + b * a.per;
+        TD* dst = dst0 + b * a.dst_stride;
+        for (long long c0 = (long long)blockIdx.x * 256 * KV_CH + threadIdx.x; c0 < nch; c0 += step) {
+            Chunk8<TS> v[KV_CH];
+#pragma unroll
+            for (int u = 0; u < KV_CH; ++u) {
+                const long long c = c0 + 256 * u;
+                if (c < nch) {
+                    if (VEC) v[u].load(src + 8 * c);
+                    else v[u].load1(src + 8 * c);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < KV_CH; ++u) {
+                const long long c = c0 + 256 * u;
+                if (c < nch) v[u].store(dst + 8 * c);
+            }
+        }
+    }
+}
+
+template <typename TS, typename TD>
+void launch_load_prefix_t(const KvLoadArgs& a, int ntensors, bool vec, cudaStream_t st) {
+    const long long blocks = (a.per / 8 + 256 * KV_CH - 1) / (256 * KV_CH);
+    const dim3 grid((unsigned)(blocks < 65536 ? blocks : 65536), (unsigned)ntensors, (unsigned)(a.B < 65535 ? a.B : 65535));
+    if (vec) k_load_prefix<TS, TD, true><<<grid, 256, 0, st>>>(a);
+    else k_load_prefix<TS, TD, false><<<grid, 256, 0, st>>>(a);
 }
 
 // Launch with programmatic dependent launch when the handle uses it (the kernel waits for its
@@ -880,22 +965,36 @@ jpi_status launch_final(jpi_handle* h, int step, int B, int C, float delta, floa
     return check_launch("final norm + Euler");
 }
 
-jpi_status launch_convert_kv(jpi_handle* h, const void* src, int src_fp32, void* dst, int B,
-                             int P, cudaStream_t st) {
-    const long long total = (long long)B * P * h->D;
-    const int g = grid_for(total, 256, 8192);
-    if (h->bf16) {
-        if (src_fp32)
-            k_convert_kv<float, __nv_bfloat16><<<g, 256, 0, st>>>((const float*)src, (__nv_bfloat16*)dst, P, h->D, h->kv_rows, total);
-        else
-            k_convert_kv<__nv_bfloat16, __nv_bfloat16><<<g, 256, 0, st>>>((const __nv_bfloat16*)src, (__nv_bfloat16*)dst, P, h->D, h->kv_rows, total);
-    } else {
-        if (src_fp32)
-            k_convert_kv<float, float><<<g, 256, 0, st>>>((const float*)src, (float*)dst, P, h->D, h->kv_rows, total);
-        else
-            k_convert_kv<__nv_bfloat16, float><<<g, 256, 0, st>>>((const __nv_bfloat16*)src, (float*)dst, P, h->D, h->kv_rows, total);
+jpi_status launch_load_prefix(jpi_handle* h, const void* const* k_layers, const void* const* v_layers, int src_fp32,
+                              int B, int P, cudaStream_t st) {
+    const size_t es = h->bf16 ? 2 : 4;
+    const size_t layer_bytes = (size_t)h->maxB * h->kv_rows * h->D * es;
+    for (int l0 = 0; l0 < h->L; l0 += KV_MAX_TENSORS / 2) {
+        const int nl = h->L - l0 < KV_MAX_TENSORS / 2 ? h->L - l0 : KV_MAX_TENSORS / 2;
+        KvLoadArgs a;
+        a.B = B;
+        a.per = (long long)P * h->D;
+        a.dst_stride = (long long)h->kv_rows * h->D;
+        uintptr_t bits = 0;
+        for (int i = 0; i < nl; ++i) {
+            a.src[2 * i] = k_layers[l0 + i];
+            a.src[2 * i + 1] = v_layers[l0 + i];
+            a.dst[2 * i] = (char*)h->kv_k + (l0 + i) * layer_bytes;
+            a.dst[2 * i + 1] = (char*)h->kv_v + (l0 + i) * layer_bytes;
+            bits |= (uintptr_t)k_layers[l0 + i] | (uintptr_t)v_layers[l0 + i];
+        }
+        const bool vec = (bits & 15) == 0;
+        using bf = __nv_bfloat16;
+        if (h->bf16) {
+            if (src_fp32) launch_load_prefix_t<float, bf>(a, 2 * nl, vec, st);
+            else launch_load_prefix_t<bf, bf>(a, 2 * nl, vec, st);
+        } else {
+            if (src_fp32) launch_load_prefix_t<float, float>(a, 2 * nl, vec, st);
+            else launch_load_prefix_t<bf, float>(a, 2 * nl, vec, st);
+        }
+        JPI_TRY(check_launch("prefix KV copy"));
     }
-    return check_launch("prefix KV conversion");
+    return JPI_OK;
 }
 
 }  // namespace jpi
