@@ -161,8 +161,9 @@ struct jpi_handle {
     // Tensor-core path: one plan per projection (QKV, O, gate/up, down) and tensor maps
     // (4 per layer, same order).
     jpi::GemmPlan plans[4];
-    int big_min_tokens[4] = {512, 128, 128, 128};   // per projection kind: from this many tokens the large-M GEMM
+    int big_min_tokens[4] = {400, 128, 128, 128};   // per projection kind: from this many tokens the large-M GEMM
     int big_split = 0;          // K split of the large-M residual projections (0: chosen per launch)
+    int resid_rows = -1;        // tokens-on-rows kernel for those (-1: chosen per launch)
     int big_clusters[4] = {0, 0, 0, 0};   // co-resident large-M clusters of 1, 2, 4, 8 CTAs
     int attn_t5_min_batch = 3;  // batches of at least this many requests use the tcgen05 attention
     bool attn_t5 = false;       // its tensor maps and attributes are ready
@@ -176,7 +177,8 @@ struct jpi_handle {
     std::vector<CUtensorMap> tmaps;
     bool mod_tc = false;        // modulation vectors on tensor cores (mod_tc.cu)
     CUtensorMap mod_map;        // the stacked modulation matrix [(6L+2) W][W] as 128 x 64 boxes
-    CUtensorMap xmaps[3];       // B operands: hx, o, z
+    CUtensorMap xmaps[3];       // activation operands hx, o, z as 64-row boxes
+    CUtensorMap xmaps_rows[3];  // and as 128-row boxes
 
     // State.
     int cur_batch = 0, cur_prefix = 0;

@@ -133,6 +133,7 @@ __host__ __device__ __forceinline__ GemmSmem gemm_layout(int kpb, int splits, bo
 
 #include "gemm_kernel.cuh"
 #include "gemm_big.cuh"
+#include "gemm_rows.cuh"
 
 // ---------------------------------------------------------------------------------------------
 // Host side: packing, plans, tensor maps, launches.
@@ -301,7 +302,8 @@ int big_clusters(const jpi_handle* h, int S) {
     return h->big_clusters[i] > 0 ? h->big_clusters[i] : h->num_sms / S;
 }
 
-int big_split(const jpi_handle* h, int kind, int units, int nkb) {
+int big_split(const jpi_handle* h, int kind, int units, int nkb, long* cost_out = nullptr) {
+    if (cost_out) *cost_out = 0;
     if (kind != G_O && kind != G_DOWN) return 1;
     if (h->big_split > 0) return nkb % h->big_split == 0 ? h->big_split : 1;
     int best = 1;
@@ -315,7 +317,46 @@ int big_split(const jpi_handle* h, int kind, int units, int nkb) {
             best = S;
         }
     }
+    if (cost_out) *cost_out = best_cost;
     return best;
+}
+
+// Whether a residual projection takes the tokens-on-rows kernel (128 x 256 tiles, no K split): when
+// its waves of whole tiles, a k-block costing 5/4 of a 128 x 128 tile's (48 against 32 KB into the
+// SM, more of them in flight), cost less than the best split of the other kernel.
+bool resid_rows(const jpi_handle* h, int kind, int Mt, const GemmPlan& pl) {
+    if (h->resid_rows >= 0) return h->resid_rows != 0;
+    long other = 0;
+    big_split(h, kind, pl.ntiles * ((Mt + BIG_NT - 1) / BIG_NT), pl.nkb, &other);
+    if (other == 0) return false;   // a fixed split
+    const long tiles = (long)((pl.ntiles + 1) / 2) * ((Mt + 127) / 128);
+    const long waves = (tiles + h->num_sms - 1) / h->num_sms;
+    return waves * pl.nkb * 5 < other * 4;
+}
+
+template <int KIND>
+jpi_status launch_gemm_rows(jpi_handle* h, const GemmPlan& pl, const CUtensorMap& wmap, const CUtensorMap& xmap,
+                            const GemmArgs& a, cudaStream_t st) {
+    constexpr int TT = (KIND == G_QKV || KIND == G_GU) ? 2 * XS_TOKENS : 128;
+    const int tiles = ((pl.ntiles + 1) / 2) * std::max(1, (a.Mt + TT - 1) / TT);
+    GemmArgs ar = a;
+    ar.ntiles = pl.ntiles;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)std::min(tiles, h->num_sms));   // persistent, one CTA per SM
+    cfg.blockDim = dim3(RT_THREADS);
+    cfg.dynamicSmemBytes = RT_SMEM;
+    cfg.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = h->pdl ? 1 : 0;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_tc_gemm_rows<KIND>, wmap, xmap, ar);
+    if (e != cudaSuccess) {
+        set_error("tensor-core GEMM launch failed: %s", cudaGetErrorString(e));
+        return JPI_ERR_CUDA;
+    }
+    return JPI_OK;
 }
 
 template <int KIND, int S>
@@ -467,7 +508,9 @@ jpi_status tc_prepare(jpi_handle* h) {
         }
         JPI_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     }
-    auto big1 = {k_tc_gemm_big<G_QKV, 1>, k_tc_gemm_big<G_O, 1>, k_tc_gemm_big<G_GU, 1>, k_tc_gemm_big<G_DOWN, 1>};
+    for (auto k : {k_tc_gemm_rows<G_QKV>, k_tc_gemm_rows<G_O>, k_tc_gemm_rows<G_GU>, k_tc_gemm_rows<G_DOWN>})
+        JPI_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, RT_SMEM));
+    auto big1 = {k_tc_gemm_big<G_O, 1>, k_tc_gemm_big<G_DOWN, 1>};
     for (auto k : big1)
         JPI_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 1024 + big_smem_bytes<1>()));
     JPI_CUDA_TRY(cudaFuncSetAttribute(k_tc_gemm_big<G_O, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 1024 + big_smem_bytes<2>()));
@@ -504,9 +547,14 @@ jpi_status tc_prepare(jpi_handle* h) {
     // JPI_BIG_SPLIT=S fixes the K split of the large-M residual projections (1, 2, 4 or 8).
     const char* split_env = std::getenv("JPI_BIG_SPLIT");
     if (split_env) h->big_split = std::atoi(split_env);
-    // Launches with at least this many tokens use the large-M kernels (full K per CTA). The
-    // gate/up projection (64 weight tiles at pi0.5 sizes) fills the GPU with them from 128 tokens;
-    // the narrower ones (8-20 weight tiles) keep the K-split kernel up to 512 tokens (measured).
+    // JPI_BIG_RESID_ROWS=0 / 1 fixes the kernel of those projections (1: tokens on the MMA's rows).
+    const char* rows_env = std::getenv("JPI_BIG_RESID_ROWS");
+    if (rows_env) h->resid_rows = std::atoi(rows_env) != 0 ? 1 : 0;
+    // Launches with at least this many tokens use the large-M kernels. The gate/up projection (64
+    // weight tiles at pi0.5 sizes) fills the GPU with them from 128 tokens (165 tokens: 11.0 us on
+    // the K-split kernel's tiles, 9.4 on the rows kernel), the residual ones with a K split; QKV (20
+    // weight tiles) keeps the K-split kernel below 400 tokens (306 tokens: 11.6 against 12.5 us; 408:
+    // 12.9 against 12.5).
     // JPI_BIG_GEMM_MIN_TOKENS sets one threshold for all four.
     const char* big_env = std::getenv("JPI_BIG_GEMM_MIN_TOKENS");
     if (big_env)
@@ -564,6 +612,9 @@ jpi_status tc_prepare(jpi_handle* h) {
     JPI_TRY(make_tmap(h->hx, (uint64_t)xs_tiles(h->maxMt) * 64, h->W, NT, &h->xmaps[0]));
     JPI_TRY(make_tmap(h->o, h->maxMt, h->HD, NT, &h->xmaps[1]));
     JPI_TRY(make_tmap(h->z, h->maxMt, h->F, NT, &h->xmaps[2]));
+    JPI_TRY(make_tmap(h->hx, (uint64_t)xs_tiles(h->maxMt) * 64, h->W, 128, &h->xmaps_rows[0]));
+    JPI_TRY(make_tmap(h->o, h->maxMt, h->HD, 128, &h->xmaps_rows[1]));
+    JPI_TRY(make_tmap(h->z, h->maxMt, h->F, 128, &h->xmaps_rows[2]));
     JPI_TRY(mod_tc_prepare(h));
     // JPI_BATCH_INVARIANT=1: every launch makes the choices it makes for one request (K-split
     // projections, split-KV attention with a single request's key split), so a request's result
@@ -588,10 +639,14 @@ jpi_status tc_launch_op(jpi_handle* h, int op, int l, int step, int B, int C, cu
     // the norm-fed kind after them reads as many slots as its producer left.
     auto big = [&](int kind) { return h->big_min_tokens[kind] > 0 && Mt >= h->big_min_tokens[kind]; };
     auto slots_left = [&](int kind) { return big(kind) ? plans[kind].ntiles : plans[kind].ntiles * plans[kind].splits; };
-    auto run = [&](auto kind_tag, const GemmPlan& pl, const CUtensorMap& wm, const CUtensorMap& xm,
+    auto run = [&](auto kind_tag, const GemmPlan& pl, const CUtensorMap& wm, int xi,
                    const GemmArgs& a) -> jpi_status {
         constexpr int KIND = decltype(kind_tag)::value;
-        return big(KIND) ? launch_gemm_big<KIND>(h, pl, wm, xm, a, st) : launch_gemm<KIND>(h, pl, wm, xm, a, st);
+        if (!big(KIND)) return launch_gemm<KIND>(h, pl, wm, h->xmaps[xi], a, st);
+        if (KIND == G_QKV || KIND == G_GU || resid_rows(h, KIND, Mt, pl))
+            return launch_gemm_rows<KIND>(h, pl, wm, h->xmaps_rows[xi], a, st);
+        if constexpr (KIND == G_O || KIND == G_DOWN) return launch_gemm_big<KIND>(h, pl, wm, h->xmaps[xi], a, st);
+        return JPI_ERR_UNSUPPORTED;
     };
     using KQ = std::integral_constant<int, G_QKV>;
     using KO = std::integral_constant<int, G_O>;
@@ -608,7 +663,7 @@ jpi_status tc_launch_op(jpi_handle* h, int op, int l, int step, int B, int C, cu
             a.kst = (__nv_bfloat16*)h->kv_k + kv_layer;
             a.vst = (__nv_bfloat16*)h->kv_v + kv_layer;
             a.rope = h->rope_tab;
-            return run(KQ{}, pl, h->tmaps[4 * l + G_QKV], h->xmaps[0], a);
+            return run(KQ{}, pl, h->tmaps[4 * l + G_QKV], 0, a);
         }
         case 3:
             // Batched launches: one CTA per 128 query rows over all keys (tcgen05, no split);
@@ -626,14 +681,14 @@ jpi_status tc_launch_op(jpi_handle* h, int op, int l, int step, int B, int C, cu
             a.beta_next = ms + 4 * W;
             a.gamma = ms + 2 * W;
             a.ss_out = h->ss;
-            return run(KO{}, pl, h->tmaps[4 * l + G_O], h->xmaps[1], a);
+            return run(KO{}, pl, h->tmaps[4 * l + G_O], 1, a);
         }
         case 5: {
             const GemmPlan& pl = plans[G_GU];
             GemmArgs a = base_args(h, B, C, pl);
             a.nslot = slots_left(G_O);   // left by O
             a.z = (__nv_bfloat16*)h->z;
-            return run(KG{}, pl, h->tmaps[4 * l + G_GU], h->xmaps[0], a);
+            return run(KG{}, pl, h->tmaps[4 * l + G_GU], 0, a);
         }
         case 6: {
             const GemmPlan& pl = plans[G_DOWN];
@@ -646,7 +701,7 @@ jpi_status tc_launch_op(jpi_handle* h, int op, int l, int step, int B, int C, cu
             }
             a.gamma = ms + 5 * W;
             a.ss_out = h->ss;
-            return run(KD{}, pl, h->tmaps[4 * l + G_DOWN], h->xmaps[2], a);
+            return run(KD{}, pl, h->tmaps[4 * l + G_DOWN], 2, a);
         }
         default:
             set_error("unknown layer op %d", op);
