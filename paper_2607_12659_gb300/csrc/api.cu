@@ -62,6 +62,13 @@ __global__ void k_f32_to_bf16(const float* __restrict__ src, __nv_bfloat16* __re
         dst[i] = __float2bfloat16_rn(src[i]);
 }
 
+// dst [cols][rows] = src [rows][cols] transposed (the small input matrices, once at create).
+__global__ void k_transpose(const float* __restrict__ src, float* __restrict__ dst, int rows, int cols) {
+    const long long n = (long long)rows * cols;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        dst[(i % cols) * rows + i / cols] = src[i];
+}
+
 // Moves one fp32 source tensor (host or device) to `dst` as fp32 or bf16.
 struct Uploader {
     jpi_handle* h;
@@ -132,7 +139,9 @@ jpi_status pack_weights(jpi_handle* h, const jpi_weights* w) {
     if ((size_t)HD * W > maxe) maxe = (size_t)HD * W;
     if ((size_t)W * dt > maxe) maxe = (size_t)W * dt;
     if ((size_t)h->QKV * W > maxe) maxe = (size_t)h->QKV * W;
-    if (!up.on_device || b16) JPI_TRY(dev_alloc(h, &up.tmp, maxe));
+    if ((size_t)W * Sd > maxe) maxe = (size_t)W * Sd;
+    if ((size_t)W * A > maxe) maxe = (size_t)W * A;
+    JPI_TRY(dev_alloc(h, &up.tmp, maxe));
 
     // Small fp32 tensors.
     JPI_TRY(dev_alloc(h, &h->state_in_w, (size_t)W * Sd));
@@ -144,9 +153,14 @@ jpi_status pack_weights(jpi_handle* h, const jpi_weights* w) {
     JPI_TRY(dev_alloc(h, &h->time_in_b, W));
     JPI_TRY(dev_alloc(h, &h->time_out_b, W));
     JPI_TRY(dev_alloc(h, &h->mod_b, (size_t)mod_rows(L) * W));
-    JPI_TRY(up.put(h->state_in_w, false, w->state_in_w, (size_t)W * Sd, "state_in_w"));
+    // The input matrices are kept [inputs][W], so that the embedding reads consecutive features.
+    JPI_TRY(up.put(up.tmp, false, w->state_in_w, (size_t)W * Sd, "state_in_w"));
+    k_transpose<<<256, 256>>>(up.tmp, h->state_in_w, W, Sd);
+    JPI_CUDA_TRY(cudaGetLastError());
+    JPI_TRY(up.put(up.tmp, false, w->action_in_w, (size_t)W * A, "action_in_w"));
+    k_transpose<<<256, 256>>>(up.tmp, h->action_in_w, W, A);
+    JPI_CUDA_TRY(cudaGetLastError());
     JPI_TRY(up.put(h->state_in_b, false, w->state_in_b, W, "state_in_b"));
-    JPI_TRY(up.put(h->action_in_w, false, w->action_in_w, (size_t)W * A, "action_in_w"));
     JPI_TRY(up.put(h->action_in_b, false, w->action_in_b, W, "action_in_b"));
     JPI_TRY(up.put(h->action_out_w, false, w->action_out_w, (size_t)A * W, "action_out_w"));
     JPI_TRY(up.put(h->action_out_b, false, w->action_out_b, A, "action_out_b"));
@@ -209,6 +223,15 @@ jpi_status alloc_buffers(jpi_handle* h) {
     JPI_TRY(dev_alloc(h, &h->corr, (size_t)h->maxB * JPI_MAX_CORRECTION * h->W));
     JPI_TRY(dev_alloc(h, &h->out, (size_t)h->maxB * h->maxC * h->A));
     JPI_TRY(dev_alloc(h, &h->temb, (size_t)h->maxN * h->dt));
+    {
+        // Periods of the time embedding, geometric from t_min_period to t_max_period.
+        const int half = h->dt / 2;
+        std::vector<double> period((size_t)half);
+        const double pmin = h->cfg.t_min_period, pmax = h->cfg.t_max_period;
+        for (int i = 0; i < half; ++i) period[(size_t)i] = pmin * std::pow(pmax / pmin, (double)i / (double)(half - 1));
+        JPI_TRY(dev_alloc(h, &h->t_period, (size_t)half));
+        JPI_CUDA_TRY(cudaMemcpy(h->t_period, period.data(), half * sizeof(double), cudaMemcpyHostToDevice));
+    }
     JPI_TRY(dev_alloc(h, &h->c1, (size_t)h->maxN * W));
     JPI_TRY(dev_alloc(h, &h->cond, (size_t)h->maxN * W));
     JPI_TRY(dev_alloc(h, &h->mods, (size_t)h->maxN * mod_rows(h->L) * W));
@@ -326,7 +349,7 @@ jpi_status enqueue_step(jpi_handle* h, int step, int B, int C, float delta, floa
         else
             JPI_TRY(launch_layer_simt(h, l, step, B, C, st));
     }
-    return launch_final(h, step, B, C, delta, v_out ? nullptr : h->x, v_out, nullptr, st);
+    return launch_final(h, step, B, C, delta, v_out ? nullptr : h->x, v_out, st);
 }
 
 jpi_status check_call(jpi_handle* h, int B, int C, int N) {
@@ -551,7 +574,7 @@ JPI_API jpi_status jpi_profile_op(jpi_handle* h, int op, int layer, int batch, i
                 break;
             case 1: JPI_TRY(launch_embed(h, 0, batch, chunk, h->x, st)); break;
             case 7:
-                JPI_TRY(launch_final(h, 0, batch, chunk, 0.f, nullptr, h->out, nullptr, st));
+                JPI_TRY(launch_final(h, 0, batch, chunk, 0.f, nullptr, h->out, st));
                 break;
             default:
                 if (h->tc)

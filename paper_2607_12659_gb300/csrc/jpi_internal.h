@@ -128,9 +128,9 @@ struct jpi_handle {
     float* time_in_b = nullptr;  // [W]
     void* time_out_w = nullptr;  // [W][W] TW
     float* time_out_b = nullptr; // [W]
-    float* state_in_w = nullptr; // [W][S_d] fp32
+    float* state_in_w = nullptr; // [S_d][W] fp32 (transposed at create)
     float* state_in_b = nullptr;
-    float* action_in_w = nullptr;   // [W][A] fp32
+    float* action_in_w = nullptr;   // [A][W] fp32 (transposed at create)
     float* action_in_b = nullptr;
     float* action_out_w = nullptr;  // [A][W] fp32
     float* action_out_b = nullptr;
@@ -145,6 +145,7 @@ struct jpi_handle {
     float* x = nullptr;         // [maxB][maxC][A] current actions
     float* state = nullptr;     // [maxB][S_d] staged state
     float* out = nullptr;       // [maxB][maxC][A] staged output
+    double* t_period = nullptr; // [d_t / 2] periods of the time embedding
     float* temb = nullptr;      // [maxN][d_t] time embeddings
     float* c1 = nullptr;        // [maxN][W]
     float* cond = nullptr;      // [maxN][W]
@@ -209,7 +210,7 @@ jpi_status launch_layer_simt(jpi_handle* h, int layer, int step, int batch, int 
 jpi_status launch_op_simt(jpi_handle* h, int op, int layer, int step, int batch, int chunk,
                           cudaStream_t st);
 jpi_status launch_final(jpi_handle* h, int step, int batch, int chunk, float delta,
-                        float* x_inout, float* v_out, float* out_copy, cudaStream_t st);
+                        float* x_inout, float* v_out, cudaStream_t st);
 jpi_status launch_load_prefix(jpi_handle* h, const void* const* k_layers, const void* const* v_layers, int src_fp32,
                               int B, int P, cudaStream_t st);
 

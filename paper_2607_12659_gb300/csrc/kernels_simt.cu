@@ -58,86 +58,136 @@ __device__ float block_sum(float v, float* scratch /* >= 32 floats */) {
     return t;
 }
 
+// Four consecutive elements (k a multiple of 4, rows 4-element aligned), or with VEC false four
+// elements 32 apart per lane (any K), zero past K; rows_k says which k they are.
+template <bool VEC> __device__ __forceinline__ int rows_k(int k0, int lane, int e) {
+    return VEC ? k0 + 4 * lane + e : k0 + lane + 32 * e;
+}
+template <bool VEC>
+__device__ __forceinline__ float4 rows_load(const float* p, int k0, int lane, int K) {
+    if (VEC) {
+        const int k = k0 + 4 * lane;
+        return k < K ? *reinterpret_cast<const float4*>(p + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    float v[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const int k = rows_k<false>(k0, lane, e);
+        v[e] = k < K ? p[k] : 0.f;
+    }
+    return make_float4(v[0], v[1], v[2], v[3]);
+}
+template <bool VEC>
+__device__ __forceinline__ float4 rows_load(const __nv_bfloat16* p, int k0, int lane, int K) {
+    if (VEC) {
+        const int k = k0 + 4 * lane;
+        if (k >= K) return make_float4(0.f, 0.f, 0.f, 0.f);
+        const uint2 u = *reinterpret_cast<const uint2*>(p + k);
+        return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16),
+                           __uint_as_float(u.y & 0xFFFF0000u));
+    }
+    float v[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const int k = rows_k<false>(k0, lane, e);
+        v[e] = k < K ? __bfloat162float(p[k]) : 0.f;
+    }
+    return make_float4(v[0], v[1], v[2], v[3]);
+}
+
 // ---------------------------------------------------------------------------------------------
 // Time conditioning: flow time enters the expert only through a sinusoidal embedding followed
 // by a two-layer swish MLP; the per-layer modulation vectors are a linear map of the result.
 // All of it depends on t alone, so it is evaluated once per call for every step time.
 
-// Grid (steps, ceil(half / blockDim)): one frequency i of one step time per thread (the fp64
-// pow/sin/cos are slow on this GPU; spread over the grid they run side by side).
-__global__ void k_time_embed(float* temb, int nsteps, int dt, double pmin, double pmax,
-                             double t_override) {
+// Grid (steps, ceil(half / 32)): one frequency i of one step time per thread, a warp per block (fp64
+// sin/cos are slow on this GPU, two lanes' worth a clock: spread over the SMs they run side by side).
+// The periods are tabulated at create.
+constexpr int TE_THREADS = 32;
+__global__ void k_time_embed(float* temb, const double* __restrict__ period, int nsteps, int dt, double t_override) {
+    ptx::grid_dep_launch();   // the next kernel waits for this one's results before reading them
     const int k = blockIdx.x;
     const double t = t_override >= 0.0 ? t_override : (double)k / (double)nsteps;
-    const int half = dt / 2;
-    for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < half; i += gridDim.y * blockDim.x) {
-        const double frac = (double)i / (double)(half - 1);
-        const double period = pmin * pow(pmax / pmin, frac);
-        const double theta = 2.0 * 3.14159265358979323846 * t / period;
-        temb[(size_t)k * dt + i] = (float)sin(theta);
-        temb[(size_t)k * dt + half + i] = (float)cos(theta);
-    }
+    const int half = dt / 2, i = blockIdx.y * TE_THREADS + threadIdx.x;
+    if (i >= half) return;
+    const double theta = 2.0 * 3.14159265358979323846 * t / period[i];
+    double s, c;
+    sincos(theta, &s, &c);
+    temb[(size_t)k * dt + i] = (float)s;
+    temb[(size_t)k * dt + half + i] = (float)c;
 }
 
-// Y[n][r] = act(sum_k W[r][k] X[n][k] + b[r]) for n < N (<= 8 per pass), r < R.
-// One warp per output row; X lives in shared memory.
-template <typename TW, bool SWISH>
-__global__ void k_gemv_multi(const TW* __restrict__ Wm, const float* __restrict__ bias,
-                             const float* __restrict__ X, float* __restrict__ Y, int R, int K,
-                             int N) {
-    extern __shared__ float xs[];
-    // Eight loads of each thread in flight before their stores (one at a time, every store would
-    // hold the next load back for a full round trip).
-    for (int i0 = threadIdx.x; i0 < N * K; i0 += 8 * blockDim.x) {
-        float v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int i = i0 + u * blockDim.x;
-            v[u] = i < N * K ? X[i] : 0.f;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int i = i0 + u * blockDim.x;
-            if (i < N * K) xs[i] = v[u];
-        }
-    }
-    __syncthreads();
+// Y[n][r] = act(sum_k W[r][k] X[n][k] + b[r]) for n < N <= GV_N, r < R: one warp per output row,
+// its first GV_U x 128 weights in registers before the dependency wait, X in shared memory (read as
+// 16-byte chunks, four consecutive k per lane). Launches of the time MLP are short chains: 1024 rows
+// x 1024 bf16 weights took 11 us with 2-byte weight loads issued after the inputs were staged.
+// The modulation vectors (no swish) are read by kernels before their own dependency wait: that
+// launch does not release its dependent early.
+constexpr int GV_N = 16, GV_U = 8;
+template <typename TW, bool SWISH, bool VEC>
+__global__ void __launch_bounds__(256) k_gemv_multi(const TW* __restrict__ Wm, const float* __restrict__ bias,
+                                                    const float* __restrict__ X, float* __restrict__ Y, int R, int K,
+                                                    int N) {
+    extern __shared__ __align__(16) float xs[];   // [N][K]
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    for (int r = warp; r < R; r += nwarps) {
-        const TW* wr = Wm + (size_t)r * K;
-        for (int n0 = 0; n0 < N; n0 += 8) {
-            float acc[8];
+    float4 w4[GV_U];
+    auto load = [&](int r, int kb) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) acc[j] = 0.f;
-            // Eight weights of the row loaded together, then their products in k order.
-            for (int k0 = lane; k0 < K; k0 += 32 * 8) {
-                float wv[8];
+        for (int u = 0; u < GV_U; ++u)
+            w4[u] = r < R ? rows_load<VEC>(Wm + (size_t)r * K, kb + 128 * u, lane, K) : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    load(warp, 0);
+    ptx::grid_dep_wait();
+    if (SWISH) ptx::grid_dep_launch();
+    // Eight loads of each thread in flight before their stores.
+    if (VEC) {
+        const int n4 = N * K / 4;
+        for (int i0 = threadIdx.x; i0 < n4; i0 += 8 * blockDim.x) {
+            float4 v[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int k = k0 + 32 * u;
-                    wv[u] = k < K ? ldf(wr + k) : 0.f;
-                }
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int k = k0 + 32 * u;
-                    if (k < K) {
-#pragma unroll
-                        for (int j = 0; j < 8; ++j)
-                            if (n0 + j < N) acc[j] = fmaf(wv[u], xs[(n0 + j) * K + k], acc[j]);
-                    }
-                }
+            for (int u = 0; u < 8; ++u) {
+                const int i = i0 + u * blockDim.x;
+                v[u] = i < n4 ? reinterpret_cast<const float4*>(X)[i] : make_float4(0.f, 0.f, 0.f, 0.f);
             }
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const float s = warp_sum(acc[j]);
-                if (lane == 0 && n0 + j < N) {
-                    const float y = s + bias[r];
-                    Y[(size_t)(n0 + j) * R + r] = SWISH ? swishf(y) : y;
-                }
+            for (int u = 0; u < 8; ++u) {
+                const int i = i0 + u * blockDim.x;
+                if (i < n4) reinterpret_cast<float4*>(xs)[i] = v[u];
             }
         }
+    } else {
+        for (int i = threadIdx.x; i < N * K; i += blockDim.x) xs[i] = X[i];
+    }
+    __syncthreads();
+    for (int r = warp; r < R; r += nwarps) {
+        float acc[GV_N];
+#pragma unroll
+        for (int j = 0; j < GV_N; ++j) acc[j] = 0.f;
+        for (int kb = 0; kb < K; kb += 128 * GV_U) {
+            if (kb > 0 || r != warp) load(r, kb);
+#pragma unroll
+            for (int u = 0; u < GV_U; ++u) {
+                if (kb + 128 * u >= K) break;
+#pragma unroll
+                for (int j = 0; j < GV_N; ++j)
+                    if (j < N) {
+                        const float4 x4 = rows_load<VEC>(xs + (size_t)j * K, kb + 128 * u, lane, K);
+                        acc[j] = fmaf(w4[u].x, x4.x, acc[j]);
+                        acc[j] = fmaf(w4[u].y, x4.y, acc[j]);
+                        acc[j] = fmaf(w4[u].z, x4.z, acc[j]);
+                        acc[j] = fmaf(w4[u].w, x4.w, acc[j]);
+                    }
+            }
+        }
+        const float br = bias[r];
+#pragma unroll
+        for (int j = 0; j < GV_N; ++j)
+            if (j < N) {
+                const float y = warp_sum(acc[j]) + br;
+                if (lane == 0) Y[(size_t)j * R + r] = SWISH ? swishf(y) : y;
+            }
     }
 }
 
@@ -218,12 +268,13 @@ __global__ void __launch_bounds__(256) k_mod_gemv(const TW* __restrict__ Wm, con
 // ---------------------------------------------------------------------------------------------
 // Token embedding: row 0 of each request is the state token, rows 1..nctx-1 the correction
 // items (context tokens, taken as given), then the C action tokens.
-// Block = 128 features of up to TPB tokens that share one input matrix: blockIdx.y counts groups of
-// action tokens first, then groups of state and context tokens. A thread keeps its feature's weight
-// row in registers for all of them (its 128 bytes are a line of their own, so with one token per
-// block every token fetched 16 KB of weights per 128 features again: 382 us at 3264 tokens x 1024
-// features, bound by those reads; the outputs alone are 20 MB, 3 us) and reads the tokens' inputs
-// from shared memory as broadcasts. The sums keep the order of one token at a time.
+// Block = 512 features (four per thread, a warp per 128-feature slice) of up to tpb tokens that share
+// one input matrix: blockIdx.y counts groups of action tokens first, then groups of state and context
+// tokens. A thread keeps its features' weights in registers for all of the block's tokens and reads
+// the tokens' inputs from shared memory as broadcasts. What bounds it: with a token per block, the
+// weight rows (a line per feature) were fetched again for every token (382 us at 3264 tokens x 1024
+// features); with a feature per thread, the instructions around each token's 32 products (31 us).
+// The outputs alone are 20 MB, 3 us.
 // For the tensor-core path it also writes the operand of the first layer's norm-fed projection
 // (xs = bf16((1 + sigma) * h) at row xs_row(m), and beta in the last row of every 64-row tile) and
 // each token's sum of squares over the 128 features (ss[slice][m]).
@@ -240,10 +291,14 @@ struct EmbedArgs {
 constexpr int EMB_MAX_TPB = 16;
 constexpr int EMB_K = 32;     // inputs per token kept in registers / shared memory
 
+__device__ __forceinline__ uint2 pack_bf16x4(float a, float b, float c, float d) {
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(a, b), hi = __floats2bfloat162_rn(c, d);
+    return make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+}
+
 __global__ void __launch_bounds__(128) k_embed(const EmbedArgs a) {
     __shared__ __align__(16) float in_s[EMB_MAX_TPB][EMB_K];
-    __shared__ float part[EMB_MAX_TPB][4];
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31;
     const bool act = (int)blockIdx.y < a.action_groups;
     // Tokens [j0, j0 + nt) of this block's kind: action token j = (request j / C, action j mod C),
     // else context token j = (request j / nctx, row j mod nctx).
@@ -253,36 +308,25 @@ __global__ void __launch_bounds__(128) k_embed(const EmbedArgs a) {
     const int K = act ? a.A : a.Sd;
     const int Kr = min(K, EMB_K);
     const float* Wm = act ? a.Wa : a.Ws;
-    const int n = blockIdx.x * 128 + tid;
+    const int n = (blockIdx.x * 128 + tid) * 4;   // first of four features (W is a multiple of 32)
     const bool live = n < a.W;
-    // Everything but x (the previous step's actions) is ready before the dependency wait.
-    float wv[EMB_K];
-    float bv = 0.f, sg = 0.f, bt = 0.f;
+    // The weights depend on nothing upstream. Products past K multiply zeros.
+    float4 wv[EMB_K];   // input k of the four features (the matrices are stored [K][W])
+    float4 bv = make_float4(0.f, 0.f, 0.f, 0.f), sg = bv, bt = bv;
+#pragma unroll
+    for (int k = 0; k < EMB_K; ++k)
+        wv[k] = k < K && live ? __ldg(reinterpret_cast<const float4*>(Wm + (size_t)k * a.W + n)) : bv;
     if (live) {
-        const float* wr = Wm + (size_t)n * K;
-        if (K % 4 == 0) {
-#pragma unroll
-            for (int k = 0; k < EMB_K; k += 4) {
-                const float4 w4 = k < K ? __ldg(reinterpret_cast<const float4*>(wr + k)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                wv[k] = w4.x;
-                wv[k + 1] = w4.y;
-                wv[k + 2] = w4.z;
-                wv[k + 3] = w4.w;
-            }
-        } else {
-#pragma unroll
-            for (int k = 0; k < EMB_K; ++k) wv[k] = k < K ? wr[k] : 0.f;
-        }
-        bv = (act ? a.ba : a.bs)[n];
-        if (a.xs) {
-            sg = a.sigma[n];
-            bt = a.beta[n];
-        }
+        bv = *reinterpret_cast<const float4*>((act ? a.ba : a.bs) + n);
     }
     // Launched with programmatic dependent launch: x comes from the previous step's final kernel;
     // the next kernel may start its weight prefetch at once.
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
+    if (live && a.xs) {
+        sg = *reinterpret_cast<const float4*>(a.sigma + n);
+        bt = *reinterpret_cast<const float4*>(a.beta + n);
+    }
     // Inputs of token j: its action row, or its request's state (context rows past 0 have none).
     auto input = [&](int j) { return act ? a.x + (size_t)j * a.A : a.state + (size_t)(j / a.nctx) * a.Sd; };
     for (int i = tid; i < nt * EMB_K; i += 128) {
@@ -290,49 +334,62 @@ __global__ void __launch_bounds__(128) k_embed(const EmbedArgs a) {
         in_s[tt][k] = k < Kr ? input(j0 + tt)[k] : 0.f;
     }
     __syncthreads();
+    int b = j0 / per, i = j0 - b * per;   // request and row within its kind, advanced token by token
     for (int tt = 0; tt < nt; ++tt) {
-        const int j = j0 + tt;
-        const int b = j / per, i = (act ? a.nctx : 0) + j - b * per;   // request, row in its suffix
-        const int m = b * a.S + i;
-        float v = 0.f;
+        const int m = b * a.S + (act ? a.nctx : 0) + i;
+        float v[4] = {0.f, 0.f, 0.f, 0.f};
         if (live) {
             if (!act && i > 0) {
-                v = a.corr[((size_t)b * (a.nctx - 1) + (i - 1)) * a.W + n];
+                const float4 c = *reinterpret_cast<const float4*>(a.corr + ((size_t)b * (a.nctx - 1) + (i - 1)) * a.W + n);
+                v[0] = c.x;
+                v[1] = c.y;
+                v[2] = c.z;
+                v[3] = c.w;
             } else {
-                float acc = 0.f;
                 const float4* iv = reinterpret_cast<const float4*>(in_s[tt]);
+                auto add = [&](const float4& w, float x) {
+                    v[0] = fmaf(w.x, x, v[0]);
+                    v[1] = fmaf(w.y, x, v[1]);
+                    v[2] = fmaf(w.z, x, v[2]);
+                    v[3] = fmaf(w.w, x, v[3]);
+                };
 #pragma unroll
                 for (int k = 0; k < EMB_K; k += 4) {
                     const float4 x4 = iv[k / 4];
-                    if (k < K) acc = fmaf(wv[k], x4.x, acc);
-                    if (k + 1 < K) acc = fmaf(wv[k + 1], x4.y, acc);
-                    if (k + 2 < K) acc = fmaf(wv[k + 2], x4.z, acc);
-                    if (k + 3 < K) acc = fmaf(wv[k + 3], x4.w, acc);
+                    add(wv[k], x4.x);
+                    add(wv[k + 1], x4.y);
+                    add(wv[k + 2], x4.z);
+                    add(wv[k + 3], x4.w);
                 }
-                const float* in = input(j);
-                for (int k = EMB_K; k < K; ++k) acc = fmaf(Wm[(size_t)n * K + k], in[k], acc);
-                v = acc + bv;
+                if (K > EMB_K) {
+                    const float* in = input(j0 + tt);
+                    for (int k = EMB_K; k < K; ++k)
+                        add(__ldg(reinterpret_cast<const float4*>(Wm + (size_t)k * a.W + n)), in[k]);
+                }
+                v[0] += bv.x;
+                v[1] += bv.y;
+                v[2] += bv.z;
+                v[3] += bv.w;
             }
-            a.hres[(size_t)m * a.W + n] = v;
-            if (a.xs) a.xs[(size_t)xs_row(m) * a.W + n] = __float2bfloat16_rn((1.f + sg) * v);
+            *reinterpret_cast<float4*>(a.hres + (size_t)m * a.W + n) = make_float4(v[0], v[1], v[2], v[3]);
+            if (a.xs)
+                *reinterpret_cast<uint2*>(a.xs + (size_t)xs_row(m) * a.W + n) =
+                    pack_bf16x4((1.f + sg.x) * v[0], (1.f + sg.y) * v[1], (1.f + sg.z) * v[2], (1.f + sg.w) * v[3]);
         }
-        if (a.ss) {
-            const float t = warp_sum(v * v);
-            if ((tid & 31) == 0) part[tt][tid >> 5] = t;
+        if (a.ss) {   // W is a multiple of 128 then: a warp is one slice
+            const float t = warp_sum(fmaf(v[0], v[0], v[1] * v[1]) + fmaf(v[2], v[2], v[3] * v[3]));
+            if (lane == 0 && live) a.ss[(size_t)(n >> 7) * a.ss_ld + m] = t;
+        }
+        if (++i == per) {
+            i = 0;
+            ++b;
         }
     }
     if (a.xs && live) {
         // Tile z's beta row: block y takes tiles y tpb .. (the blocks' token slots cover the tiles).
         const int z0 = blockIdx.y * a.tpb, z1 = min(z0 + a.tpb, xs_tiles(a.B * a.S));
-        for (int z = z0; z < z1; ++z) a.xs[((size_t)z * 64 + 63) * a.W + n] = __float2bfloat16_rn(bt);
-    }
-    if (a.ss) {
-        __syncthreads();
-        if (tid < nt) {
-            const int j = j0 + tid, b = j / per, i = (act ? a.nctx : 0) + j - b * per;
-            a.ss[(size_t)blockIdx.x * a.ss_ld + b * a.S + i] =
-                (part[tid][0] + part[tid][2]) + (part[tid][1] + part[tid][3]);
-        }
+        for (int z = z0; z < z1; ++z)
+            *reinterpret_cast<uint2*>(a.xs + ((size_t)z * 64 + 63) * a.W + n) = pack_bf16x4(bt.x, bt.y, bt.z, bt.w);
     }
 }
 
@@ -368,43 +425,6 @@ struct RowsArgs {
     const float2* rope;
     int S, H, D, P, kv_rows;
 };
-
-// Four consecutive elements (k a multiple of 4, rows 4-element aligned), or with VEC false four
-// elements 32 apart per lane (any K), zero past K. kidx(lane) says which k they are.
-template <bool VEC> __device__ __forceinline__ int rows_k(int k0, int lane, int e) {
-    return VEC ? k0 + 4 * lane + e : k0 + lane + 32 * e;
-}
-template <bool VEC>
-__device__ __forceinline__ float4 rows_load(const float* p, int k0, int lane, int K) {
-    if (VEC) {
-        const int k = k0 + 4 * lane;
-        return k < K ? *reinterpret_cast<const float4*>(p + k) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    float v[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const int k = rows_k<false>(k0, lane, e);
-        v[e] = k < K ? p[k] : 0.f;
-    }
-    return make_float4(v[0], v[1], v[2], v[3]);
-}
-template <bool VEC>
-__device__ __forceinline__ float4 rows_load(const __nv_bfloat16* p, int k0, int lane, int K) {
-    if (VEC) {
-        const int k = k0 + 4 * lane;
-        if (k >= K) return make_float4(0.f, 0.f, 0.f, 0.f);
-        const uint2 u = *reinterpret_cast<const uint2*>(p + k);
-        return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16),
-                           __uint_as_float(u.y & 0xFFFF0000u));
-    }
-    float v[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const int k = rows_k<false>(k0, lane, e);
-        v[e] = k < K ? __bfloat162float(p[k]) : 0.f;
-    }
-    return make_float4(v[0], v[1], v[2], v[3]);
-}
 
 template <typename T, int KIND, bool VEC, int KS>
 __global__ void __launch_bounds__(32 * ROWS_WARPS) k_rows_gemm(const RowsArgs a) {
@@ -825,34 +845,129 @@ __global__ void __launch_bounds__(32 * AR_WARPS) k_attn_rows(const T* __restrict
 // ---------------------------------------------------------------------------------------------
 // Final adaptive RMSNorm of an action row, velocity v = u W_out^T + b_out, Euler update
 // x <- x + delta v (or, for a single forward, v itself).
-// One CTA of FIN_THREADS per action row. The row's values (FIN_CAP per thread at most, all loads
-// in flight together) give the norm; the normalised row goes to shared memory; then thread t
-// takes output a0 + t / 8 over the 16-byte column chunks t mod 8, t mod 8 + 8, .. (a group of 8
-// threads reads 128 contiguous bytes per step) and the group adds its 8 partial sums.
+// One CTA of FIN_THREADS per FR action rows. The rows' values give the norms and the normalised rows
+// go to shared memory; then a warp takes four outputs of all FR rows, a lane four consecutive columns
+// of every 128 (FR + 4 16-byte loads per 16 FR products), and the sums are reduced over the lanes.
+// With one row per CTA, each CTA reads all of W_out (128 KB at 32 x 1024) from L2: 32 us for 3200
+// rows; FR = 1 stays for few rows, where the CTAs run side by side and the chain is shortest.
+// A row's sums do not depend on FR: its squares are added as 256 strided partials in the tree of one
+// CTA per row (FR = 1), whichever warp owns the row, and its products in the same lanes and order.
 constexpr int FIN_THREADS = 256;
 constexpr int FIN_CAP = 16;   // W <= 4096
-__global__ void __launch_bounds__(FIN_THREADS) k_final(const float* __restrict__ hres, const float* __restrict__ sigma,
-                        const float* __restrict__ beta, const float* __restrict__ Wout,
-                        const float* __restrict__ bout, float* __restrict__ x,
-                        float* __restrict__ vout, float* __restrict__ outcopy, int S, int nctx, int C,
-                        int W, int A, float eps, float delta) {
-    extern __shared__ float us[];        // [W]
+constexpr size_t FIN_SMEM_MAX = 100 * 1024;   // rows of one CTA (two CTAs per SM)
+struct FinalArgs {
+    const float *hres, *sigma, *beta, *Wout, *bout;
+    float *x, *vout;
+    int rows, S, nctx, C, W, A;   // rows: action rows of all requests
+    float eps, delta;
+};
+
+// Sums v over the lanes (reduce-scatter, partners 16, 8, .., 1 lanes apart): lane L is left with the
+// totals of values L NV / 32 .. in v[0 .. max(NV / 32, 1)) (for NV < 32, 32 / NV lanes share one).
+template <int NV>
+__device__ __forceinline__ void lane_reduce(float (&v)[NV], int lane) {
+    int n = NV;
+#pragma unroll
+    for (int sh = 16; sh > 0; sh >>= 1) {
+        if (n > 1) {
+            n >>= 1;
+            const bool hi = (lane & sh) != 0;
+#pragma unroll
+            for (int i = 0; i < NV / 2; ++i) {
+                if (i >= n) break;
+                const float send = hi ? v[i] : v[i + n], keep = hi ? v[i + n] : v[i];
+                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, sh);
+            }
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], sh);
+        }
+    }
+}
+
+// Outputs of the FR normalised rows us [FR][W] of the CTA (rows bj0 ..). w0: the first PRE steps of
+// the warp's first four rows of W_out.
+template <int FR, int PRE>
+__device__ __forceinline__ void final_outputs(const FinalArgs& a, const float* us, int bj0, float4 (&w0)[PRE][4]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int o0 = 4 * warp; o0 < a.A; o0 += 4 * (FIN_THREADS / 32)) {
+        float v[4 * FR];   // row r, output o0 + s at 4 r + s
+#pragma unroll
+        for (int i = 0; i < 4 * FR; ++i) v[i] = 0.f;
+        auto step = [&](int k0, const float4 (&w4)[4]) {
+#pragma unroll
+            for (int r = 0; r < FR; ++r) {
+                const int k = k0 + 4 * lane;
+                const float4 u4 = k < a.W ? *reinterpret_cast<const float4*>(us + (size_t)r * a.W + k)
+                                          : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int s = 0; s < 4; ++s) {
+                    float t = v[4 * r + s];
+                    t = fmaf(u4.x, w4[s].x, t);
+                    t = fmaf(u4.y, w4[s].y, t);
+                    t = fmaf(u4.z, w4[s].z, t);
+                    v[4 * r + s] = fmaf(u4.w, w4[s].w, t);
+                }
+            }
+        };
+        int k0 = 0;
+        if (o0 == 4 * warp) {
+#pragma unroll
+            for (int q = 0; q < PRE; ++q) step(128 * q, w0[q]);
+            k0 = 128 * PRE;
+        }
+#pragma unroll 2
+        for (; k0 < a.W; k0 += 128) {
+            float4 w4[4];
+#pragma unroll
+            for (int s = 0; s < 4; ++s)
+                w4[s] = rows_load<true>(a.Wout + (size_t)min(o0 + s, a.A - 1) * a.W, k0, lane, a.W);
+            step(k0, w4);
+        }
+        lane_reduce<4 * FR>(v, lane);
+        constexpr int PER = FR >= 8 ? FR / 8 : 1, SHARE = FR >= 8 ? 1 : 8 / FR;   // values per lane, lanes per value
+#pragma unroll
+        for (int e = 0; e < PER; ++e) {
+            const int idx = lane / SHARE * PER + e, r = idx >> 2, o = o0 + (idx & 3);
+            if (lane % SHARE != 0 || o >= a.A || bj0 + r >= a.rows) continue;
+            const float vel = v[e] + a.bout[o];
+            const size_t at = (size_t)(bj0 + r) * a.A + o;
+            if (a.vout) a.vout[at] = vel;
+            if (a.x) a.x[at] = a.x[at] + a.delta * vel;
+        }
+    }
+}
+
+// The first PRE steps of W_out rows 4 warp .. + 3 (weights: before the dependency wait).
+template <int PRE>
+__device__ __forceinline__ void final_prefetch(const FinalArgs& a, float4 (&w0)[PRE][4]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int q = 0; q < PRE; ++q)
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+            w0[q][s] = rows_load<true>(a.Wout + (size_t)min(4 * warp + s, a.A - 1) * a.W, 128 * q, lane, a.W);
+}
+
+__global__ void __launch_bounds__(FIN_THREADS) k_final(const FinalArgs a) {
+    extern __shared__ __align__(16) float us[];        // [W]
     __shared__ float scratch[32];
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, W = a.W;
     const int bj = blockIdx.x;           // request b, action j
-    const int b = bj / C, j = bj % C;
+    const int b = bj / a.C, j = bj % a.C;
     // The modulation (scale, shift) of this thread's features, before the dependency wait.
     float sg[FIN_CAP], bt[FIN_CAP];
 #pragma unroll
     for (int q = 0; q < FIN_CAP; ++q) {
         const int k = tid + FIN_THREADS * q;
-        sg[q] = k < W ? sigma[k] : 0.f;
-        bt[q] = k < W ? beta[k] : 0.f;
+        sg[q] = k < W ? a.sigma[k] : 0.f;
+        bt[q] = k < W ? a.beta[k] : 0.f;
     }
+    float4 w0[4][4];
+    final_prefetch(a, w0);
     // Launched with programmatic dependent launch: h comes from the last layer's down projection.
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-    const float* hr = hres + ((size_t)b * S + nctx + j) * W;
+    const float* hr = a.hres + ((size_t)b * a.S + a.nctx + j) * W;
     float hv[FIN_CAP];
 #pragma unroll
     for (int q = 0; q < FIN_CAP; ++q) {
@@ -864,43 +979,59 @@ __global__ void __launch_bounds__(FIN_THREADS) k_final(const float* __restrict__
     for (int q = 0; q < FIN_CAP; ++q) ss = fmaf(hv[q], hv[q], ss);
     for (int k = tid + FIN_THREADS * FIN_CAP; k < W; k += FIN_THREADS) ss = fmaf(hr[k], hr[k], ss);   // W > 4096
     ss = block_sum(ss, scratch);
-    const float rinv = rsqrtf(ss / (float)W + eps);
+    const float rinv = rsqrtf(ss / (float)W + a.eps);
 #pragma unroll
     for (int q = 0; q < FIN_CAP; ++q) {
         const int k = tid + FIN_THREADS * q;
         if (k < W) us[k] = hv[q] * rinv * (1.f + sg[q]) + bt[q];
     }
     for (int k = tid + FIN_THREADS * FIN_CAP; k < W; k += FIN_THREADS)
-        us[k] = hr[k] * rinv * (1.f + sigma[k]) + beta[k];
+        us[k] = hr[k] * rinv * (1.f + a.sigma[k]) + a.beta[k];
     __syncthreads();
-    const int ks = tid & 7;
-    const int n4 = W >> 2;   // W is a multiple of 32 (checked at create)
-    const float4* us4 = reinterpret_cast<const float4*>(us);
-    for (int a0 = 0; a0 < A; a0 += FIN_THREADS / 8) {
-        const int a = a0 + (tid >> 3);
-        float acc = 0.f;
-        if (a < A) {
-            const float4* wr = reinterpret_cast<const float4*>(Wout + (size_t)a * W);
+    final_outputs<1>(a, us, bj, w0);
+}
+
+// FR rows per CTA: a warp per row (then per row + 8) computes the norm.
+template <int FR>
+__global__ void __launch_bounds__(FIN_THREADS) k_final_rows(const FinalArgs a) {
+    extern __shared__ __align__(16) float us[];        // [FR][W]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = a.W;
+    const int bj0 = blockIdx.x * FR;
+    float4 w0[1][4];
+    final_prefetch(a, w0);
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
+    for (int r = warp; r < FR && bj0 + r < a.rows; r += FIN_THREADS / 32) {
+        const int bj = bj0 + r, b = bj / a.C, j = bj - b * a.C;
+        const float* hr = a.hres + ((size_t)b * a.S + a.nctx + j) * W;
+        float* ur = us + (size_t)r * W;
+        // Partial w of this lane is thread 32 w + lane of k_final: columns 32 w + lane + 256 q.
+        float ps[8];
+#pragma unroll
+        for (int w = 0; w < 8; ++w) ps[w] = 0.f;
+        for (int k0 = 0; k0 < W; k0 += 2 * FIN_THREADS) {
+            float hv[16];
+#pragma unroll
+            for (int w = 0; w < 16; ++w) {
+                const int k = k0 + 32 * w + lane;
+                hv[w] = k < W ? hr[k] : 0.f;
+            }
+#pragma unroll
+            for (int w = 0; w < 16; ++w) {
+                const int k = k0 + 32 * w + lane;
+                ps[w & 7] = fmaf(hv[w], hv[w], ps[w & 7]);
+                if (k < W) ur[k] = hv[w];
+            }
+        }
+#pragma unroll
+        for (int w = 0; w < 8; ++w) ps[w] = warp_sum(ps[w]);
+        const float ss = ((ps[0] + ps[4]) + (ps[2] + ps[6])) + ((ps[1] + ps[5]) + (ps[3] + ps[7]));
+        const float rinv = rsqrtf(ss / (float)W + a.eps);
 #pragma unroll 8
-            for (int c = ks; c < n4; c += 8) {
-                const float4 w4 = __ldg(wr + c), u4 = us4[c];
-                acc = fmaf(u4.x, w4.x, fmaf(u4.y, w4.y, fmaf(u4.z, w4.z, fmaf(u4.w, w4.w, acc))));
-            }
-        }
-        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-        acc += __shfl_xor_sync(0xffffffffu, acc, 4);
-        if (ks == 0 && a < A) {
-            const float v = acc + bout[a];
-            const size_t idx = (size_t)bj * A + a;
-            if (vout) vout[idx] = v;
-            if (x) {
-                const float xn = x[idx] + delta * v;
-                x[idx] = xn;
-                if (outcopy) outcopy[idx] = xn;
-            }
-        }
+        for (int k = lane; k < W; k += 32) ur[k] = ur[k] * rinv * (1.f + a.sigma[k]) + a.beta[k];
     }
+    __syncthreads();
+    final_outputs<FR>(a, us, bj0, w0);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1173,9 +1304,30 @@ jpi_status op_simt(jpi_handle* h, int op, int l, int step, int B, int C, cudaStr
     }
 }
 
-// Step times are processed in groups of at most 8 so the shared-memory copy of the inputs
-// stays at 8 x max(W, d_t) floats whatever the step count.
-constexpr int TC_GROUP = 8;
+// Step times per launch of k_gemv_multi: its shared copy of the inputs is that many x max(W, d_t)
+// floats, kept within 200 KB.
+int tc_group(const jpi_handle* h) {
+    const size_t row = sizeof(float) * (size_t)(h->W > h->dt ? h->W : h->dt);
+    int g = GV_N;
+    while (g > 1 && g * row > 200 * 1024) g /= 2;
+    return g;
+}
+
+// Y [N][R] = act(X [N][K] Wm [R][K]^T + bias) by k_gemv_multi, tc_group step times per launch.
+template <typename T, bool SWISH>
+void launch_gemv(jpi_handle* h, const T* Wm, const float* bias, const float* X, float* Y, int R, int K, int N,
+                 cudaStream_t st) {
+    const int group = tc_group(h);
+    const dim3 grid(grid_for((long long)R * 32, 256, 1024)), blk(256);
+    for (int n0 = 0; n0 < N; n0 += group) {
+        const int g = N - n0 < group ? N - n0 : group;
+        const size_t smem = sizeof(float) * (size_t)g * K;
+        const float* x = X + (size_t)n0 * K;
+        float* y = Y + (size_t)n0 * R;
+        if (K % 4 == 0) launch_pdl(h, grid, blk, smem, st, k_gemv_multi<T, SWISH, true>, Wm, bias, x, y, R, K, g);
+        else launch_pdl(h, grid, blk, smem, st, k_gemv_multi<T, SWISH, false>, Wm, bias, x, y, R, K, g);
+    }
+}
 
 // Modulation step times per pass of k_mod_gemv (its shared copy of X is MOD_GROUP x W floats).
 constexpr int MOD_GROUP = 16;
@@ -1195,14 +1347,10 @@ void launch_mod_gemv(jpi_handle* h, const float* X, float* Y, int R, cudaStream_
 template <typename T>
 jpi_status mod_gemv(jpi_handle* h, int g, const float* X, float* Y, int R, cudaStream_t st) {
     if (std::is_same<T, __nv_bfloat16>::value && h->mod_tc) return launch_mod_tc(h, X, Y, g, st);
-    // Few rows (four per thread would leave most SMs without a warp): a warp per row instead, eight
-    // step times a launch (3584 rows x 256 columns: 19 us with four rows per thread on 14 CTAs).
+    // Few rows (four per thread would leave most SMs without a warp): a warp per row instead
+    // (3584 rows x 256 columns: 19 us with four rows per thread on 14 CTAs).
     if (R < MOD_RT * 64 * h->num_sms) {
-        for (int n0 = 0; n0 < g; n0 += TC_GROUP) {
-            const int ng = g - n0 < TC_GROUP ? g - n0 : TC_GROUP;
-            k_gemv_multi<T, false><<<grid_for((long long)R * 32, 256, 1024), 256, sizeof(float) * ng * h->W, st>>>(
-                (const T*)h->mod_w, h->mod_b, X + (size_t)n0 * h->W, Y + (size_t)n0 * R, R, h->W, ng);
-        }
+        launch_gemv<T, false>(h, (const T*)h->mod_w, h->mod_b, X, Y, R, h->W, g, st);
         return JPI_OK;
     }
     switch (g) {
@@ -1227,55 +1375,64 @@ jpi_status set_mod_attrs(int smem) {
     return JPI_OK;
 }
 
+// Time MLP and modulation vectors of N step times from their embeddings temb [N][d_t].
 template <typename T>
-jpi_status time_cond(jpi_handle* h, int N, cudaStream_t st) {
-    const int W = h->W, dt = h->dt;
-    const int R = mod_rows(h->L) * W;
-    const dim3 blk(256);
-    for (int n0 = 0; n0 < N; n0 += TC_GROUP) {
-        const int g = (N - n0) < TC_GROUP ? (N - n0) : TC_GROUP;
-        k_gemv_multi<T, true><<<grid_for((long long)W * 32, 256, 1024), blk, sizeof(float) * g * dt, st>>>(
-            (const T*)h->time_in_w, h->time_in_b, h->temb + (size_t)n0 * dt, h->c1 + (size_t)n0 * W, W, dt, g);
-        k_gemv_multi<T, true><<<grid_for((long long)W * 32, 256, 1024), blk, sizeof(float) * g * W, st>>>(
-            (const T*)h->time_out_w, h->time_out_b, h->c1 + (size_t)n0 * W, h->cond + (size_t)n0 * W, W, W, g);
-    }
+jpi_status time_cond(jpi_handle* h, int N, const float* temb, float* c1, float* cond, cudaStream_t st) {
+    const int W = h->W, dt = h->dt, R = mod_rows(h->L) * W;
+    launch_gemv<T, true>(h, (const T*)h->time_in_w, h->time_in_b, temb, c1, W, dt, N, st);
+    launch_gemv<T, true>(h, (const T*)h->time_out_w, h->time_out_b, c1, cond, W, W, N, st);
     for (int n0 = 0; n0 < N; n0 += MOD_GROUP) {
         const int g = (N - n0) < MOD_GROUP ? (N - n0) : MOD_GROUP;
-        JPI_TRY(mod_gemv<T>(h, g, h->cond + (size_t)n0 * W, h->mods + (size_t)n0 * R, R, st));
+        JPI_TRY(mod_gemv<T>(h, g, cond + (size_t)n0 * W, h->mods + (size_t)n0 * R, R, st));
     }
     return check_launch("time conditioning");
+}
+
+template <typename T>
+jpi_status set_gemv_attrs(int smem) {
+    JPI_CUDA_TRY(cudaFuncSetAttribute(k_gemv_multi<T, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    JPI_CUDA_TRY(cudaFuncSetAttribute(k_gemv_multi<T, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    JPI_CUDA_TRY(cudaFuncSetAttribute(k_gemv_multi<T, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    JPI_CUDA_TRY(cudaFuncSetAttribute(k_gemv_multi<T, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    return JPI_OK;
 }
 
 }  // namespace
 
 jpi_status configure_simt_kernels(jpi_handle* h) {
-    const int gemv_smem = (int)(sizeof(float) * (size_t)TC_GROUP * (h->W > h->dt ? h->W : h->dt));
+    const int gemv_smem = (int)(sizeof(float) * (size_t)tc_group(h) * (h->W > h->dt ? h->W : h->dt));
     const int mod_smem = (int)(sizeof(float) * (size_t)MOD_GROUP * h->W);
     int dev = 0;
     JPI_CUDA_TRY(cudaGetDevice(&dev));
     JPI_CUDA_TRY(cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, dev));
+    JPI_CUDA_TRY(cudaFuncSetAttribute(k_final_rows<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FIN_SMEM_MAX));
+    JPI_CUDA_TRY(cudaFuncSetAttribute(k_final_rows<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FIN_SMEM_MAX));
     if (h->bf16) {
-        using T = __nv_bfloat16;
-        JPI_CUDA_TRY(cudaFuncSetAttribute(k_gemv_multi<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemv_smem));
-        JPI_CUDA_TRY(cudaFuncSetAttribute(k_gemv_multi<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemv_smem));
-        JPI_TRY(set_mod_attrs<T>(mod_smem));
+        JPI_TRY(set_gemv_attrs<__nv_bfloat16>(gemv_smem));
+        JPI_TRY(set_mod_attrs<__nv_bfloat16>(mod_smem));
     } else {
-        using T = float;
-        JPI_CUDA_TRY(cudaFuncSetAttribute(k_gemv_multi<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemv_smem));
-        JPI_CUDA_TRY(cudaFuncSetAttribute(k_gemv_multi<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemv_smem));
+        JPI_TRY(set_gemv_attrs<float>(gemv_smem));
         JPI_TRY(set_mod_attrs<float>(mod_smem));
     }
     return JPI_OK;
 }
 
-jpi_status launch_time_embed(jpi_handle* h, int nsteps, double t_override, cudaStream_t st) {
-    k_time_embed<<<dim3(nsteps, (h->dt / 2 + 127) / 128), 128, 0, st>>>(h->temb, nsteps, h->dt, h->cfg.t_min_period,
-                                                                      h->cfg.t_max_period, t_override);
+namespace {
+// Embeddings of the step times k / nsteps, or of one given time (t_override >= 0).
+jpi_status time_embed_into(jpi_handle* h, float* temb, int nsteps, double t_override, cudaStream_t st) {
+    k_time_embed<<<dim3(nsteps, (h->dt / 2 + TE_THREADS - 1) / TE_THREADS), TE_THREADS, 0, st>>>(
+        temb, h->t_period, nsteps, h->dt, t_override);
     return check_launch("time embedding");
+}
+}  // namespace
+
+jpi_status launch_time_embed(jpi_handle* h, int nsteps, double t_override, cudaStream_t st) {
+    return time_embed_into(h, h->temb, nsteps, t_override, st);
 }
 
 jpi_status launch_time_conditioning(jpi_handle* h, int nsteps, cudaStream_t st) {
-    return h->bf16 ? time_cond<__nv_bfloat16>(h, nsteps, st) : time_cond<float>(h, nsteps, st);
+    return h->bf16 ? time_cond<__nv_bfloat16>(h, nsteps, h->temb, h->c1, h->cond, st)
+                   : time_cond<float>(h, nsteps, h->temb, h->c1, h->cond, st);
 }
 
 // Time conditioning of one step time with caller-chosen scratch: sinusoid into temb [d_t],
@@ -1283,30 +1440,12 @@ jpi_status launch_time_conditioning(jpi_handle* h, int nsteps, cudaStream_t st) 
 // vectors go to the handle's step-0 slot, as with launch_time_conditioning(h, 1, ...).
 jpi_status launch_time_conditioning_into(jpi_handle* h, double t, float* temb, float* c1,
                                          float* cond, cudaStream_t st) {
-    const int W = h->W, dt = h->dt;
-    const int R = mod_rows(h->L) * W;
-    k_time_embed<<<dim3(1, (dt / 2 + 127) / 128), 128, 0, st>>>(temb, 1, dt, h->cfg.t_min_period, h->cfg.t_max_period, t);
-    const dim3 blk(256);
-    if (h->bf16) {
-        using T = __nv_bfloat16;
-        k_gemv_multi<T, true><<<grid_for((long long)W * 32, 256, 1024), blk, sizeof(float) * dt, st>>>(
-            (const T*)h->time_in_w, h->time_in_b, temb, c1, W, dt, 1);
-        k_gemv_multi<T, true><<<grid_for((long long)W * 32, 256, 1024), blk, sizeof(float) * W, st>>>(
-            (const T*)h->time_out_w, h->time_out_b, c1, cond, W, W, 1);
-        JPI_TRY(mod_gemv<T>(h, 1, cond, h->mods, R, st));
-    } else {
-        using T = float;
-        k_gemv_multi<T, true><<<grid_for((long long)W * 32, 256, 1024), blk, sizeof(float) * dt, st>>>(
-            (const T*)h->time_in_w, h->time_in_b, temb, c1, W, dt, 1);
-        k_gemv_multi<T, true><<<grid_for((long long)W * 32, 256, 1024), blk, sizeof(float) * W, st>>>(
-            (const T*)h->time_out_w, h->time_out_b, c1, cond, W, W, 1);
-        JPI_TRY(mod_gemv<T>(h, 1, cond, h->mods, R, st));
-    }
-    return check_launch("time conditioning (caller scratch)");
+    JPI_TRY(time_embed_into(h, temb, 1, t, st));
+    return h->bf16 ? time_cond<__nv_bfloat16>(h, 1, temb, c1, cond, st) : time_cond<float>(h, 1, temb, c1, cond, st);
 }
 
 jpi_status launch_embed(jpi_handle* h, int step, int B, int C, const float* x, cudaStream_t st) {
-    const int slices = (h->W + 127) / 128, nctx = h->n_ctx();
+    const int slices = (h->W + 511) / 512, nctx = h->n_ctx();
     // Scale and shift of layer 0's attention norm at this step.
     const float* ms = h->mods + (size_t)step * mod_rows(h->L) * h->W;
     EmbedArgs a;
@@ -1330,9 +1469,9 @@ jpi_status launch_embed(jpi_handle* h, int step, int B, int C, const float* x, c
     a.W = h->W;
     a.Sd = h->Sd;
     a.A = h->A;
-    // About eight blocks per SM (a small batch keeps one token per block, the shortest chain), at
-    // most EMB_MAX_TPB tokens each.
-    const long long want = 8ll * h->num_sms;
+    // About two blocks per SM (a small batch keeps one token per block, the shortest chain), at most
+    // EMB_MAX_TPB tokens each.
+    const long long want = 2ll * h->num_sms;
     const long long tpb = ((long long)B * a.S * slices + want - 1) / want;
     a.tpb = (int)(tpb < 1 ? 1 : tpb > EMB_MAX_TPB ? EMB_MAX_TPB : tpb);
     a.action_groups = (B * C + a.tpb - 1) / a.tpb;
@@ -1352,13 +1491,35 @@ jpi_status launch_layer_simt(jpi_handle* h, int layer, int step, int B, int C, c
     return JPI_OK;
 }
 
-jpi_status launch_final(jpi_handle* h, int step, int B, int C, float delta, float* x_inout,
-                        float* v_out, float* out_copy, cudaStream_t st) {
-    const int W = h->W;
+jpi_status launch_final(jpi_handle* h, int step, int B, int C, float delta, float* x_inout, float* v_out,
+                        cudaStream_t st) {
+    const int W = h->W, rows = B * C;
     const float* ms = h->mods + (size_t)step * mod_rows(h->L) * W + (size_t)6 * h->L * W;
-    launch_pdl(h, dim3(B * C), dim3(FIN_THREADS), sizeof(float) * W, st, k_final, (const float*)h->h, ms, ms + W,
-               (const float*)h->action_out_w, (const float*)h->action_out_b, x_inout, v_out, out_copy,
-               C + h->n_ctx(), h->n_ctx(), C, W, h->A, h->cfg.rms_eps, delta);
+    FinalArgs a;
+    a.hres = h->h;
+    a.sigma = ms;
+    a.beta = ms + W;
+    a.Wout = h->action_out_w;
+    a.bout = h->action_out_b;
+    a.x = x_inout;
+    a.vout = v_out;
+    a.rows = rows;
+    a.S = C + h->n_ctx();
+    a.nctx = h->n_ctx();
+    a.C = C;
+    a.W = W;
+    a.A = h->A;
+    a.eps = h->cfg.rms_eps;
+    a.delta = delta;
+    // One row per CTA up to two CTAs per SM, then 4, then 8 rows (while they fit the shared memory).
+    const int fr = rows <= 2 * h->num_sms ? 1 : rows <= 8 * h->num_sms ? 4 : 8;
+    const size_t row = sizeof(float) * (size_t)W;
+    if (fr == 8 && 8 * row <= FIN_SMEM_MAX)
+        launch_pdl(h, dim3((rows + 7) / 8), dim3(FIN_THREADS), 8 * row, st, k_final_rows<8>, a);
+    else if (fr >= 4 && 4 * row <= FIN_SMEM_MAX)
+        launch_pdl(h, dim3((rows + 3) / 4), dim3(FIN_THREADS), 4 * row, st, k_final_rows<4>, a);
+    else
+        launch_pdl(h, dim3(rows), dim3(FIN_THREADS), row, st, k_final, a);
     return check_launch("final norm + Euler");
 }
 
