@@ -45,14 +45,14 @@ int t5_splits(const jpi_handle* h, int blocks, int nb_all) {
 template <int D>
 jpi_status prepare_t5(jpi_handle* h) {
     JPI_CUDA_TRY(cudaFuncSetAttribute(k_attn_t5<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      1024 + T5Smem<D>::TOTAL));
+                                      T5Smem<D>::BYTES));
     // Co-resident clusters of s CTAs along z (the key splits of one row block).
     h->t5_clusters[1] = h->num_sms;
     for (int s = 2; s <= T5_MAX_SPLIT; ++s) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(h->num_sms / s), 1, (unsigned)s);
         cfg.blockDim = dim3(T5_THREADS);
-        cfg.dynamicSmemBytes = 1024 + T5Smem<D>::TOTAL;
+        cfg.dynamicSmemBytes = T5Smem<D>::BYTES;
         cudaLaunchAttribute at;
         at.id = cudaLaunchAttributeClusterDimension;
         at.val.clusterDim.x = 1;
@@ -90,7 +90,7 @@ jpi_status launch_t5(jpi_handle* h, int l, int B, int C, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(rblocks, B, splits);
     cfg.blockDim = dim3(T5_THREADS);
-    cfg.dynamicSmemBytes = 1024 + T5Smem<D>::TOTAL;
+    cfg.dynamicSmemBytes = T5Smem<D>::BYTES;
     cfg.stream = st;
     cudaLaunchAttribute attrs[2];
     int n = 0;

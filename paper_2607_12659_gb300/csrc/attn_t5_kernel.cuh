@@ -11,21 +11,31 @@
 //
 // One CTA = 128 query rows of one request over all of its keys, in blocks of 64 keys (two TMEM
 // score buffers and two shared-memory P buffers, so block i+1's softmax overlaps block i's P V):
-//   warp 0  one thread: bulk tensor copies of the query tile once, then K blocks through a
-//           two-slot ring (K of block i+2 as soon as S_i is done);
-//   warp 1  one thread: V blocks through a two-slot ring of their own (V of block i+2 once
-//           P_i V_i is done); prefix blocks of either may be fetched before the dependency wait;
+//   warp 0  one thread: bulk tensor copies of the query tile once, then K blocks through a ring of
+//           NS slots (K of block i+NS as soon as S_i is done);
+//   warp 1  one thread: V blocks through a ring of their own (V of block i+NS once P_i V_i is
+//           done); prefix blocks of either may be fetched before the dependency wait;
 //   warp 2  one thread: S_i = Q K_i^T (M = 128, N = 64, K = D) into one of two TMEM score
 //           buffers: S_0, S_1, then S_{i+2} as soon as P_i is written (its score buffer is free);
 //   warp 3  one thread: O += P_i V_i (M = 128, N = D, K = 64) into the TMEM output with V read
 //           as an MN-major operand straight from its bulk copy, as soon as P_i and V_i are in.
 //           The two MMA chains are issued by two threads, so neither waits on the other's issue
 //           (one thread issues an N = 64 MMA every ~50-75 cycles, longer than it runs);
-//   warps 4-7  one query row per thread (its TMEM lane): scale, mask, block maximum, softmax
-//           probabilities P_i written to shared memory (bf16, 128-byte swizzled K-major rows).
+//   warps 4-11  two threads per query row (its TMEM lane), 32 of the block's keys each: scale, mask,
+//           block maximum (the halves' exchanged through shared memory), softmax probabilities P_i
+//           written to shared memory (bf16, 128-byte swizzled K-major rows). One thread per row took
+//           about a microsecond per block, longer than the block's MMAs, and set the rate.
 //           The running maximum is only moved, and O rescaled in TMEM, when a block's maximum
 //           exceeds it by more than 8 (log2 units), so probabilities stay below 2^8.
 // At the end every row is divided by its sum and written as bf16. All waits are bounded.
+//
+// Head dim 256 (QT): the query tile is the A operand from tensor memory instead of shared memory, where
+// its 64 KB make room for a third K and V slot. It lands in V slots 1 and 2, the softmax warps copy
+// their rows to TMEM columns 384.. (two bf16 a column), and V_1, V_2 follow. What bounds a block of 64
+// keys (33 of them per CTA at batch 64, prefix 2048; 70.7 us a launch with one softmax thread per row,
+// two slots and MMAs issued under `lane == 0`): the chain from scores through softmax to P V. Two
+// threads per row, single-thread issue the compiler knows of (ptx::elect_one, 72.1 -> 67.6 us) and the
+// third slot (67.6 -> 63.5 us) each shorten it; 17.6 -> 15.2 us at 16 requests and two key splits.
 // Key splits (gridDim.z = S > 1, the S CTAs of a row block forming a cluster along z): CTA s takes
 // the key blocks [s nb / S, (s + 1) nb / S). Past its key loop each CTA writes its rows'
 // unnormalised fp32 outputs and (m, l) to its slot of a workspace in global memory (row-fastest,
@@ -49,8 +59,8 @@ namespace {
 constexpr int T5_ERR_LOAD = 1, T5_ERR_MMA = 2;
 constexpr int T5_ROWS = 128;
 constexpr int T5_KEYS = 64;
-constexpr int T5_STAGES = 2;
-constexpr int T5_THREADS = 256;
+constexpr int T5_THREADS = 384;
+constexpr int T5_COMBINE = 256;   // threads that combine key splits
 constexpr uint64_t T5_WAIT_NS = 200ull * 1000 * 1000;
 constexpr float T5_RESCALE = 8.f;   // log2 units
 
@@ -68,15 +78,21 @@ struct T5Args {
 
 template <int D>
 struct T5Smem {
-    static constexpr int QBYTES = T5_ROWS * D * 2;        // D/64 blocks of [128 rows][128 B]
+    static constexpr bool QT = D == 256;                  // queries in tensor memory
+    static constexpr int NS = QT ? 3 : 2;                 // K and V slots
+    static constexpr int QBYTES = QT ? 0 : T5_ROWS * D * 2;   // D/64 blocks of [128 rows][128 B]
     static constexpr int KVBYTES = T5_KEYS * D * 2;       // D/64 blocks of [64 rows][128 B]
     static constexpr int STAGE = 2 * KVBYTES;             // ring slot s: K then V
     static constexpr int ST_OFF = QBYTES;
     static constexpr int PBYTES = T5_ROWS * T5_KEYS * 2;      // one P buffer [128 rows][128 B]
-    static constexpr int P_OFF = ST_OFF + T5_STAGES * STAGE;   // two P buffers
-    static constexpr int BAR_OFF = P_OFF + 2 * PBYTES;
-    static constexpr int TOTAL = BAR_OFF + 256;
-    static constexpr int TMEM_COLS = D == 256 ? 512 : 256;   // 2 score buffers of 64 + O (D)
+    static constexpr int P_OFF = ST_OFF + NS * STAGE;          // two P buffers
+    static constexpr int XM_OFF = P_OFF + 2 * PBYTES;          // [2 blocks][2 key halves][128 rows] maxima
+    static constexpr int BAR_OFF = XM_OFF + 4 * T5_ROWS * 4;
+    static constexpr int TOTAL = BAR_OFF + 192;
+    static constexpr int BYTES = TOTAL;   // of a launch (the array is declared 1024-byte aligned)
+    static_assert(BYTES <= 227 * 1024, "fits an SM");
+    static constexpr int TMEM_COLS = D == 256 ? 512 : 256;   // 2 score buffers of 64 + O (D) (+ Q, 128)
+    static constexpr uint32_t TMEM_Q = 384;
 };
 
 __device__ __forceinline__ uint32_t pack_bf16x2_t5(float lo, float hi) {
@@ -118,12 +134,12 @@ __device__ __forceinline__ void t5_combine(const T5Args& a, size_t cta, int r_lo
     }
     __syncthreads();
     constexpr int IB = 32 / S;
-    const int nitems = nown * (D / 4);
-    for (int base = tid; base < nitems; base += IB * T5_THREADS) {
+    const int nitems = tid < T5_COMBINE ? nown * (D / 4) : 0;
+    for (int base = tid; base < nitems; base += IB * T5_COMBINE) {
         float4 v[IB][S];
 #pragma unroll
         for (int i = 0; i < IB; ++i) {
-            const int idx = base + i * T5_THREADS;
+            const int idx = base + i * T5_COMBINE;
             if (idx < nitems) {
                 const int c = idx / nown, rr = idx - c * nown;
 #pragma unroll
@@ -133,7 +149,7 @@ __device__ __forceinline__ void t5_combine(const T5Args& a, size_t cta, int r_lo
         }
 #pragma unroll
         for (int i = 0; i < IB; ++i) {
-            const int idx = base + i * T5_THREADS;
+            const int idx = base + i * T5_COMBINE;
             if (idx < nitems) {
                 const int c = idx / nown, rr = idx - c * nown;
                 const int R = row0 + r_lo + rr;
@@ -164,9 +180,10 @@ __device__ __forceinline__ void t5_combine_rows(const T5Args& a, size_t cta, int
                                                 const float2* own_ml, int row0, int nrows, int b, bool ok_all,
                                                 int tid) {
     constexpr int NOWN = T5_ROWS / S;          // rows per split: 64 or 32
-    constexpr int CSTEP = T5_THREADS / NOWN;   // chunks one pass of the block covers
+    constexpr int CSTEP = T5_COMBINE / NOWN;   // chunks one pass covers
     constexpr int NI = (D / 4) / CSTEP;        // chunks per thread
-    static_assert(T5_THREADS % NOWN == 0 && (D / 4) % CSTEP == 0, "rows and chunks tile the block");
+    static_assert(T5_COMBINE % NOWN == 0 && (D / 4) % CSTEP == 0, "rows and chunks tile the block");
+    if (tid >= T5_COMBINE) return;
     const int rr = tid % NOWN, cb = tid / NOWN, r_lo = split * NOWN;
     float2 ml[S];
     float4 v[NI][S];
@@ -223,29 +240,33 @@ __global__ void __launch_bounds__(T5_THREADS, 1) k_attn_t5(const __grid_constant
                                                            const __grid_constant__ CUtensorMap vmap,
                                                            const __grid_constant__ T5Args a) {
     using L = T5Smem<D>;
+    constexpr bool QT = L::QT;
+    constexpr int NS = L::NS;
     constexpr int NDB = D / 64;   // 64-column blocks of a row
     constexpr uint32_t IDESC_S = ptx::idesc_bf16_f32(T5_ROWS, T5_KEYS);
     constexpr uint32_t IDESC_PV = ptx::idesc_bf16_f32(T5_ROWS, D) | (1u << 16);   // B MN-major
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
+    extern __shared__ __align__(1024) uint8_t t5_smem_raw[];
+    uint8_t* smem = t5_smem_raw;
     uint8_t* qs = smem;
     uint8_t* stages = smem + L::ST_OFF;
     uint8_t* ps = smem + L::P_OFF;
+    float* xmax = (float*)(smem + L::XM_OFF);
     uint64_t* bars = (uint64_t*)(smem + L::BAR_OFF);
     uint64_t* qfull = bars;                       // 1
     uint64_t* sfull = bars + 1;                   // 2: score buffer b ready
-    uint64_t* pfull = bars + 3;                   // 2: P buffer b written by the 128 softmax threads
+    uint64_t* pfull = bars + 3;                   // 2: P buffer b written by the 256 softmax threads
     uint64_t* odone = bars + 5;                   // 2: P V of the block in P buffer b done
-    // K and V have their own rings (slot i mod 2), so K of block i+2 is fetched as soon as
-    // S_i is done and V of block i+2 once P_i V_i is done.
-    uint64_t* kfull = bars + 7;                   // T5_STAGES
-    uint64_t* vfull = kfull + T5_STAGES;
-    uint64_t* kempty = vfull + T5_STAGES;
-    uint64_t* vempty = kempty + T5_STAGES;
-    uint32_t* tmem_slot = (uint32_t*)(vempty + T5_STAGES);
+    // K and V have their own rings (slot i mod NS), so K of block i+NS is fetched as soon as
+    // S_i is done and V of block i+NS once P_i V_i is done.
+    uint64_t* kfull = bars + 7;                   // NS
+    uint64_t* vfull = kfull + NS;
+    uint64_t* kempty = vfull + NS;
+    uint64_t* vempty = kempty + NS;
+    uint64_t* qready = vempty + NS;               // QT: every softmax thread has its row in TMEM
+    uint32_t* tmem_slot = (uint32_t*)(qready + 1);
     int* flag = (int*)(tmem_slot + 1);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = ptx::warp_index(), lane = tid & 31;
     const int rb = blockIdx.x, b = blockIdx.y;
     const int nrows = a.S * a.H, nk = a.P + a.S;
     const int row0 = rb * T5_ROWS;
@@ -265,10 +286,11 @@ __global__ void __launch_bounds__(T5_THREADS, 1) k_attn_t5(const __grid_constant
         ptx::mbar_init(&sfull[0], 1);
         ptx::mbar_init(&sfull[1], 1);
         for (int b2 = 0; b2 < 2; ++b2) {
-            ptx::mbar_init(&pfull[b2], 128);
+            ptx::mbar_init(&pfull[b2], 256);
             ptx::mbar_init(&odone[b2], 1);
         }
-        for (int s = 0; s < T5_STAGES; ++s) {
+        ptx::mbar_init(qready, 256);
+        for (int s = 0; s < NS; ++s) {
             ptx::mbar_init(&kfull[s], 1);
             ptx::mbar_init(&vfull[s], 1);
             ptx::mbar_init(&kempty[s], 1);
@@ -284,37 +306,48 @@ __global__ void __launch_bounds__(T5_THREADS, 1) k_attn_t5(const __grid_constant
 
     if (warp <= 1) {
         // Warp 0 streams Q and K, warp 1 streams V.
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             const bool is_v = warp == 1;
             const uint64_t pol = ptx::l2_policy_evict_first();
             const int kv0 = (a.layer * a.maxB + b) * a.kv_rows;
             uint64_t* fullb = is_v ? vfull : kfull;
             uint64_t* emptyb = is_v ? vempty : kempty;
             const CUtensorMap* map = is_v ? &vmap : &kmap;
-            // Block i into ring slot i mod 2: NDB column boxes.
+            // Block i into ring slot i mod NS: NDB column boxes.
             auto load = [&](int i) {
-                const int sl = i % T5_STAGES;
+                const int sl = i % NS;
                 uint8_t* base = stages + sl * L::STAGE + (is_v ? L::KVBYTES : 0);
                 ptx::mbar_expect_tx(&fullb[sl], (uint32_t)L::KVBYTES);
                 for (int db = 0; db < NDB; ++db)
                     ptx::tma_load_2d(base + db * (T5_KEYS * 128), map, &fullb[sl], db * 64,
                                      kv0 + (blk0 + i) * T5_KEYS, pol);
             };
-            // First use of both slots: blocks made only of prefix keys were written before this
-            // graph ran and are fetched before the dependency wait.
+            // First use of the slots: blocks made only of prefix keys were written before this
+            // graph ran and are fetched before the dependency wait (QT: of V only block 0, the other
+            // slots take the query tile first).
+            const int early = QT && is_v ? 1 : NS;
             int first = 0;
-            while (first < T5_STAGES && first < nb && (blk0 + first + 1) * T5_KEYS <= a.P) load(first++);
+            while (first < early && first < nb && (blk0 + first + 1) * T5_KEYS <= a.P) load(first++);
             if (!is_v) ptx::prefetch_tmap(&qmap);
             ptx::grid_dep_wait();
             if (!is_v) {
-                ptx::mbar_expect_tx(qfull, (uint32_t)L::QBYTES);
-                for (int db = 0; db < NDB; ++db)
-                    ptx::tma_load_2d(qs + db * (T5_ROWS * 128), &qmap, qfull, db * 64, b * nrows + row0, pol);
+                ptx::mbar_expect_tx(qfull, (uint32_t)(T5_ROWS * D * 2));
+                for (int db = 0; db < NDB; ++db) {
+                    uint8_t* dst = QT ? stages + (1 + db / 2) * L::STAGE + L::KVBYTES + (db % 2) * (T5_ROWS * 128)
+                                      : qs + db * (T5_ROWS * 128);
+                    ptx::tma_load_2d(dst, &qmap, qfull, db * 64, b * nrows + row0, pol);
+                }
             }
-            for (; first < T5_STAGES && first < nb; ++first) load(first);
-            // Block j once the MMAs that read block j - 2 (S_{j-2}, or P_{j-2} V_{j-2}) are done.
-            for (int j = T5_STAGES; j < nb; ++j) {
-                if (!ptx::mbar_wait_bounded(&emptyb[j % T5_STAGES], ((j - 2) >> 1) & 1, T5_WAIT_NS)) {
+            bool ok = true;
+            if (QT && is_v) {
+                for (; first < 1 && first < nb; ++first) load(first);
+                ok = ptx::mbar_wait_bounded(qready, 0, T5_WAIT_NS);
+                if (!ok) *flag = T5_ERR_LOAD;
+            }
+            for (; ok && first < NS && first < nb; ++first) load(first);
+            // Block j once the MMAs that read block j - NS (S_{j-NS}, or P_{j-NS} V_{j-NS}) are done.
+            for (int j = NS; ok && j < nb; ++j) {
+                if (!ptx::mbar_wait_bounded(&emptyb[j % NS], (j / NS - 1) & 1, T5_WAIT_NS)) {
                     *flag = T5_ERR_LOAD;
                     break;
                 }
@@ -322,26 +355,32 @@ __global__ void __launch_bounds__(T5_THREADS, 1) k_attn_t5(const __grid_constant
             }
         }
     } else if (warp == 2) {
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             const uint32_t qb = ptx::smem_u32(qs), sb = ptx::smem_u32(stages);
-            bool good = ptx::mbar_wait_bounded(qfull, 0, T5_WAIT_NS);
-            // S_i = Q K_i^T into score buffer i mod 2; K slot i mod 2 is released when it is done.
+            bool good = ptx::mbar_wait_bounded(QT ? qready : qfull, 0, T5_WAIT_NS);
+            // S_i = Q K_i^T into score buffer i mod 2; K slot i mod NS is released when it is done.
             auto issue_s = [&](int i) {
-                const int sl = i % T5_STAGES;
-                if (!ptx::mbar_wait_bounded(&kfull[sl], (i >> 1) & 1, T5_WAIT_NS)) good = false;
+                const int sl = i % NS;
+                if (!ptx::mbar_wait_bounded(&kfull[sl], (i / NS) & 1, T5_WAIT_NS)) good = false;
                 ptx::tc_fence_after();
                 if (good) {
-                    const uint32_t kb = sb + sl * L::STAGE;
+                    const uint64_t kb = ptx::desc_sw128(sb + sl * L::STAGE), qd = ptx::desc_sw128(qb);
+#pragma unroll
                     for (int db = 0; db < NDB; ++db)
 #pragma unroll
-                        for (int kk = 0; kk < 4; ++kk)
-                            ptx::mma_bf16(tmem + (uint32_t)(64 * (i & 1)),
-                                          ptx::desc_sw128(qb + db * (T5_ROWS * 128) + kk * 32),
-                                          ptx::desc_sw128(kb + db * (T5_KEYS * 128) + kk * 32), IDESC_S,
-                                          (db | kk) != 0);
+                        for (int kk = 0; kk < 4; ++kk) {
+                            const uint64_t kd = ptx::desc_add(kb, db * (T5_KEYS * 128) + kk * 32);
+                            const uint32_t d = tmem + (uint32_t)(64 * (i & 1));
+                            if constexpr (QT)
+                                ptx::mma_bf16_ta(d, tmem + L::TMEM_Q + (uint32_t)(8 * (4 * db + kk)), kd, IDESC_S,
+                                                 (db | kk) != 0);
+                            else
+                                ptx::mma_bf16(d, ptx::desc_add(qd, db * (T5_ROWS * 128) + kk * 32), kd, IDESC_S,
+                                              (db | kk) != 0);
+                        }
                 }
                 ptx::mma_commit(&sfull[i & 1]);
-                if (i + T5_STAGES < nb) ptx::mma_commit(&kempty[sl]);
+                if (i + NS < nb) ptx::mma_commit(&kempty[sl]);
             };
             if (nb > 0) issue_s(0);
             if (nb > 1) issue_s(1);
@@ -354,72 +393,105 @@ __global__ void __launch_bounds__(T5_THREADS, 1) k_attn_t5(const __grid_constant
             if (!good) *flag = T5_ERR_MMA;
         }
     } else if (warp == 3) {
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             const uint32_t sb = ptx::smem_u32(stages), pb = ptx::smem_u32(ps);
             bool good = true;
             for (int i = 0; i < nb; ++i) {
-                const int sl = i % T5_STAGES;
+                const int sl = i % NS;
                 if (!ptx::mbar_wait_bounded(&pfull[i & 1], (i >> 1) & 1, T5_WAIT_NS)) good = false;
-                if (!ptx::mbar_wait_bounded(&vfull[sl], (i >> 1) & 1, T5_WAIT_NS)) good = false;
+                if (!ptx::mbar_wait_bounded(&vfull[sl], (i / NS) & 1, T5_WAIT_NS)) good = false;
                 ptx::tc_fence_after();
                 if (good) {
-                    const uint32_t vb = sb + sl * L::STAGE + L::KVBYTES;
-                    const uint32_t pbi = pb + (uint32_t)((i & 1) * L::PBYTES);
+                    const uint64_t vb = ptx::desc_sw128_mn(sb + sl * L::STAGE + L::KVBYTES, T5_KEYS * 128, 1024);
+                    const uint64_t pbi = ptx::desc_sw128(pb + (uint32_t)((i & 1) * L::PBYTES));
 #pragma unroll
                     for (int kk = 0; kk < T5_KEYS / 16; ++kk)
-                        ptx::mma_bf16(tmem + 128u, ptx::desc_sw128(pbi + kk * 32),
-                                      ptx::desc_sw128_mn(vb + kk * 16 * 128, T5_KEYS * 128, 1024), IDESC_PV,
+                        ptx::mma_bf16(tmem + 128u, ptx::desc_add(pbi, kk * 32), ptx::desc_add(vb, kk * 16 * 128), IDESC_PV,
                                       (i | kk) != 0);
                 }
-                if (i + T5_STAGES < nb) ptx::mma_commit(&vempty[sl]);
+                if (i + NS < nb) ptx::mma_commit(&vempty[sl]);
                 ptx::mma_commit(&odone[i & 1]);
             }
             if (!good) *flag = T5_ERR_MMA;
         }
     } else {
-        // ---- softmax: one query row per thread ----
-        const int row = (warp & 3) * 32 + lane;
+        // ---- softmax: two threads per query row, half of a block's keys each ----
+        const int row = (warp & 3) * 32 + lane, half = (warp - 4) >> 2;
         const int R = row0 + row;
         const bool valid = R < nrows;
         // Visible keys: state and context rows see the prefix and each other; padding rows none.
         const int nvis = !valid ? 0 : R / a.H < a.nctx ? a.P + a.nctx : nk;
         const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-        float m_used = -INFINITY, l = 0.f;
+        const uint32_t pair_bar = 1 + (warp & 3);   // the two warps of these 32 rows
+        float m_used = -INFINITY, l = 0.f;          // m_used is the same in both threads of a row
         bool good = true;
+        if constexpr (QT) {
+            // This row of the query tile from its staging (V slots 1 and 2, 128-byte swizzled rows)
+            // to TMEM, half of it per thread: column 32 db + 4 c + e holds elements 64 db + 8 c + 2 e, + 1.
+            if (!ptx::mbar_wait_bounded(qfull, 0, T5_WAIT_NS)) good = false;
+#pragma unroll
+            for (int d2 = 0; d2 < NDB / 2; ++d2) {
+                const int db = half * (NDB / 2) + d2;
+                const uint8_t* src = stages + (1 + db / 2) * L::STAGE + L::KVBYTES + (db % 2) * (T5_ROWS * 128) + row * 128;
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf) {
+                    uint32_t rq[16];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        const uint4 v = *(const uint4*)(src + (((4 * hf + c) ^ (row & 7)) << 4));
+                        rq[4 * c] = v.x;
+                        rq[4 * c + 1] = v.y;
+                        rq[4 * c + 2] = v.z;
+                        rq[4 * c + 3] = v.w;
+                    }
+                    ptx::tmem_st_x16(lane_base + L::TMEM_Q + (uint32_t)(32 * db + 16 * hf), rq);
+                }
+            }
+            ptx::tmem_st_wait();
+            ptx::tc_fence_before();
+            ptx::mbar_arrive(qready);
+        }
+        constexpr int HK = T5_KEYS / 2;   // keys per thread
         for (int i = 0; i < nb; ++i) {
             if (!ptx::mbar_wait_bounded(&sfull[i & 1], (i >> 1) & 1, T5_WAIT_NS)) good = false;
             ptx::tc_fence_after();
-            // The block's 64 raw scores: four loads in flight, one wait.
-            uint32_t r[4][16];
+            // This thread's 32 raw scores.
+            uint32_t r[2][16];
             {
-                const uint32_t sa = lane_base + (uint32_t)(64 * (i & 1));
+                const uint32_t sa = lane_base + (uint32_t)(64 * (i & 1) + HK * half);
                 ptx::tmem_ld_x16(sa, r[0]);
                 ptx::tmem_ld_x16(sa + 16u, r[1]);
-                ptx::tmem_ld_x16(sa + 32u, r[2]);
-                ptx::tmem_ld_x16(sa + 48u, r[3]);
                 ptx::tmem_ld_wait();
             }
-            // Keys of this block the row sees: all of them except in the last block(s).
-            const int vis = nvis - (blk0 + i) * T5_KEYS;
-            const bool full = vis >= T5_KEYS;
+            // Keys of this half block the row sees: all of them except in the last block(s).
+            const int vis = nvis - (blk0 + i) * T5_KEYS - HK * half;
+            const bool full = __all_sync(0xffffffffu, vis >= HK);   // warp-uniform
             // Block maximum in log2 units (the scale is positive, so it commutes with the max);
-            // four independent chains.
+            // four independent chains, then the other half's through shared memory.
             float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+            if (full) {
 #pragma unroll
-            for (int j = 0; j < 16; ++j)
+                for (int j = 0; j < HK; ++j) m4[j & 3] = fmaxf(m4[j & 3], __uint_as_float(r[j >> 4][j & 15]));
+            } else {
 #pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    if (full || 16 * q + j < vis) m4[q] = fmaxf(m4[q], __uint_as_float(r[q][j]));
-            const float mb = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * a.scale_log2;
+                for (int j = 0; j < HK; ++j)
+                    if (j < vis) m4[j & 3] = fmaxf(m4[j & 3], __uint_as_float(r[j >> 4][j & 15]));
+            }
+            float mb = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+            float* xm = xmax + (i & 1) * 2 * T5_ROWS + row;
+            xm[half * T5_ROWS] = mb;
+            ptx::named_bar_sync(pair_bar, 64);
+            mb = fmaxf(mb, xm[(1 - half) * T5_ROWS]) * a.scale_log2;
             const bool move = mb > m_used + T5_RESCALE;
             const float alpha = !move ? 1.f : m_used == -INFINITY ? 0.f : ex2(m_used - mb);
-            // TMEM loads and stores are warp-collective: the warp rescales together, lanes whose
-            // maximum stays put multiply by 1. O is settled once P V of the previous block is done.
+            // TMEM loads and stores are warp-collective: the warp rescales together (its half of the
+            // columns), lanes whose maximum stays put multiply by 1. O is settled once P V of the
+            // previous block is done.
             if (__any_sync(0xffffffffu, move && i > 0 && m_used != -INFINITY)) {
                 if (!ptx::mbar_wait_bounded(&odone[(i - 1) & 1], ((i - 1) >> 1) & 1, T5_WAIT_NS)) good = false;
                 ptx::tc_fence_after();
 #pragma unroll 1
-                for (int c0 = 0; c0 < D; c0 += 16) {
+                for (int c0 = half * (D / 2); c0 < (half + 1) * (D / 2); c0 += 16) {
                     uint32_t ro[16];
                     ptx::tmem_ld_x16(lane_base + 128u + (uint32_t)c0, ro);
                     ptx::tmem_ld_wait();
@@ -438,34 +510,44 @@ __global__ void __launch_bounds__(T5_THREADS, 1) k_attn_t5(const __grid_constant
             const bool seen = m_used != -INFINITY;
             const float neg_m = seen ? -m_used : 0.f;
             float l4[4] = {0.f, 0.f, 0.f, 0.f};
-            uint32_t pk[T5_KEYS / 2];
+            uint32_t pk[HK / 2];
+            if (full && __all_sync(0xffffffffu, seen)) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-#pragma unroll
-                for (int j = 0; j < 16; j += 2) {
-                    const int k = 16 * q + j;
-                    float p0 = ex2(fmaf(__uint_as_float(r[q][j]), a.scale_log2, neg_m));
-                    float p1 = ex2(fmaf(__uint_as_float(r[q][j + 1]), a.scale_log2, neg_m));
-                    if (!full || !seen) {
-                        p0 = (seen && k < vis) ? p0 : 0.f;
-                        p1 = (seen && k + 1 < vis) ? p1 : 0.f;
-                    }
-                    l4[q] += p0 + p1;
+                for (int k = 0; k < HK; k += 2) {
+                    const float p0 = ex2(fmaf(__uint_as_float(r[k >> 4][k & 15]), a.scale_log2, neg_m));
+                    const float p1 = ex2(fmaf(__uint_as_float(r[k >> 4][(k + 1) & 15]), a.scale_log2, neg_m));
+                    l4[(k >> 1) & 3] += p0 + p1;
                     pk[k / 2] = pack_bf16x2_t5(p0, p1);
                 }
+            } else {
+#pragma unroll
+                for (int k = 0; k < HK; k += 2) {
+                    float p0 = ex2(fmaf(__uint_as_float(r[k >> 4][k & 15]), a.scale_log2, neg_m));
+                    float p1 = ex2(fmaf(__uint_as_float(r[k >> 4][(k + 1) & 15]), a.scale_log2, neg_m));
+                    p0 = (seen && k < vis) ? p0 : 0.f;
+                    p1 = (seen && k + 1 < vis) ? p1 : 0.f;
+                    l4[(k >> 1) & 3] += p0 + p1;
+                    pk[k / 2] = pack_bf16x2_t5(p0, p1);
+                }
+            }
             l += (l4[0] + l4[1]) + (l4[2] + l4[3]);
             // P buffer i mod 2 is free once P V of block i - 2 is done.
             if (i >= 2 && !ptx::mbar_wait_bounded(&odone[i & 1], ((i - 2) >> 1) & 1, T5_WAIT_NS)) good = false;
             ptx::tc_fence_after();
-            // Row `row` of P: 8 chunks of 16 bytes, chunk c at position c ^ (row mod 8).
+            // Row `row` of P: 8 chunks of 16 bytes (this thread's four), chunk c at position c ^ (row mod 8).
             uint4* prow = (uint4*)(ps + (i & 1) * L::PBYTES + row * 128);
 #pragma unroll
-            for (int c = 0; c < 8; ++c)
-                prow[c ^ (row & 7)] = make_uint4(pk[4 * c], pk[4 * c + 1], pk[4 * c + 2], pk[4 * c + 3]);
+            for (int c = 0; c < 4; ++c)
+                prow[(4 * half + c) ^ (row & 7)] = make_uint4(pk[4 * c], pk[4 * c + 1], pk[4 * c + 2], pk[4 * c + 3]);
             ptx::fence_proxy_async_smem();
             ptx::tc_fence_before();
             ptx::mbar_arrive(&pfull[i & 1]);
         }
+        // The row's sum: both halves, in order.
+        float* xl = xmax + (nb & 1) * 2 * T5_ROWS + row;   // not the buffer of the last block's maxima
+        xl[half * T5_ROWS] = l;
+        ptx::named_bar_sync(pair_bar, 64);
+        l = xl[0] + xl[T5_ROWS];
         // Every P V is done (both buffers' last commits observed, so none arrives after exit).
         if (nb >= 2 && !ptx::mbar_wait_bounded(&odone[(nb - 2) & 1], ((nb - 2) >> 1) & 1, T5_WAIT_NS)) good = false;
         if (nb >= 1 && !ptx::mbar_wait_bounded(&odone[(nb - 1) & 1], ((nb - 1) >> 1) & 1, T5_WAIT_NS)) good = false;
@@ -477,7 +559,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) k_attn_t5(const __grid_constant
         const float inv = l > 0.f ? 1.f / l : 0.f;
         __nv_bfloat16* orow = a.o + ((size_t)b * nrows + R) * D;
 #pragma unroll 1
-        for (int c0 = 0; c0 < D && nsplit == 1; c0 += 32) {
+        for (int c0 = half * (D / 2); c0 < (half + 1) * (D / 2) && nsplit == 1; c0 += 32) {
             uint32_t r[2][16];
             ptx::tmem_ld_x16(lane_base + 128u + (uint32_t)c0, r[0]);
             ptx::tmem_ld_x16(lane_base + 128u + (uint32_t)(c0 + 16), r[1]);
@@ -502,20 +584,21 @@ __global__ void __launch_bounds__(T5_THREADS, 1) k_attn_t5(const __grid_constant
         // ---- combine the key splits of this row block through the workspace ----
         const size_t cta = ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * nsplit;   // split 0 of the row block
         // With 2 or 4 splits the rows this CTA combines are whole warps' rows: those warps keep
-        // their partials in shared memory (over the query tile; every MMA is done) and their
+        // their partials in shared memory (from its start, over the query tile or the K/V slots; every
+        // copy has been consumed and every MMA is done) and their
         // (m, l) over the P buffers.
         const bool rows_fixed = nsplit == 2 || nsplit == 4;
         const int nown_fixed = rows_fixed ? T5_ROWS / nsplit : 0;
         float4* own = reinterpret_cast<float4*>(smem);
         float2* own_ml = reinterpret_cast<float2*>(ps);
         if (warp >= 4) {
-            const int row = (warp & 3) * 32 + lane;
+            const int row = (warp & 3) * 32 + lane, half = (warp - 4) >> 2;   // half of the columns
             const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
             const bool mine = rows_fixed && row / nown_fixed == split;   // warp-uniform
             float4* dst = mine ? own + (row - split * nown_fixed) : a.ws + (cta + split) * (size_t)(D / 4) * T5_ROWS + row;
             const int stride = mine ? nown_fixed : T5_ROWS;
 #pragma unroll 1
-            for (int c0 = 0; c0 < D; c0 += 32) {
+            for (int c0 = half * (D / 2); c0 < (half + 1) * (D / 2); c0 += 32) {
                 uint32_t r[2][16];
                 ptx::tmem_ld_x16(lane_base + 128u + (uint32_t)c0, r[0]);
                 ptx::tmem_ld_x16(lane_base + 128u + (uint32_t)(c0 + 16), r[1]);
@@ -526,7 +609,8 @@ __global__ void __launch_bounds__(T5_THREADS, 1) k_attn_t5(const __grid_constant
                         make_float4(__uint_as_float(r[v >> 2][4 * (v & 3)]), __uint_as_float(r[v >> 2][4 * (v & 3) + 1]),
                                     __uint_as_float(r[v >> 2][4 * (v & 3) + 2]), __uint_as_float(r[v >> 2][4 * (v & 3) + 3]));
             }
-            if (mine) own_ml[row - split * nown_fixed] = make_float2(x_m, x_l);
+            if (half != 0) {
+            } else if (mine) own_ml[row - split * nown_fixed] = make_float2(x_m, x_l);
             else a.wml[(cta + split) * T5_ROWS + row] = make_float2(x_m, x_l);
         }
         // Every split's rows are in the workspace (the barrier orders global memory at cluster scope;
@@ -534,7 +618,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) k_attn_t5(const __grid_constant
         ptx::tc_fence_before();
         ptx::cluster_sync_all();
         ptx::tc_fence_after();
-        float* wsm = reinterpret_cast<float*>(smem);   // [rows][S] weights, over the query tile
+        float* wsm = reinterpret_cast<float*>(smem);   // [rows][S] weights, over the same bytes
         const int rps = (T5_ROWS + nsplit - 1) / nsplit;
         const int r_lo = split * rps;
         const int nown = max(0, min(T5_ROWS, r_lo + rps) - r_lo);

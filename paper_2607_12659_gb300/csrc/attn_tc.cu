@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(AT_THREADS) k_attn_tc(const __grid_constant__ 
     uint64_t* qbar = rbar + 1;                           // the query tile's bulk copies
     uint64_t* kvbar = rbar + 2;                          // [NBUF] each K/V buffer's bulk copies
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = ptx::warp_index(), lane = tid & 31;
     const int rg = warp & 1, kh = warp >> 1;             // row group, key half / column half
     const int rb = blockIdx.x, b = blockIdx.z;
     const int nrows = a.S * a.H, nk = a.P + a.S;
@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(AT_THREADS) k_attn_tc(const __grid_constant__ 
     // A first block made only of prefix keys (written before this graph ran) is fetched before
     // the dependency wait; one holding suffix keys (written by the QKV kernel) after it.
     const bool early = min(k_end, k_begin + KB) <= a.P;
-    if (tid == 0) {
+    if (warp == 0 && ptx::elect_one()) {
         ptx::prefetch_tmap(&qmap);
         if (early) load_block(k_begin, 0);
     }
@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(AT_THREADS) k_attn_tc(const __grid_constant__ 
 
     // Query block: D/64 bulk tensor copies of 32 rows (rows past this request's S*H rows are
     // the next request's or zero fill; their results are never stored).
-    if (tid == 0) {
+    if (warp == 0 && ptx::elect_one()) {
         ptx::mbar_expect_tx(qbar, (uint32_t)(AT_ROWS * D * 2));
         for (int db = 0; db < D / 64; ++db)
             ptx::tma_load_2d(qs + db * (AT_ROWS * 128), &qmap, qbar, db * 64, b * nrows + row0, pol);
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(AT_THREADS) k_attn_tc(const __grid_constant__ 
         // Block jb sits in buffer jb mod NBUF (its (jb / NBUF)-th use); with two buffers the next
         // block is fetched into the other one while this one is processed.
         const int bi = NBUF == 2 ? (jb & 1) : 0;
-        if (tid == 0) {
+        if (warp == 0 && ptx::elect_one()) {
             if (NBUF == 2 && key0 + KB < k_end) load_block(key0 + KB, bi ^ 1);
             if (NBUF == 1 && key0 != k_begin) load_block(key0, 0);
         }

@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(BIG_THREADS, 1) k_tc_gemm_big(const __grid_con
     uint32_t* tmem_slot = (uint32_t*)(pfree + 1);
     int* flag = (int*)(tmem_slot + 1);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = ptx::warp_index(), lane = tid & 31;
     const int rank = S == 1 ? 0 : (int)ptx::cluster_rank();
     const int nkb = a.nkb / S;                 // K blocks of this CTA
     const int kb0 = rank * nkb;
@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(BIG_THREADS, 1) k_tc_gemm_big(const __grid_con
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             const uint64_t pol = ptx::l2_policy_evict_first();
             auto load_w = [&](int tile, int kb, int s) {
                 ptx::mbar_expect_tx(&full[s], (uint32_t)BIG_STAGE_BYTES);
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(BIG_THREADS, 1) k_tc_gemm_big(const __grid_con
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             const uint32_t base = ptx::smem_u32(stages);
             bool good = true;
             int it = 0;
@@ -169,10 +169,10 @@ __global__ void __launch_bounds__(BIG_THREADS, 1) k_tc_gemm_big(const __grid_con
                     if (good && !ptx::mbar_wait_bounded(&full[s], n & 1, WAIT_LIMIT_NS)) good = false;
                     ptx::tc_fence_after();
                     if (good) {
-                        const uint32_t w = base + s * BIG_STAGE_BYTES, x = w + TILE_BYTES;
+                        const uint64_t w = ptx::desc_sw128(base + s * BIG_STAGE_BYTES), x = ptx::desc_add(w, TILE_BYTES);
 #pragma unroll
                         for (int kk = 0; kk < KBLK / 16; ++kk)
-                            ptx::mma_bf16(acc, ptx::desc_sw128(w + kk * 32), ptx::desc_sw128(x + kk * 32), IDESC,
+                            ptx::mma_bf16(acc, ptx::desc_add(w, kk * 32), ptx::desc_add(x, kk * 32), IDESC,
                                           (kb | kk) != 0);
                     }
                     ptx::mma_commit(&empty[s]);

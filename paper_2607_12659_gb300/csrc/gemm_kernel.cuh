@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_tc_gemm(const __grid_consta
     uint32_t* tmem_slot = (uint32_t*)(bars + 4);
     int* flag = (int*)(tmem_slot + 1);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = ptx::warp_index(), lane = tid & 31;
     const int rank = (int)ptx::cluster_rank();
     const int tile = blockIdx.x / a.splits;
     const int kb0 = rank * a.kpb;
@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_tc_gemm(const __grid_consta
     const uint32_t tmem = *tmem_slot;
 
     // Weight tiles depend on nothing upstream: start streaming them before the dependency wait.
-    if (tid == 0) {
+    if (warp == 0 && ptx::elect_one()) {
         const uint64_t pol = ptx::l2_policy_evict_first();
         ptx::mbar_expect_tx(&bars[0], (uint32_t)(a.kpb * TILE_BYTES));
         for (int j = 0; j < a.kpb; ++j)
@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_tc_gemm(const __grid_consta
         const int tt = blockIdx.y;   // token tile
         const int tok0 = tt * TT;
         // ---- 1. B operand (64 rows from row tt * 64 of the operand buffer) ----
-        if (tid == 0) {
+        if (warp == 0 && ptx::elect_one()) {
             const uint64_t pol = ptx::l2_policy_evict_first();
             ptx::mbar_expect_tx(&bars[1], (uint32_t)(a.kpb * XBLK_BYTES));
             for (int j = 0; j < a.kpb; ++j)
@@ -146,20 +146,19 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_tc_gemm(const __grid_consta
             ptx::mbar_expect_tx(&bars[3], (uint32_t)((a.splits - 1) * 2 * npairs * 128));
 
         // ---- 2. MMA: D[128 rows][64 columns] over this CTA's K blocks ----
-        if (tid == 0 && *flag == 0) {
+        if (warp == 0 && ptx::elect_one()) {
             bool ok_in = ptx::mbar_wait_bounded(&bars[1], 0, WAIT_LIMIT_NS);
             if (ok_in) ok_in = ptx::mbar_wait_bounded(&bars[0], 0, WAIT_LIMIT_NS);
             if (!ok_in) {
                 *flag = DEV_TIMEOUT_WEIGHTS;
             } else {
                 ptx::tc_fence_after();
-                const uint32_t wbase = ptx::smem_u32(wsm), xbase = ptx::smem_u32(xsm);
+                const uint64_t wd = ptx::desc_sw128(ptx::smem_u32(wsm)), xd = ptx::desc_sw128(ptx::smem_u32(xsm));
                 for (int j = 0; j < a.kpb; ++j)
 #pragma unroll
                     for (int kk = 0; kk < KBLK / 16; ++kk)
-                        ptx::mma_bf16(tmem, ptx::desc_sw128(wbase + j * TILE_BYTES + kk * 32),
-                                      ptx::desc_sw128(xbase + j * XBLK_BYTES + kk * 32), IDESC,
-                                      (j | kk) != 0);
+                        ptx::mma_bf16(tmem, ptx::desc_add(wd, j * TILE_BYTES + kk * 32),
+                                      ptx::desc_add(xd, j * XBLK_BYTES + kk * 32), IDESC, (j | kk) != 0);
             }
             // Committed even after a timeout so that the wait below completes.
             ptx::mma_commit(&bars[2]);

@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(RT_THREADS, 1) k_tc_gemm_rows(const __grid_con
     uint32_t* tmem_slot = (uint32_t*)(acce + 2);
     int* flag = (int*)(tmem_slot + 1);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = ptx::warp_index(), lane = tid & 31;
     const int nkb = a.nkb;
     const int ntn = (a.ntiles + 1) / 2, ntm = (a.Mt + TT - 1) / TT;
     const int total = ntn * ntm;
@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(RT_THREADS, 1) k_tc_gemm_rows(const __grid_con
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             const uint64_t pol = ptx::l2_policy_evict_first();
             // Both weight tiles' k-blocks (rows past the last tile arrive as zeros).
             auto load_w = [&](int tn, int kb, int s) {
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(RT_THREADS, 1) k_tc_gemm_rows(const __grid_con
                 (void)ptx::mbar_wait_bounded(&full[i % RT_STAGES], (i / RT_STAGES) & 1, WAIT_LIMIT_NS);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             const uint32_t base = ptx::smem_u32(stages);
             bool good = true;
             int it = 0;
@@ -136,10 +136,10 @@ __global__ void __launch_bounds__(RT_THREADS, 1) k_tc_gemm_rows(const __grid_con
                     if (good && !ptx::mbar_wait_bounded(&full[s], n & 1, WAIT_LIMIT_NS)) good = false;
                     ptx::tc_fence_after();
                     if (good) {
-                        const uint32_t x = base + s * RT_STAGE_BYTES, w = x + RT_XBYTES;
+                        const uint64_t x = ptx::desc_sw128(base + s * RT_STAGE_BYTES), w = ptx::desc_add(x, RT_XBYTES);
 #pragma unroll
                         for (int kk = 0; kk < KBLK / 16; ++kk)
-                            ptx::mma_bf16(acc, ptx::desc_sw128(x + kk * 32), ptx::desc_sw128(w + kk * 32), IDESC,
+                            ptx::mma_bf16(acc, ptx::desc_add(x, kk * 32), ptx::desc_add(w, kk * 32), IDESC,
                                           (kb | kk) != 0);
                     }
                     ptx::mma_commit(&empty[s]);

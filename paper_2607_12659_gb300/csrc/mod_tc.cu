@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(MT_THREADS, 1) k_mod_tc(const __grid_constant_
     uint32_t* tmem_slot = (uint32_t*)(acce + 2);
     int* flag = (int*)(tmem_slot + 1);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = ptx::warp_index(), lane = tid & 31;
     const int ntiles = R / MT_ROWS;
     const int t0 = blockIdx.x, dt = gridDim.x;
     const int my_tiles = t0 < ntiles ? (ntiles - t0 + dt - 1) / dt : 0;
@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(MT_THREADS, 1) k_mod_tc(const __grid_constant_
     };
     // The weights do not depend on the previous kernel: fill the ring before waiting for it.
     const int npre = total < MT_STAGES ? total : MT_STAGES;
-    if (tid == 0)
+    if (warp == 0 && ptx::elect_one())
         for (int it = 0; it < npre; ++it) load(it);
     ptx::grid_dep_wait();
 
@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(MT_THREADS, 1) k_mod_tc(const __grid_constant_
     __syncthreads();
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             int issued = npre;
             for (int it = npre; it < total; ++it) {
                 const int s = it % MT_STAGES, n = it / MT_STAGES;
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(MT_THREADS, 1) k_mod_tc(const __grid_constant_
                     *flag = DEV_TIMEOUT_WEIGHTS;
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             constexpr uint32_t IDESC = ptx::idesc_bf16_f32(MT_ROWS, MT_N);
             const uint32_t rbase = ptx::smem_u32(ring), xbase = ptx::smem_u32(xop);
             bool good = true;

@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pf_gemm(const __grid_constant
     uint32_t* tmem_slot = (uint32_t*)(acce + 2);
     int* flag = (int*)(tmem_slot + 1);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = ptx::warp_index(), lane = tid & 31;
     const int nkb = (a.K + PG_KBLK - 1) / PG_KBLK;
     const int ntn = (a.N + PG_TN - 1) / PG_TN, ntm = (a.M + PG_TM - 1) / PG_TM;
     const int total = ntn * ntm * a.ksplit;
@@ -441,7 +441,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pf_gemm(const __grid_constant
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             int it = 0, issued = 0;
             bool ok = true;
             for (int u = u0; u < total && ok; u += du) {
@@ -468,7 +468,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pf_gemm(const __grid_constant
                     *flag = PF_DEV_TIMEOUT_LOAD;
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             constexpr uint32_t IDESC = ptx::idesc_bf16_f32(PG_TM, PG_TN);
             const uint32_t base = ptx::smem_u32(stages);
             bool good = true;
@@ -485,10 +485,10 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pf_gemm(const __grid_constant
                     if (good && !ptx::mbar_wait_bounded(&full[s], n & 1, PG_WAIT_NS)) good = false;
                     ptx::tc_fence_after();
                     if (good) {
-                        const uint32_t x = base + (uint32_t)(s * PG_STAGE_BYTES), w = x + PG_XBYTES;
+                        const uint64_t x = ptx::desc_sw128(base + (uint32_t)(s * PG_STAGE_BYTES)), w = ptx::desc_add(x, PG_XBYTES);
 #pragma unroll
                         for (int kk = 0; kk < PG_KBLK / 16; ++kk)
-                            ptx::mma_bf16(acc, ptx::desc_sw128(x + kk * 32), ptx::desc_sw128(w + kk * 32), IDESC,
+                            ptx::mma_bf16(acc, ptx::desc_add(x, kk * 32), ptx::desc_add(w, kk * 32), IDESC,
                                           (kb != kb_lo) || (kk != 0));
                     }
                     ptx::mma_commit(&empty[s]);
@@ -774,7 +774,7 @@ jpi_status attention_t5(jpi_prefill_handle* h, cudaStream_t st, const __nv_bfloa
     a.o = h->o;
     a.err = h->dev_err;
     const dim3 grid((unsigned)((nrows + jpi::T5_ROWS - 1) / jpi::T5_ROWS), (unsigned)batch);
-    jpi::k_attn_t5<D><<<grid, jpi::T5_THREADS, 1024 + jpi::T5Smem<D>::TOTAL, st>>>(qmap, kmap, vmap, a);
+    jpi::k_attn_t5<D><<<grid, jpi::T5_THREADS, jpi::T5Smem<D>::BYTES, st>>>(qmap, kmap, vmap, a);
     PF_CUDA(cudaGetLastError());
     return JPI_OK;
 }
@@ -858,9 +858,9 @@ jpi_status setup(jpi_prefill_handle* h, const jpi_prefill_config* c, const jpi_p
     PF_CUDA(cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, device));
     PF_CUDA(cudaFuncSetAttribute(k_pf_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM));
     PF_CUDA(cudaFuncSetAttribute(jpi::k_attn_t5<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 1024 + jpi::T5Smem<128>::TOTAL));
+                                 jpi::T5Smem<128>::BYTES));
     PF_CUDA(cudaFuncSetAttribute(jpi::k_attn_t5<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 1024 + jpi::T5Smem<256>::TOTAL));
+                                 jpi::T5Smem<256>::BYTES));
     PF_TRY(pf_alloc(h, &h->dev_err, 1));
     PF_CUDA(cudaMemset(h->dev_err, 0, sizeof(int)));
     float* staging = nullptr;
