@@ -16,7 +16,7 @@
 //   warp 1  one thread: V blocks through a ring of their own (V of block i+NS once P_i V_i is
 //           done); prefix blocks of either may be fetched before the dependency wait;
 //   warp 2  one thread: S_i = Q K_i^T (M = 128, N = 64, K = D) into one of two TMEM score
-//           buffers: S_0, S_1, then S_{i+2} as soon as P_i is written (its score buffer is free);
+//           buffers: S_0, S_1, then S_{i+2} as soon as the softmax has read S_i into registers;
 //   warp 3  one thread: O += P_i V_i (M = 128, N = D, K = 64) into the TMEM output with V read
 //           as an MN-major operand straight from its bulk copy, as soon as P_i and V_i are in.
 //           The two MMA chains are issued by two threads, so neither waits on the other's issue
@@ -263,7 +263,8 @@ __global__ void __launch_bounds__(T5_THREADS, 1) k_attn_t5(const __grid_constant
     uint64_t* kempty = vfull + NS;
     uint64_t* vempty = kempty + NS;
     uint64_t* qready = vempty + NS;               // QT: every softmax thread has its row in TMEM
-    uint32_t* tmem_slot = (uint32_t*)(qready + 1);
+    uint64_t* sfree = qready + 1;                 // 2: score buffer b has been read by the softmax threads
+    uint32_t* tmem_slot = (uint32_t*)(sfree + 2);
     int* flag = (int*)(tmem_slot + 1);
 
     const int tid = threadIdx.x, warp = ptx::warp_index(), lane = tid & 31;
@@ -287,6 +288,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) k_attn_t5(const __grid_constant
         ptx::mbar_init(&sfull[1], 1);
         for (int b2 = 0; b2 < 2; ++b2) {
             ptx::mbar_init(&pfull[b2], 256);
+            ptx::mbar_init(&sfree[b2], 256);
             ptx::mbar_init(&odone[b2], 1);
         }
         ptx::mbar_init(qready, 256);
@@ -384,9 +386,9 @@ __global__ void __launch_bounds__(T5_THREADS, 1) k_attn_t5(const __grid_constant
             };
             if (nb > 0) issue_s(0);
             if (nb > 1) issue_s(1);
-            // S_{i+2} once P_i is written: the softmax of block i has read score buffer i mod 2.
+            // S_{i+2} once the softmax of block i has read score buffer i mod 2.
             for (int i = 0; i + 2 < nb; ++i) {
-                if (!ptx::mbar_wait_bounded(&pfull[i & 1], (i >> 1) & 1, T5_WAIT_NS)) good = false;
+                if (!ptx::mbar_wait_bounded(&sfree[i & 1], (i >> 1) & 1, T5_WAIT_NS)) good = false;
                 ptx::tc_fence_after();
                 issue_s(i + 2);
             }
@@ -462,6 +464,8 @@ __global__ void __launch_bounds__(T5_THREADS, 1) k_attn_t5(const __grid_constant
                 ptx::tmem_ld_x16(sa, r[0]);
                 ptx::tmem_ld_x16(sa + 16u, r[1]);
                 ptx::tmem_ld_wait();
+                ptx::tc_fence_before();
+                ptx::mbar_arrive(&sfree[i & 1]);
             }
             // Keys of this half block the row sees: all of them except in the last block(s).
             const int vis = nvis - (blk0 + i) * T5_KEYS - HK * half;
