@@ -23,6 +23,7 @@
 #include <cstdint>
 #include <cstdio>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "jpi_prefill.h"
@@ -73,6 +74,7 @@ __global__ void k_pf_cast(const float* __restrict__ src, __nv_bfloat16* __restri
 
 // h = x (fp32 or bf16 embeddings) as the fp32 residual stream.
 __global__ void k_pf_load_x(const void* __restrict__ x, int x_fp32, float* __restrict__ h, long long n) {
+    jpi::ptx::grid_dep_launch();   // the next kernel waits for this one's results
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         h[i] = x_fp32 ? static_cast<const float*>(x)[i] : __bfloat162float(static_cast<const __nv_bfloat16*>(x)[i]);
 }
@@ -118,6 +120,8 @@ __global__ void __launch_bounds__(RB) k_pf_rmsnorm(const float* __restrict__ h, 
                                                    TO* __restrict__ y, long long rows, int W, float eps) {
     __shared__ float red[RB / 32];
     const int t = threadIdx.x, n4 = W >> 2;
+    jpi::ptx::grid_dep_wait();
+    jpi::ptx::grid_dep_launch();
     for (long long r = blockIdx.x; r < rows; r += gridDim.x) {
         const float4* hr = reinterpret_cast<const float4*>(h + r * W);
         if (n4 <= RB * RB_CAP) {
@@ -155,6 +159,8 @@ __global__ void k_pf_rope_scatter(const float* __restrict__ qkv, const float2* _
                                   int D) {
     const int half = D / 2, secs = H + 2, slots = secs * half;
     constexpr int RS_BATCH = 8;   // slots of a thread whose loads are in flight together
+    jpi::ptx::grid_dep_wait();
+    jpi::ptx::grid_dep_launch();
     for (long long r = blockIdx.x; r < (long long)B * P; r += gridDim.x) {   // r = b P + p
         const int p = (int)(r % P), b = (int)(r / P);
         const float* row = qkv + r * (long long)secs * D;
@@ -202,6 +208,8 @@ __global__ void __launch_bounds__(256) k_pf_softmax(const float* __restrict__ s,
                                                     long long rows, int n, int ld) {
     const int lane = threadIdx.x & 31;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
+    jpi::ptx::grid_dep_wait();
+    jpi::ptx::grid_dep_launch();
     for (long long r = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < rows; r += nwarps) {
         const float* sr = s + r * ld;
         __nv_bfloat16* pr = p + r * ld;
@@ -242,45 +250,48 @@ __global__ void __launch_bounds__(256) k_pf_softmax(const float* __restrict__ s,
     }
 }
 
-// After a product split over K ranges: h += (part_0 + part_1 + ...) in range order (parts [rows][W]
-// fp32, `pstride` elements apart), then, when w is set, the next RMSNorm y = h / sqrt(mean(h^2) +
-// eps) * (1 + w) as k_pf_rmsnorm computes it.
+// Stream-K pieces of tile t (nkb k-blocks each) over T units and G CTAs: first CTA and count.
+__host__ __device__ __forceinline__ int pg_cta_of(long long x, long long T, int G) {
+    return (int)(((x + 1) * G - 1) / T);
+}
+__host__ __device__ __forceinline__ int pg_pieces(int t, int nkb, long long T, int G) {
+    return pg_cta_of((long long)(t + 1) * nkb - 1, T, G) - pg_cta_of((long long)t * nkb, T, G) + 1;
+}
+
+// After a stream-K product: h += (piece 0 + piece 1 + ...) of each 128 x 256 tile in order (pieces
+// [rows][W] fp32, `pstride` elements apart; ntm row tiles, nkb k-blocks a tile dealt to G CTAs), then,
+// when w is set, the next RMSNorm y = h / sqrt(mean(h^2) + eps) * (1 + w) as k_pf_rmsnorm computes it.
 template <typename TO>
 __global__ void __launch_bounds__(RB) k_pf_residual_norm(float* __restrict__ h, const float* __restrict__ parts,
-                                                         int nparts, long long pstride, const float* __restrict__ w,
-                                                         TO* __restrict__ y, long long rows, int W, float eps) {
+                                                         long long pstride, int ntm, int nkb, long long T, int G,
+                                                         const float* __restrict__ w, TO* __restrict__ y, long long rows,
+                                                         int W, float eps) {
     __shared__ float red[RB / 32];
     const int t = threadIdx.x, n4 = W >> 2;
+    jpi::ptx::grid_dep_wait();
+    jpi::ptx::grid_dep_launch();
     for (long long r = blockIdx.x; r < rows; r += gridDim.x) {
         float4* hr = reinterpret_cast<float4*>(h + r * W);
-        // h + (part_0 + part_1 + ...) for float4 i.
-        auto update = [&](int i) {
-            float4 d = reinterpret_cast<const float4*>(parts + r * W)[i];
-            for (int q = 1; q < nparts; ++q) {
-                const float4 e = reinterpret_cast<const float4*>(parts + (size_t)q * pstride + r * W)[i];
-                d = make_float4(d.x + e.x, d.y + e.y, d.z + e.z, d.w + e.w);
-            }
-            const float4 o = hr[i];
-            const float4 v = make_float4(o.x + d.x, o.y + d.y, o.z + d.z, o.w + d.w);
-            hr[i] = v;
-            return v;
-        };
+        const int tm = (int)(r >> 7);
+        // Pieces of the tile that holds float4 i of this row (256 columns are 64 float4).
+        auto pieces = [&](int i) { return pg_pieces((i >> 6) * ntm + tm, nkb, T, G); };
+        auto part = [&](int q) { return reinterpret_cast<const float4*>(parts + (size_t)q * pstride + r * W); };
         if (n4 <= RB * RB_CAP) {
-            // Passes over the row held in registers: part 0, each further part, then h.
+            // Passes over the row held in registers: piece 0, each further piece, then h.
             float4 v[RB_CAP];
-            const float4* p0 = reinterpret_cast<const float4*>(parts + r * W);
+            int np[RB_CAP], most = 0;
 #pragma unroll
             for (int k = 0; k < RB_CAP; ++k) {
                 const int i = t + RB * k;
-                v[k] = i < n4 ? p0[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+                np[k] = i < n4 ? pieces(i) : 0;
+                most = max(most, np[k]);
+                v[k] = i < n4 ? part(0)[i] : make_float4(0.f, 0.f, 0.f, 0.f);
             }
-            for (int q = 1; q < nparts; ++q) {
-                const float4* pq = reinterpret_cast<const float4*>(parts + (size_t)q * pstride + r * W);
+            for (int q = 1; q < most; ++q) {
 #pragma unroll
                 for (int k = 0; k < RB_CAP; ++k) {
-                    const int i = t + RB * k;
-                    if (i < n4) {
-                        const float4 e = pq[i];
+                    if (q < np[k]) {
+                        const float4 e = part(q)[t + RB * k];
                         v[k] = make_float4(v[k].x + e.x, v[k].y + e.y, v[k].z + e.z, v[k].w + e.w);
                     }
                 }
@@ -312,7 +323,18 @@ __global__ void __launch_bounds__(RB) k_pf_residual_norm(float* __restrict__ h, 
             }
         } else {
             float s = 0.f;
-            for (int i = t; i < n4; i += RB) s += sq4(update(i));
+            for (int i = t; i < n4; i += RB) {
+                float4 d = part(0)[i];
+                const int np = pieces(i);
+                for (int q = 1; q < np; ++q) {
+                    const float4 e = part(q)[i];
+                    d = make_float4(d.x + e.x, d.y + e.y, d.z + e.z, d.w + e.w);
+                }
+                const float4 o = hr[i];
+                const float4 v = make_float4(o.x + d.x, o.y + d.y, o.z + d.z, o.w + d.w);
+                hr[i] = v;
+                s += sq4(v);
+            }
             if (!w) continue;
             const float rinv = 1.f / sqrtf(block_sum_rb(s, red) / (float)W + eps);
             for (int i = t; i < n4; i += RB) store_normed4(y, w, r, W, i, hr[i], rinv);
@@ -347,19 +369,24 @@ struct LayerW {
 // The products: Y[m][n] = alpha sum_k X[m][k] W[n][k] (+ Y[m][n]), X [M][K] and W [N][K] row-major
 // bf16, Y fp32 or bf16, fp32 accumulation. One output tile = 128 rows of X (the MMA's M) x 256
 // rows of W (its N) over the whole K range, in TMEM as [X row = lane][W row = column]: each k-block
-// brings 48 KB into the SM for 2 M multiply-adds (a 128 x 128 tile brings 32 KB for 1 M, and one
-// SM takes in only about 85 GB/s from L2), and only the token dimension, 816 rows at Gemma-2B
-// sizes, is padded. Persistent: one CTA per SM walks the tiles u = blockIdx.x, + gridDim.x, ...
-// with the X tile fastest, so the CTAs that run together share one W tile through L2 and every W
-// tile is read from HBM once (W is the large operand: 134 MB for gate/up, X 3.3 MB):
+// brings 48 KB into the SM for 2 M multiply-adds (a 128 x 128 tile brings 32 KB for 1 M), and only the
+// token dimension, 816 rows at Gemma-2B sizes, is padded. Persistent: one CTA per SM walks the tiles
+// u = blockIdx.x, + gridDim.x, ... with the X tile fastest, so the CTAs that run together share one W
+// tile through L2 and every W tile is read from HBM once (W is the large operand: 134 MB for
+// gate/up, X 3.3 MB):
 //   warp 0  one thread streams (X block, W block) pairs of 64 K-columns by bulk tensor copies
 //           (128-byte swizzle; rows and columns past the tensors' extents arrive as zeros) into a
-//           ring of PG_STAGES stages;
+//           ring of PG_STAGES stages (W blocks of the first stages before the dependency wait);
 //   warp 1  one thread issues the tcgen05.mma chain (M = 128, N = 256, K = 16 each) into one of two
 //           TMEM accumulators and releases each stage through tcgen05.commit;
-//   warps 2-5  one TMEM lane (X row m) per thread: 16 columns (W rows n) at a time, scaled by
-//           alpha, added to Y when accumulating, stored as 16 consecutive elements of row m, after
-//           which the accumulator goes back to the MMA thread.
+//   warps 2-5  one TMEM lane (X row m) per thread. Every warp passes its 32 rows through 4 KB of
+//           shared memory of its own, 128 bytes of a row at a time (16-byte chunks XOR-swizzled by the
+//           row), and writes 128-byte pieces of four rows per instruction (a row per thread, each
+//           store touched 32 lines). The QKV form applies the rotary coding there and scatters q, k
+//           and v, which replaced an fp32 round trip through memory and a kernel of its own.
+// Stream-K (args.stream): a product with fewer tiles than SMs deals its (tile, k-block) units out
+// evenly, CTA c taking [c T / G, (c + 1) T / G); each piece of a tile goes to its own partial buffer
+// (piece p of a tile: the p-th CTA that touches it), and the consumer adds a tile's pieces in order.
 // Every wait is bounded; a timeout records a device error in the handle's word and the CTA returns.
 
 constexpr int PG_TM = 128;                                      // X rows per tile (MMA M)
@@ -371,7 +398,8 @@ constexpr int PG_WBYTES = PG_TN * PG_KBLK * 2;                  // 32 KB
 constexpr int PG_STAGE_BYTES = PG_XBYTES + PG_WBYTES;
 constexpr int PG_THREADS = 192;
 constexpr uint64_t PG_WAIT_NS = 200ull * 1000 * 1000;
-constexpr size_t PG_SMEM = 1024 + (size_t)PG_STAGES * PG_STAGE_BYTES + 128;
+constexpr int PG_STAGING = 32 * 128;                            // one epilogue warp: 32 rows of 128 bytes
+constexpr size_t PG_SMEM = 1024 + (size_t)PG_STAGES * PG_STAGE_BYTES + 4 * PG_STAGING + 128;
 
 enum PfDeviceError { PF_DEV_OK = 0, PF_DEV_TIMEOUT_LOAD = 1, PF_DEV_TIMEOUT_MMA = 2 };
 
@@ -383,13 +411,20 @@ struct PfGemmArgs {
     int vec;              // Y and ldy allow 16-byte stores of 16 consecutive elements
     void* Y;
     long long ldy;        // elements
-    // K split: k-blocks in ksplit consecutive ranges; range s writes its partial products to
-    // Y + s * ysplit (fp32, never accumulating), summed in range order by the consumer.
-    int ksplit;
+    // Stream-K: piece p of a tile writes Y + p * ysplit (fp32, never accumulating).
+    int stream;
     long long ysplit;
     // GeGLU: W tile t holds gate rows 128 t.. then the up rows of the same features; Y is bf16
     // z [M][ldy] = gelu_tanh(alpha gate) * (alpha up) for the nz features.
     int geglu, nz;
+    int w_const;          // W is a weight matrix (not an output of an earlier kernel)
+    // QKV (D = 128 or 256): columns are H query heads, the key head and the values, D each; rotated
+    // queries to q [M][H][D], rotated keys and the values of row m = b P + p to kd / vd + b kv_stride +
+    // p D. rope[p][j] = (cos, sin) of pair j.
+    int qkv, H, D, P;
+    const float2* rope;
+    __nv_bfloat16 *q, *kd, *vd;
+    long long kv_stride;
     int* err;
 };
 
@@ -400,7 +435,8 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pf_gemm(const __grid_constant
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
     uint8_t* stages = smem;                                  // [stage][X 16 KB | W 32 KB]
-    uint64_t* full = (uint64_t*)(smem + (size_t)PG_STAGES * PG_STAGE_BYTES);
+    uint8_t* staging = smem + (size_t)PG_STAGES * PG_STAGE_BYTES;   // [4 warps][32 rows][128 B]
+    uint64_t* full = (uint64_t*)(staging + 4 * PG_STAGING);
     uint64_t* empty = full + PG_STAGES;
     uint64_t* accf = empty + PG_STAGES;
     uint64_t* acce = accf + 2;
@@ -410,16 +446,26 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pf_gemm(const __grid_constant
     const int tid = threadIdx.x, warp = ptx::warp_index(), lane = tid & 31;
     const int nkb = (a.K + PG_KBLK - 1) / PG_KBLK;
     const int ntn = (a.N + PG_TN - 1) / PG_TN, ntm = (a.M + PG_TM - 1) / PG_TM;
-    const int total = ntn * ntm * a.ksplit;
-    const int u0 = blockIdx.x, du = gridDim.x;
-    // Unit u: X tile fastest, then W tile, then K range; k-blocks [kb_lo, kb_hi) of the range.
-    const int nkr = (nkb + a.ksplit - 1) / a.ksplit;
-    auto unit = [&](int u, int& tm, int& tn, int& sk, int& kb_lo, int& kb_hi) {
+    const int tiles = ntn * ntm;
+    // Segment j of this CTA: a tile (X tile fastest) and k-blocks [kb_lo, kb_hi) of it.
+    const long long T = (long long)tiles * nkb;
+    const long long x0 = a.stream ? blockIdx.x * T / gridDim.x : 0, x1 = a.stream ? (blockIdx.x + 1) * T / gridDim.x : 0;
+    const int first = a.stream ? (int)(x0 / nkb) : (int)blockIdx.x, dstep = a.stream ? 1 : (int)gridDim.x;
+    const int nseg = a.stream ? (x1 > x0 ? (int)((x1 - 1) / nkb) - first + 1 : 0)
+                              : (first < tiles ? (tiles - first + dstep - 1) / dstep : 0);
+    auto segment = [&](int j, int& tm, int& tn, int& piece, int& kb_lo, int& kb_hi) {
+        const int u = first + j * dstep;
         tm = u % ntm;
-        tn = (u / ntm) % ntn;
-        sk = u / (ntm * ntn);
-        kb_lo = sk * nkr;
-        kb_hi = min(nkb, kb_lo + nkr);
+        tn = u / ntm;
+        piece = 0;
+        kb_lo = 0;
+        kb_hi = nkb;
+        if (a.stream) {
+            const long long base = (long long)u * nkb;
+            kb_lo = x0 > base ? (int)(x0 - base) : 0;
+            kb_hi = x1 < base + nkb ? (int)(x1 - base) : nkb;
+            piece = (int)blockIdx.x - pg_cta_of(base, T, gridDim.x);
+        }
     };
 
     if (warp == 1) {
@@ -444,9 +490,28 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pf_gemm(const __grid_constant
         if (ptx::elect_one()) {
             int it = 0, issued = 0;
             bool ok = true;
-            for (int u = u0; u < total && ok; u += du) {
-                int tm, tn, sk, kb_lo, kb_hi;
-                unit(u, tm, tn, sk, kb_lo, kb_hi);
+            auto load_w = [&](int tn, int kb, int s) {
+                ptx::mbar_expect_tx(&full[s], (uint32_t)PG_STAGE_BYTES);
+                ptx::tma_load_2d_plain(stages + (size_t)s * PG_STAGE_BYTES + PG_XBYTES, &wmap, &full[s], kb * PG_KBLK,
+                                       tn * PG_TN);
+            };
+            auto load_x = [&](int tm, int kb, int s) {
+                ptx::tma_load_2d_plain(stages + (size_t)s * PG_STAGE_BYTES, &xmap, &full[s], kb * PG_KBLK, tm * PG_TM);
+            };
+            // The weights depend on nothing upstream: the first segment's first stages.
+            int npre = 0;
+            if (a.w_const && nseg > 0) {
+                int tm, tn, piece, kb_lo, kb_hi;
+                segment(0, tm, tn, piece, kb_lo, kb_hi);
+                npre = min(PG_STAGES, kb_hi - kb_lo);
+                issued = npre;
+                for (int i = 0; i < npre; ++i) load_w(tn, kb_lo + i, i);
+            }
+            ptx::prefetch_tmap(&xmap);
+            ptx::grid_dep_wait();
+            for (int j = 0; j < nseg && ok; ++j) {
+                int tm, tn, piece, kb_lo, kb_hi;
+                segment(j, tm, tn, piece, kb_lo, kb_hi);
                 for (int kb = kb_lo; kb < kb_hi; ++kb, ++it) {
                     const int s = it % PG_STAGES, n = it / PG_STAGES;
                     if (it >= PG_STAGES && !ptx::mbar_wait_bounded(&empty[s], (n - 1) & 1, PG_WAIT_NS)) {
@@ -454,11 +519,9 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pf_gemm(const __grid_constant
                         ok = false;
                         break;
                     }
-                    uint8_t* st = stages + (size_t)s * PG_STAGE_BYTES;
-                    ptx::mbar_expect_tx(&full[s], (uint32_t)PG_STAGE_BYTES);
-                    ptx::tma_load_2d_plain(st, &xmap, &full[s], kb * PG_KBLK, tm * PG_TM);
-                    ptx::tma_load_2d_plain(st + PG_XBYTES, &wmap, &full[s], kb * PG_KBLK, tn * PG_TN);
-                    issued = it + 1;
+                    if (it >= npre) load_w(tn, kb, s);
+                    load_x(tm, kb, s);
+                    issued = max(issued, it + 1);
                 }
             }
             // Nothing may land in this CTA's shared memory after it exits: wait for the last copy
@@ -473,13 +536,13 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pf_gemm(const __grid_constant
             const uint32_t base = ptx::smem_u32(stages);
             bool good = true;
             int it = 0;
-            for (int u = u0, j = 0; u < total; u += du, ++j) {
+            for (int j = 0; j < nseg; ++j) {
                 const int buf = j & 1;
                 if (j >= 2 && !ptx::mbar_wait_bounded(&acce[buf], ((j - 2) >> 1) & 1, PG_WAIT_NS)) good = false;
                 ptx::tc_fence_after();
                 const uint32_t acc = tmem + (uint32_t)(buf * PG_TN);
-                int tm, tn, sk, kb_lo, kb_hi;
-                unit(u, tm, tn, sk, kb_lo, kb_hi);
+                int tm, tn, piece, kb_lo, kb_hi;
+                segment(j, tm, tn, piece, kb_lo, kb_hi);
                 for (int kb = kb_lo; kb < kb_hi; ++kb, ++it) {
                     const int s = it % PG_STAGES, n = it / PG_STAGES;
                     if (good && !ptx::mbar_wait_bounded(&full[s], n & 1, PG_WAIT_NS)) good = false;
@@ -499,105 +562,186 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pf_gemm(const __grid_constant
             if (!good) *flag = PF_DEV_TIMEOUT_MMA;
         }
     } else {
-        const int row = (warp & 3) * 32 + lane;   // TMEM lane: X row of the tile
-        const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-        for (int u = u0, j = 0; u < total; u += du, ++j) {
+        const int qd = warp & 3, row = qd * 32 + lane;   // TMEM lane: X row of the tile
+        uint8_t* stg = staging + qd * PG_STAGING;
+        // Through the staging, lane l handles 16-byte chunk l mod 8 of rows 4 i + l / 8 of the warp's 32.
+        const int sr = lane >> 3, sc = lane & 7;
+        auto own_chunk = [&](int c) { return (uint4*)(stg + lane * 128 + ((c ^ (lane & 7)) << 4)); };
+        auto row_chunk = [&](int r, int c) { return (const uint4*)(stg + r * 128 + ((c ^ (r & 7)) << 4)); };
+        auto pack2 = [](float lo, float hi) {
+            const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+            return *reinterpret_cast<const uint32_t*>(&v);
+        };
+        ptx::grid_dep_wait();   // outputs may still be read by the previous kernel
+        for (int j = 0; j < nseg; ++j) {
             const int buf = j & 1;
-            int tm, tn, sk, kb_lo, kb_hi;
-            unit(u, tm, tn, sk, kb_lo, kb_hi);
-            const bool ok = ptx::mbar_wait_bounded(&accf[buf], (j >> 1) & 1, PG_WAIT_NS) && *flag == 0;
+            int tm, tn, piece, kb_lo, kb_hi;
+            segment(j, tm, tn, piece, kb_lo, kb_hi);
+            if (!ptx::mbar_wait_bounded(&accf[buf], (j >> 1) & 1, PG_WAIT_NS)) *flag = PF_DEV_TIMEOUT_MMA;
+            const bool ok = __all_sync(0xffffffffu, *flag == 0);
             ptx::tc_fence_after();
-            const int m = tm * PG_TM + row;
-            const bool live = ok && m < a.M;
-            if (a.geglu) {
-                // Gate columns c0.. and up columns 128 + c0.. of this tile: 16 features of z.
-                for (int c0 = 0; c0 < PG_TN / 2; c0 += 16) {
-                    uint32_t rg[16], ru[16];
-                    ptx::tmem_ld_x16(lane_base + (uint32_t)(buf * PG_TN + c0), rg);
-                    ptx::tmem_ld_x16(lane_base + (uint32_t)(buf * PG_TN + PG_TN / 2 + c0), ru);
-                    ptx::tmem_ld_wait();
-                    const int f0 = tn * (PG_TN / 2) + c0;
-                    if (!live || f0 >= a.nz) continue;
-                    float v[16];
+            // The last accumulator is complete: the next kernel's CTAs may come in.
+            if (j + 1 == nseg) ptx::grid_dep_launch();
+            const uint32_t acc = tmem + (uint32_t)(buf * PG_TN) + ((uint32_t)(qd * 32) << 16);
+            const int m0 = tm * PG_TM + qd * 32;   // the warp's first row
+            // Stream-K: this piece of the tile has its own partial buffer.
+            void* Y = a.stream ? (void*)(static_cast<float*>(a.Y) + (size_t)piece * a.ysplit) : a.Y;
+            if (a.qkv) {
+                // Steps of 16 rotary pairs: columns c1.. and c1 + D / 2.. of one head section.
+                const int half = a.D >> 1;
+                int pos[8];
+                size_t qo[8], kvo[8];
 #pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        v[i] = gelu_tanh_f(a.alpha * __uint_as_float(rg[i])) * (a.alpha * __uint_as_float(ru[i]));
-                    __nv_bfloat16* z = static_cast<__nv_bfloat16*>(a.Y) + (size_t)m * a.ldy + f0;
-                    if (a.vec && f0 + 16 <= a.nz) {
-                        uint32_t p[8];
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            __nv_bfloat162 t = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-                            p[i] = *reinterpret_cast<uint32_t*>(&t);
-                        }
-                        reinterpret_cast<uint4*>(z)[0] = make_uint4(p[0], p[1], p[2], p[3]);
-                        reinterpret_cast<uint4*>(z)[1] = make_uint4(p[4], p[5], p[6], p[7]);
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < 16; ++i)
-                            if (f0 + i < a.nz) z[i] = __float2bfloat16_rn(v[i]);
-                    }
+                for (int i = 0; i < 8; ++i) {
+                    const int m = min(m0 + 4 * i + sr, a.M - 1), b = m / a.P;
+                    pos[i] = m - b * a.P;
+                    qo[i] = (size_t)m * a.H * a.D;
+                    kvo[i] = (size_t)b * a.kv_stride + (size_t)pos[i] * a.D;
                 }
-                ptx::tc_fence_before();
-                ptx::mbar_arrive(&acce[buf]);
-                if (!ok && lane == 0) *flag = PF_DEV_TIMEOUT_MMA;
-                continue;
-            }
-            // K range sk writes its own partial (never accumulating).
-            void* Yu = a.ksplit > 1 ? (void*)(static_cast<float*>(a.Y) + (size_t)sk * a.ysplit) : a.Y;
-            const bool accum = a.accumulate && a.ksplit == 1;
-            for (int c0 = 0; c0 < PG_TN; c0 += 16) {
-                uint32_t r[16];
-                ptx::tmem_ld_x16(lane_base + (uint32_t)(buf * PG_TN + c0), r);
-                ptx::tmem_ld_wait();
-                const int n0 = tn * PG_TN + c0;
-                if (!live || n0 >= a.N) continue;
-                float v[16];
+#pragma unroll 1
+                for (int s = 0; s < PG_TN / 32; ++s) {
+                    const int sl = 16 * s / half, j0 = 16 * s - sl * half;   // section of the tile, first pair
+                    const int sec = tn * (PG_TN / a.D) + sl, c1 = sl * a.D + j0;
+                    const bool rot = sec <= a.H, in = sec < a.H + 2;
+                    float4 cs[8];
 #pragma unroll
-                for (int i = 0; i < 16; ++i) v[i] = a.alpha * __uint_as_float(r[i]);
-                const size_t o = (size_t)m * a.ldy + n0;
-                if (a.vec && n0 + 16 <= a.N) {
-                    if (a.out_bf16) {
-                        uint4* y = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(Yu) + o);
-                        uint32_t p[8];
+                    for (int i = 0; i < 8; ++i)
+                        cs[i] = rot ? __ldg((const float4*)(a.rope + (size_t)pos[i] * half + j0) + sc)
+                                    : make_float4(1.f, 0.f, 1.f, 0.f);
+                    uint32_t r1[16], r2[16];
+                    ptx::tmem_ld_x16(acc + (uint32_t)c1, r1);
+                    ptx::tmem_ld_x16(acc + (uint32_t)(c1 + half), r2);
+                    ptx::tmem_ld_wait();
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            __nv_bfloat162 t = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-                            p[i] = *reinterpret_cast<uint32_t*>(&t);
-                        }
-                        y[0] = make_uint4(p[0], p[1], p[2], p[3]);
-                        y[1] = make_uint4(p[4], p[5], p[6], p[7]);
-                    } else {
-                        float4* y = reinterpret_cast<float4*>(static_cast<float*>(Yu) + o);
+                    for (int c = 0; c < 8; ++c) *own_chunk(c) = make_uint4(r1[2 * c], r1[2 * c + 1], r2[2 * c], r2[2 * c + 1]);
+                    __syncwarp();
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            float4 t = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-                            if (accum) {
-                                const float4 old = y[q];
-                                t.x += old.x;
-                                t.y += old.y;
-                                t.z += old.z;
-                                t.w += old.w;
-                            }
-                            y[q] = t;
-                        }
+                    for (int i = 0; i < 8; ++i) {
+                        const uint4 v = *row_chunk(4 * i + sr, sc);
+                        const float ua = __uint_as_float(v.x), ub = __uint_as_float(v.y);
+                        const float va = __uint_as_float(v.z), vb = __uint_as_float(v.w);
+                        if (!ok || !in || m0 + 4 * i + sr >= a.M) continue;
+                        __nv_bfloat16* d = (sec < a.H ? a.q + qo[i] + (size_t)sec * a.D : (sec == a.H ? a.kd : a.vd) + kvo[i]) +
+                                           j0 + 2 * sc;
+                        *(uint32_t*)d = pack2(ua * cs[i].x - va * cs[i].y, ub * cs[i].z - vb * cs[i].w);
+                        *(uint32_t*)(d + half) = pack2(va * cs[i].x + ua * cs[i].y, vb * cs[i].z + ub * cs[i].w);
                     }
-                } else {
+                    __syncwarp();
+                }
+            } else if (!a.vec) {
+                // Outputs that take no 16-byte access: a row per thread, element by element.
+                const int m = m0 + lane;
+                const int nc = a.geglu ? PG_TN / 2 : PG_TN, nlim = a.geglu ? a.nz : a.N;
+                for (int c0 = 0; c0 < nc; c0 += 16) {
+                    uint32_t r[16], r2[16];
+                    ptx::tmem_ld_x16(acc + (uint32_t)c0, r);
+                    if (a.geglu) ptx::tmem_ld_x16(acc + (uint32_t)(PG_TN / 2 + c0), r2);
+                    ptx::tmem_ld_wait();
+                    const int n0 = tn * nc + c0;
+                    if (!ok || m >= a.M) continue;
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
-                        if (n0 + i >= a.N) continue;
-                        if (a.out_bf16) {
-                            static_cast<__nv_bfloat16*>(Yu)[o + i] = __float2bfloat16_rn(v[i]);
+                        if (n0 + i >= nlim) continue;
+                        const size_t o = (size_t)m * a.ldy + n0 + i;
+                        float v = a.alpha * __uint_as_float(r[i]);
+                        if (a.geglu) v = gelu_tanh_f(v) * (a.alpha * __uint_as_float(r2[i]));
+                        if (a.geglu || a.out_bf16) static_cast<__nv_bfloat16*>(Y)[o] = __float2bfloat16_rn(v);
+                        else static_cast<float*>(Y)[o] = a.accumulate ? static_cast<float*>(Y)[o] + v : v;
+                    }
+                }
+            } else if (a.geglu || a.out_bf16) {
+                // 64 bf16 outputs of a row per pass (GeGLU: gate columns c.. and up columns 128 + c..).
+                const int nc = a.geglu ? PG_TN / 2 : PG_TN, nlim = a.geglu ? a.nz : a.N;
+                for (int c0 = 0; c0 < nc; c0 += 64) {
+                    const int n0 = tn * nc + c0;
+                    if (n0 >= nlim) break;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        uint32_t r[16], r2[16];
+                        ptx::tmem_ld_x16(acc + (uint32_t)(c0 + 16 * q), r);
+                        if (a.geglu) ptx::tmem_ld_x16(acc + (uint32_t)(PG_TN / 2 + c0 + 16 * q), r2);
+                        ptx::tmem_ld_wait();
+                        uint32_t o[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            float v0 = a.alpha * __uint_as_float(r[2 * i]), v1 = a.alpha * __uint_as_float(r[2 * i + 1]);
+                            if (a.geglu) {
+                                v0 = gelu_tanh_f(v0) * (a.alpha * __uint_as_float(r2[2 * i]));
+                                v1 = gelu_tanh_f(v1) * (a.alpha * __uint_as_float(r2[2 * i + 1]));
+                            }
+                            o[i] = pack2(v0, v1);
+                        }
+                        *own_chunk(2 * q) = make_uint4(o[0], o[1], o[2], o[3]);
+                        *own_chunk(2 * q + 1) = make_uint4(o[4], o[5], o[6], o[7]);
+                    }
+                    __syncwarp();
+                    const int n = n0 + 8 * sc;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int m = m0 + 4 * i + sr;
+                        const uint4 v = *row_chunk(4 * i + sr, sc);
+                        if (!ok || m >= a.M) continue;
+                        __nv_bfloat16* y = static_cast<__nv_bfloat16*>(Y) + (size_t)m * a.ldy + n;
+                        if (n + 8 <= nlim) {
+                            *(uint4*)y = v;
                         } else {
-                            float* y = static_cast<float*>(Yu) + o + i;
-                            *y = accum ? *y + v[i] : v[i];
+                            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                            for (int e = 0; e < 8; ++e)
+                                if (n + e < nlim)
+                                    reinterpret_cast<unsigned short*>(y)[e] = (unsigned short)(w[e / 2] >> (16 * (e & 1)));
                         }
                     }
+                    __syncwarp();
+                }
+            } else {
+                // 32 fp32 outputs of a row per pass.
+                const bool accum = a.accumulate && !a.stream;
+                for (int c0 = 0; c0 < PG_TN; c0 += 32) {
+                    const int n0 = tn * PG_TN + c0;
+                    if (n0 >= a.N) break;
+                    const int n = n0 + 4 * sc;
+                    float4 old[8];   // before the accumulator is read: the loads overlap it
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int m = m0 + 4 * i + sr;
+                        old[i] = accum && m < a.M && n + 4 <= a.N
+                                     ? *(const float4*)(static_cast<const float*>(Y) + (size_t)m * a.ldy + n)
+                                     : make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
+                    uint32_t r[2][16];
+                    ptx::tmem_ld_x16(acc + (uint32_t)c0, r[0]);
+                    ptx::tmem_ld_x16(acc + (uint32_t)(c0 + 16), r[1]);
+                    ptx::tmem_ld_wait();
+#pragma unroll
+                    for (int c = 0; c < 8; ++c)
+                        *own_chunk(c) = make_uint4(r[c >> 2][4 * (c & 3)], r[c >> 2][4 * (c & 3) + 1],
+                                                   r[c >> 2][4 * (c & 3) + 2], r[c >> 2][4 * (c & 3) + 3]);
+                    __syncwarp();
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int m = m0 + 4 * i + sr;
+                        const uint4 u = *row_chunk(4 * i + sr, sc);
+                        if (!ok || m >= a.M) continue;
+                        const float4 v = make_float4(old[i].x + a.alpha * __uint_as_float(u.x),
+                                                     old[i].y + a.alpha * __uint_as_float(u.y),
+                                                     old[i].z + a.alpha * __uint_as_float(u.z),
+                                                     old[i].w + a.alpha * __uint_as_float(u.w));
+                        float* y = static_cast<float*>(Y) + (size_t)m * a.ldy + n;
+                        if (n + 4 <= a.N) {
+                            *(float4*)y = v;
+                        } else {
+                            const float w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                            for (int e = 0; e < 4; ++e)
+                                if (n + e < a.N) y[e] = accum ? y[e] + w[e] : w[e];
+                        }
+                    }
+                    __syncwarp();
                 }
             }
             ptx::tc_fence_before();
             ptx::mbar_arrive(&acce[buf]);
-            if (!ok && lane == 0) *flag = PF_DEV_TIMEOUT_MMA;
         }
     }
 
@@ -612,6 +756,8 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pf_gemm(const __grid_constant
 __global__ void k_pf_transpose(const __nv_bfloat16* __restrict__ v, __nv_bfloat16* __restrict__ vt, int P, int D,
                                int ldt) {
     __shared__ __nv_bfloat16 t[32][33];
+    jpi::ptx::grid_dep_wait();
+    jpi::ptx::grid_dep_launch();
     const int p0 = blockIdx.x * 32, d0 = blockIdx.y * 32;
     for (int i = threadIdx.y; i < 32; i += blockDim.y) {
         const int p = p0 + i, d = d0 + threadIdx.x;
@@ -649,11 +795,11 @@ struct jpi_prefill_handle {
     float2* rope = nullptr;          // [Pm][D / 2]
     float* h = nullptr;              // [Bm Pm][W] residual stream
     __nv_bfloat16* xn = nullptr;     // [Bm Pm][W] GEMM operand: normed h
-    float* qkv = nullptr;            // [Bm Pm][(H + 2) D]
+    float* qkv = nullptr;            // [Bm Pm][(H + 2) D] (head dims without the fused epilogue)
     __nv_bfloat16* q = nullptr;      // [Bm Pm][H][D]
     __nv_bfloat16* o = nullptr;      // [Bm Pm][H D]
     __nv_bfloat16* z = nullptr;      // [Bm Pm][F] GeGLU output (the gate/up product's epilogue)
-    float* part = nullptr;           // partial products of a K-split projection
+    float* part = nullptr;           // pieces of a stream-K residual product
     long long part_elems = 0;        // floats `part` holds
     int Fp = 0;                      // F rounded up to 128: gate/up tiles of 128 features
     float* sc = nullptr;             // [H Pm][Pp] scores of one request
@@ -661,6 +807,7 @@ struct jpi_prefill_handle {
     __nv_bfloat16* vt = nullptr;     // [D][Pp] one request's values, transposed
     int* dev_err = nullptr;          // device error word of the GEMM's bounded waits
     int num_sms = 0;
+    bool qkv_fused() const { return D == 128 || D == 256; }
 };
 
 namespace {
@@ -703,17 +850,35 @@ jpi_status make_map(const void* base, long long rows, long long cols, long long 
     return JPI_OK;
 }
 
+// Launch with programmatic dependent launch: the kernel waits for its predecessor (griddepcontrol)
+// before it touches what that reads or writes, and starts its weight copies before. A failed launch
+// leaves its error for the cudaGetLastError check that follows.
+template <typename... KArgs, typename... Args>
+void pdl(cudaStream_t st, dim3 grid, dim3 block, size_t smem, void (*k)(KArgs...), Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    (void)cudaLaunchKernelEx(&cfg, k, args...);
+}
+
 // Y [M][N] (leading dimension ldy; fp32, or bf16 when y_bf16) = alpha X [M][K] W[N][K]^T, plus Y
-// when accumulating. X and W are bf16 with leading dimensions ldx and ldw. With ksplit > 1 the
-// k-blocks are cut into ksplit ranges and range s writes fp32 Y + s * ysplit (not accumulating);
-// with nz > 0, Y is the bf16 GeGLU output z [M][ldy] of nz features (gate/up tiles packed).
+// when accumulating. X and W are bf16 with leading dimensions ldx and ldw; w_const: W is a weight
+// matrix. `more` sets the fields of the other forms (GeGLU, QKV, stream-K); grid > 0 fixes the CTAs.
+template <typename F>
 jpi_status row_gemm(jpi_prefill_handle* h, cudaStream_t st, const __nv_bfloat16* X, long long ldx,
-                    const __nv_bfloat16* Wm, long long ldw, void* Y, bool y_bf16, long long ldy, int M, int N,
-                    int K, float alpha, bool accumulate, int ksplit = 1, long long ysplit = 0, int nz = 0) {
+                    const __nv_bfloat16* Wm, long long ldw, bool w_const, void* Y, bool y_bf16, long long ldy, int M,
+                    int N, int K, float alpha, bool accumulate, int grid, F&& more) {
     CUtensorMap wmap, xmap;
     PF_TRY(make_map(Wm, N, K, ldw, PG_TN, &wmap));
     PF_TRY(make_map(X, M, K, ldx, PG_TM, &xmap));
-    PfGemmArgs a;
+    PfGemmArgs a = {};
     a.M = M;
     a.N = N;
     a.K = K;
@@ -723,29 +888,38 @@ jpi_status row_gemm(jpi_prefill_handle* h, cudaStream_t st, const __nv_bfloat16*
     a.Y = Y;
     a.ldy = ldy;
     a.vec = (reinterpret_cast<uintptr_t>(Y) % 16 == 0 && ldy % (y_bf16 ? 8 : 4) == 0) ? 1 : 0;
-    a.ksplit = ksplit;
-    a.ysplit = ysplit;
-    a.geglu = nz > 0 ? 1 : 0;
-    a.nz = nz;
+    a.w_const = w_const ? 1 : 0;
     a.err = h->dev_err;
-    const long long tiles = (long long)((N + PG_TN - 1) / PG_TN) * ((M + PG_TM - 1) / PG_TM) * ksplit;
-    const int grid = (int)(tiles < h->num_sms ? tiles : h->num_sms);
-    k_pf_gemm<<<grid, PG_THREADS, PG_SMEM, st>>>(wmap, xmap, a);
+    more(a);
+    if (grid <= 0) {
+        const long long tiles = (long long)((N + PG_TN - 1) / PG_TN) * ((M + PG_TM - 1) / PG_TM);
+        grid = (int)(tiles < h->num_sms ? tiles : h->num_sms);
+    }
+    pdl(st, dim3(grid), dim3(PG_THREADS), PG_SMEM, k_pf_gemm, wmap, xmap, a);
     PF_CUDA(cudaGetLastError());
     return JPI_OK;
 }
+jpi_status row_gemm(jpi_prefill_handle* h, cudaStream_t st, const __nv_bfloat16* X, long long ldx,
+                    const __nv_bfloat16* Wm, long long ldw, bool w_const, void* Y, bool y_bf16, long long ldy, int M,
+                    int N, int K, float alpha, bool accumulate) {
+    return row_gemm(h, st, X, ldx, Wm, ldw, w_const, Y, y_bf16, ldy, M, N, K, alpha, accumulate, 0, [](PfGemmArgs&) {});
+}
 
-// K ranges for a product with few output tiles (at small B x P the O and down projections have
-// 56 tiles at Gemma-2B sizes): as many as keep one wave on the GPU, at most 4, each of at least
-// 8 k-blocks, and only while the partials [M][N] fit.
-int split_for(const jpi_prefill_handle* h, int M, int N, int K) {
+// CTAs a residual product [M][N] over K is dealt out to (stream-K), or 0: whole tiles, accumulated in
+// place. Up to 4/5 of a wave of tiles (at Gemma-2B sizes and 816 tokens O and down have 56: dealt out,
+// every CTA takes 11.8 of O's and 94.3 of down's k-blocks; two K ranges per tile kept 112 of 152 SMs
+// busy, 16 and 128 k-blocks each), at most 8 CTAs a tile and 8 k-blocks a CTA.
+int stream_grid(int num_sms, int M, int N, int K) {
     const long long tiles = (long long)((N + PG_TN - 1) / PG_TN) * ((M + PG_TM - 1) / PG_TM);
     const int nkb = (K + PG_KBLK - 1) / PG_KBLK;
-    int s = 1;
-    while (s < 4 && tiles * (s + 1) <= h->num_sms && nkb / (s + 1) >= 8 &&
-           (long long)(s + 1) * M * N <= h->part_elems)
-        ++s;
-    return s;
+    if (tiles * 5 > num_sms * 4ll) return 0;
+    const long long g = std::min<long long>(std::min<long long>(num_sms, 8 * tiles), tiles * nkb / 8);
+    return g > tiles ? (int)g : 0;
+}
+// Most pieces a tile of such a product has.
+int stream_pieces(int grid, int M, int N) {
+    const int tiles = ((N + PG_TN - 1) / PG_TN) * ((M + PG_TM - 1) / PG_TM);
+    return (grid + tiles - 1) / tiles + 1;
 }
 
 // Attention of the requests of one layer on the tcgen05 attention kernel: the queries h->q
@@ -774,7 +948,8 @@ jpi_status attention_t5(jpi_prefill_handle* h, cudaStream_t st, const __nv_bfloa
     a.o = h->o;
     a.err = h->dev_err;
     const dim3 grid((unsigned)((nrows + jpi::T5_ROWS - 1) / jpi::T5_ROWS), (unsigned)batch);
-    jpi::k_attn_t5<D><<<grid, jpi::T5_THREADS, jpi::T5Smem<D>::BYTES, st>>>(qmap, kmap, vmap, a);
+    pdl(st, grid, dim3(jpi::T5_THREADS), jpi::T5Smem<D>::BYTES, jpi::k_attn_t5<D>, qmap, kmap,
+        vmap, a);
     PF_CUDA(cudaGetLastError());
     return JPI_OK;
 }
@@ -902,15 +1077,16 @@ jpi_status setup(jpi_prefill_handle* h, const jpi_prefill_config* c, const jpi_p
     PF_TRY(pf_alloc(h, &h->h, Mm * W));
     PF_TRY(pf_alloc(h, &h->xn, Mm * W));
     PF_TRY(pf_alloc(h, &h->z, Mm * F));
-    // Partials of K-split projections (N = W): a split needs at most num_sms / 2 output tiles,
-    // so a part has at most that many 128-row tiles of rows, and there are at most 4 parts.
-    {
-        const long long ntn = (h->W + PG_TN - 1) / PG_TN;
-        const long long rows2 = std::min<long long>((long long)Mm, (h->num_sms / 2 / ntn) * PG_TM);
-        h->part_elems = 4 * rows2 * h->W;
-        if (h->part_elems > 0) PF_TRY(pf_alloc(h, &h->part, (size_t)h->part_elems));
-    }
-    PF_TRY(pf_alloc(h, &h->qkv, Mm * (size_t)h->QKV));
+    // Pieces of the residual products (O and down) that are dealt out by stream-K: the most any token
+    // count up to the maximum needs (pieces x 128-row tiles).
+    for (long long m = 1; m <= (long long)((Mm + PG_TM - 1) / PG_TM); ++m)
+        for (int K : {h->H * h->D, h->F}) {
+            const int M = (int)std::min<long long>(m * PG_TM, (long long)Mm), g = stream_grid(h->num_sms, M, h->W, K);
+            if (g > 0) h->part_elems = std::max(h->part_elems, (long long)stream_pieces(g, M, h->W) * M * h->W);
+        }
+    if (h->part_elems > 0) PF_TRY(pf_alloc(h, &h->part, (size_t)h->part_elems));
+    // Head dims 128 and 256 rotate and scatter in the product's epilogue; others through fp32.
+    if (!h->qkv_fused()) PF_TRY(pf_alloc(h, &h->qkv, Mm * (size_t)h->QKV));
     PF_TRY(pf_alloc(h, &h->q, Mm * HD));
     PF_TRY(pf_alloc(h, &h->o, Mm * HD));
     PF_TRY(pf_alloc(h, &h->sc, (size_t)h->H * h->Pm * h->Pp));
@@ -975,23 +1151,61 @@ JPI_API jpi_status jpi_prefill_run(jpi_prefill_handle* h, const void* x, int x_i
 
     k_pf_load_x<<<grid_for(M * W), 256, 0, st>>>(x, x_is_fp32, h->h, M * W);
     PF_CUDA(cudaGetLastError());
-    // After a K-split down projection, the step that adds its partials to h also writes the next
-    // layer's attention norm into xn.
-    bool xn_ready = false;
-    const long long pstride = M * W;   // elements between the parts of a split product
+    // A residual product (O or down): dealt out by stream-K with its pieces added by the row kernel
+    // that also writes the next norm, or whole tiles accumulated into h and the norm alone after it.
+    // norm null: no norm follows.
+    const dim3 rows_grid(grid_for(M, 1, 16384));
+    auto residual = [&](const __nv_bfloat16* X, int K, const __nv_bfloat16* Wm, const float* norm, auto* y) -> jpi_status {
+        using TO = std::remove_reference_t<decltype(*y)>;
+        const int g = stream_grid(h->num_sms, (int)M, W, K);
+        if (g > 0) {
+            const long long pstride = M * W;   // elements between the pieces
+            PF_TRY(row_gemm(h, st, X, K, Wm, K, true, h->part, false, W, (int)M, W, K, 1.f, false, g, [&](PfGemmArgs& a) {
+                a.stream = 1;
+                a.ysplit = pstride;
+            }));
+            const int ntm = (int)((M + PG_TM - 1) / PG_TM), nkb = (K + PG_KBLK - 1) / PG_KBLK;
+            const long long T = (long long)((W + PG_TN - 1) / PG_TN) * ntm * nkb;
+            pdl(st, rows_grid, dim3(RB), 0, k_pf_residual_norm<TO>, h->h, (const float*)h->part, pstride, ntm, nkb, T, g,
+                norm, y, M, W, eps);
+        } else {
+            PF_TRY(row_gemm(h, st, X, K, Wm, K, true, h->h, false, W, (int)M, W, K, 1.f, true));
+            if (norm) pdl(st, rows_grid, dim3(RB), 0, k_pf_rmsnorm<TO>, (const float*)h->h, norm, y, M, W, eps);
+        }
+        PF_CUDA(cudaGetLastError());
+        return JPI_OK;
+    };
+    pdl(st, rows_grid, dim3(RB), 0, k_pf_rmsnorm<__nv_bfloat16>, (const float*)h->h, (const float*)h->layers[0].attn_norm,
+        h->xn, M, W, eps);
+    PF_CUDA(cudaGetLastError());
     for (int l = 0; l < h->L; ++l) {
         const LayerW& lw = h->layers[(size_t)l];
         __nv_bfloat16* kd = static_cast<__nv_bfloat16*>(k_layers[l]);
         __nv_bfloat16* vd = static_cast<__nv_bfloat16*>(v_layers[l]);
-        // Attention sublayer.
-        if (!xn_ready) {
-            k_pf_rmsnorm<__nv_bfloat16><<<grid_for(M, 1, 16384), RB, 0, st>>>(h->h, lw.attn_norm, h->xn, M, W, eps);
+        // Attention sublayer: projections, rotary coding, scatter into q and the caller's KV store.
+        if (h->qkv_fused()) {
+            // The attention below reads the destinations by bulk tensor copies; this epilogue stores
+            // pairs of elements.
+            if ((reinterpret_cast<uintptr_t>(kd) | reinterpret_cast<uintptr_t>(vd)) & 15)
+                return pfail(JPI_ERR_INVALID_ARG, "a GEMM operand is not 16-byte aligned (address or row stride)");
+            PF_TRY(row_gemm(h, st, h->xn, W, lw.wqkv, W, true, h->q, true, H * D, (int)M, h->QKV, W, 1.f, false, 0,
+                            [&](PfGemmArgs& a) {
+                                a.qkv = 1;
+                                a.H = H;
+                                a.D = D;
+                                a.P = P;
+                                a.rope = h->rope;
+                                a.q = h->q;
+                                a.kd = kd;
+                                a.vd = vd;
+                                a.kv_stride = request_stride;
+                            }));
+        } else {
+            PF_TRY(row_gemm(h, st, h->xn, W, lw.wqkv, W, true, h->qkv, false, h->QKV, (int)M, h->QKV, W, 1.f, false));
+            pdl(st, rows_grid, dim3(256), 0, k_pf_rope_scatter, (const float*)h->qkv, (const float2*)h->rope, h->q, kd, vd,
+                request_stride, batch, P, H, D);
             PF_CUDA(cudaGetLastError());
         }
-        PF_TRY(row_gemm(h, st, h->xn, W, lw.wqkv, W, h->qkv, false, h->QKV, (int)M, h->QKV, W, 1.f, false));
-        k_pf_rope_scatter<<<grid_for(M, 1, 16384), 256, 0, st>>>(h->qkv, h->rope, h->q, kd, vd,
-                                                                             request_stride, batch, P, H, D);
-        PF_CUDA(cudaGetLastError());
         // Attention: on the tcgen05 attention kernel (scores and probabilities never leave the
         // SM), else per request through the GEMM: scores, softmax, V^T, probabilities times V.
         const bool t5 = (D == 128 || D == 256) && request_stride % D == 0 && request_stride / D <= INT32_MAX;
@@ -1004,49 +1218,23 @@ JPI_API jpi_status jpi_prefill_run(jpi_prefill_handle* h, const void* x, int x_i
             const __nv_bfloat16* kb = kd + (size_t)b * request_stride;  // [P][D]
             const __nv_bfloat16* vb = vd + (size_t)b * request_stride;  // [P][D]
             __nv_bfloat16* ob = h->o + (size_t)b * P * H * D;           // [(P H)][D] = [P][H D]
-            PF_TRY(row_gemm(h, st, qb, D, kb, D, h->sc, false, Pp, P * H, P, D, scale, false));
-            k_pf_softmax<<<grid_for((long long)P * H * 32), 256, 0, st>>>(h->sc, h->pr, (long long)P * H, P, Pp);
+            PF_TRY(row_gemm(h, st, qb, D, kb, D, false, h->sc, false, Pp, P * H, P, D, scale, false));
+            pdl(st, dim3(grid_for((long long)P * H * 32)), dim3(256), 0, k_pf_softmax, (const float*)h->sc, h->pr,
+                (long long)P * H, P, Pp);
             PF_CUDA(cudaGetLastError());
-            k_pf_transpose<<<dim3((P + 31) / 32, (D + 31) / 32), dim3(32, 8), 0, st>>>(vb, h->vt, P, D, Pp);
+            pdl(st, dim3((P + 31) / 32, (D + 31) / 32), dim3(32, 8), 0, k_pf_transpose, vb, h->vt, P, D, Pp);
             PF_CUDA(cudaGetLastError());
-            PF_TRY(row_gemm(h, st, h->pr, Pp, h->vt, Pp, ob, true, D, P * H, D, P, 1.f, false));
+            PF_TRY(row_gemm(h, st, h->pr, Pp, h->vt, Pp, false, ob, true, D, P * H, D, P, 1.f, false));
         }
-        // Output projection into the residual stream, then the MLP norm: split over K when the
-        // product has too few tiles to fill the GPU (partials added in order with the norm).
-        const int so = split_for(h, (int)M, W, H * D);
-        if (so > 1) {
-            PF_TRY(row_gemm(h, st, h->o, H * D, lw.wo, H * D, h->part, false, W, (int)M, W, H * D, 1.f, false, so,
-                            pstride));
-            k_pf_residual_norm<__nv_bfloat16><<<grid_for(M, 1, 16384), RB, 0, st>>>(h->h, h->part, so, pstride,
-                                                                                  lw.mlp_norm, h->xn, M, W, eps);
-        } else {
-            PF_TRY(row_gemm(h, st, h->o, H * D, lw.wo, H * D, h->h, false, W, (int)M, W, H * D, 1.f, true));
-            k_pf_rmsnorm<__nv_bfloat16><<<grid_for(M, 1, 16384), RB, 0, st>>>(h->h, lw.mlp_norm, h->xn, M, W, eps);
-        }
-        PF_CUDA(cudaGetLastError());
+        PF_TRY(residual(h->o, H * D, lw.wo, lw.mlp_norm, h->xn));
         // MLP sublayer: gate/up with GeGLU in its epilogue (z bf16), then down into the residual.
-        PF_TRY(row_gemm(h, st, h->xn, W, lw.wgu, W, h->z, true, F, (int)M, 2 * h->Fp, W, 1.f, false, 1, 0, F));
-        const int sd = split_for(h, (int)M, W, F);
-        if (sd > 1) {
-            PF_TRY(row_gemm(h, st, h->z, F, lw.wd, F, h->part, false, W, (int)M, W, F, 1.f, false, sd, pstride));
-            if (l + 1 < h->L) {
-                k_pf_residual_norm<__nv_bfloat16><<<grid_for(M, 1, 16384), RB, 0, st>>>(
-                    h->h, h->part, sd, pstride, h->layers[(size_t)l + 1].attn_norm, h->xn, M, W, eps);
-                xn_ready = true;
-            } else if (out_final) {
-                k_pf_residual_norm<float><<<grid_for(M, 1, 16384), RB, 0, st>>>(h->h, h->part, sd, pstride,
-                                                                            h->final_norm, out_final, M, W, eps);
-            } else {
-                k_pf_residual_norm<float><<<grid_for(M, 1, 16384), RB, 0, st>>>(h->h, h->part, sd, pstride, nullptr,
-                                                                            nullptr, M, W, eps);
-            }
-        } else {
-            PF_TRY(row_gemm(h, st, h->z, F, lw.wd, F, h->h, false, W, (int)M, W, F, 1.f, true));
-            xn_ready = false;
-            if (l + 1 == h->L && out_final)
-                k_pf_rmsnorm<float><<<grid_for(M, 1, 16384), RB, 0, st>>>(h->h, h->final_norm, out_final, M, W, eps);
-        }
-        PF_CUDA(cudaGetLastError());
+        PF_TRY(row_gemm(h, st, h->xn, W, lw.wgu, W, true, h->z, true, F, (int)M, 2 * h->Fp, W, 1.f, false, 0,
+                        [&](PfGemmArgs& a) {
+                            a.geglu = 1;
+                            a.nz = F;
+                        }));
+        if (l + 1 < h->L) PF_TRY(residual(h->z, F, lw.wd, h->layers[(size_t)l + 1].attn_norm, h->xn));
+        else PF_TRY(residual(h->z, F, lw.wd, out_final ? h->final_norm : nullptr, out_final));
     }
     return JPI_OK;
 }
