@@ -379,8 +379,8 @@ struct LayerW {
 //           ring of PG_STAGES stages (W blocks of the first stages before the dependency wait);
 //   warp 1  one thread issues the tcgen05.mma chain (M = 128, N = 256, K = 16 each) into one of two
 //           TMEM accumulators and releases each stage through tcgen05.commit;
-//   warps 2-5  one TMEM lane (X row m) per thread. Every warp passes its 32 rows through 4 KB of
-//           shared memory of its own, 128 bytes of a row at a time (16-byte chunks XOR-swizzled by the
+//   warps 2-9  one TMEM lane (X row m) per thread, two groups of four warps with half of the columns
+//           each. Every warp passes its 32 rows through 4 KB of shared memory of its own, 128 bytes of a row at a time (16-byte chunks XOR-swizzled by the
 //           row), and writes 128-byte pieces of four rows per instruction (a row per thread, each
 //           store touched 32 lines). The QKV form applies the rotary coding there and scatters q, k
 //           and v, which replaced an fp32 round trip through memory and a kernel of its own.
@@ -396,10 +396,11 @@ constexpr int PG_STAGES = 4;
 constexpr int PG_XBYTES = PG_TM * PG_KBLK * 2;                  // 16 KB
 constexpr int PG_WBYTES = PG_TN * PG_KBLK * 2;                  // 32 KB
 constexpr int PG_STAGE_BYTES = PG_XBYTES + PG_WBYTES;
-constexpr int PG_THREADS = 192;
+constexpr int PG_EPI = 256;                                     // epilogue threads: two groups of four warps
+constexpr int PG_THREADS = 64 + PG_EPI;
 constexpr uint64_t PG_WAIT_NS = 200ull * 1000 * 1000;
 constexpr int PG_STAGING = 32 * 128;                            // one epilogue warp: 32 rows of 128 bytes
-constexpr size_t PG_SMEM = 1024 + (size_t)PG_STAGES * PG_STAGE_BYTES + 4 * PG_STAGING + 128;
+constexpr size_t PG_SMEM = 1024 + (size_t)PG_STAGES * PG_STAGE_BYTES + 8 * PG_STAGING + 128;
 
 enum PfDeviceError { PF_DEV_OK = 0, PF_DEV_TIMEOUT_LOAD = 1, PF_DEV_TIMEOUT_MMA = 2 };
 
@@ -435,8 +436,8 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pf_gemm(const __grid_constant
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
     uint8_t* stages = smem;                                  // [stage][X 16 KB | W 32 KB]
-    uint8_t* staging = smem + (size_t)PG_STAGES * PG_STAGE_BYTES;   // [4 warps][32 rows][128 B]
-    uint64_t* full = (uint64_t*)(staging + 4 * PG_STAGING);
+    uint8_t* staging = smem + (size_t)PG_STAGES * PG_STAGE_BYTES;   // [8 warps][32 rows][128 B]
+    uint64_t* full = (uint64_t*)(staging + 8 * PG_STAGING);
     uint64_t* empty = full + PG_STAGES;
     uint64_t* accf = empty + PG_STAGES;
     uint64_t* acce = accf + 2;
@@ -476,8 +477,8 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pf_gemm(const __grid_constant
         for (int i = 0; i < 2 * PG_STAGES; ++i) ptx::mbar_init(&full[i], 1);
         ptx::mbar_init(&accf[0], 1);
         ptx::mbar_init(&accf[1], 1);
-        ptx::mbar_init(&acce[0], 128);
-        ptx::mbar_init(&acce[1], 128);
+        ptx::mbar_init(&acce[0], PG_EPI);
+        ptx::mbar_init(&acce[1], PG_EPI);
         ptx::fence_mbar_init();
         *flag = 0;
     }
@@ -562,8 +563,9 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pf_gemm(const __grid_constant
             if (!good) *flag = PF_DEV_TIMEOUT_MMA;
         }
     } else {
-        const int qd = warp & 3, row = qd * 32 + lane;   // TMEM lane: X row of the tile
-        uint8_t* stg = staging + qd * PG_STAGING;
+        // One TMEM lane (X row of the tile) per thread; group g of four warps takes half of the columns.
+        const int qd = warp & 3, g = (warp - 2) >> 2;
+        uint8_t* stg = staging + (warp - 2) * PG_STAGING;
         // Through the staging, lane l handles 16-byte chunk l mod 8 of rows 4 i + l / 8 of the warp's 32.
         const int sr = lane >> 3, sc = lane & 7;
         auto own_chunk = [&](int c) { return (uint4*)(stg + lane * 128 + ((c ^ (lane & 7)) << 4)); };
@@ -590,16 +592,15 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pf_gemm(const __grid_constant
                 // Steps of 16 rotary pairs: columns c1.. and c1 + D / 2.. of one head section.
                 const int half = a.D >> 1;
                 int pos[8];
-                size_t qo[8], kvo[8];
+                size_t kvo[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     const int m = min(m0 + 4 * i + sr, a.M - 1), b = m / a.P;
                     pos[i] = m - b * a.P;
-                    qo[i] = (size_t)m * a.H * a.D;
                     kvo[i] = (size_t)b * a.kv_stride + (size_t)pos[i] * a.D;
                 }
 #pragma unroll 1
-                for (int s = 0; s < PG_TN / 32; ++s) {
+                for (int s = g * (PG_TN / 64); s < (g + 1) * (PG_TN / 64); ++s) {
                     const int sl = 16 * s / half, j0 = 16 * s - sl * half;   // section of the tile, first pair
                     const int sec = tn * (PG_TN / a.D) + sl, c1 = sl * a.D + j0;
                     const bool rot = sec <= a.H, in = sec < a.H + 2;
@@ -621,7 +622,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pf_gemm(const __grid_constant
                         const float ua = __uint_as_float(v.x), ub = __uint_as_float(v.y);
                         const float va = __uint_as_float(v.z), vb = __uint_as_float(v.w);
                         if (!ok || !in || m0 + 4 * i + sr >= a.M) continue;
-                        __nv_bfloat16* d = (sec < a.H ? a.q + qo[i] + (size_t)sec * a.D : (sec == a.H ? a.kd : a.vd) + kvo[i]) +
+                        __nv_bfloat16* d = (sec < a.H ? a.q + ((size_t)(m0 + 4 * i + sr) * a.H + sec) * a.D : (sec == a.H ? a.kd : a.vd) + kvo[i]) +
                                            j0 + 2 * sc;
                         *(uint32_t*)d = pack2(ua * cs[i].x - va * cs[i].y, ub * cs[i].z - vb * cs[i].w);
                         *(uint32_t*)(d + half) = pack2(va * cs[i].x + ua * cs[i].y, vb * cs[i].z + ub * cs[i].w);
@@ -632,7 +633,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pf_gemm(const __grid_constant
                 // Outputs that take no 16-byte access: a row per thread, element by element.
                 const int m = m0 + lane;
                 const int nc = a.geglu ? PG_TN / 2 : PG_TN, nlim = a.geglu ? a.nz : a.N;
-                for (int c0 = 0; c0 < nc; c0 += 16) {
+                for (int c0 = g * nc / 2; c0 < (g + 1) * nc / 2; c0 += 16) {
                     uint32_t r[16], r2[16];
                     ptx::tmem_ld_x16(acc + (uint32_t)c0, r);
                     if (a.geglu) ptx::tmem_ld_x16(acc + (uint32_t)(PG_TN / 2 + c0), r2);
@@ -652,7 +653,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pf_gemm(const __grid_constant
             } else if (a.geglu || a.out_bf16) {
                 // 64 bf16 outputs of a row per pass (GeGLU: gate columns c.. and up columns 128 + c..).
                 const int nc = a.geglu ? PG_TN / 2 : PG_TN, nlim = a.geglu ? a.nz : a.N;
-                for (int c0 = 0; c0 < nc; c0 += 64) {
+                for (int c0 = g * nc / 2; c0 < (g + 1) * nc / 2; c0 += 64) {
                     const int n0 = tn * nc + c0;
                     if (n0 >= nlim) break;
 #pragma unroll
@@ -697,7 +698,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pf_gemm(const __grid_constant
             } else {
                 // 32 fp32 outputs of a row per pass.
                 const bool accum = a.accumulate && !a.stream;
-                for (int c0 = 0; c0 < PG_TN; c0 += 32) {
+                for (int c0 = g * PG_TN / 2; c0 < (g + 1) * PG_TN / 2; c0 += 32) {
                     const int n0 = tn * PG_TN + c0;
                     if (n0 >= a.N) break;
                     const int n = n0 + 4 * sc;
@@ -807,6 +808,8 @@ struct jpi_prefill_handle {
     __nv_bfloat16* vt = nullptr;     // [D][Pp] one request's values, transposed
     int* dev_err = nullptr;          // device error word of the GEMM's bounded waits
     int num_sms = 0;
+    int t5_clusters[5] = {};         // row blocks whose s-CTA clusters of the attention are co-resident
+    void *t5_ws = nullptr, *t5_wml = nullptr;   // its key-split workspace: partial outputs, (m, l)
     bool qkv_fused() const { return D == 128 || D == 256; }
 };
 
@@ -906,14 +909,22 @@ jpi_status row_gemm(jpi_prefill_handle* h, cudaStream_t st, const __nv_bfloat16*
 }
 
 // CTAs a residual product [M][N] over K is dealt out to (stream-K), or 0: whole tiles, accumulated in
-// place. Up to 4/5 of a wave of tiles (at Gemma-2B sizes and 816 tokens O and down have 56: dealt out,
-// every CTA takes 11.8 of O's and 94.3 of down's k-blocks; two K ranges per tile kept 112 of 152 SMs
-// busy, 16 and 128 k-blocks each), at most 8 CTAs a tile and 8 k-blocks a CTA.
+// place. Up to 4/5 of a wave of tiles, at most 8 CTAs a tile and at least 8 k-blocks a CTA. A CTA that
+// cuts across tiles writes a piece for each, worth about PG_PIECE_KB k-blocks, so the choice is between
+// every SM (each CTA two pieces) and the whole number of CTAs per tile that fits (one piece): at
+// Gemma-2B sizes and 816 tokens (56 tiles) down (256 k-blocks a tile) takes 152 CTAs of 94.3 k-blocks,
+// O (32) 112 of 16.
+constexpr int PG_PIECE_KB = 8;
 int stream_grid(int num_sms, int M, int N, int K) {
     const long long tiles = (long long)((N + PG_TN - 1) / PG_TN) * ((M + PG_TM - 1) / PG_TM);
     const int nkb = (K + PG_KBLK - 1) / PG_KBLK;
     if (tiles * 5 > num_sms * 4ll) return 0;
-    const long long g = std::min<long long>(std::min<long long>(num_sms, 8 * tiles), tiles * nkb / 8);
+    const long long most = std::min<long long>(std::min<long long>(num_sms, 8 * tiles), tiles * nkb / 8);
+    const long long whole = most / tiles * tiles;
+    if (whole <= 0) return 0;
+    const long long kb_most = (tiles * nkb + most - 1) / most + 2 * PG_PIECE_KB;
+    const long long kb_whole = (nkb + whole / tiles - 1) / (whole / tiles) + PG_PIECE_KB;
+    const long long g = kb_most < kb_whole ? most : whole;
     return g > tiles ? (int)g : 0;
 }
 // Most pieces a tile of such a product has.
@@ -947,9 +958,30 @@ jpi_status attention_t5(jpi_prefill_handle* h, cudaStream_t st, const __nv_bfloa
     a.scale_log2 = 1.4426950408889634f / sqrtf((float)D);
     a.o = h->o;
     a.err = h->dev_err;
-    const dim3 grid((unsigned)((nrows + jpi::T5_ROWS - 1) / jpi::T5_ROWS), (unsigned)batch);
-    pdl(st, grid, dim3(jpi::T5_THREADS), jpi::T5Smem<D>::BYTES, jpi::k_attn_t5<D>, qmap, kmap,
-        vmap, a);
+    // Key splits (a cluster of 4 or 2 CTAs per row block) while they are co-resident: 51 row blocks
+    // at 816 tokens and 8 heads leave two thirds of the SMs idle unsplit.
+    const int rblocks = (int)((nrows + jpi::T5_ROWS - 1) / jpi::T5_ROWS), nb = (P + jpi::T5_KEYS - 1) / jpi::T5_KEYS;
+    int splits = 1;
+    for (int s = 4; s >= 2 && splits == 1; s /= 2)
+        if (h->t5_ws && nb >= s && (long long)rblocks * batch <= h->t5_clusters[s]) splits = s;
+    a.ws = reinterpret_cast<float4*>(h->t5_ws);
+    a.wml = reinterpret_cast<float2*>(h->t5_wml);
+    const dim3 grid((unsigned)rblocks, (unsigned)batch, (unsigned)splits);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(jpi::T5_THREADS);
+    cfg.dynamicSmemBytes = jpi::T5Smem<D>::BYTES;
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = 1;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = (unsigned)splits;
+    cfg.attrs = at;
+    cfg.numAttrs = splits > 1 ? 2 : 1;
+    (void)cudaLaunchKernelEx(&cfg, jpi::k_attn_t5<D>, qmap, kmap, vmap, a);
     PF_CUDA(cudaGetLastError());
     return JPI_OK;
 }
@@ -1036,6 +1068,35 @@ jpi_status setup(jpi_prefill_handle* h, const jpi_prefill_config* c, const jpi_p
                                  jpi::T5Smem<128>::BYTES));
     PF_CUDA(cudaFuncSetAttribute(jpi::k_attn_t5<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  jpi::T5Smem<256>::BYTES));
+    if (h->qkv_fused()) {
+        // Attention key splits: clusters that fit at once, and a workspace slot per CTA.
+        for (int s = 2; s <= 4; s *= 2) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)(h->num_sms / s), 1, (unsigned)s);
+            cfg.blockDim = dim3(jpi::T5_THREADS);
+            cfg.dynamicSmemBytes = D == 256 ? jpi::T5Smem<256>::BYTES : jpi::T5Smem<128>::BYTES;
+            cudaLaunchAttribute at;
+            at.id = cudaLaunchAttributeClusterDimension;
+            at.val.clusterDim.x = 1;
+            at.val.clusterDim.y = 1;
+            at.val.clusterDim.z = (unsigned)s;
+            cfg.attrs = &at;
+            cfg.numAttrs = 1;
+            int n = 0;
+            const cudaError_t e = D == 256 ? cudaOccupancyMaxActiveClusters(&n, jpi::k_attn_t5<256>, &cfg)
+                                           : cudaOccupancyMaxActiveClusters(&n, jpi::k_attn_t5<128>, &cfg);
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                n = 0;
+            }
+            h->t5_clusters[s] = std::min(n, h->num_sms / s);
+        }
+        uint8_t* ws = nullptr;
+        const size_t part = (size_t)h->num_sms * (D / 4) * jpi::T5_ROWS * sizeof(float4);
+        PF_TRY(pf_alloc(h, &ws, part + (size_t)h->num_sms * jpi::T5_ROWS * sizeof(float2)));
+        h->t5_ws = ws;
+        h->t5_wml = ws + part;
+    }
     PF_TRY(pf_alloc(h, &h->dev_err, 1));
     PF_CUDA(cudaMemset(h->dev_err, 0, sizeof(int)));
     float* staging = nullptr;
