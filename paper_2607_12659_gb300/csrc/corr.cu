@@ -87,6 +87,24 @@ struct LinArgs {
     int ldy;
     int rows, in, out, gelu;
     int hs_items, hs_heads, hs_dh;   // head-select mode when hs_items > 0
+    // Forms of the streamed product only (k_corr_linear_pipe):
+    int res_mod;             // > 0: residual row r mod res_mod (a table shared by the requests)
+    const float* x2;         // columns join.. of row r come from row r / x2_div of x2 (null: none)
+    int join, x2_div, ldx2;
+    int seg_out, seg_rows;   // features below seg_out: rows 0 .. seg_rows - 1 of seg_x into seg_y instead
+    const float* seg_x;
+    int seg_ldx;
+    float* seg_y;
+    int seg_ldy;
+    const float *ln_g, *ln_b;   // LayerNorm of every input row (width `in`) before the product
+    float ln_eps;
+    int att_heads_dh;        // attention form: head dim; x holds q, k at + d and v at + 2 d (d = in)
+    float att_scale;
+    // Confidence of the heads: CTAs past lin_ctas (one per request of conf_items rows) compute
+    // conf[b] = conf_w . mean of the request's normalised rows + conf_b.
+    int lin_ctas, conf_items;
+    const float *conf_w, *conf_b;
+    float* conf;
 };
 
 template <typename TW, bool VEC>
@@ -263,25 +281,169 @@ __global__ void __launch_bounds__(256) k_corr_linear16(const LinArgs a) {
 // chunks per weight chunk and was bound by those L1 reads); the per-feature sums are reduced over
 // the block in a fixed order. No waits that can spin: the copies are waited with
 // cp.async.wait_group.
+//
+// Forms that take a neighbouring kernel in, because at a handful of rows every launch of the chain
+// costs 4-5 us whatever it computes:
+//   LP_LN    LayerNorm of the input rows (in <= 2048, at most LP_LN_ROWS rows): every CTA computes the
+//            rows' mean and variance first (a warp per row, two passes over registers), then
+//            normalises each chunk as it loads it;
+//   LP_ATTN  multi-head attention among four tokens (rows r0 .. r0 + 3 are one request's): the thread's
+//            chunk of the attention output is computed in registers from its chunk of q, k and v, the
+//            scores summed over the head's lanes by shuffles;
+// and, in every form, a residual table indexed by row mod n, an input joined from two sources, a first
+// segment of features with rows of its own, and the confidence head on CTAs of its own.
 constexpr int LP_ROWS = 8;
 constexpr int LP_XR = 4;          // activation rows per pass
 constexpr int LP_MAX_IN = 4096;
+constexpr int LP_LN_ROWS = 32;
+enum { LP_PLAIN = 0, LP_LN = 1, LP_ATTN = 2 };
 __host__ __device__ constexpr int lp_stages(int in) {
     return in <= 2048 ? 4 : 3;
 }
-template <int NST>
-__global__ void __launch_bounds__(256) k_corr_linear_pipe(const LinArgs a) {
+
+// Mean and 1 / sqrt(biased variance + eps) of rows r0, r0 + step, .. (< rows) of x (width d <= 2048, a
+// multiple of 4, 16-byte aligned rows), one warp per row, into mr[r - base].
+__device__ __forceinline__ void lp_row_stats(const float* x, int ldx, int r0, int step, int rows, int d, float eps,
+                                             float2* mr, int base) {
+    const int lane = threadIdx.x & 31, d4 = d >> 2;
+    for (int r = r0; r < rows; r += step) {
+        const float4* xr = reinterpret_cast<const float4*>(x + (size_t)r * ldx);
+        float4 v[16];
+        float s = 0.f;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            const int i = lane + 32 * k;
+            v[k] = i < d4 ? xr[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int k = 0; k < 16; ++k) s += (v[k].x + v[k].y) + (v[k].z + v[k].w);
+        const float mean = warp_sum(s) / (float)d;
+        float var = 0.f;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            if (lane + 32 * k >= d4) break;
+            const float t0 = v[k].x - mean, t1 = v[k].y - mean, t2 = v[k].z - mean, t3 = v[k].w - mean;
+            var = fmaf(t0, t0, fmaf(t1, t1, fmaf(t2, t2, fmaf(t3, t3, var))));
+        }
+        const float rstd = 1.f / sqrtf(warp_sum(var) / (float)d + eps);
+        if (lane == 0) mr[r - base] = make_float2(mean, rstd);
+    }
+}
+
+__device__ __forceinline__ void lp_load8(const float* p, float (&x)[8]) {
+    const float4 x0 = *reinterpret_cast<const float4*>(p), x1 = *reinterpret_cast<const float4*>(p + 4);
+    x[0] = x0.x; x[1] = x0.y; x[2] = x0.z; x[3] = x0.w;
+    x[4] = x1.x; x[5] = x1.y; x[6] = x1.z; x[7] = x1.w;
+}
+
+// Columns 8 c .. 8 c + 7 of the attention output of four tokens, c this thread's chunk: base points at
+// the chunk of the first token's query, rows ldx apart, keys d and values 2 d further on. The dh / 8
+// lanes of a head (a power of two within a warp) sum its scores; every lane of the warp takes part.
+__device__ __forceinline__ void attn4_chunk(const float* base, int ldx, int d, int dh, float scale, float (&x)[4][8]) {
+    float q[4][8], k[4][8], v[4][8], s[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        lp_load8(base + (size_t)i * ldx, q[i]);
+        lp_load8(base + (size_t)i * ldx + d, k[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) lp_load8(base + (size_t)i * ldx + 2 * d, v[i]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            float t = 0.f;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) t = fmaf(q[i][e], k[j][e], t);
+            s[i][j] = t;
+        }
+    for (int sh = dh / 16; sh > 0; sh >>= 1)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) s[i][j] += __shfl_xor_sync(0xffffffffu, s[i][j], sh);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        float mx = -INFINITY, den = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            s[i][j] *= scale;
+            mx = fmaxf(mx, s[i][j]);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            s[i][j] = expf(s[i][j] - mx);
+            den += s[i][j];
+        }
+        const float inv = 1.f / den;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            float t = 0.f;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) t = fmaf(s[i][j], v[j][e], t);
+            x[i][e] = t * inv;
+        }
+    }
+}
+
+// The same attention as a launch of its own (one CTA per request; o [4 B][d]): bit for bit what the
+// LP_ATTN form computes, for batches where computing it in every CTA of the product takes longer.
+__global__ void __launch_bounds__(256) k_corr_attn4(const float* __restrict__ qkv, float* __restrict__ o, int d, int dh,
+                                                    float scale) {
+    jpi::ptx::grid_dep_wait();
+    jpi::ptx::grid_dep_launch();
+    const int nch = d / 8, c = (int)threadIdx.x < nch ? threadIdx.x : 0;
+    float x[4][8];
+    attn4_chunk(qkv + (size_t)blockIdx.x * 4 * 3 * d + 8 * c, 3 * d, d, dh, scale, x);
+    if ((int)threadIdx.x >= nch) return;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        float4* y = reinterpret_cast<float4*>(o + ((size_t)blockIdx.x * 4 + i) * d + 8 * c);
+        y[0] = make_float4(x[i][0], x[i][1], x[i][2], x[i][3]);
+        y[1] = make_float4(x[i][4], x[i][5], x[i][6], x[i][7]);
+    }
+}
+
+template <int NST, int MODE>
+__global__ void __launch_bounds__(256) k_corr_linear_pipe(const __grid_constant__ LinArgs a) {
     extern __shared__ __align__(128) uint8_t lp_smem[];
     __shared__ float red[8][LP_ROWS * LP_XR];
+    __shared__ float2 mr[LP_LN_ROWS];   // LayerNorm: (mean, 1 / std) of each row
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int in = a.in, nch = in / 8;
+    if (MODE == LP_LN && a.conf && (int)blockIdx.x >= a.lin_ctas) {
+        // The confidence of request b: features tid, tid + 256, .. of the mean normalised row.
+        jpi::ptx::grid_dep_wait();
+        jpi::ptx::grid_dep_launch();
+        const int b = blockIdx.x - a.lin_ctas, n = a.conf_items;
+        lp_row_stats(a.x, a.ldx, b * n + warp, 8, (b + 1) * n, in, a.ln_eps, mr, b * n);
+        __syncthreads();
+        float s = 0.f;
+        for (int c = tid; c < in; c += 256) {
+            float m = 0.f;
+            for (int i = 0; i < n; ++i)
+                m += (a.x[(size_t)(b * n + i) * a.ldx + c] - mr[i].x) * mr[i].y * a.ln_g[c] + a.ln_b[c];
+            s = fmaf(a.conf_w[c], m / (float)n, s);
+        }
+        s = warp_sum(s);
+        if (lane == 0) red[0][warp] = s;
+        __syncthreads();
+        if (tid == 0) {
+            float v = 0.f;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) v += red[0][w];
+            a.conf[b] = v + a.conf_b[0];
+        }
+        return;
+    }
     const int sbytes = LP_ROWS * in * 2;
     const int ngroups = (a.out + LP_ROWS - 1) / LP_ROWS;
+    const int nctas = a.lin_ctas;
     const uint8_t* W = static_cast<const uint8_t*>(a.w);
-    // Group k of this CTA: blockIdx.x + k gridDim.x; its rows into stage k mod NST (one commit
+    // Group k of this CTA: blockIdx.x + k nctas; its rows into stage k mod NST (one commit
     // group per k, empty past the last group, so the group count stays uniform).
     auto issue = [&](int k) {
-        const int g = blockIdx.x + k * gridDim.x;
+        const int g = blockIdx.x + k * nctas;
         if (g < ngroups) {
             const int rows = min(LP_ROWS, a.out - g * LP_ROWS);
             const int chunks = rows * nch;
@@ -295,15 +457,25 @@ __global__ void __launch_bounds__(256) k_corr_linear_pipe(const LinArgs a) {
     for (int k = 0; k < NST - 1; ++k) issue(k);
     jpi::ptx::grid_dep_wait();
     jpi::ptx::grid_dep_launch();
-    for (int k = 0; blockIdx.x + k * gridDim.x < ngroups; ++k) {
+    if (MODE == LP_LN) {
+        lp_row_stats(a.x, a.ldx, warp, 8, a.rows, in, a.ln_eps, mr, 0);
+        __syncthreads();
+    }
+    for (int k = 0; blockIdx.x + k * nctas < ngroups; ++k) {
         issue(k + NST - 1);
         asm volatile("cp.async.wait_group %0;" ::"n"(NST - 1) : "memory");
         __syncthreads();   // stage k mod NST holds group k for every thread
-        const int o0 = (blockIdx.x + k * gridDim.x) * LP_ROWS;
+        const int o0 = (blockIdx.x + k * nctas) * LP_ROWS;
         const int nout = min(LP_ROWS, a.out - o0);
         const uint4* wst = reinterpret_cast<const uint4*>(lp_smem + (size_t)(k % NST) * sbytes);
-        for (int r0 = 0; r0 < a.rows; r0 += LP_XR) {
-            const int nr = min(LP_XR, a.rows - r0);
+        // Rows, input and output of this group's segment (seg_out is a multiple of LP_ROWS). The
+        // segment's input rows are rows of x: their statistics are found by the address.
+        const bool seg = o0 < a.seg_out;
+        const int rows = seg ? a.seg_rows : a.rows, ldx = seg ? a.seg_ldx : a.ldx, ldy = seg ? a.seg_ldy : a.ldy;
+        const float* xb = seg ? a.seg_x : a.x;
+        float* yb = seg ? a.seg_y : a.y;
+        for (int r0 = 0; r0 < rows; r0 += LP_XR) {
+            const int nr = min(LP_XR, rows - r0);
             // The bias and residual of this thread's output (thread o LP_XR + q writes feature
             // o0 + o of row r0 + q), fetched before the products so their latency hides there.
             float bias_v = 0.f, res_v = 0.f;
@@ -311,7 +483,8 @@ __global__ void __launch_bounds__(256) k_corr_linear_pipe(const LinArgs a) {
                 const int o = tid / LP_XR, q = tid % LP_XR;
                 if (o < nout && q < nr) {
                     if (a.bias) bias_v = a.bias[o0 + o];
-                    if (a.res) res_v = a.res[(size_t)(r0 + q) * a.ldr + o0 + o];
+                    const int rr = a.res_mod > 0 ? (r0 + q) % a.res_mod : r0 + q;
+                    if (a.res) res_v = a.res[(size_t)rr * a.ldr + o0 + o];
                 }
             }
             float acc[LP_ROWS][LP_XR];
@@ -319,19 +492,8 @@ __global__ void __launch_bounds__(256) k_corr_linear_pipe(const LinArgs a) {
             for (int o = 0; o < LP_ROWS; ++o)
 #pragma unroll
                 for (int q = 0; q < LP_XR; ++q) acc[o][q] = 0.f;
-            for (int c = tid; c < nch; c += 256) {
-                float x[LP_XR][8];
-#pragma unroll
-                for (int q = 0; q < LP_XR; ++q) {
-                    float4 x0 = make_float4(0.f, 0.f, 0.f, 0.f), x1 = x0;
-                    if (q < nr) {
-                        const float* xr = a.x + (size_t)(r0 + q) * a.ldx + 8 * c;
-                        x0 = *reinterpret_cast<const float4*>(xr);
-                        x1 = *reinterpret_cast<const float4*>(xr + 4);
-                    }
-                    x[q][0] = x0.x; x[q][1] = x0.y; x[q][2] = x0.z; x[q][3] = x0.w;
-                    x[q][4] = x1.x; x[q][5] = x1.y; x[q][6] = x1.z; x[q][7] = x1.w;
-                }
+            // Chunk c (8 columns) of rows r0 .. r0 + 3 against the group's weight rows.
+            auto product = [&](int c, const float (&x)[LP_XR][8]) {
 #pragma unroll
                 for (int o = 0; o < LP_ROWS; ++o) {
                     if (o >= nout) break;
@@ -351,6 +513,40 @@ __global__ void __launch_bounds__(256) k_corr_linear_pipe(const LinArgs a) {
                         for (int e = 0; e < 8; ++e) t = fmaf(w[e], x[q][e], t);
                         acc[o][q] = t;
                     }
+                }
+            };
+            if constexpr (MODE == LP_ATTN) {
+                // One chunk per thread (in <= 2048).
+                const int c = tid < nch ? tid : 0;
+                float x[LP_XR][8];
+                attn4_chunk(xb + (size_t)r0 * ldx + 8 * c, ldx, in, a.att_heads_dh, a.att_scale, x);
+                if (tid < nch) product(tid, x);
+            } else {
+                for (int c = tid; c < nch; c += 256) {
+                    float x[LP_XR][8];
+                    float gv[8], bv[8];
+                    if (MODE == LP_LN) {
+                        lp_load8(a.ln_g + 8 * c, gv);
+                        lp_load8(a.ln_b + 8 * c, bv);
+                    }
+#pragma unroll
+                    for (int q = 0; q < LP_XR; ++q) {
+                        if (q < nr) {
+                            const bool second = a.x2 && 8 * c >= a.join;
+                            lp_load8(second ? a.x2 + (size_t)((r0 + q) / a.x2_div) * a.ldx2 + (8 * c - a.join)
+                                         : xb + (size_t)(r0 + q) * ldx + 8 * c, x[q]);
+                            if (MODE == LP_LN) {
+                                // Row of x this is (a segment's rows are a subset of them).
+                                const float2 st = mr[seg ? (int)((a.seg_x - a.x + (size_t)(r0 + q) * ldx) / a.ldx) : r0 + q];
+#pragma unroll
+                                for (int e = 0; e < 8; ++e) x[q][e] = (x[q][e] - st.x) * st.y * gv[e] + bv[e];
+                            }
+                        } else {
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) x[q][e] = 0.f;
+                        }
+                    }
+                    product(c, x);
                 }
             }
             // (feature o, row q) sums: over the warp's lanes, then over the 8 warps in order. The
@@ -386,7 +582,7 @@ __global__ void __launch_bounds__(256) k_corr_linear_pipe(const LinArgs a) {
                     v += bias_v;
                     if (a.gelu) v = gelu_tanh_f(v);
                     if (a.res) v += res_v;
-                    a.y[(size_t)r * a.ldy + of] = v;
+                    yb[(size_t)r * ldy + of] = v;
                 }
             }
             __syncthreads();   // red is reused by the next pass
@@ -605,7 +801,8 @@ constexpr size_t CORR_SCORES_SMEM = (size_t)(CORR_MAX_M + 32) * CORR_KPAD * size
 // VEC: dv a multiple of 4 and hv aligned to four elements, so the staging moves four features
 // per load; every thread's staging loads are issued before any of its stores (one at a time, each
 // store would hold the next load back for a full L2 round trip).
-template <typename THV, bool VEC>
+// RM: query rows per thread, 8 RM >= M.
+template <typename THV, bool VEC, int RM>
 __global__ void __launch_bounds__(256) k_corr_scores(const float* __restrict__ qk, const THV* __restrict__ hv,
                                                      float* __restrict__ part, int M, int T, int dv) {
     // Launched with programmatic dependent launch: wait for the previous kernel's results, then
@@ -623,9 +820,9 @@ __global__ void __launch_bounds__(256) k_corr_scores(const float* __restrict__ q
         // rows and 8 token rows at most.
         const int k4 = threadIdx.x & 63, r0 = threadIdx.x >> 6, kk = 4 * k4;
         const bool kin = kk < cn;
-        float4 qa[CORR_MAX_M / 4], hb4[8];
+        float4 qa[2 * RM], hb4[8];
 #pragma unroll
-        for (int i = 0; i < CORR_MAX_M / 4; ++i) {
+        for (int i = 0; i < 2 * RM; ++i) {
             const int m = r0 + 4 * i;
             qa[i] = (m < M && kin) ? *reinterpret_cast<const float4*>(qk + (size_t)m * dv + c0 + kk)
                                    : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -636,16 +833,13 @@ __global__ void __launch_bounds__(256) k_corr_scores(const float* __restrict__ q
             hb4[i] = (j < T && kin) ? load4(hb + (size_t)j * dv + c0 + kk) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
-        for (int i = 0; i < CORR_MAX_M / 4; ++i) {
-            const int m = r0 + 4 * i;
-            if (m < M) *reinterpret_cast<float4*>(as + m * CORR_KPAD + kk) = qa[i];
-        }
+        for (int i = 0; i < 2 * RM; ++i) *reinterpret_cast<float4*>(as + (r0 + 4 * i) * CORR_KPAD + kk) = qa[i];
 #pragma unroll
         for (int i = 0; i < 8; ++i) *reinterpret_cast<float4*>(bs + (r0 + 4 * i) * CORR_KPAD + kk) = hb4[i];
     } else {
-        for (int idx = threadIdx.x; idx < M * CORR_KCHUNK; idx += 256) {
+        for (int idx = threadIdx.x; idx < 8 * RM * CORR_KCHUNK; idx += 256) {
             const int m = idx / CORR_KCHUNK, kk = idx % CORR_KCHUNK;
-            as[m * CORR_KPAD + kk] = kk < cn ? qk[(size_t)m * dv + c0 + kk] : 0.f;
+            as[m * CORR_KPAD + kk] = m < M && kk < cn ? qk[(size_t)m * dv + c0 + kk] : 0.f;
         }
         for (int idx = threadIdx.x; idx < 32 * CORR_KCHUNK; idx += 256) {
             const int t = idx / CORR_KCHUNK, kk = idx % CORR_KCHUNK, j = j0 + t;
@@ -653,35 +847,43 @@ __global__ void __launch_bounds__(256) k_corr_scores(const float* __restrict__ q
         }
     }
     __syncthreads();
-    constexpr int RM = CORR_MAX_M / 16;   // rows per thread at most
-    const int mg = threadIdx.x >> 4, jg = threadIdx.x & 15;
-    float acc[RM][2];
+    // Thread (kg, mg, jg) takes features 64 kg .. of the chunk, query rows mg + 8 r and tokens jg + 8 u:
+    // per four features 8 + RM 16-byte loads for 16 RM products (RM = 4 for M <= 32, else 8).
+    const int kg = threadIdx.x >> 6, mg = (threadIdx.x >> 3) & 7, jg = threadIdx.x & 7;
+    float acc[RM][4];
 #pragma unroll
-    for (int r = 0; r < RM; ++r) acc[r][0] = acc[r][1] = 0.f;
-    const float4* b0 = reinterpret_cast<const float4*>(bs + jg * CORR_KPAD);
-    const float4* b1 = reinterpret_cast<const float4*>(bs + (jg + 16) * CORR_KPAD);
+    for (int r = 0; r < RM; ++r)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[r][u] = 0.f;
+    const float* ap = as + mg * CORR_KPAD + 64 * kg;
+    const float* bp = bs + jg * CORR_KPAD + 64 * kg;
 #pragma unroll 4
-    for (int k4 = 0; k4 < CORR_KCHUNK / 4; ++k4) {
-        const float4 x0 = b0[k4], x1 = b1[k4];
+    for (int k = 0; k < 64; k += 4) {
+        float4 x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = *reinterpret_cast<const float4*>(bp + 8 * u * CORR_KPAD + k);
 #pragma unroll
         for (int r = 0; r < RM; ++r) {
-            const int m = mg + 16 * r;
-            if (m < M) {
-                const float4 q = reinterpret_cast<const float4*>(as + m * CORR_KPAD)[k4];
-                acc[r][0] = fmaf(q.w, x0.w, fmaf(q.z, x0.z, fmaf(q.y, x0.y, fmaf(q.x, x0.x, acc[r][0]))));
-                acc[r][1] = fmaf(q.w, x1.w, fmaf(q.z, x1.z, fmaf(q.y, x1.y, fmaf(q.x, x1.x, acc[r][1]))));
-            }
+            const float4 q = *reinterpret_cast<const float4*>(ap + 8 * r * CORR_KPAD + k);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                acc[r][u] = fmaf(q.w, x[u].w, fmaf(q.z, x[u].z, fmaf(q.y, x[u].y, fmaf(q.x, x[u].x, acc[r][u]))));
         }
     }
+    // The four feature groups' sums in order, through shared memory (over the staged operands).
+    __syncthreads();
+    float* sums = as;   // [4][8 RM rows][33]
 #pragma unroll
-    for (int r = 0; r < RM; ++r) {
-        const int m = mg + 16 * r;
-        if (m >= M) continue;
+    for (int r = 0; r < RM; ++r)
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int j = j0 + jg + 16 * u;
-            if (j < T) part[(((size_t)b * gridDim.y + kc) * M + m) * T + j] = acc[r][u];
-        }
+        for (int u = 0; u < 4; ++u) sums[(kg * 8 * RM + mg + 8 * r) * 33 + jg + 8 * u] = acc[r][u];
+    __syncthreads();
+    for (int idx = threadIdx.x; idx < M * 32; idx += 256) {
+        const int m = idx >> 5, u = idx & 31, j = j0 + u;
+        float v = 0.f;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) v += sums[(g * 8 * RM + m) * 33 + u];
+        if (j < T) part[(((size_t)b * gridDim.y + kc) * M + m) * T + j] = v;
     }
 }
 
@@ -743,9 +945,11 @@ __global__ void __launch_bounds__(256) k_corr_softmax_sum(const float* __restric
 // (tid mod 128, tid / 128) takes columns 2 cg, 2 cg + 1 of the CTA's 256 and rows mg RH .. + RH - 1
 // (RH = 16 for M <= 32, else 32), token after token in order; the chunk's probabilities sit in
 // shared memory transposed ([token][row], read as 16-byte broadcasts) and each token's two values
-// come in one load, eight tokens' loads in flight together. The token chunks are added in order
+// come in one load, CORR_TB tokens' loads in flight together (a chunk of 64 tokens eight at a time
+// was eight L2 round trips in a row on 104 CTAs). The token chunks are added in order
 // by k_corr_wsum_reduce.
-constexpr int CORR_TCHUNK = 64;
+constexpr int CORR_TCHUNK = 32;
+constexpr int CORR_TB = 16;     // tokens whose values a thread has in flight
 constexpr int CORR_PTS = CORR_MAX_M + 4;   // row stride of the transposed probabilities
 
 template <typename THV>
@@ -771,17 +975,17 @@ __global__ void __launch_bounds__(256) k_corr_wsum(const float* __restrict__ p, 
     const int b = blockIdx.z, tc = blockIdx.y;
     const int j0 = tc * CORR_TCHUNK, jn = min(CORR_TCHUNK, T - j0);
     {
-        // Thread t loads token t mod 64 of rows t / 64, t / 64 + 4, .. (coalesced along the
+        // Thread t loads token t mod 32 of rows t / 32, t / 32 + 8, .. (coalesced along the
         // tokens, all loads before the transposed stores); rows past M are zero.
-        const int jj = threadIdx.x & 63, r0 = threadIdx.x >> 6;
-        float pv[CORR_PTS / 4];
+        const int jj = threadIdx.x & 31, r0 = threadIdx.x >> 5;
+        float pv[CORR_MAX_M / 8];
 #pragma unroll
-        for (int i = 0; i < CORR_PTS / 4; ++i) {
-            const int r = r0 + 4 * i;
+        for (int i = 0; i < CORR_MAX_M / 8; ++i) {
+            const int r = r0 + 8 * i;
             pv[i] = (jj < jn && r < M) ? p[((size_t)b * M + r) * T + j0 + jj] : 0.f;
         }
 #pragma unroll
-        for (int i = 0; i < CORR_PTS / 4; ++i) pt[jj][r0 + 4 * i] = pv[i];
+        for (int i = 0; i < CORR_MAX_M / 8; ++i) pt[jj][r0 + 8 * i] = pv[i];
     }
     __syncthreads();
     const int cg = threadIdx.x & 127, mg = threadIdx.x >> 7;
@@ -792,10 +996,10 @@ __global__ void __launch_bounds__(256) k_corr_wsum(const float* __restrict__ p, 
 #pragma unroll
     for (int i = 0; i < RH; ++i) acc[i][0] = acc[i][1] = 0.f;
     const THV* hb = hv + ((size_t)b * T + j0) * dv + c;
-    for (int jb = 0; jb < jn; jb += 8) {
-        float2 hvv[8];
+    for (int jb = 0; jb < jn; jb += CORR_TB) {
+        float2 hvv[CORR_TB];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
+        for (int u = 0; u < CORR_TB; ++u) {
             hvv[u] = make_float2(0.f, 0.f);
             if (jb + u < jn) {
                 const THV* hp = hb + (size_t)(jb + u) * dv;
@@ -804,7 +1008,7 @@ __global__ void __launch_bounds__(256) k_corr_wsum(const float* __restrict__ p, 
             }
         }
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
+        for (int u = 0; u < CORR_TB; ++u) {
             const float4* prow = reinterpret_cast<const float4*>(&pt[jb + u][m0]);
 #pragma unroll
             for (int i4 = 0; i4 < RH / 4; ++i4) {
@@ -1119,11 +1323,57 @@ void pdl(cudaStream_t st, dim3 grid, dim3 block, size_t smem, void (*k)(KArgs...
     (void)cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...);
 }
 
+// Whether a product can stream its weights through shared memory (k_corr_linear_pipe): bf16 rows of
+// 16-byte chunks up to LP_MAX_IN, 16-byte aligned activations.
+bool pipe_ok(const jpi_corr_handle* h, const float* x, int ldx, const void* w, int in) {
+    return h->bf16 && in % 8 == 0 && in <= LP_MAX_IN && ldx % 4 == 0 && ((uintptr_t)x & 15) == 0 &&
+           ((uintptr_t)w & 15) == 0;
+}
+// Whether its LayerNorm form takes `rows` rows of the module's width: every CTA computes the rows'
+// statistics, up to two rows per warp (about the time of one; more would cost what the launch saved).
+bool ln_fused(const jpi_corr_handle* h, const float* x, int ldx, const void* w, int rows) {
+    return pipe_ok(h, x, ldx, w, h->d) && h->d <= 2048 && rows <= 16;
+}
+
+// By persistent CTAs, one per SM at most (plus `extra` for the confidence head).
+jpi_status launch_pipe(const jpi_corr_handle* h, cudaStream_t st, int mode, LinArgs a, int extra = 0) {
+    const int groups = (a.out + LP_ROWS - 1) / LP_ROWS;
+    a.lin_ctas = groups < h->num_sms ? groups : h->num_sms;
+    const int nst = lp_stages(a.in);
+    const size_t smem = (size_t)nst * LP_ROWS * a.in * 2;
+    const dim3 grid(a.lin_ctas + extra), block(256);
+    if (mode == LP_LN) pdl(st, grid, block, smem, k_corr_linear_pipe<4, LP_LN>, a);
+    else if (mode == LP_ATTN) pdl(st, grid, block, smem, k_corr_linear_pipe<4, LP_ATTN>, a);
+    else if (nst == 4) pdl(st, grid, block, smem, k_corr_linear_pipe<4, LP_PLAIN>, a);
+    else pdl(st, grid, block, smem, k_corr_linear_pipe<3, LP_PLAIN>, a);
+    JPI_CUDA_TRY(cudaGetLastError());
+    return JPI_OK;
+}
+
+// Arguments of y [rows][out] = act(x [rows][in] w^T + bias) + res.
+LinArgs lin_args(const float* x, int ldx, const void* w, const float* bias, const float* res, int ldr, float* y, int ldy,
+                 int rows, int in, int out, bool gelu) {
+    LinArgs a = {};
+    a.x = x;
+    a.ldx = ldx;
+    a.w = w;
+    a.bias = bias;
+    a.res = res;
+    a.ldr = ldr;
+    a.y = y;
+    a.ldy = ldy;
+    a.rows = rows;
+    a.in = in;
+    a.out = out;
+    a.gelu = gelu ? 1 : 0;
+    return a;
+}
+
 jpi_status linear(const jpi_corr_handle* h, cudaStream_t st, const float* x, int ldx, const void* w,
                   const float* bias, const float* res, int ldr, float* y, int ldy, int rows, int in,
                   int out, bool gelu, int hs_items = 0) {
     if (rows <= 0 || out <= 0) return JPI_OK;
-    LinArgs a;
+    LinArgs a = {};
     a.x = x;
     a.ldx = ldx;
     a.w = w;
@@ -1141,19 +1391,7 @@ jpi_status linear(const jpi_corr_handle* h, cudaStream_t st, const float* x, int
     a.hs_dh = h->Dh;
     const bool vec = in % 4 == 0 && ldx % 4 == 0 && ((uintptr_t)x & 15) == 0 &&
                      ((uintptr_t)w & (h->bf16 ? 7 : 15)) == 0;
-    // bf16 rows of 16-byte chunks up to LP_MAX_IN, no head-select: streamed through shared memory
-    // by persistent CTAs, one per SM at most.
-    if (h->bf16 && hs_items == 0 && in % 8 == 0 && in <= LP_MAX_IN && ldx % 4 == 0 && ((uintptr_t)x & 15) == 0 &&
-        ((uintptr_t)w & 15) == 0) {
-        const int groups = (out + LP_ROWS - 1) / LP_ROWS;
-        const int nb = groups < h->num_sms ? groups : h->num_sms;
-        const int nst = lp_stages(in);
-        const size_t smem = (size_t)nst * LP_ROWS * in * 2;
-        if (nst == 4) pdl(st, dim3(nb), dim3(256), smem, k_corr_linear_pipe<4>, a);
-        else pdl(st, dim3(nb), dim3(256), smem, k_corr_linear_pipe<3>, a);
-        JPI_CUDA_TRY(cudaGetLastError());
-        return JPI_OK;
-    }
+    if (hs_items == 0 && pipe_ok(h, x, ldx, w, in)) return launch_pipe(h, st, LP_PLAIN, a);
     // Other bf16 rows of 16-byte chunks: the streaming kernel, with 2 or 4 warps per output
     // feature while that keeps at least 256 inputs a warp and brings the launch towards 2048 warps.
     if (h->bf16 && in % 8 == 0 && ldx % 4 == 0 && ((uintptr_t)x & 15) == 0 && ((uintptr_t)w & 15) == 0) {
@@ -1194,6 +1432,22 @@ jpi_status layernorm(const jpi_corr_handle* h, cudaStream_t st, const float* x, 
     return JPI_OK;
 }
 
+// y = act(LN(x) w^T + bias) over rows of the module's width: one launch where ln_fused, else the
+// LayerNorm into u first.
+jpi_status ln_linear(const jpi_corr_handle* h, cudaStream_t st, const float* x, const float* g, const float* b, float* u,
+                     const void* w, const float* bias, float* y, int rows, int out, bool gelu) {
+    const int d = h->d;
+    if (ln_fused(h, x, d, w, rows)) {
+        LinArgs a = lin_args(x, d, w, bias, nullptr, 0, y, out, rows, d, out, gelu);
+        a.ln_g = g;
+        a.ln_b = b;
+        a.ln_eps = h->cfg.ln_eps;
+        return launch_pipe(h, st, LP_LN, a);
+    }
+    JPI_TRY(layernorm(h, st, x, d, g, b, u, d, rows));
+    return linear(h, st, u, d, w, bias, nullptr, 0, y, out, rows, d, out, gelu);
+}
+
 jpi_status attention(const jpi_corr_handle* h, cudaStream_t st, const float* q, int ldq, const float* k,
                      int ldk, const float* v, int ldv, float* o, int ldo, int B, int nq, int nk) {
     AttnSmallArgs a;
@@ -1220,12 +1474,26 @@ jpi_status attention(const jpi_corr_handle* h, cudaStream_t st, const float* q, 
 // One pre-LN block over `rows` rows of x (rows = B n, n tokens per request), in place.
 jpi_status block(const jpi_corr_handle* h, cudaStream_t st, const BlockDev& w, float* x, int B, int n) {
     const int d = h->d, rows = B * n;
-    JPI_TRY(layernorm(h, st, x, d, w.ln1_w, w.ln1_b, h->u, d, rows));
-    JPI_TRY(linear(h, st, h->u, d, w.wqkv, w.bqkv, nullptr, 0, h->qkv, 3 * d, rows, d, 3 * d, false));
-    JPI_TRY(attention(h, st, h->qkv, 3 * d, h->qkv + d, 3 * d, h->qkv + 2 * d, 3 * d, h->o, d, B, n, n));
-    JPI_TRY(linear(h, st, h->o, d, w.wo, w.bo, x, d, x, d, rows, d, d, false));
-    JPI_TRY(layernorm(h, st, x, d, w.ln2_w, w.ln2_b, h->u, d, rows));
-    JPI_TRY(linear(h, st, h->u, d, w.w1, w.b1, nullptr, 0, h->hid, h->F, rows, d, h->F, true));
+    JPI_TRY(ln_linear(h, st, x, w.ln1_w, w.ln1_b, h->u, w.wqkv, w.bqkv, h->qkv, rows, 3 * d, false));
+    // Attention among four tokens goes into the output product for one or two requests (every CTA
+    // computes it: more requests take longer there than in a launch of their own). Which kernels run
+    // must not show in a request's result, so both ways compute the same sums.
+    const bool four = n == LP_XR && (h->Dh & (h->Dh - 1)) == 0 && d <= 2048 && pipe_ok(h, h->qkv, 3 * d, w.wo, d);
+    if (four && B <= 2) {
+        LinArgs a = lin_args(h->qkv, 3 * d, w.wo, w.bo, x, d, x, d, rows, d, d, false);
+        a.att_heads_dh = h->Dh;
+        a.att_scale = 1.f / sqrtf((float)h->Dh);
+        JPI_TRY(launch_pipe(h, st, LP_ATTN, a));
+    } else {
+        if (four) {
+            pdl(st, dim3(B), dim3(256), 0, k_corr_attn4, (const float*)h->qkv, h->o, d, h->Dh, 1.f / sqrtf((float)h->Dh));
+            JPI_CUDA_TRY(cudaGetLastError());
+        } else {
+            JPI_TRY(attention(h, st, h->qkv, 3 * d, h->qkv + d, 3 * d, h->qkv + 2 * d, 3 * d, h->o, d, B, n, n));
+        }
+        JPI_TRY(linear(h, st, h->o, d, w.wo, w.bo, x, d, x, d, rows, d, d, false));
+    }
+    JPI_TRY(ln_linear(h, st, x, w.ln2_w, w.ln2_b, h->u, w.w1, w.b1, h->hid, rows, h->F, true));
     JPI_TRY(linear(h, st, h->hid, h->F, w.w2, w.b2, x, d, x, d, rows, h->F, d, false));
     return JPI_OK;
 }
@@ -1378,17 +1646,17 @@ jpi_status setup(jpi_corr_handle* h, const jpi_corr_config* c, const jpi_corr_we
     JPI_TRY(corr_alloc(h, &h->out_st, B * (size_t)h->Ti * h->d));
     JPI_TRY(corr_alloc(h, &h->out_conf, (size_t)B));
     JPI_CUDA_TRY(cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking));
-    JPI_CUDA_TRY(cudaFuncSetAttribute(k_corr_scores<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)CORR_SCORES_SMEM));
-    JPI_CUDA_TRY(cudaFuncSetAttribute(k_corr_scores<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)CORR_SCORES_SMEM));
-    JPI_CUDA_TRY(cudaFuncSetAttribute(k_corr_scores<__nv_bfloat16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)CORR_SCORES_SMEM));
-    JPI_CUDA_TRY(cudaFuncSetAttribute(k_corr_scores<__nv_bfloat16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)CORR_SCORES_SMEM));
-    JPI_CUDA_TRY(cudaFuncSetAttribute(k_corr_linear_pipe<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      4 * LP_ROWS * 2048 * 2));
-    JPI_CUDA_TRY(cudaFuncSetAttribute(k_corr_linear_pipe<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    JPI_CUDA_TRY(cudaFuncSetAttribute(k_corr_scores<float, true, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SCORES_SMEM));
+    JPI_CUDA_TRY(cudaFuncSetAttribute(k_corr_scores<float, true, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SCORES_SMEM));
+    JPI_CUDA_TRY(cudaFuncSetAttribute(k_corr_scores<float, false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SCORES_SMEM));
+    JPI_CUDA_TRY(cudaFuncSetAttribute(k_corr_scores<float, false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SCORES_SMEM));
+    JPI_CUDA_TRY(cudaFuncSetAttribute(k_corr_scores<__nv_bfloat16, true, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SCORES_SMEM));
+    JPI_CUDA_TRY(cudaFuncSetAttribute(k_corr_scores<__nv_bfloat16, true, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SCORES_SMEM));
+    JPI_CUDA_TRY(cudaFuncSetAttribute(k_corr_scores<__nv_bfloat16, false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SCORES_SMEM));
+    JPI_CUDA_TRY(cudaFuncSetAttribute(k_corr_scores<__nv_bfloat16, false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SCORES_SMEM));
+    for (auto k : {k_corr_linear_pipe<4, LP_PLAIN>, k_corr_linear_pipe<4, LP_LN>, k_corr_linear_pipe<4, LP_ATTN>})
+        JPI_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * LP_ROWS * 2048 * 2));
+    JPI_CUDA_TRY(cudaFuncSetAttribute(k_corr_linear_pipe<3, LP_PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       3 * LP_ROWS * LP_MAX_IN * 2));
     {
         int dev = 0;
@@ -1417,9 +1685,9 @@ jpi_status enqueue_compress(jpi_corr_handle* h, const void* hvlm, int vlm_is_fp3
     if (vlm_is_fp32) {
         const float* hv = static_cast<const float*>(hvlm);
         if (dv % 4 == 0 && ((uintptr_t)hv & 15) == 0)
-            pdl(st, dim3(gs), dim3(256), CORR_SCORES_SMEM, k_corr_scores<float, true>, h->qk, hv, h->scp, M, n_tokens, dv);
+            pdl(st, dim3(gs), dim3(256), CORR_SCORES_SMEM, M <= 32 ? k_corr_scores<float, true, 4> : k_corr_scores<float, true, 8>, h->qk, hv, h->scp, M, n_tokens, dv);
         else
-            pdl(st, dim3(gs), dim3(256), CORR_SCORES_SMEM, k_corr_scores<float, false>, h->qk, hv, h->scp, M, n_tokens, dv);
+            pdl(st, dim3(gs), dim3(256), CORR_SCORES_SMEM, M <= 32 ? k_corr_scores<float, false, 4> : k_corr_scores<float, false, 8>, h->qk, hv, h->scp, M, n_tokens, dv);
         pdl(st, dim3(batch * M), dim3(256), 0, k_corr_softmax_sum, h->scp, h->sc, M, n_tokens, nkc);
         const bool pair = dv % 2 == 0 && ((uintptr_t)hv & 7) == 0;
         if (M <= 32) {
@@ -1432,9 +1700,9 @@ jpi_status enqueue_compress(jpi_corr_handle* h, const void* hvlm, int vlm_is_fp3
     } else {
         const __nv_bfloat16* hv = static_cast<const __nv_bfloat16*>(hvlm);
         if (dv % 4 == 0 && ((uintptr_t)hv & 7) == 0)
-            pdl(st, dim3(gs), dim3(256), CORR_SCORES_SMEM, k_corr_scores<__nv_bfloat16, true>, h->qk, hv, h->scp, M, n_tokens, dv);
+            pdl(st, dim3(gs), dim3(256), CORR_SCORES_SMEM, M <= 32 ? k_corr_scores<__nv_bfloat16, true, 4> : k_corr_scores<__nv_bfloat16, true, 8>, h->qk, hv, h->scp, M, n_tokens, dv);
         else
-            pdl(st, dim3(gs), dim3(256), CORR_SCORES_SMEM, k_corr_scores<__nv_bfloat16, false>, h->qk, hv, h->scp, M, n_tokens, dv);
+            pdl(st, dim3(gs), dim3(256), CORR_SCORES_SMEM, M <= 32 ? k_corr_scores<__nv_bfloat16, false, 4> : k_corr_scores<__nv_bfloat16, false, 8>, h->qk, hv, h->scp, M, n_tokens, dv);
         pdl(st, dim3(batch * M), dim3(256), 0, k_corr_softmax_sum, h->scp, h->sc, M, n_tokens, nkc);
         const bool pair = dv % 2 == 0 && ((uintptr_t)hv & 3) == 0;
         if (M <= 32) {
@@ -1451,8 +1719,7 @@ jpi_status enqueue_compress(jpi_corr_handle* h, const void* hvlm, int vlm_is_fp3
     // queries' residual, the MLP, and the output LayerNorm.
     JPI_TRY(linear(h, st, h->gs, dv, h->qf_ca_wv, h->qf_ca_bv, nullptr, 0, h->o, d, rows, dv, d, false, T));
     JPI_TRY(linear(h, st, h->o, d, h->qf_ca_wo, h->qf_ca_bo, h->x1b, d, h->xf, d, rows, d, d, false));
-    JPI_TRY(layernorm(h, st, h->xf, d, h->qf_ln3_w, h->qf_ln3_b, h->u, d, rows));
-    JPI_TRY(linear(h, st, h->u, d, h->qf_w1, h->qf_b1, nullptr, 0, h->hid, h->F, rows, d, h->F, true));
+    JPI_TRY(ln_linear(h, st, h->xf, h->qf_ln3_w, h->qf_ln3_b, h->u, h->qf_w1, h->qf_b1, h->hid, rows, h->F, true));
     JPI_TRY(linear(h, st, h->hid, h->F, h->qf_w2, h->qf_b2, h->xf, d, h->xf, d, rows, h->F, d, false));
     JPI_TRY(layernorm(h, st, h->xf, d, h->qf_lnf_w, h->qf_lnf_b, out, d, rows));
     return JPI_OK;
@@ -1465,27 +1732,69 @@ jpi_status enqueue_predict(jpi_corr_handle* h, const float* state, const float* 
     const BlockDev& ab = h->ab;
     // Action tokens: MLP, plus the position row of each action.
     JPI_TRY(linear(h, st, actions, h->A, h->act_w1, h->act_b1, nullptr, 0, h->t1, d, ra, h->A, d, true));
-    JPI_TRY(linear(h, st, h->t1, d, h->act_w2, h->act_b2, nullptr, 0, h->xa, d, ra, d, d, false));
-    pdl(st, dim3(grid_for((long long)ra * d)), dim3(256), 0, k_corr_add_pos, h->xa, h->act_pos, batch, delta, d);
-    JPI_CUDA_TRY(cudaGetLastError());
+    if (pipe_ok(h, h->t1, d, h->act_w2, d)) {
+        LinArgs a = lin_args(h->t1, d, h->act_w2, h->act_b2, h->act_pos, d, h->xa, d, ra, d, d, false);
+        a.res_mod = delta;
+        JPI_TRY(launch_pipe(h, st, LP_PLAIN, a));
+    } else {
+        JPI_TRY(linear(h, st, h->t1, d, h->act_w2, h->act_b2, nullptr, 0, h->xa, d, ra, d, d, false));
+        pdl(st, dim3(grid_for((long long)ra * d)), dim3(256), 0, k_corr_add_pos, h->xa, h->act_pos, batch, delta, d);
+        JPI_CUDA_TRY(cudaGetLastError());
+    }
     // Block ab, kept at the last action of each request only: keys and values of every action,
     // the query, attention output, residual and MLP of the last.
-    JPI_TRY(layernorm(h, st, h->xa, d, ab.ln1_w, ab.ln1_b, h->ua, d, ra));
-    JPI_TRY(linear(h, st, h->ua, d, tw_rows(h, ab.wqkv, (size_t)d, (size_t)d), ab.bqkv + d, nullptr, 0, h->kva,
-                   2 * d, ra, d, 2 * d, false));
     const size_t last = (size_t)(delta - 1) * d;
-    JPI_TRY(linear(h, st, h->ua + last, delta * d, ab.wqkv, ab.bqkv, nullptr, 0, h->ql, d, batch, d, d, false));
+    const bool abln = ln_fused(h, h->xa, d, ab.wqkv, ra);
+    if (!abln) JPI_TRY(layernorm(h, st, h->xa, d, ab.ln1_w, ab.ln1_b, h->ua, d, ra));
+    const float* uin = abln ? h->xa : h->ua;
+    if (pipe_ok(h, uin, d, ab.wqkv, d)) {
+        // One product: its first d features (the queries) over the last actions, the rest over all.
+        LinArgs a = lin_args(uin, d, ab.wqkv, ab.bqkv, nullptr, 0, h->kva - d, 2 * d, ra, d, 3 * d, false);
+        a.seg_out = d;
+        a.seg_rows = batch;
+        a.seg_x = uin + last;
+        a.seg_ldx = delta * d;
+        a.seg_y = h->ql;
+        a.seg_ldy = d;
+        a.ln_g = ab.ln1_w;
+        a.ln_b = ab.ln1_b;
+        a.ln_eps = h->cfg.ln_eps;
+        JPI_TRY(launch_pipe(h, st, abln ? LP_LN : LP_PLAIN, a));
+    } else {
+        JPI_TRY(linear(h, st, h->ua, d, tw_rows(h, ab.wqkv, (size_t)d, (size_t)d), ab.bqkv + d, nullptr, 0, h->kva,
+                       2 * d, ra, d, 2 * d, false));
+        JPI_TRY(linear(h, st, h->ua + last, delta * d, ab.wqkv, ab.bqkv, nullptr, 0, h->ql, d, batch, d, d, false));
+    }
     JPI_TRY(attention(h, st, h->ql, d, h->kva, 2 * d, h->kva + d, 2 * d, h->ol, d, batch, 1, delta));
     JPI_TRY(linear(h, st, h->ol, d, ab.wo, ab.bo, h->xa + last, delta * d, h->xl, d, batch, d, d, false));
-    JPI_TRY(layernorm(h, st, h->xl, d, ab.ln2_w, ab.ln2_b, h->ul, d, batch));
-    JPI_TRY(linear(h, st, h->ul, d, ab.w1, ab.b1, nullptr, 0, h->hidl, F, batch, d, F, true));
+    JPI_TRY(ln_linear(h, st, h->xl, ab.ln2_w, ab.ln2_b, h->ul, ab.w1, ab.b1, h->hidl, batch, F, true));
     JPI_TRY(linear(h, st, h->hidl, F, ab.w2, ab.b2, h->xl, d, h->xl, d, batch, F, d, false));
     // Join: [compressed token ; action summary] projected back to the module width.
-    pdl(st, dim3(grid_for((long long)rows * 2 * d)), dim3(256), 0, k_corr_join, state, h->xl, h->xj, batch, T, d);
-    JPI_CUDA_TRY(cudaGetLastError());
-    JPI_TRY(linear(h, st, h->xj, 2 * d, h->fuse_w, h->fuse_b, nullptr, 0, h->xf, d, rows, 2 * d, d, false));
+    if (pipe_ok(h, state, d, h->fuse_w, 2 * d)) {
+        LinArgs a = lin_args(state, d, h->fuse_w, h->fuse_b, nullptr, 0, h->xf, d, rows, 2 * d, d, false);
+        a.join = d;
+        a.x2 = h->xl;
+        a.x2_div = T;
+        a.ldx2 = d;
+        JPI_TRY(launch_pipe(h, st, LP_PLAIN, a));
+    } else {
+        pdl(st, dim3(grid_for((long long)rows * 2 * d)), dim3(256), 0, k_corr_join, state, h->xl, h->xj, batch, T, d);
+        JPI_CUDA_TRY(cudaGetLastError());
+        JPI_TRY(linear(h, st, h->xj, 2 * d, h->fuse_w, h->fuse_b, nullptr, 0, h->xf, d, rows, 2 * d, d, false));
+    }
     for (int i = 0; i < h->J; ++i) JPI_TRY(block(h, st, h->jb[(size_t)i], h->xf, batch, T));
     // Heads.
+    if (ln_fused(h, h->xf, d, h->corr_w, rows)) {
+        LinArgs a = lin_args(h->xf, d, h->corr_w, h->corr_b, nullptr, 0, out, d, rows, d, d, false);
+        a.ln_g = h->head_ln_w;
+        a.ln_b = h->head_ln_b;
+        a.ln_eps = h->cfg.ln_eps;
+        a.conf_items = T;
+        a.conf_w = h->conf_w;
+        a.conf_b = h->conf_b;
+        a.conf = conf;
+        return launch_pipe(h, st, LP_LN, a, batch);
+    }
     JPI_TRY(layernorm(h, st, h->xf, d, h->head_ln_w, h->head_ln_b, h->u, d, rows));
     JPI_TRY(linear(h, st, h->u, d, h->corr_w, h->corr_b, nullptr, 0, out, d, rows, d, d, false));
     pdl(st, dim3(batch), dim3(256), 0, k_corr_confidence, h->u, h->conf_w, h->conf_b, conf, T, d);
