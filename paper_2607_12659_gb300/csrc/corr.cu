@@ -21,8 +21,6 @@
 #include "jpi_internal.h"
 #include "ptx.h"
 
-#include <map>
-#include <tuple>
 #include "jpi_corr.h"
 
 #include <cmath>
@@ -404,13 +402,20 @@ __global__ void __launch_bounds__(256) k_corr_attn4(const float* __restrict__ qk
     }
 }
 
-template <int NST, int MODE>
+// SPLIT = 2 (in <= 1024, more than four rows): the two halves of the block take four of a group's
+// features each over all chunks, and a pass takes eight rows; otherwise threads past in / 8 chunks would
+// idle, and every four rows cost a reduction over the block. The sums are the same either way.
+template <int NST, int MODE, int SPLIT>
 __global__ void __launch_bounds__(256) k_corr_linear_pipe(const __grid_constant__ LinArgs a) {
+    constexpr int XR = LP_XR * SPLIT, FPT = LP_ROWS / SPLIT;   // rows per pass, features per thread
+    constexpr int CT = 256 / SPLIT;                            // threads that share a feature's chunks
+    static_assert(MODE != LP_ATTN || SPLIT == 1, "the attention form takes four rows");
     extern __shared__ __align__(128) uint8_t lp_smem[];
-    __shared__ float red[8][LP_ROWS * LP_XR];
+    __shared__ float red[8][32];
     __shared__ float2 mr[LP_LN_ROWS];   // LayerNorm: (mean, 1 / std) of each row
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int in = a.in, nch = in / 8;
+    const int ct = tid % CT, f0 = tid / CT * FPT;   // first chunk, first feature of a group
     if (MODE == LP_LN && a.conf && (int)blockIdx.x >= a.lin_ctas) {
         // The confidence of request b: features tid, tid + 256, .. of the mean normalised row.
         jpi::ptx::grid_dep_wait();
@@ -474,30 +479,30 @@ __global__ void __launch_bounds__(256) k_corr_linear_pipe(const __grid_constant_
         const int rows = seg ? a.seg_rows : a.rows, ldx = seg ? a.seg_ldx : a.ldx, ldy = seg ? a.seg_ldy : a.ldy;
         const float* xb = seg ? a.seg_x : a.x;
         float* yb = seg ? a.seg_y : a.y;
-        for (int r0 = 0; r0 < rows; r0 += LP_XR) {
-            const int nr = min(LP_XR, rows - r0);
-            // The bias and residual of this thread's output (thread o LP_XR + q writes feature
+        for (int r0 = 0; r0 < rows; r0 += XR) {
+            const int nr = min(XR, rows - r0);
+            // The bias and residual of this thread's output (thread o XR + q writes feature
             // o0 + o of row r0 + q), fetched before the products so their latency hides there.
             float bias_v = 0.f, res_v = 0.f;
-            if (tid < LP_ROWS * LP_XR) {
-                const int o = tid / LP_XR, q = tid % LP_XR;
+            if (tid < LP_ROWS * XR) {
+                const int o = tid / XR, q = tid % XR;
                 if (o < nout && q < nr) {
                     if (a.bias) bias_v = a.bias[o0 + o];
                     const int rr = a.res_mod > 0 ? (r0 + q) % a.res_mod : r0 + q;
                     if (a.res) res_v = a.res[(size_t)rr * a.ldr + o0 + o];
                 }
             }
-            float acc[LP_ROWS][LP_XR];
+            float acc[FPT][XR];
 #pragma unroll
-            for (int o = 0; o < LP_ROWS; ++o)
+            for (int o = 0; o < FPT; ++o)
 #pragma unroll
-                for (int q = 0; q < LP_XR; ++q) acc[o][q] = 0.f;
-            // Chunk c (8 columns) of rows r0 .. r0 + 3 against the group's weight rows.
-            auto product = [&](int c, const float (&x)[LP_XR][8]) {
+                for (int q = 0; q < XR; ++q) acc[o][q] = 0.f;
+            // Chunk c (8 columns) of rows r0 .. against this thread's weight rows of the group.
+            auto product = [&](int c, const float (&x)[XR][8]) {
 #pragma unroll
-                for (int o = 0; o < LP_ROWS; ++o) {
-                    if (o >= nout) break;
-                    const uint4 wv = wst[(size_t)o * nch + c];
+                for (int o = 0; o < FPT; ++o) {
+                    if (f0 + o >= nout) break;
+                    const uint4 wv = wst[(size_t)(f0 + o) * nch + c];
                     const uint32_t u[4] = {wv.x, wv.y, wv.z, wv.w};
                     float w[8];
 #pragma unroll
@@ -507,7 +512,7 @@ __global__ void __launch_bounds__(256) k_corr_linear_pipe(const __grid_constant_
                         w[2 * e + 1] = f.y;
                     }
 #pragma unroll
-                    for (int q = 0; q < LP_XR; ++q) {
+                    for (int q = 0; q < XR; ++q) {
                         float t = acc[o][q];
 #pragma unroll
                         for (int e = 0; e < 8; ++e) t = fmaf(w[e], x[q][e], t);
@@ -522,28 +527,33 @@ __global__ void __launch_bounds__(256) k_corr_linear_pipe(const __grid_constant_
                 attn4_chunk(xb + (size_t)r0 * ldx + 8 * c, ldx, in, a.att_heads_dh, a.att_scale, x);
                 if (tid < nch) product(tid, x);
             } else {
-                for (int c = tid; c < nch; c += 256) {
-                    float x[LP_XR][8];
+                for (int c = ct; c < nch; c += CT) {
+                    float x[XR][8];
                     float gv[8], bv[8];
                     if (MODE == LP_LN) {
                         lp_load8(a.ln_g + 8 * c, gv);
                         lp_load8(a.ln_b + 8 * c, bv);
                     }
+                    const bool second = a.x2 && 8 * c >= a.join;
+                    const float* xc = xb + (size_t)r0 * ldx + 8 * c;
 #pragma unroll
-                    for (int q = 0; q < LP_XR; ++q) {
+                    for (int q = 0; q < XR; ++q) {
                         if (q < nr) {
-                            const bool second = a.x2 && 8 * c >= a.join;
                             lp_load8(second ? a.x2 + (size_t)((r0 + q) / a.x2_div) * a.ldx2 + (8 * c - a.join)
-                                         : xb + (size_t)(r0 + q) * ldx + 8 * c, x[q]);
-                            if (MODE == LP_LN) {
-                                // Row of x this is (a segment's rows are a subset of them).
-                                const float2 st = mr[seg ? (int)((a.seg_x - a.x + (size_t)(r0 + q) * ldx) / a.ldx) : r0 + q];
-#pragma unroll
-                                for (int e = 0; e < 8; ++e) x[q][e] = (x[q][e] - st.x) * st.y * gv[e] + bv[e];
-                            }
+                                            : xc + (size_t)q * ldx, x[q]);
                         } else {
 #pragma unroll
                             for (int e = 0; e < 8; ++e) x[q][e] = 0.f;
+                        }
+                    }
+                    if (MODE == LP_LN) {
+#pragma unroll
+                        for (int q = 0; q < XR; ++q) {
+                            if (q >= nr) break;
+                            // Row of x this is (a segment's rows are a subset of them).
+                            const float2 st = mr[seg ? (int)((a.seg_x - a.x + (size_t)(r0 + q) * ldx) / a.ldx) : r0 + q];
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) x[q][e] = (x[q][e] - st.x) * st.y * gv[e] + bv[e];
                         }
                     }
                     product(c, x);
@@ -553,13 +563,13 @@ __global__ void __launch_bounds__(256) k_corr_linear_pipe(const __grid_constant_
             // warp sum is a reduce-scatter: at offset 16, 8, .., 1 each lane keeps the half of its
             // pairs whose bit matches its own and adds its partner's partial of them (the same
             // pairwise sums as a butterfly per pair, 31 shuffles instead of 160); lane p ends
-            // with pair p = o LP_XR + q.
-            static_assert(LP_ROWS * LP_XR == 32, "one pair per lane");
+            // with pair p = o XR + q of its half's features.
+            static_assert(FPT * XR == 32, "one pair per lane");
             float pv[32];
 #pragma unroll
-            for (int o = 0; o < LP_ROWS; ++o)
+            for (int o = 0; o < FPT; ++o)
 #pragma unroll
-                for (int q = 0; q < LP_XR; ++q) pv[o * LP_XR + q] = acc[o][q];
+                for (int q = 0; q < XR; ++q) pv[o * XR + q] = acc[o][q];
 #pragma unroll
             for (int sh = 16; sh > 0; sh >>= 1) {
                 const bool hi = (lane & sh) != 0;
@@ -572,11 +582,12 @@ __global__ void __launch_bounds__(256) k_corr_linear_pipe(const __grid_constant_
             }
             red[warp][lane] = pv[0];
             __syncthreads();
-            if (tid < LP_ROWS * LP_XR) {
-                const int o = tid / LP_XR, q = tid % LP_XR;
+            if (tid < LP_ROWS * XR) {
+                // Thread o XR + q: lane tid mod 32 of the warps of half tid / 32, in warp order.
+                const int o = tid / XR, q = tid % XR;
                 float v = 0.f;
 #pragma unroll
-                for (int w8 = 0; w8 < 8; ++w8) v += red[w8][tid];
+                for (int w8 = 0; w8 < 8 / SPLIT; ++w8) v += red[(tid >> 5) * (8 / SPLIT) + w8][lane];
                 const int of = o0 + o, r = r0 + q;
                 if (o < nout && q < nr) {
                     v += bias_v;
@@ -1191,13 +1202,6 @@ struct jpi_corr_handle {
     float *scp = nullptr, *gsp = nullptr;   // partials: [B][dv / 256][M][Tm], [B][Tm / 64][M][dv]
     float* conf_scratch = nullptr;                                        // [B]
 
-    // Graph replay: the calls copy their inputs into these buffers, replay the kernel sequence
-    // captured once per (call, batch, tokens or delta, input type), and copy the outputs out.
-    void* in_vlm = nullptr;                                               // [B][Tm][dv], fp32 or bf16
-    float *in_state = nullptr, *in_act = nullptr;                         // [B T'][d], [B Dm][A]
-    float *out_st = nullptr, *out_conf = nullptr;                         // [B T'][d], [B]
-    cudaStream_t cap = nullptr;
-    std::map<std::tuple<int, int, int, int>, cudaGraphExec_t> graphs;
 };
 
 namespace {
@@ -1306,8 +1310,12 @@ jpi_status put_block(jpi_corr_handle* h, bool dev, BlockDev* out, const jpi_corr
 // ---------------------------------------------------------------- launchers
 
 // Every kernel of a call is launched with programmatic dependent launch (each waits for its
-// predecessor at its start), so in the captured graph a kernel's launch overlaps the previous
-// kernel's tail. A failed launch leaves its error for the cudaGetLastError check that follows.
+// predecessor at its start), so a kernel's launch overlaps the previous kernel's tail. The calls
+// enqueue their kernels on the caller's pointers: a graph of them, captured once per shape, needed
+// every input copied in and every output copied out, which took more of the GPU's time (10 us of 62 per
+// compress, 12 of 109 per predict at batch 1) than the host's 27 launches leave it idle (none: they
+// take the host less time than the kernels run). A failed launch leaves its error for the
+// cudaGetLastError check that follows.
 template <typename... KArgs, typename... Args>
 void pdl(cudaStream_t st, dim3 grid, dim3 block, size_t smem, void (*k)(KArgs...), Args&&... args) {
     cudaLaunchConfig_t cfg = {};
@@ -1342,10 +1350,13 @@ jpi_status launch_pipe(const jpi_corr_handle* h, cudaStream_t st, int mode, LinA
     const int nst = lp_stages(a.in);
     const size_t smem = (size_t)nst * LP_ROWS * a.in * 2;
     const dim3 grid(a.lin_ctas + extra), block(256);
-    if (mode == LP_LN) pdl(st, grid, block, smem, k_corr_linear_pipe<4, LP_LN>, a);
-    else if (mode == LP_ATTN) pdl(st, grid, block, smem, k_corr_linear_pipe<4, LP_ATTN>, a);
-    else if (nst == 4) pdl(st, grid, block, smem, k_corr_linear_pipe<4, LP_PLAIN>, a);
-    else pdl(st, grid, block, smem, k_corr_linear_pipe<3, LP_PLAIN>, a);
+    const bool split = a.in <= 1024 && a.rows > LP_XR;
+    if (mode == LP_LN && split) pdl(st, grid, block, smem, k_corr_linear_pipe<4, LP_LN, 2>, a);
+    else if (mode == LP_LN) pdl(st, grid, block, smem, k_corr_linear_pipe<4, LP_LN, 1>, a);
+    else if (mode == LP_ATTN) pdl(st, grid, block, smem, k_corr_linear_pipe<4, LP_ATTN, 1>, a);
+    else if (split) pdl(st, grid, block, smem, k_corr_linear_pipe<4, LP_PLAIN, 2>, a);
+    else if (nst == 4) pdl(st, grid, block, smem, k_corr_linear_pipe<4, LP_PLAIN, 1>, a);
+    else pdl(st, grid, block, smem, k_corr_linear_pipe<3, LP_PLAIN, 1>, a);
     JPI_CUDA_TRY(cudaGetLastError());
     return JPI_OK;
 }
@@ -1640,12 +1651,6 @@ jpi_status setup(jpi_corr_handle* h, const jpi_corr_config* c, const jpi_corr_we
     JPI_TRY(corr_alloc(h, &h->gs, B * M * dv));
     JPI_TRY(corr_alloc(h, &h->scp, B * (size_t)((dv + CORR_KCHUNK - 1) / CORR_KCHUNK) * M * h->Tm));
     JPI_TRY(corr_alloc(h, &h->gsp, B * (size_t)((h->Tm + CORR_TCHUNK - 1) / CORR_TCHUNK) * M * dv));
-    JPI_TRY(corr_alloc(h, reinterpret_cast<float**>(&h->in_vlm), B * (size_t)h->Tm * dv));
-    JPI_TRY(corr_alloc(h, &h->in_state, B * (size_t)h->Ti * h->d));
-    JPI_TRY(corr_alloc(h, &h->in_act, B * (size_t)h->Dm * h->A));
-    JPI_TRY(corr_alloc(h, &h->out_st, B * (size_t)h->Ti * h->d));
-    JPI_TRY(corr_alloc(h, &h->out_conf, (size_t)B));
-    JPI_CUDA_TRY(cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking));
     JPI_CUDA_TRY(cudaFuncSetAttribute(k_corr_scores<float, true, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SCORES_SMEM));
     JPI_CUDA_TRY(cudaFuncSetAttribute(k_corr_scores<float, true, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SCORES_SMEM));
     JPI_CUDA_TRY(cudaFuncSetAttribute(k_corr_scores<float, false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SCORES_SMEM));
@@ -1654,9 +1659,10 @@ jpi_status setup(jpi_corr_handle* h, const jpi_corr_config* c, const jpi_corr_we
     JPI_CUDA_TRY(cudaFuncSetAttribute(k_corr_scores<__nv_bfloat16, true, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SCORES_SMEM));
     JPI_CUDA_TRY(cudaFuncSetAttribute(k_corr_scores<__nv_bfloat16, false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SCORES_SMEM));
     JPI_CUDA_TRY(cudaFuncSetAttribute(k_corr_scores<__nv_bfloat16, false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CORR_SCORES_SMEM));
-    for (auto k : {k_corr_linear_pipe<4, LP_PLAIN>, k_corr_linear_pipe<4, LP_LN>, k_corr_linear_pipe<4, LP_ATTN>})
+    for (auto k : {k_corr_linear_pipe<4, LP_PLAIN, 1>, k_corr_linear_pipe<4, LP_PLAIN, 2>, k_corr_linear_pipe<4, LP_LN, 1>,
+                   k_corr_linear_pipe<4, LP_LN, 2>, k_corr_linear_pipe<4, LP_ATTN, 1>})
         JPI_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * LP_ROWS * 2048 * 2));
-    JPI_CUDA_TRY(cudaFuncSetAttribute(k_corr_linear_pipe<3, LP_PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    JPI_CUDA_TRY(cudaFuncSetAttribute(k_corr_linear_pipe<3, LP_PLAIN, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       3 * LP_ROWS * LP_MAX_IN * 2));
     {
         int dev = 0;
@@ -1802,32 +1808,6 @@ jpi_status enqueue_predict(jpi_corr_handle* h, const float* state, const float* 
     return JPI_OK;
 }
 
-// The graph of one call shape, captured on the handle's own stream the first time it is asked for.
-template <typename F>
-jpi_status corr_graph(jpi_corr_handle* h, std::tuple<int, int, int, int> key, F&& enqueue, cudaGraphExec_t* out) {
-    auto it = h->graphs.find(key);
-    if (it != h->graphs.end()) {
-        *out = it->second;
-        return JPI_OK;
-    }
-    cudaGraph_t g = nullptr;
-    JPI_CUDA_TRY(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
-    const jpi_status s = enqueue(h->cap);
-    const cudaError_t e = cudaStreamEndCapture(h->cap, &g);
-    if (s != JPI_OK) {
-        if (g) cudaGraphDestroy(g);
-        return s;
-    }
-    if (e != cudaSuccess) return cfail(JPI_ERR_CUDA, "graph capture failed: %s", cudaGetErrorString(e));
-    cudaGraphExec_t ex = nullptr;
-    const cudaError_t ei = cudaGraphInstantiate(&ex, g, 0);
-    cudaGraphDestroy(g);
-    if (ei != cudaSuccess) return cfail(JPI_ERR_CUDA, "graph instantiate failed: %s", cudaGetErrorString(ei));
-    h->graphs[key] = ex;
-    *out = ex;
-    return JPI_OK;
-}
-
 }  // namespace
 
 extern "C" {
@@ -1846,7 +1826,6 @@ JPI_API jpi_status jpi_corr_create(const jpi_corr_config* cfg, const jpi_corr_we
     if (s != JPI_OK) {
         cudaStreamSynchronize(nullptr);   // let any conversion in flight finish before its buffers go
         cudaGetLastError();
-        if (h->cap) cudaStreamDestroy(h->cap);
         for (void* p : h->allocs) cudaFree(p);
         delete h;
         return s;
@@ -1859,8 +1838,6 @@ JPI_API jpi_status jpi_corr_destroy(jpi_corr_handle* h) {
     jpi::clear_error();
     if (!h) return JPI_OK;
     cudaDeviceSynchronize();
-    for (auto& kv : h->graphs) cudaGraphExecDestroy(kv.second);
-    if (h->cap) cudaStreamDestroy(h->cap);
     for (void* p : h->allocs) cudaFree(p);
     cudaGetLastError();
     delete h;
@@ -1877,18 +1854,7 @@ JPI_API jpi_status jpi_corr_compress(jpi_corr_handle* h, const void* h_vlm, int 
         return cfail(JPI_ERR_SHAPE, "batch %d / n_tokens %d exceed the maxima %d / %d", batch, n_tokens, h->B,
                      h->Tm);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const size_t in_bytes = (size_t)batch * n_tokens * h->dv * (vlm_is_fp32 ? 4 : 2);
-    cudaGraphExec_t ex = nullptr;
-    JPI_TRY(corr_graph(h, std::make_tuple(0, batch, n_tokens, vlm_is_fp32 ? 1 : 0),
-                       [&](cudaStream_t cs) {
-                           return enqueue_compress(h, h->in_vlm, vlm_is_fp32, batch, n_tokens, h->out_st, cs);
-                       },
-                       &ex));
-    JPI_CUDA_TRY(cudaMemcpyAsync(h->in_vlm, h_vlm, in_bytes, cudaMemcpyDeviceToDevice, st));
-    JPI_CUDA_TRY(cudaGraphLaunch(ex, st));
-    JPI_CUDA_TRY(cudaMemcpyAsync(out_state, h->out_st, (size_t)batch * h->Ti * h->d * sizeof(float),
-                                 cudaMemcpyDeviceToDevice, st));
-    return JPI_OK;
+    return enqueue_compress(h, h_vlm, vlm_is_fp32, batch, n_tokens, out_state, st);
 }
 
 JPI_API jpi_status jpi_corr_predict(jpi_corr_handle* h, const float* state, const float* actions, int batch,
@@ -1900,22 +1866,8 @@ JPI_API jpi_status jpi_corr_predict(jpi_corr_handle* h, const float* state, cons
     if (batch > h->B || delta > h->Dm)
         return cfail(JPI_ERR_SHAPE, "batch %d / delta %d exceed the maxima %d / %d", batch, delta, h->B, h->Dm);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    cudaGraphExec_t ex = nullptr;
-    JPI_TRY(corr_graph(h, std::make_tuple(1, batch, delta, 0),
-                       [&](cudaStream_t cs) {
-                           return enqueue_predict(h, h->in_state, h->in_act, batch, delta, h->out_st, h->out_conf, cs);
-                       },
-                       &ex));
-    const size_t state_bytes = (size_t)batch * h->Ti * h->d * sizeof(float);
-    JPI_CUDA_TRY(cudaMemcpyAsync(h->in_state, state, state_bytes, cudaMemcpyDeviceToDevice, st));
-    JPI_CUDA_TRY(cudaMemcpyAsync(h->in_act, actions, (size_t)batch * delta * h->A * sizeof(float),
-                                 cudaMemcpyDeviceToDevice, st));
-    JPI_CUDA_TRY(cudaGraphLaunch(ex, st));
-    JPI_CUDA_TRY(cudaMemcpyAsync(out_state, h->out_st, state_bytes, cudaMemcpyDeviceToDevice, st));
-    if (out_confidence)
-        JPI_CUDA_TRY(cudaMemcpyAsync(out_confidence, h->out_conf, (size_t)batch * sizeof(float),
-                                     cudaMemcpyDeviceToDevice, st));
-    return JPI_OK;
+    return enqueue_predict(h, state, actions, batch, delta, out_state, out_confidence ? out_confidence : h->conf_scratch,
+                           st);
 }
 
 JPI_API jpi_status jpi_corr_memory_usage(const jpi_corr_handle* h, long long* bytes) {
