@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_tc_gemm(const __grid_consta
     // write consecutive output features of one token.
     const int nitems = npairs * QUADS;
 
-    if (warp == 0) {
+    if (warp == 1) {
         ptx::tmem_alloc(tmem_slot, NT);
         ptx::tmem_relinquish();
     }
@@ -234,6 +234,11 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_tc_gemm(const __grid_consta
         ptx::tc_fence_before();
         ptx::fence_proxy_async_smem();
         __syncthreads();
+        // The accumulator has been read: give its columns back here, off the path to the exit.
+        if (warp == 1) {
+            ptx::tc_fence_after();
+            ptx::tmem_dealloc(tmem, NT);
+        }
 
         // ---- 3b. push each other rank's rows (pairs r*npairs.. and +64) to that rank ----
         ptx::cluster_wait();   // receive barriers initialised everywhere
@@ -369,9 +374,5 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_tc_gemm(const __grid_consta
     // Pairs the arrival after the receive wait.
     ptx::cluster_wait();
 
-    if (tid == 0 && *flag != 0) set_device_error(a.err, *flag);
-    ptx::tc_fence_before();
-    __syncthreads();
-    ptx::tc_fence_after();
-    if (warp == 0) ptx::tmem_dealloc(tmem, NT);
+    if (*flag != 0) set_device_error(a.err, *flag);   // by any thread that saw it
 }
