@@ -191,9 +191,12 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_tc_gemm(const __grid_consta
                 rinv_s[c] = r;
             }
         }
-        if (!ptx::mbar_wait_bounded(&bars[2], 0, WAIT_LIMIT_NS)) *flag = DEV_TIMEOUT_MMA;
+        // Published here, while the MMAs run: the column scales and the MMA thread's flag; and every
+        // CTA's receive barrier is initialised by now.
         __syncthreads();
-        const bool ok = *flag == 0;
+        ptx::cluster_wait();
+        if (!ptx::mbar_wait_bounded(&bars[2], 0, WAIT_LIMIT_NS)) *flag = DEV_TIMEOUT_MMA;
+        const bool ok = __all_sync(0xffffffffu, *flag == 0);
         ptx::tc_fence_after();
 
         // ---- 3a. TMEM -> fp16 partial in shared memory (warp w: lanes 32 (w mod 4), half w / 4).
@@ -233,25 +236,29 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_tc_gemm(const __grid_consta
         }
         ptx::tc_fence_before();
         ptx::fence_proxy_async_smem();
-        __syncthreads();
+
+        // ---- 3b. push each other rank's rows (pairs r*npairs.. and +64) to that rank ----
+        // The 32 rows of TMEM lane group qd = warp mod 4 are written by two warps (one per column
+        // half) and hold whole chunks of npairs rows: as soon as both warps are through, lane i of the
+        // first sends chunk i to the rank that owns it (with npairs = 64 there is nobody to send to).
+        if (a.splits > 1) {
+            const int qd = warp & 3, per = 32 / npairs;
+            ptx::named_bar_sync(2 + qd, 64);
+            const int r = (qd & 1) * per + lane;
+            if (warp < 4 && lane < per && r != rank) {
+                const uint32_t chunk = (uint32_t)(npairs * 128);
+                const int slot = rank < r ? rank : rank - 1;   // owner r stores senders != r in order
+                const uint32_t dst =
+                    ptx::dsmem_map(ptx::smem_u32(recv + ((size_t)slot * 2 + (qd >> 1)) * npairs * 64), (uint32_t)r);
+                ptx::bulk_copy_to_cluster(dst, part + (size_t)(32 * qd + lane * npairs) * 64, chunk,
+                                          ptx::dsmem_map(ptx::smem_u32(&bars[3]), (uint32_t)r));
+            }
+        }
+        __syncthreads();   // every row of this CTA's own partial is written (the exchange is under way)
         // The accumulator has been read: give its columns back here, off the path to the exit.
         if (warp == 1) {
             ptx::tc_fence_after();
             ptx::tmem_dealloc(tmem, NT);
-        }
-
-        // ---- 3b. push each other rank's rows (pairs r*npairs.. and +64) to that rank ----
-        ptx::cluster_wait();   // receive barriers initialised everywhere
-        // Lane r of warp 0 sends rank r its rows (the copies to all ranks issue together).
-        if (warp == 0 && lane < a.splits && lane != rank) {
-            const int r = lane;
-            const uint32_t chunk = (uint32_t)(npairs * 128);
-            const uint32_t bar_u = ptx::smem_u32(&bars[3]);
-            const int slot = rank < r ? rank : rank - 1;   // owner r stores senders != r in order
-            const uint32_t dst = ptx::dsmem_map(ptx::smem_u32(recv + (size_t)slot * 2 * npairs * 64), (uint32_t)r);
-            const uint32_t rbar = ptx::dsmem_map(bar_u, (uint32_t)r);
-            ptx::bulk_copy_to_cluster(dst, part + (size_t)r * npairs * 64, chunk, rbar);
-            ptx::bulk_copy_to_cluster(dst + chunk, part + (size_t)(r * npairs + 64) * 64, chunk, rbar);
         }
         if (!ptx::mbar_wait_bounded(&bars[3], 0, WAIT_LIMIT_NS)) *flag = DEV_TIMEOUT_MMA;
         // Everything addressed to this CTA has landed (seen through its own mbarrier); once all
