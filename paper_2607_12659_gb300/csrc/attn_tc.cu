@@ -168,8 +168,7 @@ __global__ void __launch_bounds__(AT_THREADS) k_attn_tc(const __grid_constant__ 
     // before the first push (published by fence.mbarrier_init, so the arrival is relaxed).
     ptx::cluster_arrive_relaxed();
 
-    // K and V blocks by bulk tensor copies (one thread): D/64 column blocks x KB/32 boxes of 32
-    // rows each. Rows past the split's last key are whatever the store holds there (finite:
+    // K and V blocks by bulk tensor copies (one thread): D/64 column blocks of KB rows each. Rows past the split's last key are whatever the store holds there (finite:
     // zero-initialised, or other requests' and layers' keys); their scores are masked.
     const uint32_t qs_u = ptx::smem_u32(qs), ks_u = ptx::smem_u32(ks), vs_u = ptx::smem_u32(vs);
     const int kv_row_b = a.kv_row0 + b * a.kv_rows;      // this request's key 0 in the maps
@@ -178,13 +177,12 @@ __global__ void __launch_bounds__(AT_THREADS) k_attn_tc(const __grid_constant__ 
         uint8_t* kd = ks + buf * KV_BUF;
         uint8_t* vd = vs + buf * KV_BUF;
         ptx::mbar_expect_tx(&kvbar[buf], KV_BUF);
-        for (int db = 0; db < D / 64; ++db)
-            for (int hb = 0; hb < KB / 32; ++hb) {
-                const uint32_t off = (uint32_t)(db * (KB * 128) + hb * (32 * 128));
-                const int y = kv_row_b + key0 + hb * 32;
-                ptx::tma_load_2d(kd + off, &kmap, &kvbar[buf], db * 64, y, pol);
-                ptx::tma_load_2d(vd + off, &vmap, &kvbar[buf], db * 64, y, pol);
-            }
+#pragma unroll
+        for (int db = 0; db < D / 64; ++db) {
+            const uint32_t off = (uint32_t)(db * (KB * 128));
+            ptx::tma_load_2d(kd + off, &kmap, &kvbar[buf], db * 64, kv_row_b + key0, pol);
+            ptx::tma_load_2d(vd + off, &vmap, &kvbar[buf], db * 64, kv_row_b + key0, pol);
+        }
     };
     // A first block made only of prefix keys (written before this graph ran) is fetched before
     // the dependency wait; one holding suffix keys (written by the QKV kernel) after it.
@@ -204,6 +202,9 @@ __global__ void __launch_bounds__(AT_THREADS) k_attn_tc(const __grid_constant__ 
             ptx::tma_load_2d(qs + db * (AT_ROWS * 128), &qmap, qbar, db * 64, b * nrows + row0, pol);
         if (!early) load_block(k_begin, 0);
     }
+
+    // Receive barriers are initialised cluster-wide by now (waited for here, beside the loads).
+    ptx::cluster_wait();
 
     // Per-thread rows g and g + 8 of this warp's 16; their visible key count.
     const int g = lane >> 2, cq = lane & 3;
@@ -373,7 +374,6 @@ __global__ void __launch_bounds__(AT_THREADS) k_attn_tc(const __grid_constant__ 
     __syncthreads();
 
     // ---- exchange: push every other split's rows into its receive buffer ----
-    ptx::cluster_wait();
     // Lane s of warp 0 sends split s its rows (the copies to all splits issue together).
     if (warp == 0 && lane < ns && lane != rank) {
         const int s = lane;
@@ -510,8 +510,8 @@ jpi_status launch_attn_d(jpi_handle* h, int l, int B, int C, cudaStream_t st) {
     }
     cfg.attrs = attrs;
     cfg.numAttrs = n;
-    cudaError_t e = two ? cudaLaunchKernelEx(&cfg, k_attn_tc<D, 2>, h->qmap_at, h->kmap_at, h->vmap_at, a)
-                        : cudaLaunchKernelEx(&cfg, k_attn_tc<D, 1>, h->qmap_at, h->kmap_at, h->vmap_at, a);
+    cudaError_t e = two ? cudaLaunchKernelEx(&cfg, k_attn_tc<D, 2>, h->qmap_at, h->kmap_at[0], h->vmap_at[0], a)
+                        : cudaLaunchKernelEx(&cfg, k_attn_tc<D, 1>, h->qmap_at, h->kmap_at[1], h->vmap_at[1], a);
     if (e != cudaSuccess) {
         set_error("attention launch failed: %s", cudaGetErrorString(e));
         return JPI_ERR_CUDA;
@@ -548,10 +548,12 @@ jpi_status attn_tc_prepare(jpi_handle* h) {
     h->attn_force_splits = env ? std::atoi(env) : 0;
     // The query tile as 32-row boxes of 64 columns (128-byte swizzle) over q [maxMt * H][D].
     JPI_TRY(tc_make_tmap(h->q, (uint64_t)h->maxMt * h->H, h->D, AT_ROWS, &h->qmap_at));
-    // K and V of all layers [L * maxB * kv_rows][D] as 32-row boxes.
+    // K and V of all layers [L * maxB * kv_rows][D] as boxes of one key block (32 or 64 rows).
     const uint64_t kv_rows_all = (uint64_t)h->L * h->maxB * h->kv_rows;
-    JPI_TRY(tc_make_tmap(h->kv_k, kv_rows_all, h->D, 32, &h->kmap_at));
-    JPI_TRY(tc_make_tmap(h->kv_v, kv_rows_all, h->D, 32, &h->vmap_at));
+    for (int i = 0; i < 2; ++i) {
+        JPI_TRY(tc_make_tmap(h->kv_k, kv_rows_all, h->D, 32 * (i + 1), &h->kmap_at[i]));
+        JPI_TRY(tc_make_tmap(h->kv_v, kv_rows_all, h->D, 32 * (i + 1), &h->vmap_at[i]));
+    }
     switch (h->D) {
         case 64: return prepare_d<64>(h);
         case 128: return prepare_d<128>(h);

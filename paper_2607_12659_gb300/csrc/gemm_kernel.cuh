@@ -52,9 +52,12 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_tc_gemm(const __grid_consta
     const int tile = blockIdx.x / a.splits;
     const int kb0 = rank * a.kpb;
     const int npairs = 64 / a.splits, p0 = rank * npairs;
-    // Epilogue item = (column quad, owned pair) with the pair fastest, so that consecutive lanes
-    // write consecutive output features of one token.
-    const int nitems = npairs * QUADS;
+    // Epilogue item = (TW columns, owned pair) with the pair fastest, so that consecutive lanes
+    // write consecutive output features of one token. Two columns for the residual kinds: at their
+    // K split of 8 that is an item for every thread (four left half of them idle, and each item
+    // has eight residual values to fetch and update).
+    constexpr int TW = RESID ? 2 : 4;
+    const int nitems = npairs * (NT / TW);
 
     if (warp == 1) {
         ptx::tmem_alloc(tmem_slot, NT);
@@ -85,11 +88,16 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_tc_gemm(const __grid_consta
     // the residual stream h was last written two projections back (the previous norm-fed kernel
     // passed its own dependency wait, so that writer has completed). Global loads still in flight
     // at the TMEM read-out would slow it down.
-    float hv1[4] = {0.f, 0.f, 0.f, 0.f}, hv2[4] = {0.f, 0.f, 0.f, 0.f}, g1 = 0.f, g2 = 0.f;
+    float hv1[TW], hv2[TW], g1 = 0.f, g2 = 0.f;
     float sn1 = 0.f, sn2 = 0.f;
-    float2 cs[4] = {make_float2(1.f, 0.f), make_float2(1.f, 0.f), make_float2(1.f, 0.f), make_float2(1.f, 0.f)};
+    float2 cs[TW];
+#pragma unroll
+    for (int e = 0; e < TW; ++e) {
+        hv1[e] = hv2[e] = 0.f;
+        cs[e] = make_float2(1.f, 0.f);
+    }
     auto prefetch = [&](int item, int tok0) {
-        const int p = p0 + item % npairs, t0 = (item / npairs) * 4;
+        const int p = p0 + item % npairs, t0 = (item / npairs) * TW;
         const int f1 = tile * TILE_ROWS + p, f2 = f1 + 64;
         if (RESID) {
             g1 = a.gamma[f1];
@@ -100,7 +108,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_tc_gemm(const __grid_consta
             }
         }
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
+        for (int e = 0; e < TW; ++e) {
             const int tok = tok0 + t0 + e;
             hv1[e] = hv2[e] = 0.f;
             cs[e] = make_float2(1.f, 0.f);
@@ -268,15 +276,19 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_tc_gemm(const __grid_consta
         if (!EARLY_TRIGGER) ptx::grid_dep_launch();
 
         // ---- 4. rank-ordered sum of the slices (own rows read in place) + epilogue ----
-        float ssq[4] = {0.f, 0.f, 0.f, 0.f};
+        float ssq[TW];
+#pragma unroll
+        for (int e = 0; e < TW; ++e) ssq[e] = 0.f;
         for (int item = tid; item < nitems; item += GEMM_THREADS) {
             if (item != tid) prefetch(item, tok0);
-            const int pi = item % npairs, quad = item / npairs, t0 = quad * 4, p = p0 + pi;
-            // Offsets of columns t0..t0+3 and of column 63 inside a swizzled row with key p mod 8
+            const int pi = item % npairs, t0 = (item / npairs) * TW, p = p0 + pi;
+            // Offsets of columns t0.. and of column 63 inside a swizzled row with key p mod 8
             // (= (p + 64) mod 8).
-            const int off = (((quad >> 1) ^ (p & 7)) << 3) + ((quad & 1) << 2);
+            const int off = (((t0 >> 3) ^ (p & 7)) << 3) + (t0 & 7);
             const int off63 = ((7 ^ (p & 7)) << 3) + 7;
-            float4 y1 = make_float4(0.f, 0.f, 0.f, 0.f), y2 = y1;
+            float y1[TW], y2[TW];
+#pragma unroll
+            for (int e = 0; e < TW; ++e) y1[e] = y2[e] = 0.f;
             float b1 = 0.f, b2 = 0.f;
 #pragma unroll 4
             for (int r = 0; r < a.splits; ++r) {
@@ -290,8 +302,20 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_tc_gemm(const __grid_consta
                     s1 = recv + ((size_t)slot * 2 * npairs + pi) * 64;
                     s2 = recv + ((size_t)slot * 2 * npairs + npairs + pi) * 64;
                 }
-                f4add(y1, half4_to_float4(*(const uint2*)(s1 + off)));
-                f4add(y2, half4_to_float4(*(const uint2*)(s2 + off)));
+                if constexpr (TW == 4) {
+                    const float4 v1 = half4_to_float4(*(const uint2*)(s1 + off)), v2 = half4_to_float4(*(const uint2*)(s2 + off));
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        y1[e] += f4get(v1, e);
+                        y2[e] += f4get(v2, e);
+                    }
+                } else {
+                    const float2 v1 = unpack_half2(*(const uint32_t*)(s1 + off)), v2 = unpack_half2(*(const uint32_t*)(s2 + off));
+                    y1[0] += v1.x;
+                    y1[1] += v1.y;
+                    y2[0] += v2.x;
+                    y2[1] += v2.y;
+                }
                 if (NORM_IN) {
                     b1 += __half2float(s1[off63]);
                     b2 += __half2float(s2[off63]);
@@ -310,7 +334,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_tc_gemm(const __grid_consta
                 qi = tok0 + t0 - qb * a.S;
             }
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
+            for (int e = 0; e < TW; ++e) {
                 const int tok = tok0 + t0 + e;
                 const int b = qb, i = qi;   // request and position of token tok (QKV)
                 if (KIND == G_QKV && ++qi == a.S) {
@@ -318,7 +342,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_tc_gemm(const __grid_consta
                     ++qb;
                 }
                 if (t0 + e >= TT || tok >= a.Mt) continue;
-                const float u1 = f4get(y1, e) + b1, u2 = f4get(y2, e) + b2;
+                const float u1 = y1[e] + b1, u2 = y2[e] + b2;
                 if (KIND == G_QKV) {
                     const int hd = a.D >> 1;
                     float r1 = u1, r2 = u2;
@@ -346,12 +370,12 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_tc_gemm(const __grid_consta
                 }
             }
             if (RESID) {
-                // Sum over the pairs of this item's token quad: the w = min(npairs, 32) lanes
+                // Sum over the pairs of this item's tokens: the w = min(npairs, 32) lanes
                 // that share it, in a fixed butterfly order; then one lane per group records it
                 // for its 32-pair chunk (two chunks only when npairs = 64).
                 const int w = npairs < 32 ? npairs : 32;
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
+                for (int e = 0; e < TW; ++e) {
                     float v = ssq[e];
                     for (int o = 1; o < w; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
                     if ((lane & (w - 1)) == 0) ssred[(pi >> 5) * NT + t0 + e] = v;

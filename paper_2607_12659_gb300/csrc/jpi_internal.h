@@ -174,7 +174,7 @@ struct jpi_handle {
     void* t5_wml = nullptr;
     CUtensorMap amaps[3];       // attention operands: q, prefix/suffix K, V (all layers)
     CUtensorMap qmap_at;        // q as 32-row boxes for the split-KV attention
-    CUtensorMap kmap_at, vmap_at;   // K, V of all layers as 32-row boxes for it
+    CUtensorMap kmap_at[2], vmap_at[2];   // K, V of all layers as 32- and 64-row boxes for it
     std::vector<CUtensorMap> tmaps;
     bool mod_tc = false;        // modulation vectors on tensor cores (mod_tc.cu)
     CUtensorMap mod_map;        // the stacked modulation matrix [(6L+2) W][W] as 128 x 64 boxes

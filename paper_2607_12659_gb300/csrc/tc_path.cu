@@ -36,7 +36,6 @@ constexpr int TILE_BYTES = TILE_ROWS * KBLK * 2;
 constexpr int XBLK_BYTES = NT * KBLK * 2;
 constexpr int PART_BYTES = TILE_ROWS * NT * 2;  // fp16 partial of one tile (128-byte rows)
 constexpr int GEMM_THREADS = 256;
-constexpr int QUADS = NT / 4;                  // token quads per tile
 constexpr uint64_t WAIT_LIMIT_NS = 200ull * 1000 * 1000;   // 0.2 s
 
 enum GemmKind { G_QKV = 0, G_O = 1, G_GU = 2, G_DOWN = 3 };
@@ -98,12 +97,6 @@ __device__ __forceinline__ float4 half4_to_float4(uint2 v) {
     const float2 lo = __half22float2(*reinterpret_cast<__half2*>(&v.x));
     const float2 hi = __half22float2(*reinterpret_cast<__half2*>(&v.y));
     return make_float4(lo.x, lo.y, hi.x, hi.y);
-}
-__device__ __forceinline__ void f4add(float4& a, const float4& b) {
-    a.x += b.x;
-    a.y += b.y;
-    a.z += b.z;
-    a.w += b.w;
 }
 
 // Shared-memory layout of one GEMM CTA (byte offsets from the 1024-aligned base).
