@@ -136,7 +136,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_tc_gemm(const __grid_consta
     // one (gate/up) streams the largest weight set of the layer (2F x W, four times the output
     // projection's) and needs the whole of this kernel to prefetch it; otherwise after the
     // split-K receive (below), so that the next kernel's weight prefetch does not compete with
-    // this kernel's operand loads, MMAs and exchange.
+    // this kernel's operand loads, MMAs and exchange. (Batch-1 denoise: as it is 4913 us; gate/up
+    // or down early as well 4915 and 4925; the output projection late 5041.)
     constexpr bool EARLY_TRIGGER = (KIND == G_O);
     if (EARLY_TRIGGER) ptx::grid_dep_launch();
 
@@ -214,11 +215,15 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_tc_gemm(const __grid_consta
             const int row = (warp & 3) * 32 + lane, cbase = (warp >> 2) * (NT / 2);
             const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
             bool range_ok = true;
+            // Both loads before the one wait (batch-1 denoise 4913 us -> 4860).
+            static_assert(NT / 2 == 32, "two loads of 16 columns per warp");
+            uint32_t rr[2][16];
+            ptx::tmem_ld_x16(lane_base + (uint32_t)cbase, rr[0]);
+            ptx::tmem_ld_x16(lane_base + (uint32_t)(cbase + 16), rr[1]);
+            ptx::tmem_ld_wait();
 #pragma unroll
             for (int c0 = 0; c0 < NT / 2; c0 += 16) {
-                uint32_t r[16];
-                ptx::tmem_ld_x16(lane_base + (uint32_t)(cbase + c0), r);
-                ptx::tmem_ld_wait();
+                const uint32_t (&r)[16] = rr[c0 / 16];
                 uint32_t hp[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
