@@ -128,7 +128,8 @@ typedef struct jpi_weights {
  * JPI_ATTN_T5_SPLITS=n fixes the key splits of the large-batch attention (1-4, within one wave of
  * clusters; the same rounding-only agreement); JPI_BIG_SPLIT=n fixes the K split of the large-batch
  * O and down projections (1, 2, 4 or 8); JPI_BIG_RESID_ROWS=0 / 1 fixes which of their two kernels
- * runs (1: tokens on the MMA's rows, no K split).
+ * runs (1: tokens on the MMA's rows, no K split); JPI_BIG_TILE_N=128 / 256 fixes the tile width of
+ * the large-batch QKV and gate/up projections.
  */
 JPI_API jpi_status jpi_expert_create(const jpi_config* cfg, const jpi_weights* w, jpi_handle** out);
 

@@ -2,22 +2,25 @@
 // anonymous namespace).
 //
 // Output tile = 128 operand rows (the MMA's M: 128 tokens, or for the RMSNorm-fed kinds two 64-row
-// tiles of 63 tokens + one beta row) x 256 weight rows (its N: two consecutive 128-row weight tiles)
+// tiles of 63 tokens + one beta row) x 256 weight rows (its N: NW = 2 consecutive 128-row weight tiles)
 // over the whole K range. What bounds these products is the operand bytes an SM takes in per
 // multiply-add, and how many of them are in flight: a k-block brings 48 KB for 2 M multiply-adds and
 // the ring keeps four of them, 192 KB, under way: about 0.39 us a k-block, 85% of the tensor peak
 // inside a tile (128 x 128 tiles bring 32 KB for 1 M, 128 KB under way: 0.32 us a k-block of half the
 // size). Per launch, us, 128 x 128 tiles -> these: 3264 tokens (K = 1024: QKV 2560 rows 31.5 -> 21.5,
 // gate/up 8192 rows 66.3 -> 42.2; O 26.0 -> 20.4, down 39.3 -> 30.1); 408 tokens: gate/up 16.8 -> 9.8.
+// NW = 1 (norm-fed kinds) is for launches of few tiles, where half of them would leave SMs idle: twice
+// the CTAs, each with half the bytes and half the epilogue (QKV, 408 tokens: 40 tiles 11.3 us, 80 narrow
+// ones 7.5; the launcher has the rule).
 // Persistent: one CTA per SM walks the tiles u = blockIdx.x, + gridDim.x, .., the token tile fastest
 // (the CTAs that run together share one weight tile, which is read from HBM once):
 //   warp 0  one thread streams (operand block, weight block pair) by bulk tensor copies through the
 //           ring; the weight blocks of the first stages are requested before the dependency wait;
-//   warp 1  one thread issues the tcgen05.mma chain (M = 128, N = 256, K = 16 each) of a tile into one
+//   warp 1  one thread issues the tcgen05.mma chain (M = 128, N = 128 NW, K = 16 each) of a tile into one
 //           of two TMEM accumulators and releases each stage through tcgen05.commit;
 //   warps 2-9  the epilogue: a TMEM lane is a token, so the two features that rotary coding or GeGLU
-//           combine are columns of one thread. Group g of four warps takes columns 128 g .. (one
-//           weight tile). Norm-fed kinds scale by the token's 1 / rms and add W beta, which is the
+//           combine are columns of one thread. Group g of four warps takes weight tile g (NW = 1: half of
+//           the one tile's pairs). Norm-fed kinds scale by the token's 1 / rms and add W beta, which is the
 //           accumulator row of the beta row (TMEM lane 63): its warp hands the group's 128 values
 //           over through shared memory. Every warp passes its 32 rows through 4 KB of shared memory
 //           of its own (128 bytes a row, 16-byte chunks XOR-swizzled by the row), so that global
@@ -27,29 +30,31 @@
 //           Residual kinds fetch the old residual rows one 32-column step ahead.
 // All waits are bounded.
 
-constexpr int RT_N = 256;                                       // weight rows per tile (MMA N)
 constexpr int RT_XBYTES = 128 * KBLK * 2;                       // 16 KB operand block
-constexpr int RT_STAGE_BYTES = RT_XBYTES + 2 * TILE_BYTES;      // + two weight tiles' blocks
-constexpr int RT_STAGES = 4;
+constexpr int RT_RING = 192 * 1024;                             // 4 stages of 48 KB, or 6 of 32 KB
 constexpr int RT_EPI = 256;
 constexpr int RT_THREADS = 64 + RT_EPI;
 constexpr int RT_STAGING = 32 * 128;                            // one epilogue warp: 32 rows of 128 bytes
-constexpr int RT_SMEM = 1024 + RT_STAGES * RT_STAGE_BYTES + 8 * RT_STAGING + RT_N * 4 + 128;
+constexpr int RT_SMEM = 1024 + RT_RING + 8 * RT_STAGING + 2 * TILE_ROWS * 4 + 160;
 
-template <int KIND>
+template <int KIND, int NW>
 __global__ void __launch_bounds__(RT_THREADS, 1) k_tc_gemm_rows(const __grid_constant__ CUtensorMap wmap,
                                                               const __grid_constant__ CUtensorMap xmap,
                                                               const __grid_constant__ GemmArgs a) {
     constexpr bool NORM_IN = (KIND == G_QKV || KIND == G_GU);
     constexpr int TT = NORM_IN ? 2 * XS_TOKENS : 128;   // tokens per tile
+    constexpr int RT_N = NW * TILE_ROWS;                // weight rows per tile (MMA N)
+    constexpr int RT_STAGE_BYTES = RT_XBYTES + NW * TILE_BYTES;
+    constexpr int RT_STAGES = RT_RING / RT_STAGE_BYTES;
     constexpr uint32_t IDESC = ptx::idesc_bf16_f32(128, RT_N);
+    static_assert(NW == 2 || (NW == 1 && NORM_IN), "one weight tile: norm-fed kinds only");
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
-    uint8_t* stages = smem;                                             // [stage][X 16 KB | W 32 KB]
+    uint8_t* stages = smem;                                             // [stage][X 16 KB | W 16 KB each]
     uint8_t* staging = smem + RT_STAGES * RT_STAGE_BYTES;               // [8 warps][32 rows][128 B]
-    float* beta_s = (float*)(staging + 8 * RT_STAGING);                 // [256] W beta of the tile's columns
-    uint64_t* full = (uint64_t*)(beta_s + RT_N);
+    float* beta_s = (float*)(staging + 8 * RT_STAGING);                 // [2 groups][128] W beta of their columns
+    uint64_t* full = (uint64_t*)(beta_s + 2 * TILE_ROWS);
     uint64_t* empty = full + RT_STAGES;
     uint64_t* accf = empty + RT_STAGES;   // [2] accumulator holds a finished tile
     uint64_t* acce = accf + 2;            // [2] the epilogue has read it out
@@ -58,7 +63,7 @@ __global__ void __launch_bounds__(RT_THREADS, 1) k_tc_gemm_rows(const __grid_con
 
     const int tid = threadIdx.x, warp = ptx::warp_index(), lane = tid & 31;
     const int nkb = a.nkb;
-    const int ntn = (a.ntiles + 1) / 2, ntm = (a.Mt + TT - 1) / TT;
+    const int ntn = (a.ntiles + NW - 1) / NW, ntm = (a.Mt + TT - 1) / TT;
     const int total = ntn * ntm;
     const int u0 = (int)blockIdx.x, du = (int)gridDim.x;
 
@@ -83,12 +88,13 @@ __global__ void __launch_bounds__(RT_THREADS, 1) k_tc_gemm_rows(const __grid_con
     if (warp == 0) {
         if (ptx::elect_one()) {
             const uint64_t pol = ptx::l2_policy_evict_first();
-            // Both weight tiles' k-blocks (rows past the last tile arrive as zeros).
+            // The weight tiles' k-blocks (rows past the last tile arrive as zeros).
             auto load_w = [&](int tn, int kb, int s) {
                 uint8_t* ws = stages + s * RT_STAGE_BYTES + RT_XBYTES;
                 ptx::mbar_expect_tx(&full[s], (uint32_t)RT_STAGE_BYTES);
-                ptx::tma_load_2d(ws, &wmap, &full[s], 0, (2 * tn * nkb + kb) * TILE_ROWS, pol);
-                ptx::tma_load_2d(ws + TILE_BYTES, &wmap, &full[s], 0, ((2 * tn + 1) * nkb + kb) * TILE_ROWS, pol);
+#pragma unroll
+                for (int w = 0; w < NW; ++w)
+                    ptx::tma_load_2d(ws + w * TILE_BYTES, &wmap, &full[s], 0, ((NW * tn + w) * nkb + kb) * TILE_ROWS, pol);
             };
             auto load_x = [&](int tm, int kb, int s) {
                 ptx::tma_load_2d_plain(stages + s * RT_STAGE_BYTES, &xmap, &full[s], kb * KBLK, tm * 128);
@@ -150,8 +156,11 @@ __global__ void __launch_bounds__(RT_THREADS, 1) k_tc_gemm_rows(const __grid_con
             if (!good) *flag = DEV_TIMEOUT_MMA;
         }
     } else {
-        // ---- epilogue: one token (TMEM lane) per thread, columns 128 g .. 128 g + 127 ----
+        // ---- epilogue: one token (TMEM lane) per thread; group g has weight tile g of two, or half of
+        // the one tile's pairs (steps 2 g, 2 g + 1) ----
         const int g = (warp - 2) >> 2, qd = warp & 3;
+        constexpr int NST = 2 * NW;                  // this group's steps of 32 columns
+        const int st0 = NW == 1 ? NST * g : 0;
         const int row = qd * 32 + lane;
         const uint32_t bar_id = 1 + g;
         uint8_t* stg = staging + (warp - 2) * RT_STAGING;
@@ -169,7 +178,7 @@ __global__ void __launch_bounds__(RT_THREADS, 1) k_tc_gemm_rows(const __grid_con
         bool ok = true;
         for (int u = u0, j = 0; u < total; u += du, ++j) {
             const int buf = j & 1;
-            const int tm = u % ntm, tile = 2 * (u / ntm) + g;   // this group's 128-row weight tile
+            const int tm = u % ntm, tile = NW == 2 ? 2 * (u / ntm) + g : u / ntm;   // this group's 128-row weight tile
             const bool tile_live = tile < a.ntiles;
             const int f0 = tile * TILE_ROWS;
             // Global inputs that do not depend on the product, before the accumulator is waited for.
@@ -222,17 +231,18 @@ __global__ void __launch_bounds__(RT_THREADS, 1) k_tc_gemm_rows(const __grid_con
                                             : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
             };
-            fetch(0);
+            fetch(st0);
             if (!ptx::mbar_wait_bounded(&accf[buf], (j >> 1) & 1, WAIT_LIMIT_NS)) *flag = DEV_TIMEOUT_MMA;
             ptx::tc_fence_after();
             // This CTA's last accumulator is complete: the next kernel may start streaming its weights.
             if (u + du >= total) ptx::grid_dep_launch();
-            const uint32_t lb = tmem + (uint32_t)(buf * RT_N + 128 * g) + ((uint32_t)(qd * 32) << 16);
+            const uint32_t lb = tmem + (uint32_t)(buf * RT_N + (NW == 2 ? 128 * g : 0)) + ((uint32_t)(qd * 32) << 16);
             if constexpr (NORM_IN) {
                 if (qd == 1) {
                     // The beta row is this warp's lane 31 (TMEM lane 63).
 #pragma unroll
                     for (int c0 = 0; c0 < 128; c0 += 32) {
+                        if (NW == 1 && ((c0 >> 5) & 1) != g) continue;   // the other group's pairs
                         uint32_t r[2][16];
                         ptx::tmem_ld_x16(lb + (uint32_t)c0, r[0]);
                         ptx::tmem_ld_x16(lb + (uint32_t)(c0 + 16), r[1]);
@@ -250,7 +260,8 @@ __global__ void __launch_bounds__(RT_THREADS, 1) k_tc_gemm_rows(const __grid_con
                 ok = __all_sync(0xffffffffu, ok && *flag == 0);
                 const float4* bt = (const float4*)(beta_s + 128 * g);
 #pragma unroll
-                for (int st = 0; st < 4; ++st) {
+                for (int q = 0; q < NST; ++q) {
+                    const int st = st0 + q;
                     // Columns 16 st.. and 64 + 16 st..: the two features of 16 pairs.
                     uint32_t r1[16], r2[16];
                     ptx::tmem_ld_x16(lb + (uint32_t)(16 * st), r1);
@@ -294,7 +305,7 @@ __global__ void __launch_bounds__(RT_THREADS, 1) k_tc_gemm_rows(const __grid_con
                                 *(uint32_t*)(p + hd) = pack_bf16x2(va * c.x + ua * c.y, vb * c.z + ub * c.w);
                             }
                         }
-                        if (st < 3) fetch(st + 1);
+                        if (q < NST - 1) fetch(st + 1);
                         __syncwarp();
                     }
                 }
@@ -302,8 +313,18 @@ __global__ void __launch_bounds__(RT_THREADS, 1) k_tc_gemm_rows(const __grid_con
                 ptx::mbar_arrive(&acce[buf]);
                 if (KIND == G_GU) {
                     __syncwarp();
+                    if (NW == 1) {
+                        // Four chunks a row: eight rows per instruction.
+                        const int c = 4 * g + (lane & 3);
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
+                        for (int i = 0; i < 4; ++i) {
+                            const int r = 8 * i + (lane >> 2), t = tile_live ? token(tm, qd * 32 + r) : -1;
+                            const uint4 v = *row_chunk(r, c);
+                            if (t >= 0 && ok) *(uint4*)(a.z + (size_t)t * a.F + tile * 64 + 8 * c) = v;
+                        }
+                    }
+#pragma unroll
+                    for (int i = 0; i < 8 && NW == 2; ++i) {
                         const uint4 v = *row_chunk(4 * i + sr, sc);
                         if (tk[i] >= 0 && ok) *(uint4*)(a.z + (size_t)tk[i] * a.F + tile * 64 + 8 * sc) = v;
                     }

@@ -162,9 +162,10 @@ struct jpi_handle {
     // Tensor-core path: one plan per projection (QKV, O, gate/up, down) and tensor maps
     // (4 per layer, same order).
     jpi::GemmPlan plans[4];
-    int big_min_tokens[4] = {400, 128, 128, 128};   // per projection kind: from this many tokens the large-M GEMM
+    int big_min_tokens[4] = {};   // per projection kind: from this many tokens the large-M GEMM
     int big_split = 0;          // K split of the large-M residual projections (0: chosen per launch)
     int resid_rows = -1;        // tokens-on-rows kernel for those (-1: chosen per launch)
+    int rows_tile_n = 0;        // its tile width for the norm-fed projections (0: chosen per launch)
     int big_clusters[4] = {0, 0, 0, 0};   // co-resident large-M clusters of 1, 2, 4, 8 CTAs
     int attn_t5_min_batch = 3;  // batches of at least this many requests use the tcgen05 attention
     bool attn_t5 = false;       // its tensor maps and attributes are ready

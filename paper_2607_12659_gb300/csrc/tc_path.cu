@@ -327,11 +327,23 @@ bool resid_rows(const jpi_handle* h, int kind, int Mt, const GemmPlan& pl) {
     return waves * pl.nkb * 5 < other * 4;
 }
 
-template <int KIND>
+// Whether a norm-fed projection takes 128 x 128 tiles instead of 128 x 256 ones: a wave of the narrow
+// ones takes 7/11 of a wave of the wide ones (3.5 and 5.5 us at K = 1024), so while their waves
+// cost no more. pi0.5 sizes, us, narrow and wide: QKV 408 tokens 7.5 and 11.3 (one wave each), 816: 7.8
+// and 11.3, 1020: 12.3 and 11.5 (two waves and one), 2040: 17.1 and 18.4, 3264: 21.7 and 20.4; gate/up 204
+// tokens 6.8 and 8.8, 408: 10.4 and 9.1, 816: 14.2 and 14.7, 1020: 17.8 and 15.3, 3264: 44.1 and 38.6.
+bool rows_narrow(const jpi_handle* h, int Mt, const GemmPlan& pl) {
+    if (h->rows_tile_n > 0) return h->rows_tile_n == TILE_ROWS;
+    const long ntm = (Mt + 2 * XS_TOKENS - 1) / (2 * XS_TOKENS), n = h->num_sms;
+    const long narrow = (pl.ntiles * ntm + n - 1) / n, wide = ((pl.ntiles + 1) / 2 * ntm + n - 1) / n;
+    return narrow * 7 <= wide * 11;
+}
+
+template <int KIND, int NW>
 jpi_status launch_gemm_rows(jpi_handle* h, const GemmPlan& pl, const CUtensorMap& wmap, const CUtensorMap& xmap,
                             const GemmArgs& a, cudaStream_t st) {
     constexpr int TT = (KIND == G_QKV || KIND == G_GU) ? 2 * XS_TOKENS : 128;
-    const int tiles = ((pl.ntiles + 1) / 2) * std::max(1, (a.Mt + TT - 1) / TT);
+    const int tiles = ((pl.ntiles + NW - 1) / NW) * std::max(1, (a.Mt + TT - 1) / TT);
     GemmArgs ar = a;
     ar.ntiles = pl.ntiles;
     cudaLaunchConfig_t cfg = {};
@@ -344,7 +356,7 @@ jpi_status launch_gemm_rows(jpi_handle* h, const GemmPlan& pl, const CUtensorMap
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
     cfg.numAttrs = h->pdl ? 1 : 0;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_tc_gemm_rows<KIND>, wmap, xmap, ar);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_tc_gemm_rows<KIND, NW>, wmap, xmap, ar);
     if (e != cudaSuccess) {
         set_error("tensor-core GEMM launch failed: %s", cudaGetErrorString(e));
         return JPI_ERR_CUDA;
@@ -501,7 +513,8 @@ jpi_status tc_prepare(jpi_handle* h) {
         }
         JPI_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     }
-    for (auto k : {k_tc_gemm_rows<G_QKV>, k_tc_gemm_rows<G_O>, k_tc_gemm_rows<G_GU>, k_tc_gemm_rows<G_DOWN>})
+    for (auto k : {k_tc_gemm_rows<G_QKV, 1>, k_tc_gemm_rows<G_QKV, 2>, k_tc_gemm_rows<G_GU, 1>, k_tc_gemm_rows<G_GU, 2>,
+                   k_tc_gemm_rows<G_O, 2>, k_tc_gemm_rows<G_DOWN, 2>})
         JPI_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, RT_SMEM));
     auto big1 = {k_tc_gemm_big<G_O, 1>, k_tc_gemm_big<G_DOWN, 1>};
     for (auto k : big1)
@@ -543,15 +556,9 @@ jpi_status tc_prepare(jpi_handle* h) {
     // JPI_BIG_RESID_ROWS=0 / 1 fixes the kernel of those projections (1: tokens on the MMA's rows).
     const char* rows_env = std::getenv("JPI_BIG_RESID_ROWS");
     if (rows_env) h->resid_rows = std::atoi(rows_env) != 0 ? 1 : 0;
-    // Launches with at least this many tokens use the large-M kernels. The gate/up projection (64
-    // weight tiles at pi0.5 sizes) fills the GPU with them from 128 tokens (165 tokens: 11.0 us on
-    // the K-split kernel's tiles, 9.4 on the rows kernel), the residual ones with a K split; QKV (20
-    // weight tiles) keeps the K-split kernel below 400 tokens (306 tokens: 11.6 against 12.5 us; 408:
-    // 12.9 against 12.5).
-    // JPI_BIG_GEMM_MIN_TOKENS sets one threshold for all four.
-    const char* big_env = std::getenv("JPI_BIG_GEMM_MIN_TOKENS");
-    if (big_env)
-        for (int k = 0; k < 4; ++k) h->big_min_tokens[k] = std::atoi(big_env);
+    // JPI_BIG_TILE_N=128 / 256 fixes the tile width of the large-M QKV and gate/up projections.
+    const char* tile_env = std::getenv("JPI_BIG_TILE_N");
+    if (tile_env) h->rows_tile_n = std::atoi(tile_env) == TILE_ROWS ? TILE_ROWS : 2 * TILE_ROWS;
     const int rows[4] = {h->QKV, h->W, 2 * h->F, h->W};
     const int ks[4] = {h->W, h->HD, h->W, h->F};
     // The K split (and so the summation order) is chosen once per projection, for every batch
@@ -586,6 +593,17 @@ jpi_status tc_prepare(jpi_handle* h) {
             set_error("a cluster of %d CTAs with %zu bytes of shared memory does not fit", pl.splits, pl.smem);
             return JPI_ERR_UNSUPPORTED;
         }
+        // The K-split kernel runs its grid once per token tile of 63 or 64; the large-M kernels take
+        // over once its CTAs no longer all run at once (two per SM where the shared memory allows;
+        // with one, clusters leave some SMs of a GPC idle). At pi0.5 sizes that is from 190 tokens for
+        // QKV (153 tokens: 6.6 us against 7.3; 204: 10.7 against 7.4), 64 for gate/up (102: 11.1 against
+        // 6.9) and 65 for down (102: 10.7 against 9.4). O would gain up to 256 tokens (255: 7.0 against
+        // 8.4) but takes over at 128 at the latest: the K-split kernel's partial sums are fp16, the
+        // large-M kernels' fp32. JPI_BIG_GEMM_MIN_TOKENS sets one threshold for all four.
+        const int resident = 2 * (pl.smem + 1024) <= 228 * 1024 ? 2 * sms : nclusters * pl.splits;
+        const int tt = g == G_QKV || g == G_GU ? XS_TOKENS : NT;
+        h->big_min_tokens[g] = std::min(std::max(1, resident / pl.ctas) * tt + 1, g == G_QKV ? 400 : 128);
+        if (const char* big_env = std::getenv("JPI_BIG_GEMM_MIN_TOKENS")) h->big_min_tokens[g] = std::atoi(big_env);
     }
     h->tmaps.resize((size_t)4 * h->L);
     for (int l = 0; l < h->L; ++l) {
@@ -636,10 +654,12 @@ jpi_status tc_launch_op(jpi_handle* h, int op, int l, int step, int B, int C, cu
                    const GemmArgs& a) -> jpi_status {
         constexpr int KIND = decltype(kind_tag)::value;
         if (!big(KIND)) return launch_gemm<KIND>(h, pl, wm, h->xmaps[xi], a, st);
-        if (KIND == G_QKV || KIND == G_GU || resid_rows(h, KIND, Mt, pl))
-            return launch_gemm_rows<KIND>(h, pl, wm, h->xmaps_rows[xi], a, st);
-        if constexpr (KIND == G_O || KIND == G_DOWN) return launch_gemm_big<KIND>(h, pl, wm, h->xmaps[xi], a, st);
-        return JPI_ERR_UNSUPPORTED;
+        if constexpr (KIND == G_QKV || KIND == G_GU) {
+            if (rows_narrow(h, Mt, pl)) return launch_gemm_rows<KIND, 1>(h, pl, wm, h->xmaps_rows[xi], a, st);
+        } else if (!resid_rows(h, KIND, Mt, pl)) {
+            return launch_gemm_big<KIND>(h, pl, wm, h->xmaps[xi], a, st);
+        }
+        return launch_gemm_rows<KIND, 2>(h, pl, wm, h->xmaps_rows[xi], a, st);
     };
     using KQ = std::integral_constant<int, G_QKV>;
     using KO = std::integral_constant<int, G_O>;

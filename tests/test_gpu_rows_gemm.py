@@ -1,7 +1,7 @@
 """GPU: the large-M projection kernel with the tokens on the MMA's rows, forced on every projection,
 against the fp64 oracle at the edges of its tiles: token counts around one and two tiles (126 tokens
-for the norm-fed kinds, 128 for the residual kinds) and an odd number of 128-row weight tiles (the
-second half of the last 256-row tile is padding)."""
+for the norm-fed kinds, 128 for the residual kinds), an odd number of 128-row weight tiles (the
+second half of the last 256-row tile is padding) and both tile widths of the norm-fed kinds."""
 
 import pytest
 
@@ -19,11 +19,13 @@ ONE_HEAD = ODD.with_(width=256, n_heads=1, mlp_dim=512)
 
 
 @pytest.mark.parametrize("cfg", [ODD, ONE_HEAD], ids=["odd_tiles", "one_head"])
+@pytest.mark.parametrize("tile_n", ["128", "256"])
 @pytest.mark.parametrize("B,C", [(1, 1), (2, 62), (1, 126), (3, 41), (1, 127), (1, 128), (3, 84), (4, 63)])
-def test_tokens_on_rows_kernel(monkeypatch, cfg, B, C):
+def test_tokens_on_rows_kernel(monkeypatch, cfg, B, C, tile_n):
     lib()
     monkeypatch.setenv("JPI_BIG_GEMM_MIN_TOKENS", "1")
     monkeypatch.setenv("JPI_BIG_RESID_ROWS", "1")
+    monkeypatch.setenv("JPI_BIG_TILE_N", tile_n)
     P, t = 70, 0.4
     w = make_weights(cfg, 77, mod_bias_std=0.3)
     r = make_requests(cfg, 78 + B + C, B, P, C)
