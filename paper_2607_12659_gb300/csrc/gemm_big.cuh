@@ -13,14 +13,13 @@
 //           into one of two TMEM accumulators (tile j into buffer j mod 2, once the epilogue has
 //           read tile j - 2 out of it) and releases each stage through tcgen05.commit;
 //   warps 2-9  the epilogue, two groups of four warps (group g takes accumulator columns
-//           64g..64g+63, one TMEM lane = weight row per thread). The residual rows of the tile are
-//           copied into a shared fp32 tile [token][feature] with 16-byte async copies before the
-//           accumulator is waited for (fetched in dependent chunks after it, they made the epilogue
-//           as long as the tile's operand stream); one thread waits for the accumulator and the
-//           others at a named barrier. The accumulator rows are added into that tile, then the new
-//           residual, the next norm's operand and each token's sum of squares are written
-//           a token row per warp instruction (16 / 8 bytes per lane). After the read-out the TMEM
-//           buffer goes back to the MMA thread.
+//           64g..64g+63, one TMEM lane = weight row per thread). After the read-out the TMEM buffer
+//           goes back to the MMA thread. With a K split the partials are exchanged and summed as
+//           described at BigCfg. Without one the residual rows of the tile are copied into a shared
+//           fp32 tile [token][feature] with 16-byte async copies before the accumulator is waited
+//           for and the accumulator rows are added into that tile. Either way the new residual, the
+//           next norm's operand and each token's sum of squares are written a token row per warp
+//           instruction (16 / 8 bytes per lane).
 // The next kernel is released once this CTA's last accumulator is complete. All waits are
 // bounded.
 
@@ -34,15 +33,22 @@ constexpr int BIG_YBYTES = BIG_NT * BIG_HS * 4;
 
 // S CTAs of a cluster split the K range of each unit (S = 1: no split). Each CTA then owns
 // TOK = 128 / S of the unit's tokens: it sends the fp32 partial of every other CTA's tokens to that
-// CTA ([token][feature] slices, one bulk copy per peer) and sums the S partials of its own tokens in
-// rank order. The exchange buffers take shared memory from the ring, which keeps 3 (S = 2, 4) or
-// 2 (S = 8) stages of 32 KB in flight.
+// CTA and sums the S partials of its own tokens in rank order. A slice is laid out [feature / 32][token]
+// [32], so each epilogue warp's part of it (its 32 accumulator rows, all tokens) is one contiguous
+// block, which the warp sends as soon as it has written it; a receiving warp adds the partials of its
+// tokens to residual rows it holds in registers and stores the results, with no staging tile and one
+// block barrier (for the CTA's own partials). The exchange buffers take shared memory from the ring,
+// which keeps 4 (S = 2) or 3 stages of 32 KB in flight. What bounds a unit at these sizes is the chain
+// from the accumulator to the stores: block barriers around whole-slice copies and a staging tile
+// took 1.1-2.3 us longer (us, before -> now: O 153 tokens 8.3 -> 7.2, 408: 9.3 -> 7.9, 816: 11.3 -> 9.0;
+// down 10.1 -> 9.2, 11.5 -> 10.2, 15.3 -> 12.9).
 template <int S>
 struct BigCfg {
-    static constexpr int STAGES = S == 1 ? 4 : (S == 8 ? 2 : 3);
+    static constexpr int STAGES = S <= 2 ? 4 : 3;
     static constexpr int TOK = BIG_NT / S;                                 // tokens owned per CTA
-    static constexpr int SLICE = TOK * BIG_NT * 4;                         // one [TOK][128] fp32 slice
-    static constexpr int YBYTES = S == 1 ? BIG_YBYTES : TOK * BIG_HS * 4;  // staging tile
+    static constexpr int SLICE = TOK * BIG_NT * 4;                         // one fp32 slice
+    static constexpr int WBLK = TOK * 32;                                  // floats of a warp's block of it
+    static constexpr int YBYTES = S == 1 ? BIG_YBYTES : 0;                 // staging tile
     static constexpr int SEND = (S - 1) * SLICE;                           // outgoing slices
     static constexpr int RECV = S == 1 ? 0 : S * SLICE;                    // partials by rank (own one too)
 };
@@ -69,8 +75,8 @@ __global__ void __launch_bounds__(BIG_THREADS, 1) k_tc_gemm_big(const __grid_con
     uint8_t* smem = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
     uint8_t* stages = smem;                                             // [stage][W 16 KB | X 16 KB]
     float* ystage = (float*)(smem + STAGES * BIG_STAGE_BYTES);          // residual tile [token][feature]
-    float* sendb = (float*)((uint8_t*)ystage + CF::YBYTES);             // [S - 1][TOK][128] to the peers
-    float* recvb = (float*)((uint8_t*)sendb + CF::SEND);                // [S][TOK][128] by sender rank
+    float* sendb = (float*)((uint8_t*)ystage + CF::YBYTES);             // [S - 1][4][TOK][32] to the peers
+    float* recvb = (float*)((uint8_t*)sendb + CF::SEND);                // [S][4][TOK][32] by sender rank
     uint64_t* full = (uint64_t*)((uint8_t*)recvb + CF::RECV);
     uint64_t* empty = full + STAGES;
     uint64_t* accf = empty + STAGES;   // [2] accumulator buffer holds a finished tile
@@ -103,7 +109,7 @@ __global__ void __launch_bounds__(BIG_THREADS, 1) k_tc_gemm_big(const __grid_con
         ptx::mbar_init(&acce[0], BIG_EPI);
         ptx::mbar_init(&acce[1], BIG_EPI);
         ptx::mbar_init(recvf, 1);
-        ptx::mbar_init(pfree, S > 1 ? S - 1 : 1);
+        ptx::mbar_init(pfree, S > 1 ? (S - 1) * (BIG_EPI / 32) : 1);
         ptx::fence_mbar_init();
         *flag = 0;
     }
@@ -111,8 +117,8 @@ __global__ void __launch_bounds__(BIG_THREADS, 1) k_tc_gemm_big(const __grid_con
     __syncthreads();
     ptx::tc_fence_after();
     // Split K: every CTA of the cluster has initialised its barriers before any peer aims a copy or
-    // an arrival at them.
-    if (S > 1) ptx::cluster_sync_all();
+    // an arrival at them (waited for before the first exchange).
+    if (S > 1) ptx::cluster_arrive_relaxed();
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {
@@ -127,7 +133,6 @@ __global__ void __launch_bounds__(BIG_THREADS, 1) k_tc_gemm_big(const __grid_con
             auto load_x = [&](int xt, int kb, int s) {
                 uint8_t* xs = stages + s * BIG_STAGE_BYTES + TILE_BYTES;
                 ptx::tma_load_2d(xs, &xmap, &full[s], (kb0 + kb) * KBLK, xt * BIG_NT, pol);
-                ptx::tma_load_2d(xs + XBLK_BYTES, &xmap, &full[s], (kb0 + kb) * KBLK, xt * BIG_NT + NT, pol);
             };
             // Weight blocks of the first tile's first stages do not depend on the previous kernel.
             const int npre = u0 < total ? (nkb < STAGES ? nkb : STAGES) : 0;
@@ -182,6 +187,139 @@ __global__ void __launch_bounds__(BIG_THREADS, 1) k_tc_gemm_big(const __grid_con
             }
             if (!good) *flag = DEV_TIMEOUT_MMA;
         }
+    } else if constexpr (S > 1) {
+        // ---- epilogue with a K split: TMEM lane `row` (weight row) of the accumulator per thread ----
+        const int eg = (tid - 64) >> 7;   // group: accumulator columns (tokens) 64 eg ..
+        const int ew = (tid - 64) >> 5, quarter = warp & 3;
+        constexpr int TW = TOK / 8;       // tokens a warp finishes: TW ew .. of this CTA's
+        constexpr int NSL = 64 / TOK > 0 ? 64 / TOK : 1;   // slices a group's columns cover
+        ptx::grid_dep_wait();
+        bool ok = true;
+        for (int u = u0, j = 0; u < total; u += du, ++j) {
+            const int buf = j & 1;
+            const int tile = u % ntiles, xt = u / ntiles;
+            const int tok0 = xt * BIG_NT + rank * TOK + TW * ew;   // this warp's first token
+            const int f0 = tile * TILE_ROWS;
+            // Features 4 lane ..: the residual rows, gamma and the next norm's scale, in flight while the
+            // accumulator is waited for.
+            const float4 gm = *(const float4*)(a.gamma + f0 + 4 * lane);
+            const float4 sg = a.xs ? *(const float4*)(a.sigma_next + f0 + 4 * lane) : make_float4(0.f, 0.f, 0.f, 0.f);
+            float4 hr[TW];
+#pragma unroll
+            for (int k = 0; k < TW; ++k)
+                hr[k] = tok0 + k < a.Mt ? *(const float4*)(a.hres + (size_t)(tok0 + k) * a.W + f0 + 4 * lane)
+                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+            // Slices of this unit from the S - 1 peers.
+            if (tid == 64) ptx::mbar_expect_tx(recvf, (uint32_t)((S - 1) * CF::SLICE));
+            __syncwarp();
+            if (j == 0) {
+                ptx::cluster_wait();
+            } else if (!ptx::mbar_wait_cluster_bounded(pfree, (j - 1) & 1, WAIT_LIMIT_NS)) {
+                // (Every peer has summed the last unit's slices, so this CTA's outgoing slices, read by
+                // those copies, and the peers' receive slots are free again.)
+                *flag = DEV_TIMEOUT_MMA;
+            }
+            if (!ptx::mbar_wait_bounded(&accf[buf], (j >> 1) & 1, WAIT_LIMIT_NS)) *flag = DEV_TIMEOUT_MMA;
+            __syncwarp();
+            ptx::tc_fence_after();
+            // This CTA's last accumulator is complete: the next kernel may start streaming its weights.
+            if (u + du >= total) ptx::grid_dep_launch();
+            // Accumulator column c (token c of the unit) belongs to rank c / TOK: own columns go to this
+            // CTA's slot of the receive buffer, the others to the outgoing slice of their rank.
+            {
+                const uint32_t lane_base = tmem + (uint32_t)(buf * BIG_NT + 64 * eg) + ((uint32_t)(quarter * 32) << 16);
+                uint32_t r[4][16];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) ptx::tmem_ld_x16(lane_base + (uint32_t)(16 * c), r[c]);
+                ptx::tmem_ld_wait();
+                ptx::tc_fence_before();
+                ptx::mbar_arrive(&acce[buf]);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    // 16 columns never straddle two owners (TOK >= 16).
+                    const int col0 = 64 * eg + 16 * c, q = col0 / TOK;
+                    float* dst = (q == rank ? recvb + (size_t)rank * TOK * BIG_NT
+                                            : sendb + (size_t)(q < rank ? q : q - 1) * TOK * BIG_NT) +
+                                 quarter * CF::WBLK + (col0 % TOK) * 32 + lane;
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) dst[i * 32] = __uint_as_float(r[c][i]);
+                }
+            }
+            // This warp's blocks of the outgoing slices, lane i to the i-th of their ranks.
+            ptx::fence_proxy_async_smem();
+            __syncwarp();
+            if (lane < NSL && eg * NSL + lane != rank) {
+                const int q = eg * NSL + lane;
+                ptx::bulk_copy_to_cluster(
+                    ptx::dsmem_map(ptx::smem_u32(recvb + (size_t)rank * TOK * BIG_NT + quarter * CF::WBLK), (uint32_t)q),
+                    sendb + (size_t)(q < rank ? q : q - 1) * TOK * BIG_NT + quarter * CF::WBLK, (uint32_t)(CF::WBLK * 4),
+                    ptx::dsmem_map(ptx::smem_u32(recvf), (uint32_t)q));
+            }
+            ptx::named_bar_sync(1, BIG_EPI);   // the CTA's own partials
+            ok = ok && *flag == 0;
+            // The next norm's shift in the last row of each of its token tiles (this tile's rows).
+            if (a.xs && xt == 0 && ok && rank == 0 && eg == 0) {
+                const int f = f0 + quarter * 32 + lane;
+                const float bn = a.beta_next[f];
+                for (int x = 0; x < xs_tiles(a.Mt); ++x)
+                    a.xs[((size_t)x * 64 + 63) * a.W + f] = __float2bfloat16_rn(bn);
+            }
+            if (!ptx::mbar_wait_bounded(recvf, j & 1, WAIT_LIMIT_NS)) {
+                *flag = DEV_TIMEOUT_MMA;
+                ok = false;
+            }
+            // (A timeout may be seen by some lanes only: the warp decides together.)
+            ok = __all_sync(0xffffffffu, ok);
+            // Everything addressed to this CTA has landed; once all of the cluster say so every copy
+            // out of it has landed too.
+            if (u + du >= total) ptx::cluster_arrive_relaxed();
+            // n = h + gamma * (sum of the S partials in rank order); the token's sum of squares over
+            // the tile's 128 features is lane 0's butterfly total (slot `tile`).
+            float4 y[TW];
+#pragma unroll
+            for (int k = 0; k < TW; ++k) {
+                y[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int q = 0; q < S; ++q) {
+                    const float4 v = *(const float4*)(recvb + (size_t)q * TOK * BIG_NT + (lane >> 3) * CF::WBLK +
+                                                      (TW * ew + k) * 32 + 4 * (lane & 7));
+                    y[k].x += v.x;
+                    y[k].y += v.y;
+                    y[k].z += v.z;
+                    y[k].w += v.w;
+                }
+            }
+            // This warp has read its part of the receive buffer: each peer may overwrite its slot (and
+            // reuse its outgoing slices) for the next unit. One lane per peer.
+            if (u + du < total) {
+                __syncwarp();
+                if (lane < S - 1) {
+                    const int q = lane < rank ? lane : lane + 1;
+                    ptx::mbar_arrive_cluster_relaxed(ptx::dsmem_map(ptx::smem_u32(pfree), (uint32_t)q));
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < TW; ++k) {
+                const int t = tok0 + k;
+                if (t >= a.Mt || !ok) break;
+                float4 n;
+                n.x = hr[k].x + gm.x * y[k].x;
+                n.y = hr[k].y + gm.y * y[k].y;
+                n.z = hr[k].z + gm.z * y[k].z;
+                n.w = hr[k].w + gm.w * y[k].w;
+                *(float4*)(a.hres + (size_t)t * a.W + f0 + 4 * lane) = n;
+                if (a.xs)
+                    *(uint2*)(a.xs + (size_t)xs_row(t) * a.W + f0 + 4 * lane) =
+                        make_uint2(pack_bf16x2((1.f + sg.x) * n.x, (1.f + sg.y) * n.y),
+                                   pack_bf16x2((1.f + sg.z) * n.z, (1.f + sg.w) * n.w));
+                float sq = ((n.x * n.x + n.y * n.y) + n.z * n.z) + n.w * n.w;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+                if (lane == 0) a.ss_out[(size_t)tile * a.ss_ld + t] = sq;
+            }
+            // Every warp has read the CTA's own slot before the next unit rewrites it.
+            if (u + du < total) ptx::named_bar_sync(1, BIG_EPI);
+        }
     } else {
         // ---- epilogue: TMEM lane `row` (weight row) of the accumulator per thread ----
         const int eg = (tid - 64) >> 7;   // group
@@ -200,7 +338,7 @@ __global__ void __launch_bounds__(BIG_THREADS, 1) k_tc_gemm_big(const __grid_con
             if (a.xs) sg4 = *(const float4*)(a.sigma_next + f0 + 4 * lane);
 #pragma unroll
             for (int k = 0; k < TOK / 8; ++k) {
-                const int c = (TOK / 8) * ew + k, t = tok0 + rank * TOK + c;
+                const int c = (TOK / 8) * ew + k, t = tok0 + c;
                 const bool in = t < a.Mt;
                 ptx::cp_async_16(ptx::smem_u32(ystage + c * BIG_HS + 4 * lane),
                                  a.hres + (in ? (size_t)t * a.W + f0 + 4 * lane : 0), in);
@@ -212,10 +350,6 @@ __global__ void __launch_bounds__(BIG_THREADS, 1) k_tc_gemm_big(const __grid_con
             const int tok0 = xt * BIG_NT;
             fetch(tile, tok0);
             ptx::cp_async_wait_all();
-            // Split K: every peer has summed the last unit's slices, so this CTA's outgoing slices
-            // (read by those copies) and the peers' receive slots are free again.
-            if (S > 1 && tid == 64 && j > 0 && !ptx::mbar_wait_cluster_bounded(pfree, (j - 1) & 1, WAIT_LIMIT_NS))
-                *flag = DEV_TIMEOUT_MMA;
             if (tid == 64 && !ptx::mbar_wait_bounded(&accf[buf], (j >> 1) & 1, WAIT_LIMIT_NS)) *flag = DEV_TIMEOUT_MMA;
             // The residual rows are published; the MMAs of the tile are done.
             ptx::named_bar_sync(1, BIG_EPI);
@@ -227,76 +361,24 @@ __global__ void __launch_bounds__(BIG_THREADS, 1) k_tc_gemm_big(const __grid_con
                 const uint32_t lane_base = tmem + (uint32_t)(buf * BIG_NT) + ((uint32_t)((warp & 3) * 32) << 16);
                 {
                     const int f0 = tile * TILE_ROWS, f = f0 + row;
-                    if constexpr (S == 1) {
-                        // n = h + gamma * y in place of h: accumulator row `row` (feature f), 32 token
-                        // columns at a time, into column f of the [token][feature] tile.
+                    // n = h + gamma * y in place of h: accumulator row `row` (feature f), 32 token
+                    // columns at a time, into column f of the [token][feature] tile.
 #pragma unroll
-                        for (int c0 = 0; c0 < 64; c0 += 32) {
-                            uint32_t r[2][16];
-                            ptx::tmem_ld_x16(lane_base + (uint32_t)(64 * eg + c0), r[0]);
-                            ptx::tmem_ld_x16(lane_base + (uint32_t)(64 * eg + c0 + 16), r[1]);
-                            ptx::tmem_ld_wait();
+                    for (int c0 = 0; c0 < 64; c0 += 32) {
+                        uint32_t r[2][16];
+                        ptx::tmem_ld_x16(lane_base + (uint32_t)(64 * eg + c0), r[0]);
+                        ptx::tmem_ld_x16(lane_base + (uint32_t)(64 * eg + c0 + 16), r[1]);
+                        ptx::tmem_ld_wait();
 #pragma unroll
-                            for (int i = 0; i < 32; ++i) {
-                                float* hp = ystage + (64 * eg + c0 + i) * BIG_HS + row;
-                                *hp = *hp + gam * __uint_as_float(r[i >> 4][i & 15]);
-                            }
-                        }
-                        ptx::tc_fence_before();
-                        ptx::mbar_arrive(&acce[buf]);
-                    } else {
-                        // Split K: accumulator column c (token c of the unit) belongs to rank c / TOK.
-                        // Own columns go to this CTA's slot of the receive buffer, the others to the
-                        // outgoing slice of their rank ([token][feature], a warp stores 32
-                        // consecutive features of one token).
-#pragma unroll
-                        for (int c0 = 0; c0 < 64; c0 += 32) {
-                            uint32_t r[2][16];
-                            ptx::tmem_ld_x16(lane_base + (uint32_t)(64 * eg + c0), r[0]);
-                            ptx::tmem_ld_x16(lane_base + (uint32_t)(64 * eg + c0 + 16), r[1]);
-                            ptx::tmem_ld_wait();
-#pragma unroll
-                            for (int hh = 0; hh < 2; ++hh) {
-                                // 16 columns never straddle two owners (TOK >= 16).
-                                const int col0 = 64 * eg + c0 + 16 * hh, q = col0 / TOK;
-                                float* dst = (q == rank ? recvb + (size_t)rank * TOK * BIG_NT
-                                                        : sendb + (size_t)(q < rank ? q : q - 1) * TOK * BIG_NT) +
-                                             (size_t)(col0 % TOK) * BIG_NT + row;
-#pragma unroll
-                                for (int i = 0; i < 16; ++i) dst[i * BIG_NT] = __uint_as_float(r[hh][i]);
-                            }
-                        }
-                        ptx::tc_fence_before();
-                        ptx::mbar_arrive(&acce[buf]);
-                        ptx::fence_proxy_async_smem();   // the outgoing slices, for the bulk copies
-                        ptx::named_bar_sync(1, BIG_EPI);
-                        if (ew == 0) {
-                            // Slices of this unit from the S - 1 peers (lane 0), then this CTA's
-                            // slices out, lane q to peer q (the copies issue together).
-                            if (lane == 0) ptx::mbar_expect_tx(recvf, (uint32_t)((S - 1) * CF::SLICE));
-                            if (lane < S && lane != rank) {
-                                const int q = lane;
-                                const uint32_t own_slot = ptx::smem_u32(recvb + (size_t)rank * TOK * BIG_NT);
-                                const uint32_t rbar = ptx::smem_u32(recvf);
-                                ptx::bulk_copy_to_cluster(ptx::dsmem_map(own_slot, (uint32_t)q),
-                                                          sendb + (size_t)(q < rank ? q : q - 1) * TOK * BIG_NT,
-                                                          (uint32_t)CF::SLICE, ptx::dsmem_map(rbar, (uint32_t)q));
-                            }
-                            if (lane == 0 && !ptx::mbar_wait_bounded(recvf, j & 1, WAIT_LIMIT_NS)) *flag = DEV_TIMEOUT_MMA;
-                        }
-                        ptx::named_bar_sync(1, BIG_EPI);   // every partial of this CTA's tokens is here
-                        // n = h + gamma * (sum of the S partials in rank order) for tokens cc of this
-                        // CTA, feature f: a warp reads and writes 32 consecutive features.
-                        for (int cc = eg; cc < TOK; cc += 2) {
-                            float y = 0.f;
-#pragma unroll
-                            for (int q = 0; q < S; ++q) y += recvb[(size_t)(q * TOK + cc) * BIG_NT + row];
-                            float* hp = ystage + cc * BIG_HS + row;
-                            *hp = *hp + gam * y;
+                        for (int i = 0; i < 32; ++i) {
+                            float* hp = ystage + (64 * eg + c0 + i) * BIG_HS + row;
+                            *hp = *hp + gam * __uint_as_float(r[i >> 4][i & 15]);
                         }
                     }
+                    ptx::tc_fence_before();
+                    ptx::mbar_arrive(&acce[buf]);
                     // The next norm's shift in the last row of each of its token tiles (this tile's rows).
-                    if (a.xs && xt == 0 && ok && eg == 0 && rank == 0) {
+                    if (a.xs && xt == 0 && ok && eg == 0) {
                         const float bn = a.beta_next[f];
                         for (int x = 0; x < xs_tiles(a.Mt); ++x)
                             a.xs[((size_t)x * 64 + 63) * a.W + f] = __float2bfloat16_rn(bn);
@@ -309,7 +391,7 @@ __global__ void __launch_bounds__(BIG_THREADS, 1) k_tc_gemm_big(const __grid_con
                     const bool okw = __all_sync(0xffffffffu, ok);
 #pragma unroll 4
                     for (int k = 0; k < TOK / 8; ++k) {
-                        const int c = (TOK / 8) * ew + k, t = tok0 + rank * TOK + c;
+                        const int c = (TOK / 8) * ew + k, t = tok0 + c;
                         if (t >= a.Mt || !okw) break;
                         const float4 n = *(const float4*)(ystage + c * BIG_HS + 4 * lane);
                         *(float4*)(a.hres + (size_t)t * a.W + f0 + 4 * lane) = n;
@@ -323,13 +405,6 @@ __global__ void __launch_bounds__(BIG_THREADS, 1) k_tc_gemm_big(const __grid_con
                         for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
                         if (lane == 0) a.ss_out[(size_t)tile * a.ss_ld + t] = sq;
                     }
-                    // Split K: this CTA has summed its receive buffer (every value read is in the
-                    // staging tile, published by the barrier above): each peer may overwrite its slot
-                    // (and reuse its outgoing slices) for the next unit. One lane per peer.
-                    if (S > 1 && ew == 0 && lane < S - 1) {
-                        const int q = lane < rank ? lane : lane + 1;
-                        ptx::mbar_arrive_cluster_relaxed(ptx::dsmem_map(ptx::smem_u32(pfree), (uint32_t)q));
-                    }
                 }
                 // Every epilogue thread is done with the residual tile.
                 ptx::named_bar_sync(1, BIG_EPI);
@@ -340,8 +415,16 @@ __global__ void __launch_bounds__(BIG_THREADS, 1) k_tc_gemm_big(const __grid_con
     if (tid == 0 && *flag != 0) set_device_error(a.err, *flag);
     ptx::tc_fence_before();
     __syncthreads();
-    // Split K: no copy or arrival of a peer is still aimed at this CTA when it exits.
-    if (S > 1) ptx::cluster_sync_all();
     ptx::tc_fence_after();
     if (warp == 1) ptx::tmem_dealloc(tmem, 2 * BIG_NT);
+    // Split K: no copy or arrival of a peer is still aimed at this CTA when it exits (the epilogue
+    // warps arrived once their last slices had landed).
+    if (S > 1) {
+        if (warp <= 1) {
+            __syncwarp();
+            ptx::cluster_wait();
+            ptx::cluster_arrive_relaxed();
+        }
+        ptx::cluster_wait();
+    }
 }

@@ -285,8 +285,11 @@ jpi_status launch_gemm(jpi_handle* h, const GemmPlan& pl, const CUtensorMap& wma
 // Large-M variant: persistent CTAs over (weight tile, 128-row operand tile) units. The residual
 // kinds (few weight tiles, long K) may split each unit's K range over a cluster of S CTAs so that
 // the units fill the GPU: S is the one of 1, 2, 4, 8 with the fewest estimated K blocks per SM,
-// counting waves of S x units CTAs and an exchange worth BIG_SPLIT_COST K blocks for S > 1.
-constexpr int BIG_SPLIT_COST = 4;
+// counting waves of S x units CTAs and, for each, what a unit's exchange adds in K blocks of
+// about 0.23 us. Fitted at pi0.5 sizes (one, two and three waves, us; O has 32 K blocks, down 64):
+// down S = 1 19.4; S = 2 12.7, 21.4; S = 4 10.3, 15.5, 21.9; O S = 1 12.5; S = 2 9.1, 13.7; S = 4 7.9,
+// 11.8, 15.7; S = 8 9.5 (two), 13.8, 18.5 (four).
+constexpr int BIG_SPLIT_COST[9] = {0, 0, 5, 0, 9, 0, 0, 0, 14};
 
 // Clusters of S large-M CTAs that can run at once (one CTA per SM; clusters of 8 leave some SMs
 // of each GPC idle), from the occupancy query at prepare time.
@@ -304,7 +307,7 @@ int big_split(const jpi_handle* h, int kind, int units, int nkb, long* cost_out 
     for (int S = 1; S <= 8; S *= 2) {
         if (nkb % S || nkb / S < 2) continue;
         const long waves = (units + big_clusters(h, S) - 1) / big_clusters(h, S);
-        const long cost = waves * (nkb / S + (S > 1 ? BIG_SPLIT_COST : 0));
+        const long cost = waves * (nkb / S + BIG_SPLIT_COST[S]);
         if (best_cost < 0 || cost < best_cost) {
             best_cost = cost;
             best = S;
@@ -657,7 +660,7 @@ jpi_status tc_launch_op(jpi_handle* h, int op, int l, int step, int B, int C, cu
         if constexpr (KIND == G_QKV || KIND == G_GU) {
             if (rows_narrow(h, Mt, pl)) return launch_gemm_rows<KIND, 1>(h, pl, wm, h->xmaps_rows[xi], a, st);
         } else if (!resid_rows(h, KIND, Mt, pl)) {
-            return launch_gemm_big<KIND>(h, pl, wm, h->xmaps[xi], a, st);
+            return launch_gemm_big<KIND>(h, pl, wm, h->xmaps_rows[xi], a, st);
         }
         return launch_gemm_rows<KIND, 2>(h, pl, wm, h->xmaps_rows[xi], a, st);
     };
