@@ -70,6 +70,7 @@ struct T5Args {
     float scale_log2;   // log2(e) / sqrt(D)
     __nv_bfloat16* o;   // [Mt][H][D]
     int* err;
+    int b0 = 0;         // first request of this launch
     // Key splits: [CTA][D / 4][128] partial outputs and [CTA][128] (m, l), CTA = (row block,
     // request, split) in launch order; unused (null) without splits.
     float4* ws = nullptr;
@@ -268,7 +269,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) k_attn_t5(const __grid_constant
     int* flag = (int*)(tmem_slot + 1);
 
     const int tid = threadIdx.x, warp = ptx::warp_index(), lane = tid & 31;
-    const int rb = blockIdx.x, b = blockIdx.y;
+    const int rb = blockIdx.x, b = a.b0 + (int)blockIdx.y;
     const int nrows = a.S * a.H, nk = a.P + a.S;
     const int row0 = rb * T5_ROWS;
     // Key split: this CTA's key blocks blk0 .. blk0 + nb - 1 of the request's nb_all.
