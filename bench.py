@@ -48,7 +48,7 @@ NCU_TRAFFIC = {
 # The sources the expert's kernels and their launches are built from. The correction module
 # (CORRECTION_SOURCES) is compiled into the same library but none of the measured kernels uses it.
 EXPERT_SOURCES = ("api.cu", "attn_t5.cu", "attn_t5_kernel.cuh", "attn_tc.cu", "gemm_big.cuh", "gemm_kernel.cuh",
-                  "jpi_internal.h", "kernels_simt.cu", "mod_tc.cu", "noalloc.cu", "ptx.h", "tc_path.cu",
+                  "gemm_rows.cuh", "jpi_internal.h", "kernels_simt.cu", "mod_tc.cu", "noalloc.cu", "ptx.h", "tc_path.cu",
                   "tc_path.h")
 CORRECTION_SOURCES = ("corr.cu",)
 
@@ -56,8 +56,8 @@ CORRECTION_SOURCES = ("corr.cu",)
 # The sources the five batch-1 layer kernels of NCU_TRAFFIC are built and launched from (the
 # projection kernel, the split-KV attention, their launcher and shared headers): their counters
 # stay valid while these are unchanged, whatever changes elsewhere (the large-batch attention).
-TRAFFIC_SOURCES = ("attn_tc.cu", "gemm_big.cuh", "gemm_kernel.cuh", "jpi_internal.h", "ptx.h", "tc_path.cu",
-                   "tc_path.h")
+TRAFFIC_SOURCES = ("attn_tc.cu", "gemm_big.cuh", "gemm_kernel.cuh", "gemm_rows.cuh", "jpi_internal.h",
+                   "ptx.h", "tc_path.cu", "tc_path.h")
 
 
 def source_sha(files=EXPERT_SOURCES) -> str:
