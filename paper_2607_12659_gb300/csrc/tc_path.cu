@@ -1,18 +1,22 @@
 // Tensor-core path of the bf16 expert layers: tcgen05 GEMMs fed by bulk tensor copies.
 //
 // Every projection of a layer is a skinny GEMM Y[tokens][out] = X[tokens][K] W[out][K]^T with
-// tokens = batch x (chunk + 1) (51 at batch 1). It runs "swap-AB": a 128-row tile of W is the
-// A operand (M = 128), a 64-token tile of X is the B operand (N = 64), and the fp32 product
-// sits in TMEM. The K dimension of each weight tile is split across the CTAs of one thread-
-// block cluster. Each CTA loads its weight blocks with bulk tensor copies before it waits on
-// the previous kernel (weights do not depend on it); after the wait it loads its X blocks the
-// same way from the bf16 activation the previous op left in global memory (for the two
-// RMSNorm-fed projections it then applies the norm and the time-conditioned scale/shift in
-// shared memory), multiplies, and the cluster reduces its fp32 partials through distributed
-// shared memory in a fixed rank order, so results do not depend on timing. Each CTA applies
-// the epilogue to its slice of the reduced tile: rotary encoding + scatter into the query
-// buffer and KV store (QKV), GeGLU (gate/up), or the gated residual update of the fp32 stream
-// with its bf16 copy and per-token sums of squares for the next RMSNorm (O, down).
+// tokens = batch x (chunk + 1) (51 at batch 1). Three kernels share it by token count (the rules are
+// at the thresholds in tc_prepare and at rows_narrow, big_split and resid_rows below):
+//   gemm_kernel.cuh  few tokens: "swap-AB", a 128-row tile of W as the A operand (M = 128), 64 tokens
+//                    of X as B (N = 64), the fp32 product in TMEM; the K range of a weight tile split
+//                    over the CTAs of a cluster, which exchange fp16 partials through distributed
+//                    shared memory and sum them in a fixed rank order;
+//   gemm_rows.cuh    many tokens: tokens on the MMA's rows, 128 x 256 or 128 x 128 tiles over the
+//                    whole K range;
+//   gemm_big.cuh     O and down at token counts whose tiles would leave SMs idle: 128 x 128 tiles
+//                    with a K split over a cluster, fp32 partials.
+// Each loads its weight blocks with bulk tensor copies before it waits on the previous kernel
+// (weights do not depend on it), then its X blocks the same way from the bf16 activation the previous
+// op left in global memory. The RMSNorm-fed kinds read the scaled residual stream and apply 1 / rms
+// and the norm's shift in the epilogue. Epilogues: rotary encoding + scatter into the query buffer and
+// KV store (QKV), GeGLU (gate/up), or the gated residual update of the fp32 stream with the next norm's
+// bf16 operand and per-token sums of squares (O, down).
 
 #include "tc_path.h"
 #include "ptx.h"
