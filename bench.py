@@ -37,11 +37,11 @@ OP_NAMES = {2: "norm+qkv+rope", 3: "attention", 4: "o_proj+residual", 5: "norm+g
 # valid only while TRAFFIC_SOURCES hash to `source_sha256`.
 NCU_TRAFFIC = {
     # profiles/layer_kernels_pi05_forward.md (layer 1 of one eager forward, batch 1, P 816).
-    "norm+qkv+rope": {"bytes": 5489664, "source_sha256": "39321630f8ff0a0e"},
-    "attention": {"bytes": 1179648, "source_sha256": "39321630f8ff0a0e"},
-    "o_proj+residual": {"bytes": 4695808, "source_sha256": "39321630f8ff0a0e"},
-    "norm+gate_up+geglu": {"bytes": 16959744, "source_sha256": "39321630f8ff0a0e"},
-    "down_proj+residual": {"bytes": 9131776, "source_sha256": "39321630f8ff0a0e"},
+    "norm+qkv+rope": {"bytes": 5489152, "source_sha256": "be8926c37a41dfe4"},
+    "attention": {"bytes": 1165312, "source_sha256": "be8926c37a41dfe4"},
+    "o_proj+residual": {"bytes": 4690944, "source_sha256": "be8926c37a41dfe4"},
+    "norm+gate_up+geglu": {"bytes": 16957696, "source_sha256": "be8926c37a41dfe4"},
+    "down_proj+residual": {"bytes": 9127168, "source_sha256": "be8926c37a41dfe4"},
 }
 
 

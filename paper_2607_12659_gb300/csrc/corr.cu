@@ -1313,7 +1313,7 @@ jpi_status put_block(jpi_corr_handle* h, bool dev, BlockDev* out, const jpi_corr
 // predecessor at its start), so a kernel's launch overlaps the previous kernel's tail. The calls
 // enqueue their kernels on the caller's pointers: a graph of them, captured once per shape, needed
 // every input copied in and every output copied out, which took more of the GPU's time (10 us of 62 per
-// compress, 12 of 109 per predict at batch 1) than the host's 27 launches leave it idle (none: they
+// compress, 12 of 109 per predict at batch 1) than the host's 26 launches leave it idle (none: they
 // take the host less time than the kernels run). A failed launch leaves its error for the
 // cudaGetLastError check that follows.
 template <typename... KArgs, typename... Args>
