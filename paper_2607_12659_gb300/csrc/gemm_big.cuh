@@ -290,12 +290,13 @@ __global__ void __launch_bounds__(BIG_THREADS, 1) k_tc_gemm_big(const __grid_con
                 }
             }
             // This warp has read its part of the receive buffer: each peer may overwrite its slot (and
-            // reuse its outgoing slices) for the next unit. One lane per peer.
+            // reuse its outgoing slices) for the next unit. One lane per peer; a release, so that the reads
+            // of the whole warp (ordered before it by the __syncwarp) are over before the peer's next copy.
             if (u + du < total) {
                 __syncwarp();
                 if (lane < S - 1) {
                     const int q = lane < rank ? lane : lane + 1;
-                    ptx::mbar_arrive_cluster_relaxed(ptx::dsmem_map(ptx::smem_u32(pfree), (uint32_t)q));
+                    ptx::mbar_arrive_cluster(ptx::dsmem_map(ptx::smem_u32(pfree), (uint32_t)q));
                 }
             }
 #pragma unroll

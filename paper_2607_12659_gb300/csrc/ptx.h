@@ -145,11 +145,11 @@ __device__ __forceinline__ void bulk_copy_to_cluster(uint32_t dst, const void* s
         "r"(smem_u32(src)), "r"(bytes), "r"(remote_bar)
         : "memory");
 }
-// Arrival on an mbarrier of another CTA of the cluster (shared::cluster address, from dsmem_map)
-// that orders nothing: for "I have finished reading what you sent", where every read it covers
-// has already returned its value.
-__device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t bar_cluster) {
-    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
+// Arrival on an mbarrier of another CTA of the cluster (shared::cluster address, from dsmem_map), with
+// release order at cluster scope: this thread's earlier reads and writes, and those of threads it has
+// synchronised with, come before what a thread that waits on the barrier does next.
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
 }
 // Bounded wait on a local mbarrier whose phase other CTAs of the cluster complete (acquire at
 // cluster scope); gives up after `limit_ns`.

@@ -248,6 +248,46 @@ def test_pi05_large_m_k_splits(large_m_everywhere, monkeypatch):
         assert dh <= 2e-3, f"K split {S} vs 1: hidden state differs by {dh:.3g} of max |h|"
 
 
+# More 128-token tiles than clusters fit the GPU, so that a cluster of the split kernel walks three units
+# and more: the peers' release of its receive slots, the second and third phases of its barriers, and the
+# reuse of its outgoing slices. The same products summed in another order (see above), the same bits on
+# every run, and the oracle for requests of the first, a middle and the last units.
+@pytest.mark.parametrize("S,B", [(2, 78), (4, 40), (8, 21)])
+def test_large_m_k_split_several_units_per_cluster(large_m_everywhere, monkeypatch, S, B):
+    cfg = ExpertConfig(n_layers=2, width=512, n_heads=4, head_dim=128, mlp_dim=512, action_dim=7, state_dim=7,
+                       time_dim=64, precision="bf16")
+    P, C, t = 20, 99, 0.4
+    clusters = torch.cuda.get_device_properties(0).multi_processor_count // S
+    assert cfg.width // 128 * (B * (C + 1) // 128) >= 3 * clusters
+    w = make_weights(cfg, 2290, mod_bias_std=0.3)
+    r = make_requests(cfg, 2291, B, P, C)
+
+    def forward(split, reps):
+        monkeypatch.setenv("JPI_BIG_SPLIT", str(split))
+        ex = make_expert(cfg, w, max_batch=B, max_prefix=P, max_chunk=C, max_steps=1)
+        try:
+            ex.set_prefix_kv(*to_dev_kv(r, cfg))
+            s, x = torch.from_numpy(r["state"]).cuda(), torch.from_numpy(r["noise"]).cuda()
+            out = [ex.forward(s, x, t) for _ in range(reps)]
+            torch.cuda.synchronize()
+            ex.device_status()
+            return [(v.cpu().numpy(), h.cpu().numpy()) for v, h in out]
+        finally:
+            ex.close()
+
+    got, one = forward(S, 8), forward(1, 1)[0]
+    for v, h in got[1:]:
+        assert np.array_equal(v, got[0][0]) and np.array_equal(h, got[0][1]), "two runs differ"
+    dh = float(np.abs(got[0][1] - one[1]).max()) / float(np.abs(one[1]).max())
+    assert dh <= 2e-3, f"K split {S} vs 1: hidden state differs by {dh:.3g} of max |h|"
+    ids = [0, B // 2, B - 1]
+    want_v, want_h = oracle.forward_batch(r["noise"][ids], r["state"][ids], t, r["prefix_k"][:, ids],
+                                          r["prefix_v"][:, ids], w, cfg)
+    assert_close(got[0][0][ids], want_v, cfg, f"K split {S}, several units per cluster")
+    _, rel = errors(got[0][1][ids], want_h)
+    assert rel <= 1e-2, f"hidden rel-L2 {rel:.3g}"
+
+
 def test_pi05_large_m_projection_path(large_m_everywhere):
     w = make_weights(PI05, 2000)
     ex = make_expert(PI05, w, max_batch=3, max_prefix=816, max_chunk=50, max_steps=10)
