@@ -157,6 +157,7 @@ __global__ void __launch_bounds__(BIG_THREADS, 1) k_tc_gemm_big(const __grid_con
                     load_x(xt, kb, s);
                 }
             }
+            if (!ptx::ring_drain(full, STAGES, it, WAIT_LIMIT_NS)) *flag = DEV_TIMEOUT_WEIGHTS;
         }
     } else if (warp == 1) {
         if (ptx::elect_one()) {

@@ -122,10 +122,7 @@ __global__ void __launch_bounds__(RT_THREADS, 1) k_tc_gemm_rows(const __grid_con
                     load_x(tm, kb, s);
                 }
             }
-            // Nothing may land in this CTA's shared memory after it exits: the last copy into every
-            // stage (complete already unless a wait above gave up).
-            for (int i = it > RT_STAGES ? it - RT_STAGES : 0; i < it; ++i)
-                (void)ptx::mbar_wait_bounded(&full[i % RT_STAGES], (i / RT_STAGES) & 1, WAIT_LIMIT_NS);
+            if (!ptx::ring_drain(full, RT_STAGES, it, WAIT_LIMIT_NS)) *flag = DEV_TIMEOUT_WEIGHTS;
         }
     } else if (warp == 1) {
         if (ptx::elect_one()) {

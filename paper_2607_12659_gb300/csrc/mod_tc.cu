@@ -138,11 +138,7 @@ __global__ void __launch_bounds__(MT_THREADS, 1) k_mod_tc(const __grid_constant_
                 load(it);
                 issued = it + 1;
             }
-            // No copy into this CTA's shared memory is left in flight at exit: the last load of
-            // every stage has landed (at once in the normal case, where the MMAs consumed it).
-            for (int it = issued - MT_STAGES < 0 ? 0 : issued - MT_STAGES; it < issued; ++it)
-                if (!ptx::mbar_wait_bounded(&full[it % MT_STAGES], (it / MT_STAGES) & 1, MT_WAIT_NS))
-                    *flag = DEV_TIMEOUT_WEIGHTS;
+            if (!ptx::ring_drain(full, MT_STAGES, issued, MT_WAIT_NS)) *flag = DEV_TIMEOUT_WEIGHTS;
         }
     } else if (warp == 1) {
         if (ptx::elect_one()) {

@@ -525,11 +525,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pf_gemm(const __grid_constant
                     issued = max(issued, it + 1);
                 }
             }
-            // Nothing may land in this CTA's shared memory after it exits: wait for the last copy
-            // into every stage (complete already unless a wait above gave up).
-            for (int i = issued - PG_STAGES < 0 ? 0 : issued - PG_STAGES; i < issued; ++i)
-                if (!ptx::mbar_wait_bounded(&full[i % PG_STAGES], (i / PG_STAGES) & 1, PG_WAIT_NS))
-                    *flag = PF_DEV_TIMEOUT_LOAD;
+            if (!ptx::ring_drain(full, PG_STAGES, issued, PG_WAIT_NS)) *flag = PF_DEV_TIMEOUT_LOAD;
         }
     } else if (warp == 1) {
         if (ptx::elect_one()) {

@@ -63,6 +63,18 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
     }
 }
 
+// Waits (bounded) for the last copy into each of a ring's `stages` stages, `issued` copies having gone
+// round it: copy i completes phase i / stages of full[i mod stages]. Nothing may land in a CTA's shared
+// memory once it has exited, so the thread that issued the copies calls this before it leaves its role,
+// also after a wait of its own gave up (otherwise they have been consumed, and it returns at once). False if
+// a copy did not land in time.
+__device__ __forceinline__ bool ring_drain(uint64_t* full, int stages, int issued, uint64_t limit_ns) {
+    bool landed = true;
+    for (int i = issued > stages ? issued - stages : 0; i < issued; ++i)
+        landed = mbar_wait_bounded(&full[i % stages], (uint32_t)(i / stages) & 1u, limit_ns) && landed;
+    return landed;
+}
+
 // ---------------------------------------------------------------- TMA (bulk tensor copies)
 __device__ __forceinline__ uint64_t l2_policy_evict_first() {
     uint64_t pol;

@@ -27,3 +27,15 @@ def test_arrivals_on_a_peers_barrier_release_the_reads_before_them():
             found += 1
             assert arrival.startswith("mbarrier.arrive.release.cluster."), f"{name}: {arrival}"
     assert found == 1
+
+
+# The thread that fills a ring of shared-memory stages waits for its last copies before it leaves its role.
+RINGS = {"gemm_rows.cuh": "full, RT_STAGES", "gemm_big.cuh": "full, STAGES", "mod_tc.cu": "full, MT_STAGES",
+         "prefill/prefill.cu": "full, PG_STAGES"}
+
+
+def test_ring_loaders_wait_for_their_last_copies():
+    for name, ring in RINGS.items():
+        text = _source(*name.split("/"))
+        loader, rest = text.index("if (warp == 0) {"), text.index("} else if (warp == 1) {")
+        assert f"ring_drain({ring}," in text[loader:rest], name
