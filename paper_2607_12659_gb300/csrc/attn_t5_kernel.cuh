@@ -349,13 +349,17 @@ __global__ void __launch_bounds__(T5_THREADS, 1) k_attn_t5(const __grid_constant
             }
             for (; ok && first < NS && first < nb; ++first) load(first);
             // Block j once the MMAs that read block j - NS (S_{j-NS}, or P_{j-NS} V_{j-NS}) are done.
+            int issued = first;
             for (int j = NS; ok && j < nb; ++j) {
                 if (!ptx::mbar_wait_bounded(&emptyb[j % NS], (j / NS - 1) & 1, T5_WAIT_NS)) {
                     *flag = T5_ERR_LOAD;
                     break;
                 }
                 load(j);
+                issued = j + 1;
             }
+            if (!is_v && !ptx::mbar_wait_bounded(qfull, 0, T5_WAIT_NS)) *flag = T5_ERR_LOAD;
+            if (!ptx::ring_drain(fullb, NS, issued, T5_WAIT_NS)) *flag = T5_ERR_LOAD;
         }
     } else if (warp == 2) {
         if (ptx::elect_one()) {

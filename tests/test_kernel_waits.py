@@ -39,3 +39,10 @@ def test_ring_loaders_wait_for_their_last_copies():
         text = _source(*name.split("/"))
         loader, rest = text.index("if (warp == 0) {"), text.index("} else if (warp == 1) {")
         assert f"ring_drain({ring}," in text[loader:rest], name
+
+
+def test_attention_loaders_wait_for_their_last_copies():
+    text = _source("attn_t5_kernel.cuh")
+    loaders = text[text.index("if (warp <= 1) {"):text.index("} else if (warp == 2) {")]
+    assert "ring_drain(fullb, NS, issued," in loaders
+    assert "mbar_wait_bounded(qfull," in loaders
