@@ -387,9 +387,9 @@ __global__ void __launch_bounds__(RT_THREADS, 1) k_tc_gemm_rows(const __grid_con
         }
     }
 
-    if (tid == 0 && *flag != 0) set_device_error(a.err, *flag);
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
+    if (tid == 0 && *flag != 0) set_device_error(a.err, *flag);   // after every role's last word on it
     if (warp == 1) ptx::tmem_dealloc(tmem, 2 * RT_N);
 }

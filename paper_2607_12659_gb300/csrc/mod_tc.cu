@@ -196,10 +196,10 @@ __global__ void __launch_bounds__(MT_THREADS, 1) k_mod_tc(const __grid_constant_
         }
     }
 
-    if (tid == 0 && *flag != 0) atomicCAS(err, 0, *flag);
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
+    if (tid == 0 && *flag != 0) atomicCAS(err, 0, *flag);   // after every role's last word on it
     if (warp == 1) ptx::tmem_dealloc(tmem, 2 * MT_N);
 }
 

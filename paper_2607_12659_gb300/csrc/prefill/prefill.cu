@@ -742,10 +742,10 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pf_gemm(const __grid_constant
         }
     }
 
-    if (tid == 0 && *flag != 0) atomicCAS(a.err, 0, *flag);
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
+    if (tid == 0 && *flag != 0) atomicCAS(a.err, 0, *flag);   // after every role's last word on it
     if (warp == 1) ptx::tmem_dealloc(tmem, 2 * PG_TN);
 }
 

@@ -56,3 +56,13 @@ def test_single_shot_loads_are_waited_for_again_after_a_wait_gave_up():
     attn = _source("attn_tc.cu")
     gave_up = attn[attn.index("if (!landed) {"):attn.index("const uint32_t kbuf_u")]
     assert "mbar_wait_bounded(&kvbar[bi]," in gave_up and "mbar_wait_bounded(qbar," in gave_up
+
+
+def test_device_errors_are_reported_after_the_last_barrier():
+    # One thread reports for the block: a role that gives up later than it must still be heard.
+    for name in ("gemm_rows.cuh", "gemm_big.cuh", "mod_tc.cu", "attn_t5_kernel.cuh", "prefill/prefill.cu"):
+        text = _source(*name.split("/"))
+        report = [m.start() for m in re.finditer(r"if \(tid == 0 && \*flag != 0\)", text)]
+        assert len(report) == 1, name
+        last = text.rindex("*flag = ", 0, report[0])
+        assert "__syncthreads();" in text[last:report[0]], name
