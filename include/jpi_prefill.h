@@ -76,7 +76,10 @@ JPI_API jpi_status jpi_prefill_destroy(jpi_prefill_handle* h);   /* NULL is a no
  *               exactly what jpi_prefix_kv_ptr returns for a JPI_BF16 expert handle. Both arrays
  *               are host arrays of L device pointers.
  *   out_final:  device [batch][prefix_len][W] fp32, the final-layer output, or NULL.
- * 1 <= batch <= max_batch, 1 <= prefix_len <= max_prefix, request_stride >= prefix_len * D.
+ * 1 <= batch <= max_batch, 1 <= prefix_len <= max_prefix, request_stride >= prefix_len * D and a
+ * multiple of 8. Key destinations are 16-byte aligned; value destinations too where D is 128 or 256 and
+ * request_stride a multiple of D, and element-aligned otherwise. Every argument is checked before anything
+ * is enqueued.
  * Enqueued on `stream`; the inputs must stay valid until the stream reaches the call. After it,
  * jpi_commit_prefix(expert, batch, prefix_len) makes the store current for the expert.
  */

@@ -426,6 +426,7 @@ struct PfGemmArgs {
     const float2* rope;
     __nv_bfloat16 *q, *kd, *vd;
     long long kv_stride;
+    int v_pairs;          // vd takes 4-byte stores
     int* err;
 };
 
@@ -620,8 +621,18 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pf_gemm(const __grid_constant
                         if (!ok || !in || m0 + 4 * i + sr >= a.M) continue;
                         __nv_bfloat16* d = (sec < a.H ? a.q + ((size_t)(m0 + 4 * i + sr) * a.H + sec) * a.D : (sec == a.H ? a.kd : a.vd) + kvo[i]) +
                                            j0 + 2 * sc;
-                        *(uint32_t*)d = pack2(ua * cs[i].x - va * cs[i].y, ub * cs[i].z - vb * cs[i].w);
-                        *(uint32_t*)(d + half) = pack2(va * cs[i].x + ua * cs[i].y, vb * cs[i].z + ub * cs[i].w);
+                        const uint32_t w0 = pack2(ua * cs[i].x - va * cs[i].y, ub * cs[i].z - vb * cs[i].w);
+                        const uint32_t w1 = pack2(va * cs[i].x + ua * cs[i].y, vb * cs[i].z + ub * cs[i].w);
+                        if (sec > a.H && !a.v_pairs) {
+                            unsigned short* e = reinterpret_cast<unsigned short*>(d);
+                            e[0] = (unsigned short)w0;
+                            e[1] = (unsigned short)(w0 >> 16);
+                            e[half] = (unsigned short)w1;
+                            e[half + 1] = (unsigned short)(w1 >> 16);
+                        } else {
+                            *(uint32_t*)d = w0;
+                            *(uint32_t*)(d + half) = w1;
+                        }
                     }
                     __syncwarp();
                 }
@@ -1201,6 +1212,15 @@ JPI_API jpi_status jpi_prefill_run(jpi_prefill_handle* h, const void* x, int x_i
         return pfail(JPI_ERR_INVALID_ARG, "request_stride must be >= prefix_len * head_dim and a multiple of 8");
     for (int l = 0; l < h->L; ++l)
         if (!k_layers[l] || !v_layers[l]) return pfail(JPI_ERR_INVALID_ARG, "KV destination of layer %d is NULL", l);
+    // Whether the attention runs on the tcgen05 attention kernel (scores and probabilities never leave the
+    // SM), else per request through the GEMM: scores, softmax, V^T, probabilities times V. Keys are read by
+    // bulk tensor copies either way, values only by the former.
+    const bool t5 = h->qkv_fused() && request_stride % h->D == 0 && request_stride / h->D <= INT32_MAX;
+    for (int l = 0; l < h->L; ++l) {
+        const uintptr_t ka = reinterpret_cast<uintptr_t>(k_layers[l]), va = reinterpret_cast<uintptr_t>(v_layers[l]);
+        if ((ka & 15) || (va & (t5 ? 15 : 1)))
+            return pfail(JPI_ERR_INVALID_ARG, "K or V destination of layer %d is not aligned (K 16 bytes, V %d)", l, t5 ? 16 : 2);
+    }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int W = h->W, D = h->D, H = h->H, F = h->F, P = prefix_len, Pp = (P + 7) / 8 * 8;
     const long long M = (long long)batch * P;
@@ -1241,10 +1261,6 @@ JPI_API jpi_status jpi_prefill_run(jpi_prefill_handle* h, const void* x, int x_i
         __nv_bfloat16* vd = static_cast<__nv_bfloat16*>(v_layers[l]);
         // Attention sublayer: projections, rotary coding, scatter into q and the caller's KV store.
         if (h->qkv_fused()) {
-            // The attention below reads the destinations by bulk tensor copies; this epilogue stores
-            // pairs of elements.
-            if ((reinterpret_cast<uintptr_t>(kd) | reinterpret_cast<uintptr_t>(vd)) & 15)
-                return pfail(JPI_ERR_INVALID_ARG, "a GEMM operand is not 16-byte aligned (address or row stride)");
             PF_TRY(row_gemm(h, st, h->xn, W, lw.wqkv, W, true, h->q, true, H * D, (int)M, h->QKV, W, 1.f, false, 0,
                             [&](PfGemmArgs& a) {
                                 a.qkv = 1;
@@ -1256,6 +1272,7 @@ JPI_API jpi_status jpi_prefill_run(jpi_prefill_handle* h, const void* x, int x_i
                                 a.kd = kd;
                                 a.vd = vd;
                                 a.kv_stride = request_stride;
+                                a.v_pairs = reinterpret_cast<uintptr_t>(vd) % 4 == 0 ? 1 : 0;
                             }));
         } else {
             PF_TRY(row_gemm(h, st, h->xn, W, lw.wqkv, W, true, h->qkv, false, h->QKV, (int)M, h->QKV, W, 1.f, false));
@@ -1263,9 +1280,6 @@ JPI_API jpi_status jpi_prefill_run(jpi_prefill_handle* h, const void* x, int x_i
                 request_stride, batch, P, H, D);
             PF_CUDA(cudaGetLastError());
         }
-        // Attention: on the tcgen05 attention kernel (scores and probabilities never leave the
-        // SM), else per request through the GEMM: scores, softmax, V^T, probabilities times V.
-        const bool t5 = (D == 128 || D == 256) && request_stride % D == 0 && request_stride / D <= INT32_MAX;
         if (t5) {
             PF_TRY(D == 256 ? attention_t5<256>(h, st, kd, vd, batch, P, request_stride / D)
                             : attention_t5<128>(h, st, kd, vd, batch, P, request_stride / D));

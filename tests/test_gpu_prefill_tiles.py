@@ -45,3 +45,57 @@ def test_prefill_tiles(cfg, B, P, pad):
     assert rel <= REL_L2, f"final output rel-L2 {rel:.3g}"
     assert np.isfinite(out.cpu().numpy()).all()
     pre.close()
+
+
+# Value destinations that are only element-aligned, which the attention's bulk copies cannot read: taken
+# where the request stride is no multiple of the head dim (the per-request products), refused otherwise.
+@pytest.mark.parametrize("cfg", [WIDE, ODD], ids=["wide", "odd"])
+@pytest.mark.parametrize("shift", [0, 1, 2, 8])
+def test_prefill_value_destinations_at_any_element(cfg, shift):
+    import torch
+    from tests.gpu_util import errors, lib
+    lib()
+    from paper_2607_12659_gb300 import prefill
+    B, P, L, D = 2, 100, cfg.n_layers, cfg.head_dim
+    stride = P * D + 8
+    w = make_llm_weights(cfg, 141, std=0.05, norm_std=0.1)
+    x = make_prefix_embeddings(cfg, 142, B, P)
+    pre = prefill.Prefill(cfg, w, max_batch=B, max_prefix=P)
+    K = torch.full((L, B * stride), 7.0, dtype=torch.bfloat16, device="cuda")
+    V = torch.full((L, B * stride + 16), 7.0, dtype=torch.bfloat16, device="cuda")
+    out = pre.run(torch.from_numpy(x).cuda(), [K[l].data_ptr() for l in range(L)],
+                  [V[l, shift:].data_ptr() for l in range(L)], stride)
+    torch.cuda.synchronize()
+    pre.device_status()
+    Kw, Vw, want = pf.prefill_batch(x, w, cfg)
+    for l in range(L):
+        for got, ref, what in ((K[l], Kw[l], "K"), (V[l, shift:shift + B * stride], Vw[l], "V")):
+            rows = got.view(B, stride).float().cpu().numpy()
+            _, rel = errors(rows[:, :P * D].reshape(B, P, D), ref)
+            assert rel <= REL_L2, f"{what} layer {l}: rel-L2 {rel:.3g}"
+            assert (rows[:, P * D:] == 7.0).all(), f"{what} layer {l}: written past the prefix"
+        assert bool((V[l, :shift] == 7.0).all()) and bool((V[l, shift + B * stride:] == 7.0).all())
+    _, rel = errors(out.cpu().numpy(), want)
+    assert rel <= REL_L2, f"final output rel-L2 {rel:.3g}"
+    pre.close()
+
+
+@pytest.mark.parametrize("which,pad,shift", [("k", 0, 4), ("v", 0, 4), ("k", 8, 4)])
+def test_prefill_refuses_a_misaligned_layer_before_it_runs_any(which, pad, shift):
+    import torch
+    from tests.gpu_util import lib
+    lib()
+    from paper_2607_12659_gb300 import prefill
+    from paper_2607_12659_gb300.jpi import JpiError
+    cfg, P = ODD, 20
+    L, D = cfg.n_layers, cfg.head_dim
+    pre = prefill.Prefill(cfg, make_llm_weights(cfg, 151, std=0.05), max_batch=1, max_prefix=P)
+    x = torch.from_numpy(make_prefix_embeddings(cfg, 152, 1, P)).cuda()
+    kv = {n: torch.full((L, P * D + 16), 7.0, dtype=torch.bfloat16, device="cuda") for n in "kv"}
+    ptr = {n: [kv[n][l].data_ptr() for l in range(L)] for n in "kv"}
+    ptr[which][-1] += 2 * shift
+    with pytest.raises(JpiError):
+        pre.run(x, ptr["k"], ptr["v"], P * D + pad)
+    torch.cuda.synchronize()
+    assert bool((kv["k"] == 7.0).all()) and bool((kv["v"] == 7.0).all())
+    pre.close()
