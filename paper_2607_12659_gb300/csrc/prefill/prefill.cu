@@ -94,7 +94,8 @@ __device__ __forceinline__ float block_sum_rb(float v, float* red) {
     __syncthreads();   // red is reused by the next row
     return t;
 }
-// y[4 i .. 4 i + 3] of row r = v * rinv * (1 + w).
+// y[4 i .. 4 i + 3] of row r = v * rinv * (1 + w). An fp32 y is the caller's and may be only
+// element-aligned.
 template <typename TO>
 __device__ __forceinline__ void store_normed4(TO* y, const float* w, long long r, int W, int i, float4 v, float rinv) {
     const float4 g = reinterpret_cast<const float4*>(w)[i];
@@ -106,8 +107,14 @@ __device__ __forceinline__ void store_normed4(TO* y, const float* w, long long r
         u.x = *reinterpret_cast<const uint32_t*>(&lo);
         u.y = *reinterpret_cast<const uint32_t*>(&hi);
         *reinterpret_cast<uint2*>(y + r * W + 4 * i) = u;
-    } else {
+    } else if ((reinterpret_cast<uintptr_t>(y) & 15) == 0) {
         *reinterpret_cast<float4*>(y + r * W + 4 * i) = make_float4(a0, a1, a2, a3);
+    } else {
+        y += r * W + 4 * i;
+        y[0] = a0;
+        y[1] = a1;
+        y[2] = a2;
+        y[3] = a3;
     }
 }
 __device__ __forceinline__ float sq4(float4 v) {

@@ -99,3 +99,30 @@ def test_prefill_refuses_a_misaligned_layer_before_it_runs_any(which, pad, shift
     torch.cuda.synchronize()
     assert bool((kv["k"] == 7.0).all()) and bool((kv["v"] == 7.0).all())
     pre.close()
+
+
+# The final output at an address that takes no 16-byte stores, from the pieces' sum (many k-blocks a tile)
+# and after the product that accumulates in place (few): the same bits as at an aligned address.
+@pytest.mark.parametrize("cfg,P", [(ODD, 20), (WIDE, 100), (ODD.with_(mlp_dim=384), 20)])
+def test_prefill_final_output_at_any_float(cfg, P):
+    import torch
+    from tests.gpu_util import lib
+    lib()
+    from paper_2607_12659_gb300 import prefill
+    L, D, W = cfg.n_layers, cfg.head_dim, cfg.width
+    pre = prefill.Prefill(cfg, make_llm_weights(cfg, 161, std=0.05), max_batch=1, max_prefix=P)
+    x = torch.from_numpy(make_prefix_embeddings(cfg, 162, 1, P)).cuda()
+    K = torch.zeros((L, P, D), dtype=torch.bfloat16, device="cuda")
+    V = torch.zeros_like(K)
+    kp, vp = [K[l].data_ptr() for l in range(L)], [V[l].data_ptr() for l in range(L)]
+    outs = []
+    for shift in (0, 1, 2):
+        buf = torch.full((P * W + 4,), 7.0, device="cuda")
+        prefill.jpi_prefill_run(pre.handle, x, True, 1, P, kp, vp, P * D, buf[shift:])
+        torch.cuda.synchronize()
+        assert bool((buf[:shift] == 7.0).all()) and bool((buf[shift + P * W:] == 7.0).all())
+        outs.append(buf[shift:shift + P * W].clone())
+    pre.device_status()
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
+    assert bool((outs[0] != 7.0).all())
+    pre.close()
