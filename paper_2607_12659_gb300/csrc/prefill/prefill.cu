@@ -1114,7 +1114,7 @@ jpi_status setup(jpi_prefill_handle* h, const jpi_prefill_config* c, const jpi_p
     PF_TRY(pf_alloc(h, &h->dev_err, 1));
     PF_CUDA(cudaMemset(h->dev_err, 0, sizeof(int)));
     float* staging = nullptr;
-    if (!dev) PF_TRY(pf_alloc(h, &staging, F * W));
+    if (!dev) PF_TRY(pf_alloc(h, &staging, std::max({F, HD, D}) * W));   // the largest tensor put_bf16 / put_gu take
     h->layers.resize((size_t)h->L);
     for (int l = 0; l < h->L; ++l) {
         LayerW& lw = h->layers[(size_t)l];

@@ -47,6 +47,27 @@ def test_prefill_tiles(cfg, B, P, pad):
     pre.close()
 
 
+# Query weights larger than the MLP's: host tensors pass through one staging buffer.
+@pytest.mark.parametrize("over", [dict(width=64, n_heads=8, head_dim=128, mlp_dim=8),
+                                  dict(width=32, n_heads=1, head_dim=64, mlp_dim=16)])
+def test_prefill_of_more_head_than_mlp_features(over):
+    from tests.gpu_util import errors, lib
+    import torch
+    lib()
+    from paper_2607_12659_gb300 import prefill
+    cfg, P = GEMMA2B.with_(n_layers=2, **over), 40
+    w = make_llm_weights(cfg, 171, std=0.05, norm_std=0.1)
+    x = make_prefix_embeddings(cfg, 172, 1, P)
+    pre = prefill.Prefill(cfg, w, max_batch=1, max_prefix=P)
+    K, V, out = pre.into_tensors(torch.from_numpy(x).cuda())
+    torch.cuda.synchronize()
+    pre.device_status()
+    pre.close()
+    for got, ref in zip((K, V, out), pf.prefill_batch(x, w, cfg)):
+        _, rel = errors(got.float().cpu().numpy(), np.stack(ref) if isinstance(ref, list) else ref)
+        assert rel <= REL_L2, f"rel-L2 {rel:.3g}"
+
+
 # Value destinations that are only element-aligned, which the attention's bulk copies cannot read: taken
 # where the request stride is no multiple of the head dim (the per-request products), refused otherwise.
 @pytest.mark.parametrize("cfg", [WIDE, ODD], ids=["wide", "odd"])
