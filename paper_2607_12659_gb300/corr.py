@@ -17,7 +17,7 @@ from ctypes import POINTER, byref, c_float, c_int, c_longlong, c_void_p
 import numpy as np
 
 from . import jpi
-from .jpi import JPI_BF16, JPI_FP32, _check, _ptr, _stream
+from .jpi import JPI_BF16, JPI_FP32, OnStream, _check, _ptr, _stream
 
 BLOCK_FIELDS = ("ln1_w", "ln1_b", "wq", "bq", "wk", "bk", "wv", "bv", "wo", "bo",
                 "ln2_w", "ln2_b", "w1", "b1", "w2", "b2")
@@ -167,14 +167,19 @@ class Corrector:
         """h_vlm: CUDA tensor [B][T][d_vlm], float32 or bfloat16 -> [B][T'][width] float32."""
         import torch
         assert h_vlm.is_cuda and h_vlm.dim() == 3 and h_vlm.shape[2] == self.dims.d_vlm
-        h_vlm = h_vlm.contiguous()
         fp32 = h_vlm.dtype == torch.float32
         if not fp32:
             assert h_vlm.dtype == torch.bfloat16
         B, T, _ = h_vlm.shape
-        if out is None:
-            out = torch.empty((B, self.dims.n_items, self.dims.width), dtype=torch.float32,
-                              device=h_vlm.device)
+        with OnStream(stream, h_vlm.device) as on:
+            on.reads(h_vlm)
+            h_vlm = h_vlm.contiguous()
+            if out is None:
+                out = torch.empty((B, self.dims.n_items, self.dims.width), dtype=torch.float32,
+                                  device=h_vlm.device)
+                on.returns(out)
+            else:
+                on.reads(out)
         jpi_corr_compress(self.handle, h_vlm, fp32, B, T, out, stream)
         return out
 
@@ -183,13 +188,21 @@ class Corrector:
         [B][T'][width], confidence [B])."""
         import torch
         assert state.is_cuda and actions.is_cuda and actions.dim() == 3
-        state = state.contiguous().float()
-        actions = actions.contiguous().float()
         B, delta, _ = actions.shape
-        if out is None:
-            out = torch.empty_like(state)
-        if confidence is None:
-            confidence = torch.empty((B,), dtype=torch.float32, device=state.device)
+        with OnStream(stream, state.device) as on:
+            on.reads(state, actions)
+            state = state.contiguous().float()
+            actions = actions.contiguous().float()
+            if out is None:
+                out = torch.empty_like(state)
+                on.returns(out)
+            else:
+                on.reads(out)
+            if confidence is None:
+                confidence = torch.empty((B,), dtype=torch.float32, device=state.device)
+                on.returns(confidence)
+            else:
+                on.reads(confidence)
         jpi_corr_predict(self.handle, state, actions, B, delta, out, confidence, stream)
         return out, confidence
 

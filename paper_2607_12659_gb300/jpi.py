@@ -8,6 +8,7 @@ raises: there is no other implementation to fall back to.
 
 from __future__ import annotations
 
+import contextlib
 import ctypes
 import os
 import re
@@ -130,6 +131,47 @@ def _stream(stream) -> int | None:
         import torch
         return torch.cuda.current_stream().cuda_stream
     return getattr(stream, "cuda_stream", stream)
+
+
+_HERE = contextlib.nullcontext()
+
+
+class OnStream:
+    """Torch's side of a call on `stream` (a torch stream, a raw handle, or None: the current one), where that
+    is not the current stream. As a context it makes `stream` current: what is converted or allocated inside is
+    ordered with the call, and its memory is given out again in that stream's order only. `reads` keeps an input
+    from being given out again before `stream` has passed the call, `returns` a result before the current
+    stream has passed its uses there."""
+
+    def __init__(self, stream, device):
+        import torch
+        self.side = self.cur = None
+        if stream is None:
+            return
+        raw, cur = _stream(stream), torch.cuda.current_stream(device)
+        if raw != cur.cuda_stream:
+            self.cur = cur
+            self.side = (stream if isinstance(stream, torch.cuda.Stream) else
+                         torch.cuda.ExternalStream(raw, device=device) if raw else torch.cuda.default_stream(device))
+
+    def __enter__(self):
+        import torch
+        self._ctx = _HERE if self.side is None else torch.cuda.stream(self.side)
+        self._ctx.__enter__()
+        return self
+
+    def __exit__(self, *exc):
+        return self._ctx.__exit__(*exc)
+
+    def reads(self, *tensors):
+        if self.side is not None:
+            for t in tensors:
+                t.record_stream(self.side)
+
+    def returns(self, *tensors):
+        if self.side is not None:
+            for t in tensors:
+                t.record_stream(self.cur)
 
 
 # ------------------------------------------------------------------ thin C-ABI mirrors
@@ -268,8 +310,10 @@ class Expert:
         import torch
         assert k.is_cuda and v.is_cuda and k.shape == v.shape
         L, B, P, _ = k.shape
-        k = k.contiguous()
-        v = v.contiguous()
+        with OnStream(stream, k.device) as on:
+            on.reads(k, v)
+            k = k.contiguous()
+            v = v.contiguous()
         fp32 = k.dtype == torch.float32
         if not fp32:
             assert k.dtype == torch.bfloat16
@@ -285,7 +329,9 @@ class Expert:
             self.n_corr = 0
             return
         assert items.is_cuda and items.dim() == 3 and items.shape[2] == self.dims.width
-        items = items.contiguous().float()
+        with OnStream(stream, items.device) as on:
+            on.reads(items)
+            items = items.contiguous().float()
         B, T, _ = items.shape
         jpi_set_correction(self.handle, items, B, T, stream)
         self._corr = (items,)
@@ -294,8 +340,13 @@ class Expert:
     def denoise(self, state, noise, num_steps, out=None, stream=None):
         import torch
         B, C, _ = noise.shape
-        if out is None:
-            out = torch.empty_like(noise)
+        with OnStream(stream, noise.device) as on:
+            on.reads(state, noise)
+            if out is None:
+                out = torch.empty_like(noise)
+                on.returns(out)
+            else:
+                on.reads(out)
         jpi_denoise(self.handle, state, noise, B, C, num_steps, out, stream)
         return out
 
@@ -310,9 +361,12 @@ class Expert:
     def forward(self, state, x_t, t, stream=None):
         import torch
         B, C, A = x_t.shape
-        v = torch.empty_like(x_t)
-        hres = torch.empty((B, 1 + getattr(self, "n_corr", 0) + C, self.dims.width), dtype=torch.float32,
-                           device=x_t.device)
+        with OnStream(stream, x_t.device) as on:
+            on.reads(state, x_t)
+            v = torch.empty_like(x_t)
+            hres = torch.empty((B, 1 + getattr(self, "n_corr", 0) + C, self.dims.width), dtype=torch.float32,
+                               device=x_t.device)
+            on.returns(v, hres)
         jpi_expert_forward(self.handle, state, x_t, t, B, C, v, hres, stream)
         return v, hres
 

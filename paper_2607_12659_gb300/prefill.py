@@ -16,7 +16,7 @@ import numpy as np
 
 from . import build as _build
 from . import jpi
-from .jpi import STATUS_NAMES, JpiError, _ptr, _stream
+from .jpi import STATUS_NAMES, JpiError, OnStream, _ptr, _stream
 
 LIB_PATH = _build.PREFILL_LIB
 LAYER_WEIGHTS = ("attn_norm", "wq", "wk", "wv", "wo", "mlp_norm", "w_gate", "w_up", "w_down")
@@ -148,12 +148,17 @@ class Prefill:
         Returns the final-layer output [B][P][W] float32 (or None)."""
         import torch
         assert x.is_cuda and x.dim() == 3 and x.shape[2] == self.dims.width
-        x = x.contiguous()
         fp32 = x.dtype == torch.float32
         if not fp32:
             assert x.dtype == torch.bfloat16
         B, P, W = x.shape
-        out = torch.empty((B, P, W), dtype=torch.float32, device=x.device) if final else None
+        out = None
+        with OnStream(stream, x.device) as on:
+            on.reads(x)
+            x = x.contiguous()
+            if final:
+                out = torch.empty((B, P, W), dtype=torch.float32, device=x.device)
+                on.returns(out)
         jpi_prefill_run(self.handle, x, fp32, B, P, list(k_ptrs), list(v_ptrs), request_stride, out, stream)
         return out
 
@@ -162,8 +167,10 @@ class Prefill:
         import torch
         B, P, _ = x.shape
         L, D = self.dims.n_layers, self.dims.head_dim
-        K = torch.empty((L, B, P, D), dtype=torch.bfloat16, device=x.device)
-        V = torch.empty_like(K)
+        with OnStream(stream, x.device) as on:
+            K = torch.empty((L, B, P, D), dtype=torch.bfloat16, device=x.device)
+            V = torch.empty_like(K)
+            on.returns(K, V)
         out = self.run(x, [K[l].data_ptr() for l in range(L)], [V[l].data_ptr() for l in range(L)], P * D,
                        final, stream)
         return K, V, out
