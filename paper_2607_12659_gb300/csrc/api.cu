@@ -12,6 +12,7 @@
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <new>
 
@@ -398,6 +399,10 @@ JPI_API jpi_status jpi_expert_create(const jpi_config* cfg, const jpi_weights* w
         return fail(JPI_ERR_CUDA, "no CUDA device: %s", cudaGetErrorString(e));
     }
     h->tc = h->bf16 && tc_supported(h);
+    // JPI_BATCH_INVARIANT=1: every launch makes the choices it makes for one request, so a request's result
+    // is the same bit for bit alone and inside any batch, at the cost of the batched kernels.
+    const char* inv_env = std::getenv("JPI_BATCH_INVARIANT");
+    h->batch_invariant = inv_env && inv_env[0] == '1';
     if ((s = alloc_buffers(h)) != JPI_OK || (s = pack_weights(h, w)) != JPI_OK ||
         (s = configure_simt_kernels(h)) != JPI_OK || (h->tc && (s = tc_prepare(h)) != JPI_OK)) {
         std::string msg = g_err;

@@ -1218,8 +1218,11 @@ jpi_status op_simt(jpi_handle* h, int op, int l, int step, int B, int C, cudaStr
     // Measured, rows against tiles (fp32, us): QKV (2560 x 1024) 33 / 88 at 51 tokens, 109 / 122 at
     // 204 (160 tiles), 211 / 125 at 408 (280); gate/up (4096 x 1024) 164 / 215 at 102 (128), 312 / 246
     // at 204 (256); down (1024 x 4096) 212 / 286 at 408 (112), 842 / 623 at 1632 (416).
+    // The two add a product's terms in different orders: in the batch-invariant mode a launch takes what
+    // one request alone would (Mi tokens).
+    const int Mi = h->batch_invariant ? S : Mt;
     auto rows_fit = [&](int N) {
-        return (long long)((N + GB_N - 1) / GB_N) * ((Mt + GB_M - 1) / GB_M) * 4 <= 5ll * h->num_sms;
+        return (long long)((N + GB_N - 1) / GB_N) * ((Mi + GB_M - 1) / GB_M) * 4 <= 5ll * h->num_sms;
     };
     const int F = h->F, HD = h->HD, mtiles = (Mt + GB_M - 1) / GB_M;
     const float eps = h->cfg.rms_eps;
@@ -1258,7 +1261,7 @@ jpi_status op_simt(jpi_handle* h, int op, int l, int step, int B, int C, cudaStr
             return launch_rows_gemm<T, RK_QKV>(h, a, st);
         case 3: {
             // Four heads per block once one head per block would be more than four blocks per SM.
-            const bool four = h->H % 4 == 0 && (long long)Mt * h->H > 4ll * h->num_sms;
+            const bool four = h->H % 4 == 0 && (long long)Mi * h->H > 4ll * h->num_sms;
             return four ? launch_attn_rows<T, 4>(h, (const T*)h->q, kst, vst, (T*)h->o, Mt, S, st)
                         : launch_attn_rows<T, 1>(h, (const T*)h->q, kst, vst, (T*)h->o, Mt, S, st);
         }

@@ -452,13 +452,21 @@ def test_tcgen05_attention_key_splits_small_and_ragged(monkeypatch, splits):
     assert_close(vel, want_v, SMALL_BF16, f"small bf16 B3 P70, tcgen05 attention, {splits} key splits")
 
 
+# A bf16 expert whose dims the tensor-core kernels do not tile.
+UNTILED_BF16 = ExpertConfig(n_layers=2, width=160, n_heads=4, head_dim=64, mlp_dim=1030, action_dim=7, state_dim=7,
+                            time_dim=64, precision="bf16")
+
+
 # Batch invariance, bit for bit: with JPI_BATCH_INVARIANT=1 every launch makes the choices it makes
 # for a single request (the K-split projections with their fixed K split, the split-KV attention
-# with one request's key split), so request b of a batch gets exactly the actions it gets alone.
+# with one request's key split; on CUDA cores the product and attention kernels of one request's tokens),
+# so request b of a batch gets exactly the actions it gets alone. The CUDA-core cases are batches that take
+# other kernels than one request does (1020 tokens) without the switch.
 # Without the switch the attention's split and the projection kernel follow the batch size and the
 # low-order bits may move (test_pi05_batches_sampled_requests bounds that).
-@pytest.mark.parametrize("cfg,P,C,N,B", [(SMALL_BF16, 100, 13, 2, 3), (PI05, 816, 50, 10, 16)],
-                         ids=["small-bf16", "pi05"])
+@pytest.mark.parametrize("cfg,P,C,N,B", [(SMALL_BF16, 100, 13, 2, 3), (PI05, 816, 50, 10, 16), (TINY, 70, 50, 2, 20),
+                                         (UNTILED_BF16, 70, 50, 2, 20)],
+                         ids=["small-bf16", "pi05", "tiny-fp32", "untiled-bf16"])
 def test_batch_invariant_mode_is_bitwise(monkeypatch, cfg, P, C, N, B):
     monkeypatch.setenv("JPI_BATCH_INVARIANT", "1")
     w = make_weights(cfg, 2800)
