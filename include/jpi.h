@@ -129,7 +129,8 @@ typedef struct jpi_weights {
  * clusters; the same rounding-only agreement); JPI_BIG_SPLIT=n fixes the K split of the large-batch
  * O and down projections (1, 2, 4 or 8); JPI_BIG_RESID_ROWS=0 / 1 fixes which of their two kernels
  * runs (1: tokens on the MMA's rows, no K split); JPI_BIG_TILE_N=128 / 256 fixes the tile width of
- * the large-batch QKV and gate/up projections.
+ * the large-batch QKV and gate/up projections; JPI_PDL=0 launches every kernel after its predecessor has
+ * finished (no dependent launches; the same results bit for bit).
  */
 JPI_API jpi_status jpi_expert_create(const jpi_config* cfg, const jpi_weights* w, jpi_handle** out);
 

@@ -403,6 +403,9 @@ JPI_API jpi_status jpi_expert_create(const jpi_config* cfg, const jpi_weights* w
     // is the same bit for bit alone and inside any batch, at the cost of the batched kernels.
     const char* inv_env = std::getenv("JPI_BATCH_INVARIANT");
     h->batch_invariant = inv_env && inv_env[0] == '1';
+    // JPI_PDL=0: no kernel starts before its predecessor has finished.
+    const char* pdl_env = std::getenv("JPI_PDL");
+    h->pdl = !(pdl_env && pdl_env[0] == '0');
     if ((s = alloc_buffers(h)) != JPI_OK || (s = pack_weights(h, w)) != JPI_OK ||
         (s = configure_simt_kernels(h)) != JPI_OK || (h->tc && (s = tc_prepare(h)) != JPI_OK)) {
         std::string msg = g_err;

@@ -105,7 +105,7 @@ struct jpi_handle {
     int device = 0;
     bool bf16 = true;
     bool tc = false;          // tensor-core kernels in use (bf16 mode with supported dims)
-    bool pdl = true;          // programmatic dependent launch between tensor-core kernels
+    bool pdl = true;          // programmatic dependent launch between the denoise's kernels (JPI_PDL)
     int num_sms = 0;
     int attn_max_splits = 8;  // largest key-split cluster of the attention kernel
     int attn_force_splits = 0;  // > 0: key splits asked of the split-KV attention (JPI_ATTN_SPLITS)

@@ -508,8 +508,6 @@ jpi_status tc_prepare(jpi_handle* h) {
     h->num_sms = sms;
     if (attn_tc_supported(h)) JPI_TRY(attn_tc_prepare(h));
     JPI_TRY(attn_t5_prepare(h));
-    const char* pdl_env = std::getenv("JPI_PDL");
-    h->pdl = !(pdl_env && pdl_env[0] == '0');
 
     int max_cluster = 16;
     auto kernels = {k_tc_gemm<G_QKV>, k_tc_gemm<G_O>, k_tc_gemm<G_GU>, k_tc_gemm<G_DOWN>};

@@ -1,6 +1,8 @@
 """Properties of the CUDA path that hold at any size: closed forms, one step = one forward,
 determinism, graph reuse across prefixes, host/device entry points, zero-copy KV, errors."""
 
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -177,3 +179,40 @@ def test_out_of_memory_is_a_status_and_frees_everything():
     torch.cuda.synchronize()
     free1, _ = torch.cuda.mem_get_info()
     assert abs(free1 - free0) < (64 << 20)
+
+
+def _programmatic_edges(enqueue):
+    """Dependent-launch edges of the graph that enqueue(stream) captures."""
+    rt = ctypes.CDLL("libcudart.so.13")
+    stream = torch.cuda.Stream()
+    st, graph, n = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p(), ctypes.c_size_t()
+    assert rt.cudaStreamBeginCapture(st, 1) == 0   # thread-local
+    enqueue(stream)
+    assert rt.cudaStreamEndCapture(st, ctypes.byref(graph)) == 0
+    assert rt.cudaGraphGetEdges(graph, None, None, None, ctypes.byref(n)) == 0
+    nodes, data = (ctypes.c_void_p * n.value)(), (ctypes.c_ubyte * (8 * n.value))()
+    to = (ctypes.c_void_p * n.value)()
+    assert rt.cudaGraphGetEdges(graph, nodes, to, data, ctypes.byref(n)) == 0
+    rt.cudaGraphDestroy(graph)
+    return sum(data[8 * i + 2] == 1 for i in range(n.value))   # byte 2 of an edge: its type, 1 programmatic
+
+
+@pytest.mark.parametrize("cfg", [*CONFIGS, TINY.with_(precision="bf16", width=96, mlp_dim=90)],
+                         ids=["fp32", "bf16", "untiled-bf16"])
+def test_dependent_launches_can_be_switched_off(monkeypatch, cfg):
+    w, B, P, C = make_weights(cfg, 41), 2, 40, 9
+    r = make_requests(cfg, 42, B, P, C)
+    state, x = torch.from_numpy(r["state"]).cuda(), torch.from_numpy(r["noise"]).cuda()
+    edges, outs = {}, {}
+    for pdl in ("0", "1"):
+        monkeypatch.setenv("JPI_PDL", pdl)
+        ex = make_expert(cfg, w, max_batch=B, max_prefix=P, max_chunk=C, max_steps=3)
+        try:
+            outs[pdl] = gpu_denoise(ex, cfg, r, 3)
+            v = torch.empty_like(x)
+            edges[pdl] = _programmatic_edges(
+                lambda s: lib().jpi_expert_forward(ex.handle, state, x, 0.3, B, C, v, None, s))
+        finally:
+            ex.close()
+    assert edges["0"] == 0 and edges["1"] >= 5 * cfg.n_layers, edges
+    np.testing.assert_array_equal(outs["0"], outs["1"])
