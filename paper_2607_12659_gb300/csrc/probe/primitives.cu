@@ -17,11 +17,7 @@
 //                       streaming at once (median per CTA), and from a 1 GB buffer (HBM) with 152;
 //                       then with 8 and 12 copies in flight (1 and 152 CTAs, L2); then per-thread
 //                       16-byte async copies (cp.async, 256 threads, 4 x 16 KB rounds in flight),
-//                       and both at once in one CTA (a bulk-copy thread and 256 cp.async threads);
-//                       then clusters of 2 and 4 where every CTA fetches 1/2 or 1/4 of each chunk
-//                       with a multicast bulk copy into all CTAs of its cluster (bytes received per
-//                       CTA: whole chunks; 12 chunks per epoch, a cluster barrier between epochs,
-//                       and the same epochs without multicast as the control)
+//                       and both at once in one CTA (a bulk-copy thread and 256 cp.async threads)
 //   mma_cycles          tcgen05.mma issued back to back by one thread (64 in a row, and 4)
 //   dsmem_ring_us       4 KB pushed around a ring of 8 CTAs of a cluster, with a cluster barrier
 //   coresident_ctas     CTAs of 200 KB shared memory co-resident per cluster size, and whether a
@@ -245,66 +241,6 @@ __global__ void k_stream_lsu(const uint8_t* src, int nchunks, int stride, int re
     if (threadIdx.x == 0) out[blockIdx.x] = t_end[0] > t_end[1] ? t_end[0] : t_end[1];
 }
 
-// Clusters of CL CTAs (CL = 1: the same protocol without multicast), thread 0 of each, in epochs:
-// arm 12 slots of 16 KB (one arrival + 16 KB each), cluster barrier (every CTA of the cluster has
-// armed its slots and read the previous epoch's), then piece `rank` (16 KB / CL) of each of the
-// epoch's 12 chunks is fetched by a multicast bulk copy into that slot of every CTA of the
-// cluster, and each CTA waits for its 12 slots: each CTA receives 192 KB an epoch while fetching
-// 1/CL of it. Every wait is bounded; the final cluster barrier keeps each CTA alive until nothing
-// can still land in it. out[blockIdx.x] = elapsed ns.
-template <int CL>
-__global__ void k_stream_mc(const uint8_t* src, int nchunks, int stride, int epochs, unsigned long long* out,
-                            int* err) {
-    constexpr int NSLOT = 12;
-    extern __shared__ __align__(128) uint8_t sm[];
-    __shared__ __align__(8) uint64_t full[NSLOT];
-    const uint32_t rank = ptx::cluster_rank();
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < NSLOT; ++i) ptx::mbar_init(&full[i], 1);
-        ptx::fence_mbar_init();
-    }
-    __syncthreads();
-    const uint64_t t0 = ptx::globaltimer_ns();
-    constexpr uint32_t piece = 16384 / CL;
-    const uint16_t mask = (uint16_t)((1u << CL) - 1);
-    const size_t cluster_id = blockIdx.x / CL;
-    bool ok = true;
-    for (int e = 0; e < epochs; ++e) {
-        if (threadIdx.x == 0)
-            for (int i = 0; i < NSLOT; ++i) ptx::mbar_expect_tx(&full[i], 16384);
-        __syncwarp();
-        ptx::cluster_arrive();
-        ptx::cluster_wait();
-        if (threadIdx.x == 0) {
-            for (int i = 0; i < NSLOT; ++i) {
-                const size_t chunk = (cluster_id * stride + (size_t)e * NSLOT + i) % nchunks;
-                if (CL == 1)
-                    asm volatile(
-                        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                            ptx::smem_u32(sm + i * 16384)),
-                        "l"(src + chunk * 16384), "r"(16384), "r"(ptx::smem_u32(&full[i]))
-                        : "memory");
-                else
-                    asm volatile(
-                        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], "
-                        "[%1], %2, [%3], %4;" ::"r"(ptx::smem_u32(sm + i * 16384 + rank * piece)),
-                        "l"(src + chunk * 16384 + rank * piece), "r"(piece), "r"(ptx::smem_u32(&full[i])), "h"(mask)
-                        : "memory");
-            }
-            for (int i = 0; i < NSLOT; ++i)
-                if (ok && !ptx::mbar_wait_bounded(&full[i], e & 1, LIMIT_NS)) {
-                    atomicExch(err, 11);
-                    ok = false;
-                }
-        }
-        __syncwarp();
-    }
-    if (threadIdx.x == 0) out[blockIdx.x] = ptx::globaltimer_ns() - t0;
-    __syncwarp();
-    ptx::cluster_arrive();
-    ptx::cluster_wait();
-}
-
 // One thread issues `nmma` tcgen05.mma of 128 x N x 16 (bf16, fp32 accumulate) back to back.
 // out[0] = cycles to issue them, out[1] = cycles until their commit has arrived.
 template <int N>
@@ -476,7 +412,6 @@ int main() {
 
     // Streaming intake per SM: one CTA per SM (120 KB of shared memory requested, 64 KB used).
     double stream_gbs[5], hbm_gbs = 0.0, deep_gbs[4] = {0.0, 0.0, 0.0, 0.0}, lsu_gbs[4] = {0.0, 0.0, 0.0, 0.0};
-    double mc_gbs[4] = {0.0, 0.0, 0.0, 0.0};
     const int nstream[5] = {1, 8, 38, 76, 152};
     {
         uint8_t* d_l2 = nullptr;
@@ -527,37 +462,6 @@ int main() {
         lsu_gbs[1] = run_lsu(sms, 0);
         lsu_gbs[2] = run_lsu(1, 1);
         lsu_gbs[3] = run_lsu(sms, 1);
-        // Multicast within clusters of 2 and 4 (and the same protocol in clusters of 1): bytes
-        // received per CTA, 192 KB an epoch.
-        auto run_mc = [&](auto kern, int cl, int ctas) -> double {
-            CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(ctas);
-            cfg.blockDim = dim3(32);
-            cfg.dynamicSmemBytes = smem;
-            cudaLaunchAttribute at;
-            at.id = cudaLaunchAttributeClusterDimension;
-            at.val.clusterDim.x = cl;
-            at.val.clusterDim.y = 1;
-            at.val.clusterDim.z = 1;
-            cfg.attrs = &at;
-            cfg.numAttrs = 1;
-            const int epochs = 170;   // 2040 chunks of 16 KB per CTA
-            for (int rep = 0; rep < 2; ++rep) {
-                if (cudaLaunchKernelEx(&cfg, kern, (const uint8_t*)d_l2, (int)(l2_bytes / 16384), 131, epochs, d_out,
-                                       d_err) != cudaSuccess)
-                    return -1.0;
-                if (cudaDeviceSynchronize() != cudaSuccess) return -1.0;
-            }
-            if (cudaMemcpy(t.data(), d_out, 8 * ctas, cudaMemcpyDeviceToHost) != cudaSuccess) return -1.0;
-            std::vector<double> gbs;
-            for (int c = 0; c < ctas; ++c) gbs.push_back((double)epochs * 12 * 16384 / (double)t[c]);
-            return median(gbs);
-        };
-        mc_gbs[0] = run_mc(k_stream_mc<1>, 1, 152);
-        mc_gbs[1] = run_mc(k_stream_mc<2>, 2, 152);
-        mc_gbs[2] = run_mc(k_stream_mc<4>, 4, 144);
-        mc_gbs[3] = run_mc(k_stream_mc<2>, 2, 2);
         CK(cudaFree(d_l2));
         CK(cudaFree(d_hbm));
     }
@@ -650,16 +554,14 @@ int main() {
            "\"cooperative_clusters_of_8\": %s, \"stream_gbs_per_cta\": {\"l2_1\": %.1f, \"l2_8\": %.1f, "
            "\"l2_38\": %.1f, \"l2_76\": %.1f, \"l2_152\": %.1f, \"hbm_152\": %.1f, \"l2_1_depth8\": %.1f, "
            "\"l2_152_depth8\": %.1f, \"l2_1_depth12\": %.1f, \"l2_152_depth12\": %.1f, \"l2_1_cp_async\": %.1f, "
-           "\"l2_152_cp_async\": %.1f, \"l2_1_bulk_plus_cp_async\": %.1f, \"l2_152_bulk_plus_cp_async\": %.1f, "
-           "\"l2_epochs_cluster1_x152\": %.1f, \"l2_multicast_cluster2_x76\": %.1f, "
-           "\"l2_multicast_cluster4_x36\": %.1f, \"l2_multicast_cluster2_x1\": %.1f}, \"errors\": %d}\n",
+           "\"l2_152_cp_async\": %.1f, \"l2_1_bulk_plus_cp_async\": %.1f, \"l2_152_bulk_plus_cp_async\": %.1f}, "
+           "\"errors\": %d}\n",
            sms, median(flag_us), *std::min_element(flag_us.begin(), flag_us.end()),
            *std::max_element(flag_us.begin(), flag_us.end()), median(data_us),
            *std::min_element(data_us.begin(), data_us.end()), *std::max_element(data_us.begin(), data_us.end()),
            barrier_us, reduce_us, sms * 32768, load_us, mma[0], mma[1], mma[2], mma[3], ring_us, coresident[0],
            coresident[1], coresident[2], coresident[3], coresident[4], coop8 ? "true" : "false", stream_gbs[0],
            stream_gbs[1], stream_gbs[2], stream_gbs[3], stream_gbs[4], hbm_gbs, deep_gbs[0], deep_gbs[1], deep_gbs[2],
-           deep_gbs[3], lsu_gbs[0], lsu_gbs[1], lsu_gbs[2], lsu_gbs[3], mc_gbs[0], mc_gbs[1], mc_gbs[2], mc_gbs[3],
-           errs);
+           deep_gbs[3], lsu_gbs[0], lsu_gbs[1], lsu_gbs[2], lsu_gbs[3], errs);
     return 0;
 }

@@ -1,5 +1,5 @@
-"""Checks, from the kernels' sources, of ordering and exit rules that no run can be made to break safely:
-a missing release or a copy still in flight at a kernel's exit corrupts memory only now and then."""
+"""Checks, from the kernels' sources, of rules that no run can be made to break safely: a missing release or a
+copy still in flight at a kernel's exit corrupts memory only now and then."""
 
 import os
 import re
@@ -66,3 +66,9 @@ def test_device_errors_are_reported_after_the_last_barrier():
         assert len(report) == 1, name
         last = text.rindex("*flag = ", 0, report[0])
         assert "__syncthreads();" in text[last:report[0]], name
+
+
+def test_no_source_uses_cluster_multicast():
+    # The library and its probe also belong to programs that run on several GPUs.
+    for name, text in _sources():
+        assert "multicast::cluster" not in text, name
