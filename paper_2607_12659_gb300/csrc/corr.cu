@@ -1384,19 +1384,7 @@ jpi_status linear(const jpi_corr_handle* h, cudaStream_t st, const float* x, int
                   const float* bias, const float* res, int ldr, float* y, int ldy, int rows, int in,
                   int out, bool gelu, int hs_items = 0) {
     if (rows <= 0 || out <= 0) return JPI_OK;
-    LinArgs a = {};
-    a.x = x;
-    a.ldx = ldx;
-    a.w = w;
-    a.bias = bias;
-    a.res = res;
-    a.ldr = ldr;
-    a.y = y;
-    a.ldy = ldy;
-    a.rows = rows;
-    a.in = in;
-    a.out = out;
-    a.gelu = gelu ? 1 : 0;
+    LinArgs a = lin_args(x, ldx, w, bias, res, ldr, y, ldy, rows, in, out, gelu);
     a.hs_items = hs_items;
     a.hs_heads = h->H;
     a.hs_dh = h->Dh;

@@ -416,8 +416,7 @@ struct PfGemmArgs {
     float alpha;
     int accumulate;       // Y += ... (fp32 Y only)
     int out_bf16;
-    int vec;              // Y and ldy allow 16-byte stores of 16 consecutive elements
-    void* Y;
+    void* Y;              // 16-byte aligned rows
     long long ldy;        // elements
     // Stream-K: piece p of a tile writes Y + p * ysplit (fp32, never accumulating).
     int stream;
@@ -642,27 +641,6 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pf_gemm(const __grid_constant
                         }
                     }
                     __syncwarp();
-                }
-            } else if (!a.vec) {
-                // Outputs that take no 16-byte access: a row per thread, element by element.
-                const int m = m0 + lane;
-                const int nc = a.geglu ? PG_TN / 2 : PG_TN, nlim = a.geglu ? a.nz : a.N;
-                for (int c0 = g * nc / 2; c0 < (g + 1) * nc / 2; c0 += 16) {
-                    uint32_t r[16], r2[16];
-                    ptx::tmem_ld_x16(acc + (uint32_t)c0, r);
-                    if (a.geglu) ptx::tmem_ld_x16(acc + (uint32_t)(PG_TN / 2 + c0), r2);
-                    ptx::tmem_ld_wait();
-                    const int n0 = tn * nc + c0;
-                    if (!ok || m >= a.M) continue;
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        if (n0 + i >= nlim) continue;
-                        const size_t o = (size_t)m * a.ldy + n0 + i;
-                        float v = a.alpha * __uint_as_float(r[i]);
-                        if (a.geglu) v = gelu_tanh_f(v) * (a.alpha * __uint_as_float(r2[i]));
-                        if (a.geglu || a.out_bf16) static_cast<__nv_bfloat16*>(Y)[o] = __float2bfloat16_rn(v);
-                        else static_cast<float*>(Y)[o] = a.accumulate ? static_cast<float*>(Y)[o] + v : v;
-                    }
                 }
             } else if (a.geglu || a.out_bf16) {
                 // 64 bf16 outputs of a row per pass (GeGLU: gate columns c.. and up columns 128 + c..).
@@ -893,6 +871,8 @@ jpi_status row_gemm(jpi_prefill_handle* h, cudaStream_t st, const __nv_bfloat16*
                     const __nv_bfloat16* Wm, long long ldw, bool w_const, void* Y, bool y_bf16, long long ldy, int M,
                     int N, int K, float alpha, bool accumulate, int grid, F&& more) {
     CUtensorMap wmap, xmap;
+    if (reinterpret_cast<uintptr_t>(Y) % 16 || ldy % (y_bf16 ? 8 : 4))   // never: widths are multiples of 8
+        return pfail(JPI_ERR_UNSUPPORTED, "a product's output rows are not 16-byte aligned");
     PF_TRY(make_map(Wm, N, K, ldw, PG_TN, &wmap));
     PF_TRY(make_map(X, M, K, ldx, PG_TM, &xmap));
     PfGemmArgs a = {};
@@ -904,7 +884,6 @@ jpi_status row_gemm(jpi_prefill_handle* h, cudaStream_t st, const __nv_bfloat16*
     a.out_bf16 = y_bf16 ? 1 : 0;
     a.Y = Y;
     a.ldy = ldy;
-    a.vec = (reinterpret_cast<uintptr_t>(Y) % 16 == 0 && ldy % (y_bf16 ? 8 : 4) == 0) ? 1 : 0;
     a.w_const = w_const ? 1 : 0;
     a.err = h->dev_err;
     more(a);

@@ -286,9 +286,9 @@ jpi_status launch_gemm(jpi_handle* h, const GemmPlan& pl, const CUtensorMap& wma
     return JPI_OK;
 }
 
-// Large-M variant: persistent CTAs over (weight tile, 128-row operand tile) units. The residual
-// kinds (few weight tiles, long K) may split each unit's K range over a cluster of S CTAs so that
-// the units fill the GPU: S is the one of 1, 2, 4, 8 with the fewest estimated K blocks per SM,
+// K split of the large-M residual projections: persistent CTAs over (weight tile, 128-token tile) units,
+// of which they have few with a long K; splitting each unit's K range over a cluster of S CTAs fills
+// the GPU: S is the one of 1, 2, 4, 8 with the fewest estimated K blocks per SM,
 // counting waves of S x units CTAs and, for each, what a unit's exchange adds in K blocks of
 // about 0.23 us. Fitted at pi0.5 sizes (one, two and three waves, us; O has 32 K blocks, down 64):
 // down S = 1 19.4; S = 2 12.7, 21.4; S = 4 10.3, 15.5, 21.9; O S = 1 12.5; S = 2 9.1, 13.7; S = 4 7.9,
@@ -302,9 +302,8 @@ int big_clusters(const jpi_handle* h, int S) {
     return h->big_clusters[i] > 0 ? h->big_clusters[i] : h->num_sms / S;
 }
 
-int big_split(const jpi_handle* h, int kind, int units, int nkb, long* cost_out = nullptr) {
+int big_split(const jpi_handle* h, int units, int nkb, long* cost_out = nullptr) {
     if (cost_out) *cost_out = 0;
-    if (kind != G_O && kind != G_DOWN) return 1;
     if (h->big_split > 0) return nkb % h->big_split == 0 ? h->big_split : 1;
     int best = 1;
     long best_cost = -1;
@@ -324,10 +323,10 @@ int big_split(const jpi_handle* h, int kind, int units, int nkb, long* cost_out 
 // Whether a residual projection takes the tokens-on-rows kernel (128 x 256 tiles, no K split): when
 // its waves of whole tiles, a k-block costing 5/4 of a 128 x 128 tile's (48 against 32 KB into the
 // SM, more of them in flight), cost less than the best split of the other kernel.
-bool resid_rows(const jpi_handle* h, int kind, int Mt, const GemmPlan& pl) {
+bool resid_rows(const jpi_handle* h, int Mt, const GemmPlan& pl) {
     if (h->resid_rows >= 0) return h->resid_rows != 0;
     long other = 0;
-    big_split(h, kind, pl.ntiles * ((Mt + BIG_NT - 1) / BIG_NT), pl.nkb, &other);
+    big_split(h, pl.ntiles * ((Mt + BIG_NT - 1) / BIG_NT), pl.nkb, &other);
     if (other == 0) return false;   // a fixed split
     const long tiles = (long)((pl.ntiles + 1) / 2) * ((Mt + 127) / 128);
     const long waves = (tiles + h->num_sms - 1) / h->num_sms;
@@ -407,19 +406,15 @@ jpi_status launch_big_s(jpi_handle* h, int units, const CUtensorMap& wmap, const
 template <int KIND>
 jpi_status launch_gemm_big(jpi_handle* h, const GemmPlan& pl, const CUtensorMap& wmap,
                            const CUtensorMap& xmap, const GemmArgs& a, cudaStream_t st) {
-    constexpr int TT = (KIND == G_QKV || KIND == G_GU) ? 2 * XS_TOKENS : BIG_NT;
-    const int units = pl.ntiles * std::max(1, (a.Mt + TT - 1) / TT);
+    const int units = pl.ntiles * std::max(1, (a.Mt + BIG_NT - 1) / BIG_NT);
     GemmArgs ab = a;
     ab.ntiles = pl.ntiles;
-    if constexpr (KIND == G_O || KIND == G_DOWN) {
-        switch (big_split(h, KIND, units, pl.nkb)) {
-            case 2: return launch_big_s<KIND, 2>(h, units, wmap, xmap, ab, st);
-            case 4: return launch_big_s<KIND, 4>(h, units, wmap, xmap, ab, st);
-            case 8: return launch_big_s<KIND, 8>(h, units, wmap, xmap, ab, st);
-            default: break;
-        }
+    switch (big_split(h, units, pl.nkb)) {
+        case 2: return launch_big_s<KIND, 2>(h, units, wmap, xmap, ab, st);
+        case 4: return launch_big_s<KIND, 4>(h, units, wmap, xmap, ab, st);
+        case 8: return launch_big_s<KIND, 8>(h, units, wmap, xmap, ab, st);
+        default: return launch_big_s<KIND, 1>(h, units, wmap, xmap, ab, st);
     }
-    return launch_big_s<KIND, 1>(h, units, wmap, xmap, ab, st);
 }
 
 GemmArgs base_args(jpi_handle* h, int B, int C, const GemmPlan& pl) {
@@ -657,7 +652,7 @@ jpi_status tc_launch_op(jpi_handle* h, int op, int l, int step, int B, int C, cu
         if (!big(KIND)) return launch_gemm<KIND>(h, pl, wm, h->xmaps[xi], a, st);
         if constexpr (KIND == G_QKV || KIND == G_GU) {
             if (rows_narrow(h, Mt, pl)) return launch_gemm_rows<KIND, 1>(h, pl, wm, h->xmaps_rows[xi], a, st);
-        } else if (!resid_rows(h, KIND, Mt, pl)) {
+        } else if (!resid_rows(h, Mt, pl)) {
             return launch_gemm_big<KIND>(h, pl, wm, h->xmaps_rows[xi], a, st);
         }
         return launch_gemm_rows<KIND, 2>(h, pl, wm, h->xmaps_rows[xi], a, st);
