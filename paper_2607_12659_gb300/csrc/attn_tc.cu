@@ -240,8 +240,8 @@ __global__ void __launch_bounds__(AT_THREADS) k_attn_tc(const __grid_constant__ 
         const uint32_t par = NBUF == 2 ? ((jb >> 1) & 1) : (jb & 1);
         bool landed = ptx::mbar_wait_bounded(&kvbar[bi], par, 200ull * 1000 * 1000);
         if (key0 == k_begin) landed = ptx::mbar_wait_bounded(qbar, 0, 200ull * 1000 * 1000) && landed;
-        if (!landed) {
-            if (tid == 0) atomicCAS(a.err, 0, (int)DEV_TIMEOUT_WEIGHTS);
+        if (!landed && tid == 0) {
+            atomicCAS(a.err, 0, (int)DEV_TIMEOUT_WEIGHTS);
             // Nothing may land in this CTA's shared memory once it has exited.
             (void)ptx::mbar_wait_bounded(&kvbar[bi], par, 200ull * 1000 * 1000);
             (void)ptx::mbar_wait_bounded(qbar, 0, 200ull * 1000 * 1000);

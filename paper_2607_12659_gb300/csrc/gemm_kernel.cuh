@@ -165,9 +165,6 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_tc_gemm(const __grid_consta
             if (ok_in) ok_in = ptx::mbar_wait_bounded(&bars[0], 0, WAIT_LIMIT_NS);
             if (!ok_in) {
                 *flag = DEV_TIMEOUT_WEIGHTS;
-                // Nothing may land in this CTA's shared memory once it has exited.
-                (void)ptx::mbar_wait_bounded(&bars[1], 0, WAIT_LIMIT_NS);
-                (void)ptx::mbar_wait_bounded(&bars[0], 0, WAIT_LIMIT_NS);
             } else {
                 ptx::tc_fence_after();
                 const uint64_t wd = ptx::desc_sw128(ptx::smem_u32(wsm)), xd = ptx::desc_sw128(ptx::smem_u32(xsm));
@@ -418,5 +415,10 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_tc_gemm(const __grid_consta
     // Pairs the arrival after the receive wait.
     ptx::cluster_wait();
 
-    if (*flag != 0) set_device_error(a.err, *flag);   // by any thread that saw it
+    if (*flag != 0) {   // by any thread that saw it
+        set_device_error(a.err, *flag);
+        // After a wait that gave up: nothing may land in this CTA's shared memory once it has exited.
+        (void)ptx::mbar_wait_bounded(&bars[0], 0, WAIT_LIMIT_NS);
+        (void)ptx::mbar_wait_bounded(&bars[1], 0, WAIT_LIMIT_NS);
+    }
 }

@@ -51,10 +51,10 @@ def test_attention_loaders_wait_for_their_last_copies():
 def test_single_shot_loads_are_waited_for_again_after_a_wait_gave_up():
     # The K-split projection's two operand barriers, and the split-KV attention's key block and queries.
     gemm = _source("gemm_kernel.cuh")
-    gave_up = gemm[gemm.index("if (!ok_in) {"):gemm.index("const uint64_t wd =")]
+    gave_up = gemm[gemm.rindex("if (*flag != 0) {"):]
     assert "mbar_wait_bounded(&bars[0]," in gave_up and "mbar_wait_bounded(&bars[1]," in gave_up
     attn = _source("attn_tc.cu")
-    gave_up = attn[attn.index("if (!landed) {"):attn.index("const uint32_t kbuf_u")]
+    gave_up = attn[attn.index("if (!landed && tid == 0) {"):attn.index("const uint32_t kbuf_u")]
     assert "mbar_wait_bounded(&kvbar[bi]," in gave_up and "mbar_wait_bounded(qbar," in gave_up
 
 
