@@ -975,8 +975,11 @@ __device__ __forceinline__ float2 load2<__nv_bfloat16>(const __nv_bfloat16* p) {
 
 // PAIR: dv even and hv aligned to two elements, so a thread's two columns load together; else
 // each value on its own (and a last odd column alone).
+// At most 128 registers: with the loads of 16 tokens in flight the compiler takes 154 at RH = 32 and a second
+// CTA no longer fits an SM (compress, us, unbounded and bounded: 1 request x 816 tokens 53 and 48, 8 x 1500
+// 359 and 256, 32 x 1500 1440 and 963).
 template <typename THV, int RH, bool PAIR>
-__global__ void __launch_bounds__(256) k_corr_wsum(const float* __restrict__ p, const THV* __restrict__ hv,
+__global__ void __launch_bounds__(256, 2) k_corr_wsum(const float* __restrict__ p, const THV* __restrict__ hv,
                                                    float* __restrict__ part, int M, int T, int dv) {
     // Launched with programmatic dependent launch: wait for the previous kernel's results, then
     // let the next kernel's CTAs be scheduled (they wait in turn).
@@ -1199,7 +1202,7 @@ struct jpi_corr_handle {
     float *xj = nullptr, *xf = nullptr, *u = nullptr, *qkv = nullptr, *o = nullptr;   // [B T'] rows
     float* hid = nullptr;                                                 // [B T'][F]
     float *sc = nullptr, *gs = nullptr;                                   // [B][M][Tm], [B][M][dv]
-    float *scp = nullptr, *gsp = nullptr;   // partials: [B][dv / 256][M][Tm], [B][Tm / 64][M][dv]
+    float *scp = nullptr, *gsp = nullptr;   // partials: [B][dv / CORR_KCHUNK][M][Tm], [B][Tm / CORR_TCHUNK][M][dv], rounded up
     float* conf_scratch = nullptr;                                        // [B]
 
 };
