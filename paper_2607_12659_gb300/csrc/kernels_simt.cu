@@ -948,7 +948,10 @@ __device__ __forceinline__ void final_prefetch(const FinalArgs& a, float4 (&w0)[
             w0[q][s] = rows_load<true>(a.Wout + (size_t)min(4 * warp + s, a.A - 1) * a.W, 128 * q, lane, a.W);
 }
 
-__global__ void __launch_bounds__(FIN_THREADS) k_final(const FinalArgs a) {
+// One row per CTA. PRE: steps of W_out fetched before the dependency wait; CTAS: CTAs that fit an SM
+// (four steps take 162 registers, two 128).
+template <int PRE, int CTAS>
+__global__ void __launch_bounds__(FIN_THREADS, CTAS) k_final(const FinalArgs a) {
     extern __shared__ __align__(16) float us[];        // [W]
     __shared__ float scratch[32];
     const int tid = threadIdx.x, W = a.W;
@@ -962,7 +965,7 @@ __global__ void __launch_bounds__(FIN_THREADS) k_final(const FinalArgs a) {
         sg[q] = k < W ? a.sigma[k] : 0.f;
         bt[q] = k < W ? a.beta[k] : 0.f;
     }
-    float4 w0[4][4];
+    float4 w0[PRE][4];
     final_prefetch(a, w0);
     // Launched with programmatic dependent launch: h comes from the last layer's down projection.
     ptx::grid_dep_wait();
@@ -1514,15 +1517,20 @@ jpi_status launch_final(jpi_handle* h, int step, int B, int C, float delta, floa
     a.A = h->A;
     a.eps = h->cfg.rms_eps;
     a.delta = delta;
-    // One row per CTA up to two CTAs per SM, then 4, then 8 rows (while they fit the shared memory).
+    // One row per CTA while the CTAs run at once, at one or two per SM, then 4, then 8 rows (while they fit
+    // the shared memory). Measured at W = 1024, us: 150 rows 3.6 (one CTA per SM), 4.0 (two), 6.3 (4 rows); 160:
+    // 6.0, 4.1, 6.3; 300: 6.5, 4.1, 6.3; 350: 8.5, 7.4, 6.4 and 8.0 (8 rows); 1200: 7.3 (4 rows), 8.2 (8
+    // rows); 1250: 12.7, 9.7.
     const int fr = rows <= 2 * h->num_sms ? 1 : rows <= 8 * h->num_sms ? 4 : 8;
     const size_t row = sizeof(float) * (size_t)W;
     if (fr == 8 && 8 * row <= FIN_SMEM_MAX)
         launch_pdl(h, dim3((rows + 7) / 8), dim3(FIN_THREADS), 8 * row, st, k_final_rows<8>, a);
     else if (fr >= 4 && 4 * row <= FIN_SMEM_MAX)
         launch_pdl(h, dim3((rows + 3) / 4), dim3(FIN_THREADS), 4 * row, st, k_final_rows<4>, a);
+    else if (rows <= h->num_sms)
+        launch_pdl(h, dim3(rows), dim3(FIN_THREADS), row, st, k_final<4, 1>, a);
     else
-        launch_pdl(h, dim3(rows), dim3(FIN_THREADS), row, st, k_final, a);
+        launch_pdl(h, dim3(rows), dim3(FIN_THREADS), row, st, k_final<2, 2>, a);
     return check_launch("final norm + Euler");
 }
 

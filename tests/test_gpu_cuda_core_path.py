@@ -64,3 +64,21 @@ def test_correction_items_fp32():
     ex.close()
     ref = oracle.denoise_batch(r["noise"], r["state"], 2, r["prefix_k"], r["prefix_v"], w, cfg, corr=items)
     assert np.abs(got - ref).max() <= 2e-5
+
+
+# The final norm and output product at every number of rows a block takes (one with one or two blocks on an
+# SM, four, eight), at widths of less than and more than the steps fetched ahead: a request's bits do not
+# depend on it.
+@pytest.mark.parametrize("W", [256, 1120])
+def test_final_rows_same_bits_in_every_block_shape(monkeypatch, W):
+    monkeypatch.setenv("JPI_BATCH_INVARIANT", "1")
+    cfg = TINY.with_(n_layers=1, width=W, n_heads=1, head_dim=32, mlp_dim=64)
+    w, P, C = make_weights(cfg, 3, mod_bias_std=0.3), 3, 50
+    ex = make_expert(cfg, w, max_batch=26, max_prefix=P, max_chunk=C, max_steps=1)
+    got = {B: gpu_denoise(ex, cfg, make_requests(cfg, 5, B, P, C), 1) for B in (1, 3, 4, 6, 7, 26)}
+    ex.close()
+    for B in (3, 4, 6, 7):
+        assert np.array_equal(got[B], got[26][:B]), B
+    assert np.array_equal(got[1], got[26][:1])
+    ref = oracle_denoise(cfg, w, make_requests(cfg, 5, 26, P, C), 1, (0, 25))
+    assert np.abs(got[26][[0, 25]] - ref).max() <= 2e-5
