@@ -1475,9 +1475,11 @@ jpi_status launch_embed(jpi_handle* h, int step, int B, int C, const float* x, c
     a.W = h->W;
     a.Sd = h->Sd;
     a.A = h->A;
-    // About two blocks per SM (a small batch keeps one token per block, the shortest chain), at most
-    // EMB_MAX_TPB tokens each.
-    const long long want = 2ll * h->num_sms;
+    // As many blocks as run at once, three to an SM (168 registers a thread; a small batch keeps one token
+    // per block, the shortest chain), at most EMB_MAX_TPB tokens each. Measured for two, three and four to an SM,
+    // us: W = 1024 408 tokens 4.0, 3.7, 3.7; 816: 6.1, 4.9, 7.3; 1632: 9.5, 7.6, 11.6; W = 256 408
+    // tokens 2.7, 2.3, 2.3; 1632: 4.3, 3.5, 5.4.
+    const long long want = 3ll * h->num_sms;
     const long long tpb = ((long long)B * a.S * slices + want - 1) / want;
     a.tpb = (int)(tpb < 1 ? 1 : tpb > EMB_MAX_TPB ? EMB_MAX_TPB : tpb);
     a.action_groups = (B * C + a.tpb - 1) / a.tpb;
