@@ -27,7 +27,7 @@
 // index mod 8, which keeps both the TMEM write-out (one row per lane) and the reduction reads
 // free of bank conflicts without padding.
 
-template <int KIND>
+template <int KIND, int TW>
 __global__ void __launch_bounds__(GEMM_THREADS, 2) k_tc_gemm(const __grid_constant__ CUtensorMap wmap,
                                                           const __grid_constant__ CUtensorMap xmap,
                                                           const __grid_constant__ GemmArgs a) {
@@ -58,10 +58,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_tc_gemm(const __grid_consta
     const int kb0 = rank * a.kpb;
     const int npairs = 64 / a.splits, p0 = rank * npairs;
     // Epilogue item = (TW columns, owned pair) with the pair fastest, so that consecutive lanes
-    // write consecutive output features of one token. Two columns for the residual kinds: at their
-    // K split of 8 that is an item for every thread (four left half of them idle, and each item
-    // has eight residual values to fetch and update).
-    constexpr int TW = RESID ? 2 : 4;
+    // write consecutive output features of one token (TW: see tw_of in the launcher).
     const int nitems = npairs * (NT / TW);
 
     if (warp == 1) {

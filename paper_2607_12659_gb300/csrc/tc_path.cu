@@ -254,6 +254,25 @@ jpi_status pack(const float* tmp, __nv_bfloat16* dst, const int* dmap, int rows,
     return JPI_OK;
 }
 
+// Columns per epilogue item of the K-split kernel: the residual kinds take two at a split of 8 or more,
+// where that is an item for every thread (four columns leave half of them idle, and each item has eight
+// residual values to fetch and update), else four, so that a thread has few items. Measured: pi0.5 sizes, split 8,
+// denoise at batch 1 5.09 ms with four columns, 4.90 with two (and the split-KV attention's whole-block
+// copies); O of one head of 128 at W = 1024, split 1, 51 tokens 6.3 us with four, 7.4 with two.
+int tw_of(int kind, const GemmPlan& pl) {
+    return (kind == G_O || kind == G_DOWN) && pl.splits >= 8 ? 2 : 4;
+}
+using GemmFn = void (*)(CUtensorMap, CUtensorMap, GemmArgs);
+GemmFn gemm_fn(int kind, const GemmPlan& pl) {
+    const bool two = tw_of(kind, pl) == 2;
+    switch (kind) {
+        case G_QKV: return k_tc_gemm<G_QKV, 4>;
+        case G_GU: return k_tc_gemm<G_GU, 4>;
+        case G_O: return two ? k_tc_gemm<G_O, 2> : k_tc_gemm<G_O, 4>;
+        default: return two ? k_tc_gemm<G_DOWN, 2> : k_tc_gemm<G_DOWN, 4>;
+    }
+}
+
 template <int KIND>
 jpi_status launch_gemm(jpi_handle* h, const GemmPlan& pl, const CUtensorMap& wmap,
                        const CUtensorMap& xmap, const GemmArgs& a, cudaStream_t st) {
@@ -278,7 +297,7 @@ jpi_status launch_gemm(jpi_handle* h, const GemmPlan& pl, const CUtensorMap& wma
     }
     cfg.attrs = attrs;
     cfg.numAttrs = n;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_tc_gemm<KIND>, wmap, xmap, a);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_fn(KIND, pl), wmap, xmap, a);
     if (e != cudaSuccess) {
         set_error("tensor-core GEMM launch failed: %s", cudaGetErrorString(e));
         return JPI_ERR_CUDA;
@@ -505,8 +524,8 @@ jpi_status tc_prepare(jpi_handle* h) {
     JPI_TRY(attn_t5_prepare(h));
 
     int max_cluster = 16;
-    auto kernels = {k_tc_gemm<G_QKV>, k_tc_gemm<G_O>, k_tc_gemm<G_GU>, k_tc_gemm<G_DOWN>};
-    for (auto k : kernels) {
+    for (GemmFn k : {k_tc_gemm<G_QKV, 4>, k_tc_gemm<G_O, 2>, k_tc_gemm<G_O, 4>, k_tc_gemm<G_GU, 4>, k_tc_gemm<G_DOWN, 2>,
+                     k_tc_gemm<G_DOWN, 4>}) {
         if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
             cudaGetLastError();
             max_cluster = 8;
@@ -584,10 +603,7 @@ jpi_status tc_prepare(jpi_handle* h) {
         cfg.attrs = &at;
         cfg.numAttrs = 1;
         int nclusters = 0;
-        const void* fn = g == 0 ? (const void*)k_tc_gemm<G_QKV>
-                       : g == 1 ? (const void*)k_tc_gemm<G_O>
-                       : g == 2 ? (const void*)k_tc_gemm<G_GU>
-                                : (const void*)k_tc_gemm<G_DOWN>;
+        const void* fn = (const void*)gemm_fn(g, pl);
         if (cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) != cudaSuccess || nclusters < 1) {
             cudaGetLastError();
             set_error("a cluster of %d CTAs with %zu bytes of shared memory does not fit", pl.splits, pl.smem);
