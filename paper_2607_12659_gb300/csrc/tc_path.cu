@@ -615,10 +615,12 @@ jpi_status tc_prepare(jpi_handle* h) {
         // QKV (153 tokens: 6.6 us against 7.3; 204: 10.7 against 7.4), 64 for gate/up (102: 11.1 against
         // 6.9) and 65 for down (102: 10.7 against 9.4). O would gain up to 256 tokens (255: 7.0 against
         // 8.4) but takes over at 128 at the latest: the K-split kernel's partial sums are fp16, the
-        // large-M kernels' fp32. JPI_BIG_GEMM_MIN_TOKENS sets one threshold for all four.
+        // large-M kernels' fp32. QKV takes over at 512 at the latest for the same reason, which only an
+        // expert of few heads meets (W = 2048, two heads of 128, 500 tokens: 7.4 us against 10.0; W = 1024, one
+        // head: 5.8 against 7.1). JPI_BIG_GEMM_MIN_TOKENS sets one threshold for all four.
         const int resident = 2 * (pl.smem + 1024) <= 228 * 1024 ? 2 * sms : nclusters * pl.splits;
         const int tt = g == G_QKV || g == G_GU ? XS_TOKENS : NT;
-        h->big_min_tokens[g] = std::min(std::max(1, resident / pl.ctas) * tt + 1, g == G_QKV ? 400 : 128);
+        h->big_min_tokens[g] = std::min(std::max(1, resident / pl.ctas) * tt + 1, g == G_QKV ? 512 : 128);
         if (const char* big_env = std::getenv("JPI_BIG_GEMM_MIN_TOKENS")) h->big_min_tokens[g] = std::atoi(big_env);
     }
     h->tmaps.resize((size_t)4 * h->L);
