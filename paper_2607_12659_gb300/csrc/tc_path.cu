@@ -307,12 +307,16 @@ jpi_status launch_gemm(jpi_handle* h, const GemmPlan& pl, const CUtensorMap& wma
 
 // K split of the large-M residual projections: persistent CTAs over (weight tile, 128-token tile) units,
 // of which they have few with a long K; splitting each unit's K range over a cluster of S CTAs fills
-// the GPU: S is the one of 1, 2, 4, 8 with the fewest estimated K blocks per SM,
-// counting waves of S x units CTAs and, for each, what a unit's exchange adds in K blocks of
-// about 0.23 us. Fitted at pi0.5 sizes (one, two and three waves, us; O has 32 K blocks, down 64):
-// down S = 1 19.4; S = 2 12.7, 21.4; S = 4 10.3, 15.5, 21.9; O S = 1 12.5; S = 2 9.1, 13.7; S = 4 7.9,
-// 11.8, 15.7; S = 8 9.5 (two), 13.8, 18.5 (four).
-constexpr int BIG_SPLIT_COST[9] = {0, 0, 5, 0, 9, 0, 0, 0, 14};
+// the GPU. S is the one of 1, 2, 4, 8 with the least estimated time: `first` + `kb` us a k-block for the first
+// wave of units, and for each further one, which overlaps with it, the longer of `next` (its exchange and
+// epilogue) and `next_kb` a k-block. Fitted to 336 shapes (128 to 3264 tokens, 256 to 2048 output features, K of
+// 128 to 4096): what it chooses takes 0.2% longer than the best choice on average, 5% at most. Measured,
+// S = 1, 2, 4, 8, us: 1024 features, 408 tokens, K = 512 7.6, 6.1, 6.2, 13.2, K = 2048 14.4, 9.4, 8.5, 14.5, K = 4096
+// 23.1, 13.5, 11.0, 16.5; 816 tokens, K = 2048 14.4, 9.6, 12.8, 20.1; 2040 tokens, K = 2048 14.6, 15.1, 22.3, 42.5.
+struct BigCost {
+    double first, kb, next, next_kb;
+};
+constexpr BigCost BIG_COST[4] = {{5.7, .27, 4.4, .29}, {5.2, .26, 4.0, .33}, {5.05, .32, 4.0, .42}, {5.5, .42, 3.9, .50}};
 
 // Clusters of S large-M CTAs that can run at once (one CTA per SM; clusters of 8 leave some SMs
 // of each GPC idle), from the occupancy query at prepare time.
@@ -321,35 +325,40 @@ int big_clusters(const jpi_handle* h, int S) {
     return h->big_clusters[i] > 0 ? h->big_clusters[i] : h->num_sms / S;
 }
 
-int big_split(const jpi_handle* h, int units, int nkb, long* cost_out = nullptr) {
-    if (cost_out) *cost_out = 0;
+int big_split(const jpi_handle* h, int units, int nkb, double* us_out = nullptr) {
+    if (us_out) *us_out = 0.;
     if (h->big_split > 0) return nkb % h->big_split == 0 ? h->big_split : 1;
     int best = 1;
-    long best_cost = -1;
-    for (int S = 1; S <= 8; S *= 2) {
-        if (nkb % S || nkb / S < 2) continue;
+    double best_us = -1.;
+    for (int i = 0; i < 4; ++i) {
+        const int S = 1 << i;
+        if (nkb % S) continue;
+        const BigCost& c = BIG_COST[i];
+        const double kb = nkb / S;
         const long waves = (units + big_clusters(h, S) - 1) / big_clusters(h, S);
-        const long cost = waves * (nkb / S + BIG_SPLIT_COST[S]);
-        if (best_cost < 0 || cost < best_cost) {
-            best_cost = cost;
+        const double us = c.first + c.kb * kb + (double)(waves - 1) * std::max(c.next, c.next_kb * kb);
+        if (best_us < 0. || us < best_us) {
+            best_us = us;
             best = S;
         }
     }
-    if (cost_out) *cost_out = best_cost;
+    if (us_out) *us_out = best_us;
     return best;
 }
 
-// Whether a residual projection takes the tokens-on-rows kernel (128 x 256 tiles, no K split): when
-// its waves of whole tiles, a k-block costing 5/4 of a 128 x 128 tile's (48 against 32 KB into the
-// SM, more of them in flight), cost less than the best split of the other kernel.
+// Whether a residual projection takes the tokens-on-rows kernel (128 x 256 tiles, no K split): when its
+// estimate (the same fit: 8.6 us + 0.275 a k-block, a further wave 6.5 + 0.22) is less than the best
+// split's of the other kernel. Measured, this kernel and the best split, us: 1024 features, 3264 tokens, K = 2048
+// 18.5 and 20.4, K = 4096 27.7 and 32.6; 2448 tokens, K = 1024 13.6 and 13.8; 2048 features, 3264 tokens, K = 512
+// 19.9 and 17.8.
 bool resid_rows(const jpi_handle* h, int Mt, const GemmPlan& pl) {
     if (h->resid_rows >= 0) return h->resid_rows != 0;
-    long other = 0;
+    double other = 0.;
     big_split(h, pl.ntiles * ((Mt + BIG_NT - 1) / BIG_NT), pl.nkb, &other);
-    if (other == 0) return false;   // a fixed split
+    if (other == 0.) return false;   // a fixed split
     const long tiles = (long)((pl.ntiles + 1) / 2) * ((Mt + 127) / 128);
     const long waves = (tiles + h->num_sms - 1) / h->num_sms;
-    return waves * pl.nkb * 5 < other * 4;
+    return 8.6 + .275 * pl.nkb + (double)(waves - 1) * (6.5 + .22 * pl.nkb) < other;
 }
 
 // Whether a norm-fed projection takes 128 x 128 tiles instead of 128 x 256 ones: a wave of the narrow
