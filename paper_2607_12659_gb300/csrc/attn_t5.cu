@@ -122,13 +122,17 @@ jpi_status launch_t5(jpi_handle* h, int l, int B, int C, cudaStream_t st) {
         return JPI_OK;
     };
     // Requests past the last whole wave go in a launch of their own where that splits them over the
-    // keys: another wave of whole rows leaves most SMs idle. Four ways, or two from 16 key blocks (40
-    // requests, prefix 1333: 44.7 -> 38.5 us, prefix 816: 32.5 -> 29.7; two ways, 48 requests, 1333:
-    // 45.0 -> 42.6, 57 requests, 816, 14 blocks: 33.6 and 33.9).
-    const int wave = h->num_sms / rblocks, rest = wave > 0 ? B % wave : 0;
-    if (B > wave && rest > 0) {
+    // keys: another wave of whole rows leaves most SMs idle. Four ways after one or two whole waves from 8 key
+    // blocks, two ways after one from 16: with fewer blocks the exchange outweighs the keys it saves, and after more
+    // waves the blocks of a single launch no longer end together. One launch and two, us, D = 256: 42 requests,
+    // 3, 6, 8, 22 key blocks 15.8 and 19.1, 20.9 and 21.2, 23.8 and 22.6, 43.6 and 37.3; 78 requests (two waves), 7,
+    // 8, 22 blocks 33.2 and 33.7, 35.4 and 34.8, 64.0 and 60.3; 154 (four), 22 blocks 104.6 and 106.2. Two ways:
+    // 48 requests, 8, 12, 22 blocks 24.2 and 24.7, 29.9 and 29.0, 44.1 and 41.2; 86, 22 blocks 64.8 and
+    // 64.2 (D = 128: 58.3 and 60.3).
+    const int wave = h->num_sms / rblocks, whole = wave > 0 ? B / wave : 0, rest = wave > 0 ? B % wave : 0;
+    if (whole >= 1 && rest > 0) {
         const int s = splits_of(rest);
-        if (s > 2 || (s == 2 && nb_all >= 16)) {
+        if ((s > 2 && whole <= 2 && nb_all >= 8) || (s == 2 && whole == 1 && nb_all >= 16)) {
             JPI_TRY(launch(0, B - rest));
             return launch(B - rest, rest);
         }

@@ -19,8 +19,12 @@ ONE = (ExpertConfig(n_layers=1, width=128, n_heads=2, head_dim=128, mlp_dim=128,
                     time_dim=64, precision="bf16"), 5, 1)
 
 
+# Below 8 key blocks (P < 398 and 443) and at a rest of 30 there is one launch; from there on four splits, two at
+# a rest of 12 from 16 blocks; 40 is a rest of 2 past two whole waves, 78 past three (one launch).
 @pytest.mark.parametrize("shape,rest,P", [(FOUR, 1, 300), (FOUR, 9, 230), (FOUR, 12, 1000), (FOUR, 30, 300),
-                                          (ONE, 1, 300), (ONE, 37, 250)])
+                                          (ONE, 1, 300), (ONE, 37, 250), (FOUR, 1, 397), (FOUR, 1, 398),
+                                          (FOUR, 9, 500), (FOUR, 12, 909), (FOUR, 40, 520), (FOUR, 78, 450),
+                                          (ONE, 1, 510), (ONE, 37, 630)])
 def test_last_requests_split_over_the_keys(shape, rest, P):
     lib()
     cfg, C, rblocks = shape
