@@ -610,7 +610,7 @@ __global__ void k_rms_mod(const float* __restrict__ hres, const float* __restric
 }
 
 // ---------------------------------------------------------------------------------------------
-// Products with many tokens (see rows_fit below): Y[m][n] = sum_k X[m][k] W[n][k] with three epilogues:
+// Products of many tokens (see rows_fit below): Y[m][n] = sum_k X[m][k] W[n][k] with three epilogues:
 //   STORE  Y[m][n] = y
 //   RESID  Y[m][n] += gamma[n] * y            (gated residual update of h)
 //   GEGLU  Z[m][n] = gelu_tanh(y_gate) * y_up (second weight matrix W2 = up)
@@ -1167,12 +1167,14 @@ inline int grid_for(long long n, int block, int cap = 4096) {
     return (int)(g < 1 ? 1 : (g > cap ? cap : g));
 }
 
-// The product kernel of one kind: KS warps share a slot group's K range while each keeps a step of
-// 128; 16-byte (8-byte for bf16) loads when K is a multiple of 4.
+// Warps that share a slot group's K range of nst steps of 128: each keeps one at least.
+int rows_ksplit(int nst) { return nst >= 4 ? 4 : nst >= 2 ? 2 : 1; }
+
+// The product kernel of one kind; 16-byte (8-byte for bf16) loads when K is a multiple of 4.
 template <typename T, int KIND>
 jpi_status launch_rows_gemm(jpi_handle* h, const RowsArgs& a, cudaStream_t st) {
     const int groups = KIND == RK_RESID ? (a.N + 3) / 4 : KIND == RK_GEGLU ? (a.N + 1) / 2 : a.N / 4;
-    const int nst = (a.K + 127) / 128, ks = nst >= 4 ? 4 : nst >= 2 ? 2 : 1;
+    const int ks = rows_ksplit((a.K + 127) / 128);
     const int cw = ROWS_WARPS / ks;
     const dim3 grid((groups + cw - 1) / cw, (a.M + ROWS_M - 1) / ROWS_M), block(32 * ROWS_WARPS);
     const bool vec = a.K % 4 == 0;
@@ -1216,16 +1218,27 @@ jpi_status op_simt(jpi_handle* h, int op, int l, int step, int B, int C, cudaStr
         set_error("layer %d has no CUDA-core weights", l);
         return JPI_ERR_INVALID_ARG;
     }
-    // Products: 16-token rows kernel while 64 x 64 tiles of the output would leave the GPU about
-    // one tile per SM or less, else those tiles, with the norm and rotary passes of their own.
-    // Measured, rows against tiles (fp32, us): QKV (2560 x 1024) 33 / 88 at 51 tokens, 109 / 122 at
-    // 204 (160 tiles), 211 / 125 at 408 (280); gate/up (4096 x 1024) 164 / 215 at 102 (128), 312 / 246
-    // at 204 (256); down (1024 x 4096) 212 / 286 at 408 (112), 842 / 623 at 1632 (416).
+    // Products: the kernel with the smaller estimate, in us (fp32 and bf16, 792 shapes of 16 to 3264 tokens, K and
+    // N of 32 to 4096; the choice takes 0.3% longer than the better kernel on average). The rows kernel is
+    // bound by its warps' 128-wide steps and the reduction after them, the 64 x 64 tiles by their chain along K, with
+    // the norm and rotary launches before and after. Rows against tiles, us: pi0.5's QKV (2560 x 1024, fp32) 33 and 88
+    // at 51 tokens, 109 and 122 at 204, 211 and 125 at 408; down (1024 x 4096) 212 and 286 at 408; bf16, QKV of 384 x
+    // 160 16 and 24 at 306, 50 and 25 at 1224; gate/up of 1030 x 160 33 and 41 at 153, 117 and 45 at 612.
     // The two add a product's terms in different orders: in the batch-invariant mode a launch takes what
     // one request alone would (Mi tokens).
     const int Mi = h->batch_invariant ? S : Mt;
-    auto rows_fit = [&](int N) {
-        return (long long)((N + GB_N - 1) / GB_N) * ((Mi + GB_M - 1) / GB_M) * 4 <= 5ll * h->num_sms;
+    auto rows_fit = [&](int kind, int N, int K) {
+        const bool norm = kind != RK_RESID, glu = kind == RK_GEGLU;
+        const long long blocks = (long long)((N + GB_N - 1) / GB_N) * ((Mi + GB_M - 1) / GB_M);
+        const double deep = (double)((blocks + h->num_sms - 1) / h->num_sms - 1);   // tiles an SM walks past the first
+        const double chain = (K + GB_K - 1) / GB_K * (glu ? 3.16 + 1.12 * deep : 1.18 + .70 * deep);
+        const double tiles = 5.1 + (glu ? 2.7 : norm ? 7.1 : 0.) + (norm ? .00106 * Mi : 0.) + chain;
+        const int nst = (K + 127) / 128, ks = rows_ksplit(nst);
+        const double warps = (double)((glu ? 2 * N : N) + 3) / 4. * ((Mi + ROWS_M - 1) / ROWS_M);
+        const double steps = warps * (nst + .95 * (ks > 1 ? ks : 2)) / h->num_sms;
+        const double rows = 2.6 + (norm ? .9 : 0.) + 1.1 * ((nst + ks - 1) / ks) +
+                            .139 * steps * (sizeof(T) == 2 ? 1.43 : 1.) * (norm ? 1.24 : 1.);
+        return rows < tiles;
     };
     const int F = h->F, HD = h->HD, mtiles = (Mt + GB_M - 1) / GB_M;
     const float eps = h->cfg.rms_eps;
@@ -1245,7 +1258,7 @@ jpi_status op_simt(jpi_handle* h, int op, int l, int step, int B, int C, cudaStr
     a.kv_rows = h->kv_rows;
     switch (op) {
         case 2:
-            if (!rows_fit(h->QKV)) {
+            if (!rows_fit(RK_QKV, h->QKV, W)) {
                 k_rms_mod<T><<<Mt, blk, 0, st>>>(h->h, ms, ms + W, act, W, W, eps);
                 k_gemm_simt<T, T, EPI_STORE><<<dim3((h->QKV + GB_N - 1) / GB_N, mtiles), blk, 0, st>>>(
                     act, W, (const T*)lwp->wqkv, nullptr, Mt, h->QKV, W, h->qkv, h->QKV, nullptr, nullptr, 0);
@@ -1269,7 +1282,7 @@ jpi_status op_simt(jpi_handle* h, int op, int l, int step, int B, int C, cudaStr
                         : launch_attn_rows<T, 1>(h, (const T*)h->q, kst, vst, (T*)h->o, Mt, S, st);
         }
         case 4:
-            if (!rows_fit(W)) {
+            if (!rows_fit(RK_RESID, W, HD)) {
                 k_gemm_simt<T, T, EPI_RESID><<<dim3((W + GB_N - 1) / GB_N, mtiles), blk, 0, st>>>(
                     (const T*)h->o, HD, (const T*)lwp->wo, nullptr, Mt, W, HD, h->h, W, ms + 2 * W, nullptr, 0);
                 return check_launch("layer op (CUDA cores)");
@@ -1280,7 +1293,7 @@ jpi_status op_simt(jpi_handle* h, int op, int l, int step, int B, int C, cudaStr
             a.gamma = ms + 2 * W;
             return launch_rows_gemm<T, RK_RESID>(h, a, st);
         case 5:
-            if (!rows_fit(F)) {
+            if (!rows_fit(RK_GEGLU, F, W)) {
                 k_rms_mod<T><<<Mt, blk, 0, st>>>(h->h, ms + 3 * W, ms + 4 * W, act, W, W, eps);
                 k_gemm_simt<T, T, EPI_GEGLU><<<dim3((F + GB_N - 1) / GB_N, mtiles), blk, 0, st>>>(
                     act, W, (const T*)lwp->wg, (const T*)lwp->wu, Mt, F, W, nullptr, 0, nullptr, (T*)h->z, F);
@@ -1294,7 +1307,7 @@ jpi_status op_simt(jpi_handle* h, int op, int l, int step, int B, int C, cudaStr
             a.z = h->z;
             return launch_rows_gemm<T, RK_GEGLU>(h, a, st);
         case 6:
-            if (!rows_fit(W)) {
+            if (!rows_fit(RK_RESID, W, F)) {
                 k_gemm_simt<T, T, EPI_RESID><<<dim3((W + GB_N - 1) / GB_N, mtiles), blk, 0, st>>>(
                     (const T*)h->z, F, (const T*)lwp->wd, nullptr, Mt, W, F, h->h, W, ms + 5 * W, nullptr, 0);
                 return check_launch("layer op (CUDA cores)");

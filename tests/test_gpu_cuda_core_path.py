@@ -24,6 +24,7 @@ CASES = [
     (dict(width=64, n_heads=4, head_dim=32, mlp_dim=64, action_dim=40, state_dim=33), 50, 3, 50, 1),
     (dict(rope_base=0.0), 1, 33, 8, 2),
     (dict(), 20, 7, 50, 1),                                                 # 64 x 64 tiles for gate/up
+    (dict(), 31, 7, 50, 1),                                                 # and for QKV and O
 ]
 
 
