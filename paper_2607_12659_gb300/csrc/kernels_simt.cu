@@ -1276,8 +1276,12 @@ jpi_status op_simt(jpi_handle* h, int op, int l, int step, int B, int C, cudaStr
             a.rope = h->rope_tab;
             return launch_rows_gemm<T, RK_QKV>(h, a, st);
         case 3: {
-            // Four heads per block once one head per block would be more than four blocks per SM.
-            const bool four = h->H % 4 == 0 && (long long)Mi * h->H > 4ll * h->num_sms;
+            // Four heads per block, each key read once for them: at head dims to 64 always, above once one
+            // head per block would be more than two blocks per SM, which then no longer run at once. One head and
+            // four per block, 832 keys, us: D = 64, 8 heads, 9 tokens 26.0 and 20.1, 51: 58.1 and 21.5; D = 160, 38
+            // tokens (304 blocks) 37.1 and 43.5, 51 (408) 64.0 and 44.4; D = 96, 304 and 408 blocks 39.2 and
+            // 34.7, 68.8 and 35.6 (32 keys, 304 blocks: 5.3 and 5.4).
+            const bool four = h->H % 4 == 0 && (h->D <= 64 || (long long)Mi * h->H > 2ll * h->num_sms);
             return four ? launch_attn_rows<T, 4>(h, (const T*)h->q, kst, vst, (T*)h->o, Mt, S, st)
                         : launch_attn_rows<T, 1>(h, (const T*)h->q, kst, vst, (T*)h->o, Mt, S, st);
         }
