@@ -1341,7 +1341,9 @@ bool pipe_ok(const jpi_corr_handle* h, const float* x, int ldx, const void* w, i
            ((uintptr_t)w & 15) == 0;
 }
 // Whether its LayerNorm form takes `rows` rows of the module's width: every CTA computes the rows'
-// statistics, up to two rows per warp (about the time of one; more would cost what the launch saved).
+// statistics, up to two rows per warp; more cost what the launch saved (predict, LayerNorm in the products and
+// in launches of its own, us: 12 rows 135.4 and 142.7, 16 rows 146.9 and 151.3, 20 rows 178.7 and 177.2, 24
+// rows 188.0 and 184.6).
 bool ln_fused(const jpi_corr_handle* h, const float* x, int ldx, const void* w, int rows) {
     return pipe_ok(h, x, ldx, w, h->d) && h->d <= 2048 && rows <= 16;
 }
@@ -1477,11 +1479,12 @@ jpi_status attention(const jpi_corr_handle* h, cudaStream_t st, const float* q, 
 jpi_status block(const jpi_corr_handle* h, cudaStream_t st, const BlockDev& w, float* x, int B, int n) {
     const int d = h->d, rows = B * n;
     JPI_TRY(ln_linear(h, st, x, w.ln1_w, w.ln1_b, h->u, w.wqkv, w.bqkv, h->qkv, rows, 3 * d, false));
-    // Attention among four tokens goes into the output product for one or two requests (every CTA
-    // computes it: more requests take longer there than in a launch of their own). Which kernels run
-    // must not show in a request's result, so both ways compute the same sums.
+    // Attention among four tokens goes into the output product for one request (every CTA computes it:
+    // more requests take longer there than in a launch of their own; predict, in the product and in its own
+    // launch, us: one request 92.1 and 92.8, two 108.2 and 102.6, three 144.8 and 135.5). Which kernels run must not
+    // show in a request's result, so both ways compute the same sums.
     const bool four = n == LP_XR && (h->Dh & (h->Dh - 1)) == 0 && d <= 2048 && pipe_ok(h, h->qkv, 3 * d, w.wo, d);
-    if (four && B <= 2) {
+    if (four && B == 1) {
         LinArgs a = lin_args(h->qkv, 3 * d, w.wo, w.bo, x, d, x, d, rows, d, d, false);
         a.att_heads_dh = h->Dh;
         a.att_scale = 1.f / sqrtf((float)h->Dh);
