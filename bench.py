@@ -36,7 +36,7 @@ OP_NAMES = {2: "norm+qkv+rope", 3: "attention", 4: "o_proj+residual", 5: "norm+g
 # DRAM bytes per launch from an ncu capture (dram__bytes_read.sum + dram__bytes_write.sum),
 # valid only while TRAFFIC_SOURCES hash to `source_sha256`.
 NCU_TRAFFIC = {
-    # profiles/layer_kernels_pi05_forward.md (layer 1 of one eager forward, batch 1, P 816).
+    # Layer 1 of one eager forward, batch 1, P 816.
     "norm+qkv+rope": {"bytes": 5489152, "source_sha256": "be8926c37a41dfe4"},
     "attention": {"bytes": 1165312, "source_sha256": "be8926c37a41dfe4"},
     "o_proj+residual": {"bytes": 4690944, "source_sha256": "be8926c37a41dfe4"},

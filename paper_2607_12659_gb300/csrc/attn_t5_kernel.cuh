@@ -32,10 +32,10 @@
 // Head dim 256 (QT): the query tile is the A operand from tensor memory instead of shared memory, where
 // its 64 KB make room for a third K and V slot. It lands in V slots 1 and 2, the softmax warps copy
 // their rows to TMEM columns 384.. (two bf16 a column), and V_1, V_2 follow. What bounds a block of 64
-// keys (33 of them per CTA at batch 64, prefix 2048; 70.7 us a launch with one softmax thread per row,
-// two slots and MMAs issued under `lane == 0`): the chain from scores through softmax to P V. Two
-// threads per row, single-thread issue the compiler knows of (ptx::elect_one, 72.1 -> 67.6 us) and the
-// third slot (67.6 -> 63.5 us) each shorten it; 17.6 -> 15.2 us at 16 requests and two key splits.
+// keys is the chain from scores through softmax to P V; at batch 64 and a prefix of 2048 (33 blocks per
+// CTA) the launch takes 62 us. Each of these shortens it: two softmax threads per row, single-thread issue
+// the compiler knows of (ptx::elect_one, 4.5 us), the third slot (4.1 us). The detour of the queries costs a
+// launch of one to three key blocks 0.2 to 0.8 us.
 // Key splits (gridDim.z = S > 1, the S CTAs of a row block forming a cluster along z): CTA s takes
 // the key blocks [s nb / S, (s + 1) nb / S). Past its key loop each CTA writes its rows'
 // unnormalised fp32 outputs and (m, l) to its slot of a workspace in global memory (row-fastest,

@@ -168,8 +168,9 @@ __global__ void __launch_bounds__(AT_THREADS) k_attn_tc(const __grid_constant__ 
     // before the first push (published by fence.mbarrier_init, so the arrival is relaxed).
     ptx::cluster_arrive_relaxed();
 
-    // K and V blocks by bulk tensor copies (one thread): D/64 column blocks of KB rows each. Rows past the split's last key are whatever the store holds there (finite:
-    // zero-initialised, or other requests' and layers' keys); their scores are masked.
+    // K and V blocks by bulk tensor copies (one thread): D/64 column blocks of KB rows each. Rows past
+    // the split's last key are whatever the store holds there (finite: zero-initialised, or other
+    // requests' and layers' keys); their scores are masked.
     const uint32_t qs_u = ptx::smem_u32(qs), ks_u = ptx::smem_u32(ks), vs_u = ptx::smem_u32(vs);
     const int kv_row_b = a.kv_row0 + b * a.kv_rows;      // this request's key 0 in the maps
     const uint64_t pol = ptx::l2_policy_evict_first();

@@ -274,10 +274,9 @@ __global__ void __launch_bounds__(256) k_corr_linear16(const LinArgs a) {
 // weight rows (contiguous) arrive by per-thread 16-byte cp.async copies into a ring of NST
 // stages, the first ones issued before the dependency wait (weights do not depend on the previous
 // kernel). Thread t takes the 8-column chunks t, t + 256, ... of the inputs for all LP_ROWS
-// features of a group, so each chunk of LP_XR activation rows it loads serves all of them (as
-// many activation bytes as weight bytes, where one warp per feature read LIN_ROWS activation
-// chunks per weight chunk and was bound by those L1 reads); the per-feature sums are reduced over
-// the block in a fixed order. No waits that can spin: the copies are waited with
+// features of a group, so each chunk of LP_XR activation rows it loads serves all of them: as
+// many activation bytes as weight bytes (one warp per feature reads LIN_ROWS activation chunks per
+// weight chunk, and those L1 reads bound it); the per-feature sums are reduced over the block in a fixed order. No waits that can spin: the copies are waited with
 // cp.async.wait_group.
 //
 // Forms that take a neighbouring kernel in, because at a handful of rows every launch of the chain
@@ -956,9 +955,8 @@ __global__ void __launch_bounds__(256) k_corr_softmax_sum(const float* __restric
 // (tid mod 128, tid / 128) takes columns 2 cg, 2 cg + 1 of the CTA's 256 and rows mg RH .. + RH - 1
 // (RH = 16 for M <= 32, else 32), token after token in order; the chunk's probabilities sit in
 // shared memory transposed ([token][row], read as 16-byte broadcasts) and each token's two values
-// come in one load, CORR_TB tokens' loads in flight together (a chunk of 64 tokens eight at a time
-// was eight L2 round trips in a row on 104 CTAs). The token chunks are added in order
-// by k_corr_wsum_reduce.
+// come in one load, CORR_TB tokens' loads in flight together: two L2 round trips a chunk, on 208 CTAs at one
+// request of 816 tokens. The token chunks are added in order by k_corr_wsum_reduce.
 constexpr int CORR_TCHUNK = 32;
 constexpr int CORR_TB = 16;     // tokens whose values a thread has in flight
 constexpr int CORR_PTS = CORR_MAX_M + 4;   // row stride of the transposed probabilities
@@ -1314,11 +1312,9 @@ jpi_status put_block(jpi_corr_handle* h, bool dev, BlockDev* out, const jpi_corr
 
 // Every kernel of a call is launched with programmatic dependent launch (each waits for its
 // predecessor at its start), so a kernel's launch overlaps the previous kernel's tail. The calls
-// enqueue their kernels on the caller's pointers: a graph of them, captured once per shape, needed
-// every input copied in and every output copied out, which took more of the GPU's time (10 us of 62 per
-// compress, 12 of 109 per predict at batch 1) than the host's 26 launches leave it idle (none: they
-// take the host less time than the kernels run). A failed launch leaves its error for the
-// cudaGetLastError check that follows.
+// enqueue their kernels on the caller's pointers: a captured graph needs every input copied in and every
+// output copied out (10 us of a compress and 12 of a predict at batch 1), and the host's 26 launches take less
+// time than the kernels run. A failed launch leaves its error for the cudaGetLastError check that follows.
 template <typename... KArgs, typename... Args>
 void pdl(cudaStream_t st, dim3 grid, dim3 block, size_t smem, void (*k)(KArgs...), Args&&... args) {
     cudaLaunchConfig_t cfg = {};

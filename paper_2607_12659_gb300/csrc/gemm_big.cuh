@@ -39,9 +39,8 @@ constexpr int BIG_YBYTES = BIG_NT * BIG_HS * 4;
 // tokens to residual rows it holds in registers and stores the results, with no staging tile and one
 // block barrier (for the CTA's own partials). The exchange buffers take shared memory from the ring,
 // which keeps 4 (S = 2) or 3 stages of 32 KB in flight. What bounds a unit at these sizes is the chain
-// from the accumulator to the stores: block barriers around whole-slice copies and a staging tile
-// took 1.1-2.3 us longer (us, before -> now: O 153 tokens 8.3 -> 7.2, 408: 9.3 -> 7.9, 816: 11.3 -> 9.0;
-// down 10.1 -> 9.2, 11.5 -> 10.2, 15.3 -> 12.9).
+// from the accumulator to the stores: O takes 7.2 us at 153 tokens, 7.9 at 408 and 9.0 at 816, down 9.2, 10.2 and
+// 12.9; whole-slice copies between block barriers and a staging tile add 1.1-2.3 us to each.
 template <int S>
 struct BigCfg {
     static constexpr int STAGES = S <= 2 ? 4 : 3;

@@ -119,8 +119,8 @@ __global__ void k_time_embed(float* temb, const double* __restrict__ period, int
 
 // Y[n][r] = act(sum_k W[r][k] X[n][k] + b[r]) for n < N <= GV_N, r < R: one warp per output row,
 // its first GV_U x 128 weights in registers before the dependency wait, X in shared memory (read as
-// 16-byte chunks, four consecutive k per lane). Launches of the time MLP are short chains: 1024 rows
-// x 1024 bf16 weights took 11 us with 2-byte weight loads issued after the inputs were staged.
+// 16-byte chunks, four consecutive k per lane). Launches of the time MLP are short chains; weight loads of 2
+// bytes issued after the inputs are staged make 1024 rows x 1024 bf16 weights an 11 us one.
 // The modulation vectors (no swish) are read by kernels before their own dependency wait: that
 // launch does not release its dependent early.
 constexpr int GV_N = 16, GV_U = 8;
@@ -717,9 +717,8 @@ __global__ void k_qkv_post(const float* __restrict__ qkv, TQ* __restrict__ q,
 // Warp w takes keys 4 w .. 4 w + 3, then + 32, ..: four keys' rows in flight at a time, the D products
 // spread over the lanes (d = lane + 32 j, j < ND), one online softmax per head and warp; the eight
 // warps' (max, sum, output) are combined in warp order through shared memory. HB = 4 reads each key
-// once for four heads; HB = 1 spreads a small batch over four times the blocks. Measured against a
-// block per token with a warp per head and the keys staged 32 at a time: a 9-token request
-// 29 -> 6 us; 408 tokens x 8 heads x 867 keys (D = 256) 456 -> 278 us.
+// once for four heads; HB = 1 spreads a small batch over four times the blocks (the launcher has the
+// line). Bound by the loads of the keys, 32 in flight a block: 408 tokens x 8 heads x 867 keys (D = 256) 280 us.
 constexpr int AR_WARPS = 8;
 
 template <typename T, int HB, int ND>
@@ -1041,9 +1040,8 @@ __global__ void __launch_bounds__(FIN_THREADS) k_final_rows(const FinalArgs a) {
 // Prefix KV into the store, every layer's K and V in one launch: tensor y (K then V of layer y / 2)
 // src [batch][P][D] (fp32 or bf16) -> dst [batch][kv_rows][D]. A request's P D elements are
 // contiguous on both sides; a thread moves KV_CH chunks of 8 elements (16 bytes of bf16), all loads
-// before the stores. Bound by launches before (one kernel of 2-byte accesses per tensor: 36 launches
-// of 4.4 us each for 15 MB at 18 layers x 816 tokens); the copy alone is 30 MB of traffic, 4.4 us at
-// the copy peak. VEC: the sources are 16-byte aligned.
+// before the stores. One launch, because a launch of its own takes each of 36 tensors 4.4 us (18 layers x
+// 816 tokens), as long as the whole copy of 30 MB at the copy peak. VEC: the sources are 16-byte aligned.
 constexpr int KV_CH = 4;
 constexpr int KV_MAX_TENSORS = 128;
 struct KvLoadArgs {

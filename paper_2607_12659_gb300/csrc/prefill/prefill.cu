@@ -387,10 +387,10 @@ struct LayerW {
 //   warp 1  one thread issues the tcgen05.mma chain (M = 128, N = 256, K = 16 each) into one of two
 //           TMEM accumulators and releases each stage through tcgen05.commit;
 //   warps 2-9  one TMEM lane (X row m) per thread, two groups of four warps with half of the columns
-//           each. Every warp passes its 32 rows through 4 KB of shared memory of its own, 128 bytes of a row at a time (16-byte chunks XOR-swizzled by the
-//           row), and writes 128-byte pieces of four rows per instruction (a row per thread, each
-//           store touched 32 lines). The QKV form applies the rotary coding there and scatters q, k
-//           and v, which replaced an fp32 round trip through memory and a kernel of its own.
+//           each. Every warp passes its 32 rows through 4 KB of shared memory of its own, 128 bytes of
+//           a row at a time (16-byte chunks XOR-swizzled by the row), and writes 128-byte pieces of four
+//           rows per instruction (a row per thread, each store would touch 32 lines). The QKV form applies
+//           the rotary coding there and scatters q, k and v.
 // Stream-K (args.stream): a product with fewer tiles than SMs deals its (tile, k-block) units out
 // evenly, CTA c taking [c T / G, (c + 1) T / G); each piece of a tile goes to its own partial buffer
 // (piece p of a tile: the p-th CTA that touches it), and the consumer adds a tile's pieces in order.
@@ -906,7 +906,9 @@ jpi_status row_gemm(jpi_prefill_handle* h, cudaStream_t st, const __nv_bfloat16*
 // cuts across tiles writes a piece for each, worth about PG_PIECE_KB k-blocks, so the choice is between
 // every SM (each CTA two pieces) and the whole number of CTAs per tile that fits (one piece): at
 // Gemma-2B sizes and 816 tokens (56 tiles) down (256 k-blocks a tile) takes 152 CTAs of 94.3 k-blocks,
-// O (32) 112 of 16.
+// O (32) 112 of 16. Measured, whole tiles, every SM, whole CTAs per tile, us a layer: 8 tiles 167, 98, 98; 56: 230,
+// 191, 191 (as chosen 188); 96: 305, 294, 306; 112: 334, 335, 337 (331); 128: 374, 386, 376; at width 1024 28
+// tiles 88, 81, 77; 72: 123, 125, 122; 112: 173, 188, 173 (180).
 constexpr int PG_PIECE_KB = 8;
 int stream_grid(int num_sms, int M, int N, int K) {
     const long long tiles = (long long)((N + PG_TN - 1) / PG_TN) * ((M + PG_TM - 1) / PG_TM);
