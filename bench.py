@@ -37,11 +37,11 @@ OP_NAMES = {2: "norm+qkv+rope", 3: "attention", 4: "o_proj+residual", 5: "norm+g
 # valid only while TRAFFIC_SOURCES hash to `source_sha256`.
 NCU_TRAFFIC = {
     # Layer 1 of one eager forward, batch 1, P 816.
-    "norm+qkv+rope": {"bytes": 5489152, "source_sha256": "be8926c37a41dfe4"},
-    "attention": {"bytes": 1165312, "source_sha256": "be8926c37a41dfe4"},
-    "o_proj+residual": {"bytes": 4690944, "source_sha256": "be8926c37a41dfe4"},
-    "norm+gate_up+geglu": {"bytes": 16957696, "source_sha256": "be8926c37a41dfe4"},
-    "down_proj+residual": {"bytes": 9127168, "source_sha256": "be8926c37a41dfe4"},
+    "norm+qkv+rope": {"bytes": 5490176, "source_sha256": "552aefb2d4113450"},
+    "attention": {"bytes": 1165824, "source_sha256": "552aefb2d4113450"},
+    "o_proj+residual": {"bytes": 4691200, "source_sha256": "552aefb2d4113450"},
+    "norm+gate_up+geglu": {"bytes": 16958720, "source_sha256": "552aefb2d4113450"},
+    "down_proj+residual": {"bytes": 9127424, "source_sha256": "552aefb2d4113450"},
 }
 
 
