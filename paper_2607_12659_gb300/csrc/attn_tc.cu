@@ -243,9 +243,7 @@ __global__ void __launch_bounds__(AT_THREADS) k_attn_tc(const __grid_constant__ 
         if (key0 == k_begin) landed = ptx::mbar_wait_bounded(qbar, 0, 200ull * 1000 * 1000) && landed;
         if (!landed && tid == 0) {
             atomicCAS(a.err, 0, (int)DEV_TIMEOUT_WEIGHTS);
-            // Nothing may land in this CTA's shared memory once it has exited.
-            (void)ptx::mbar_wait_bounded(&kvbar[bi], par, 200ull * 1000 * 1000);
-            (void)ptx::mbar_wait_bounded(qbar, 0, 200ull * 1000 * 1000);
+            ptx::drain_two(&kvbar[bi], par, qbar, 0, 200ull * 1000 * 1000);
         }
         const uint32_t kbuf_u = ks_u + bi * KV_BUF, vbuf_u = vs_u + bi * KV_BUF;
 

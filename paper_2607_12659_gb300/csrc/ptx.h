@@ -63,6 +63,14 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
     }
 }
 
+// A second bounded wait for two copies whose first one gave up, before the CTA exits (nothing may land in
+// its shared memory after that). Not inlined: it stays out of the way of the loop it is called from.
+static __device__ __noinline__ void drain_two(uint64_t* bar0, uint32_t par0, uint64_t* bar1, uint32_t par1,
+                                              uint64_t limit_ns) {
+    (void)mbar_wait_bounded(bar0, par0, limit_ns);
+    (void)mbar_wait_bounded(bar1, par1, limit_ns);
+}
+
 // Waits (bounded) for the last copy into each of a ring's `stages` stages, `issued` copies having gone
 // round it: copy i completes phase i / stages of full[i mod stages]. Nothing may land in a CTA's shared
 // memory once it has exited, so the thread that issued the copies calls this before it leaves its role,

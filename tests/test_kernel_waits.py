@@ -55,7 +55,7 @@ def test_single_shot_loads_are_waited_for_again_after_a_wait_gave_up():
     assert "mbar_wait_bounded(&bars[0]," in gave_up and "mbar_wait_bounded(&bars[1]," in gave_up
     attn = _source("attn_tc.cu")
     gave_up = attn[attn.index("if (!landed && tid == 0) {"):attn.index("const uint32_t kbuf_u")]
-    assert "mbar_wait_bounded(&kvbar[bi]," in gave_up and "mbar_wait_bounded(qbar," in gave_up
+    assert "drain_two(&kvbar[bi], par, qbar, 0," in gave_up
 
 
 def test_device_errors_are_reported_after_the_last_barrier():
