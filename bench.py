@@ -37,11 +37,11 @@ OP_NAMES = {2: "norm+qkv+rope", 3: "attention", 4: "o_proj+residual", 5: "norm+g
 # valid only while TRAFFIC_SOURCES hash to `source_sha256`.
 NCU_TRAFFIC = {
     # Layer 1 of one eager forward, batch 1, P 816.
-    "norm+qkv+rope": {"bytes": 5490176, "source_sha256": "552aefb2d4113450"},
-    "attention": {"bytes": 1165824, "source_sha256": "552aefb2d4113450"},
-    "o_proj+residual": {"bytes": 4691200, "source_sha256": "552aefb2d4113450"},
-    "norm+gate_up+geglu": {"bytes": 16958720, "source_sha256": "552aefb2d4113450"},
-    "down_proj+residual": {"bytes": 9127424, "source_sha256": "552aefb2d4113450"},
+    "norm+qkv+rope": {"bytes": 5489920, "source_sha256": "985e1d582c9b2a1e"},
+    "attention": {"bytes": 1166848, "source_sha256": "985e1d582c9b2a1e"},
+    "o_proj+residual": {"bytes": 4691712, "source_sha256": "985e1d582c9b2a1e"},
+    "norm+gate_up+geglu": {"bytes": 16958464, "source_sha256": "985e1d582c9b2a1e"},
+    "down_proj+residual": {"bytes": 9127680, "source_sha256": "985e1d582c9b2a1e"},
 }
 
 

@@ -64,7 +64,8 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
 }
 
 // A second bounded wait for two copies whose first one gave up, before the CTA exits (nothing may land in
-// its shared memory after that). Not inlined: it stays out of the way of the loop it is called from.
+// its shared memory after that). Not inlined: no working run reaches it, yet beside the split-KV attention's key
+// loop it cost the one-request pass of the pi0.5 expert 0.2% (4891 us inlined, 4873 out of line).
 static __device__ __noinline__ void drain_two(uint64_t* bar0, uint32_t par0, uint64_t* bar1, uint32_t par1,
                                               uint64_t limit_ns) {
     (void)mbar_wait_bounded(bar0, par0, limit_ns);
